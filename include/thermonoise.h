@@ -140,17 +140,18 @@ tn_status tn_apply_operator(tn_ctx *ctx, int precision, const void *u_dev, void 
 
 /* Autotuning of the FP32 operator kernel (the element-wise apply of
  * Eq. (dg_residuals)).  Two builds of it differ only in the resident CTAs
- * per SM asked of the register allocator: variant 0 gives every thread the
- * registers the code needs, variant 1 one CTA more per SM with fewer
- * registers per thread.  They execute the same arithmetic in the same
- * order, so results are bit-identical.  The first tn_apply_operator
- * (TN_F32) or mixed-mode tn_solve after a mesh or batch is built times both
- * for every degree present (3 + 10 launches of each, CUDA events on the
+ * per SM asked of the register allocator: variant 0 three CTAs of 256
+ * threads, variant 1 two, with more registers per thread.  They execute the
+ * same arithmetic in the same order, so results are bit-identical (a mesh or
+ * batch of few elements runs a third form, bit-identical too, whatever the
+ * variant).  The first tn_apply_operator (TN_F32) or mixed-mode tn_solve after
+ * a mesh or batch is built times both for every degree present (3 + 10 applies
+ * of each, CUDA events on the
  * stream of the call, not while it is being captured; the call's y, or the
  * solver's FP32 workspace, is overwritten meanwhile) and keeps variant 1
  * only when it is faster by more than 2 %.
  * tn_apply_tuning: variant[p - 2] for p = 2..8 is 0 or 1 once settled, -1
- * before; us (may be NULL) receives 14 doubles, the time per launch in
+ * before; us (may be NULL) receives 14 doubles, the time per apply in
  * microseconds of variants 0 and 1 for each degree (0 where not timed).
  * tn_set_apply_variant fixes the variant of one degree (0 or 1; the
  * autotuner then leaves it alone) or, with -1, lets it be timed again.

@@ -14,7 +14,9 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libthermonoise.so")
-SOURCES = ["kernels.cu", "precond.cu", "solver.cu", "capi.cu", "peak.cu", "mesh.cpp"]
+SOURCES = ["apply.cu", "kernels.cu", "precond.cu", "solver.cu", "capi.cu", "peak.cu", "mesh.cpp"]
+# the operator's kernels round alike in all their forms: fused operations are written out there
+NO_CONTRACT = ["apply.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -29,6 +31,8 @@ def _compile(src, verbose_ptxas=False):
     obj = os.path.join(BUILD, os.path.basename(src) + ".o")
     cmd = [nvcc(), "-c", os.path.join(CSRC, src), "-o", obj, "-O3", "-std=c++17", "-lineinfo",
            "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"] + ARCH
+    if src in NO_CONTRACT:
+        cmd.append("-fmad=false")
     if src.endswith(".cpp"):
         cmd = [nvcc(), "-c", "-x", "c++", os.path.join(CSRC, src), "-o", obj, "-O3", "-std=c++17",
                "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"]

@@ -49,11 +49,9 @@ void dfree(T *&p) {
 struct BatchInst {
   tn::HostMesh hm;
   DevMesh dm{};
-  double *colgeo = nullptr, *slabgeo = nullptr, *layer_c = nullptr;
-  float *colgeo32 = nullptr, *slabgeo32 = nullptr, *layer_c32 = nullptr;
-  int *colnb = nullptr, *colnbf = nullptr, *slab_layer = nullptr;
+  unsigned char *tables = nullptr;  // every mesh and material table, one block
   double r0 = 1.0, F0 = 1.0;
-  long long dof_off = 0, fac_off = 0;
+  long long dof_off = 0, fac_off = 0, tr_off = 0;
   int layer_off = 0;
   bool set = false;
   std::vector<double> slab_z;
@@ -67,10 +65,58 @@ struct Batch {
   long long ndof = 0, nfac = 0;
   int n_layers = 0, n_elems = 0;
   DevMesh *d_meshes = nullptr;
-  long long *d_dof_off = nullptr, *d_fac_off = nullptr;
+  long long *d_dof_off = nullptr, *d_fac_off = nullptr, *d_tr_off = nullptr;
   int2 *d_work = nullptr, *d_lines = nullptr;
+  int4 *d_ctas = nullptr;  // CTAs of the operator's two launches
   OpSys sys;
   int2 *h_work = nullptr;  // (instance, element) in the order of the apply partials
+};
+
+// host tables gathered into one block, for one allocation and one copy
+struct TablePack {
+  std::vector<unsigned char> host;
+  size_t add(const void *src, size_t bytes) {  // offset of the copy (256-byte aligned)
+    const size_t off = (host.size() + 255) / 256 * 256;
+    host.resize(off + bytes);
+    std::memcpy(host.data() + off, src, bytes);
+    return off;
+  }
+  size_t add32(const double *src, size_t n) {  // rounded to FP32
+    const size_t off = (host.size() + 255) / 256 * 256;
+    host.resize(off + n * sizeof(float));
+    float *d = reinterpret_cast<float *>(host.data() + off);
+    for (size_t i = 0; i < n; ++i) d[i] = (float)src[i];
+    return off;
+  }
+  cudaError_t upload(unsigned char **dev) const {
+    cudaError_t e = cudaMalloc((void **)dev, host.size());
+    if (e == cudaSuccess) e = cudaMemcpy(*dev, host.data(), host.size(), cudaMemcpyHostToDevice);
+    return e;
+  }
+};
+
+// the tables of a mesh and their places in the block
+struct MeshTables {
+  size_t cg, sg, cg32, sg32, nb, nbf, sl;
+  void pack(TablePack &p, const tn::HostMesh &hm) {
+    const size_t ncg = (size_t)hm.ncol * CG_NF * hm.N * hm.N, nsg = (size_t)hm.nslab * SG_NF * hm.N;
+    cg = p.add(hm.colgeo, sizeof(double) * ncg);
+    sg = p.add(hm.slabgeo, sizeof(double) * nsg);
+    cg32 = p.add32(hm.colgeo, ncg);
+    sg32 = p.add32(hm.slabgeo, nsg);
+    nb = p.add(hm.colnb, sizeof(int) * 4 * hm.ncol);
+    nbf = p.add(hm.colnbf, sizeof(int) * 4 * hm.ncol);
+    sl = p.add(hm.slab_layer, sizeof(int) * hm.nslab);
+  }
+  void point(DevMesh &m, const unsigned char *dev) const {
+    m.colgeo = (const double *)(dev + cg);
+    m.slabgeo = (const double *)(dev + sg);
+    m.colgeo32 = (const float *)(dev + cg32);
+    m.slabgeo32 = (const float *)(dev + sg32);
+    m.colnb = (const int *)(dev + nb);
+    m.colnbf = (const int *)(dev + nbf);
+    m.slab_layer = (const int *)(dev + sl);
+  }
 };
 
 struct tn_ctx {
@@ -82,13 +128,17 @@ struct tn_ctx {
   tn::HostMesh hm;
   bool have_mesh = false, have_mat = false, have_beam = false;
   DevMesh dm{};
-  double *d_colgeo = nullptr, *d_slabgeo = nullptr, *d_layer_c = nullptr;
-  int *d_colnb = nullptr, *d_colnbf = nullptr, *d_slab_layer = nullptr;
-  float *d_colgeo32 = nullptr, *d_slabgeo32 = nullptr, *d_layer_c32 = nullptr;
+  unsigned char *d_tables = nullptr;  // every mesh table, one block
+  double *d_layer_c = nullptr;
+  float *d_layer_c32 = nullptr;
   double *slab_z_host = nullptr;
   int *slab_log_host = nullptr;
   double r0 = 1.0, F0 = 1.0;
   size_t ndof = 0;
+  // traction scratch of the operator: allocated by the first apply in the
+  // precision asked for (an FP64 one serves FP32 applies too)
+  void *trace = nullptr;
+  size_t trace_entries = 0, trace_bytes = 0;
   // workspace
   size_t ws_ndof = 0;
   double *b64 = nullptr, *diag64 = nullptr, *dinv64 = nullptr, *r64 = nullptr, *z64 = nullptr,
@@ -186,13 +236,9 @@ static void reset_tuning(tn_ctx *c) {
 static void free_mesh(tn_ctx *c) {
   free_precond(c);
   reset_tuning(c);
-  dfree(c->d_colgeo);
-  dfree(c->d_slabgeo);
-  dfree(c->d_colnb);
-  dfree(c->d_colnbf);
-  dfree(c->d_slab_layer);
-  dfree(c->d_colgeo32);
-  dfree(c->d_slabgeo32);
+  dfree(c->d_tables);
+  dfree(c->trace);
+  c->trace_bytes = 0;
   tn::free_host_mesh(&c->hm);
   std::free(c->slab_z_host);
   std::free(c->slab_log_host);
@@ -245,6 +291,21 @@ static tn_status ensure_ws(tn_ctx *c) {
   c->ws_ndof = n;
   c->ws_E = E;
   c->ws_layers = NL;
+  return TN_OK;
+}
+
+static tn_status ensure_trace(tn_ctx *c, int prec) {
+  const size_t bytes = c->trace_entries * (prec == TN_F64 ? sizeof(double) : sizeof(float));
+  if (c->trace_bytes >= bytes) return TN_OK;
+  dfree(c->trace);
+  c->trace_bytes = 0;
+  const cudaError_t e = cudaMalloc(&c->trace, bytes);
+  if (e != cudaSuccess) {
+    c->trace = nullptr;
+    cudaGetLastError();
+    return fail(TN_ENOMEM, "traction scratch of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
+  }
+  c->trace_bytes = bytes;
   return TN_OK;
 }
 
@@ -489,12 +550,11 @@ static void free_batch(tn_ctx *c) {
   if (!b) return;
   for (int i = 0; i < b->n; ++i) {
     BatchInst &q = b->inst[i];
-    dfree(q.colgeo); dfree(q.slabgeo); dfree(q.layer_c); dfree(q.colgeo32); dfree(q.slabgeo32);
-    dfree(q.layer_c32); dfree(q.colnb); dfree(q.colnbf); dfree(q.slab_layer);
+    dfree(q.tables);
     tn::free_host_mesh(&q.hm);
   }
   delete[] b->inst;
-  dfree(b->d_meshes); dfree(b->d_dof_off); dfree(b->d_fac_off); dfree(b->d_work); dfree(b->d_lines);
+  dfree(b->d_meshes); dfree(b->d_dof_off); dfree(b->d_fac_off); dfree(b->d_tr_off); dfree(b->d_work); dfree(b->d_lines); dfree(b->d_ctas);
   delete[] b->h_work;
   delete b;
   c->batch = nullptr;
@@ -510,33 +570,27 @@ static OpSys make_sys(const tn_ctx *c) {
   } else {
     s.m = &c->dm;
     s.mvar = c->apply_var[c->dm.N];
-    s.n_apply_parts = c->dm.E;
+    s.n_elems = c->dm.E;
     s.n_rz_parts = tn_zline_partials(c->dm);
   }
   s.zerr = c->wctl;
+  s.trace = c->trace;
   return s;
 }
 
 // Autotuner of the FP32 operator kernel: for every LGL count of the context
 // (the mesh, or each degree group of a batch) not yet settled, times both
 // occupancy variants on the vectors u -> y (y is overwritten) and keeps
-// variant 1 only when it is faster by more than 2 %.  Nothing is timed while
-// st is being captured into a graph.
+// variant 1 only when it is faster by more than 2 %.  Not called while st is
+// being captured into a graph.
 static tn_status ensure_tuned(tn_ctx *c, const float *u, float *y, cudaStream_t st) {
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  CU_TRY(cudaStreamIsCapturing(st, &cs), "capture status");
-  if (cs != cudaStreamCaptureStatusNone) return TN_OK;
-  const bool batch = is_batch(c);
   const OpSys s = make_sys(c);
-  const int ng = batch ? s.ngroups : 1;
-  for (int g = 0; g < ng; ++g) {
-    const int N = batch ? s.gN[g] : c->dm.N;
-    if (N < 3 || N > 9 || c->apply_set[N]) continue;
+  for (int g = 0; g < (s.m ? 1 : s.ngroups); ++g) {
+    const ApplyArgs a = s.args(g, g + 1, TN_F32, u, y);
+    const int N = s.m ? s.m->N : s.gN[g];
+    if (c->apply_set[N]) continue;
     float us[2] = {0.0f, 0.0f};
-    if (batch)
-      CU_TRY(tn_tune_apply(nullptr, N, s.meshes, s.gwork[g], s.gcount[g], s.dof_off, u, y, st, us), "tuning");
-    else
-      CU_TRY(tn_tune_apply(&c->dm, N, nullptr, nullptr, 0, nullptr, u, y, st, us), "tuning");
+    CU_TRY(tn_tune_apply(a, st, us), "tuning");
     c->apply_us[N][0] = us[0];
     c->apply_us[N][1] = us[1];
     c->apply_var[N] = us[1] < 0.98f * us[0] ? 1 : 0;
@@ -605,6 +659,7 @@ tn_status tn_create(tn_ctx **out, int device, void *cuda_stream) {
       std::memcpy(tabs.D[N], D, sizeof(double) * N * N);
     }
     e = tn_upload_lgl(&tabs);
+    if (e == cudaSuccess) e = tn_upload_lgl_apply(&tabs);
     if (e == cudaSuccess) e = tn_upload_lgl_precond(&tabs);
   }
   if (e != cudaSuccess) {
@@ -646,31 +701,10 @@ tn_status tn_build_mesh(tn_ctx *c, const tn_mesh_desc *d) {
   dfree(c->d_layer_c32);
   c->have_mat = false;
   c->hm = hm;
-  const int N2 = hm.N * hm.N;
-  cudaError_t e = cudaSuccess;
-  auto up = [&](void **dst, const void *src, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(dst, bytes);
-    if (e == cudaSuccess) e = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
-  };
-  up((void **)&c->d_colgeo, hm.colgeo, sizeof(double) * (size_t)hm.ncol * CG_NF * N2);
-  up((void **)&c->d_slabgeo, hm.slabgeo, sizeof(double) * (size_t)hm.nslab * SG_NF * hm.N);
-  up((void **)&c->d_colnb, hm.colnb, sizeof(int) * 4 * hm.ncol);
-  up((void **)&c->d_colnbf, hm.colnbf, sizeof(int) * 4 * hm.ncol);
-  up((void **)&c->d_slab_layer, hm.slab_layer, sizeof(int) * hm.nslab);
-  {
-    const size_t ncg = (size_t)hm.ncol * CG_NF * N2, nsg = (size_t)hm.nslab * SG_NF * hm.N;
-    float *f32 = (float *)std::malloc(sizeof(float) * (ncg > nsg ? ncg : nsg));
-    if (!f32) e = cudaErrorMemoryAllocation;
-    if (e == cudaSuccess) {
-      for (size_t q = 0; q < ncg; ++q) f32[q] = (float)hm.colgeo[q];
-      up((void **)&c->d_colgeo32, f32, sizeof(float) * ncg);
-    }
-    if (e == cudaSuccess) {
-      for (size_t q = 0; q < nsg; ++q) f32[q] = (float)hm.slabgeo[q];
-      up((void **)&c->d_slabgeo32, f32, sizeof(float) * nsg);
-    }
-    std::free(f32);
-  }
+  TablePack pack;
+  MeshTables tab;
+  tab.pack(pack, hm);
+  const cudaError_t e = pack.upload(&c->d_tables);
   if (e != cudaSuccess) {
     free_mesh(c);
     return cuda_fail(e, "uploading the mesh");
@@ -686,9 +720,10 @@ tn_status tn_build_mesh(tn_ctx *c, const tn_mesh_desc *d) {
   DevMesh &m = c->dm;
   m.N = hm.N; m.p = hm.p; m.E = hm.E; m.ncol = hm.ncol; m.nslab = hm.nslab; m.n_layers = hm.n_layers;
   m.bc_side = hm.bc_side; m.bc_bottom = hm.bc_bottom; m.penC = hm.penC;
-  m.colgeo = c->d_colgeo; m.slabgeo = c->d_slabgeo; m.colnb = c->d_colnb; m.colnbf = c->d_colnbf;
-  m.slab_layer = c->d_slab_layer; m.layer_c = nullptr;
-  m.colgeo32 = c->d_colgeo32; m.slabgeo32 = c->d_slabgeo32; m.layer_c32 = nullptr;
+  tab.point(m, c->d_tables);
+  m.layer_c = nullptr;
+  m.layer_c32 = nullptr;
+  c->trace_entries = (size_t)tn_trace_entries(hm.N) * hm.E;
   m.penC32 = (float)hm.penC;
   c->ndof = (size_t)3 * hm.N * hm.N * hm.N * hm.E;
   c->have_mesh = true;
@@ -787,12 +822,14 @@ tn_status tn_set_beam(tn_ctx *c, double r0, double F0) {
 
 static tn_status batch_finalize(tn_ctx *c) {
   Batch *b = c->batch;
-  long long dof = 0, fac = 0;
+  long long dof = 0, fac = 0, tre = 0;
   int lay = 0, elems = 0;
   for (int i = 0; i < b->n; ++i) {
     BatchInst &q = b->inst[i];
     q.dof_off = dof;
     q.fac_off = fac;
+    q.tr_off = tre;
+    tre += tn_trace_entries(q.hm.N) * q.hm.E;
     q.layer_off = lay;
     const long long M = 3LL * q.hm.N;
     dof += 3LL * q.hm.N * q.hm.N * q.hm.N * q.hm.E;
@@ -803,9 +840,11 @@ static tn_status batch_finalize(tn_ctx *c) {
   }
   b->ndof = dof; b->nfac = fac; b->n_layers = lay; b->n_elems = elems;
   std::vector<int2> work, lines;
+  std::vector<int4> ctas, adds;
   OpSys &s = b->sys;
   s = OpSys();
   int rz = 0;
+  const bool few = tn_apply_few(elems);
   for (int N = TN_MIN_N; N <= TN_MAX_N; ++N) {
     const int w0 = (int)work.size(), l0 = (int)lines.size();
     for (int i = 0; i < b->n; ++i) {
@@ -816,6 +855,13 @@ static tn_status batch_finalize(tn_ctx *c) {
     }
     if ((int)work.size() == w0) continue;
     const int g = s.ngroups++;
+    auto split = [&](std::vector<int4> &v, int eb) {
+      for (int w = w0; w < (int)work.size(); w += eb)
+        v.push_back(make_int4(N, w, std::min(eb, (int)work.size() - w), 0));
+      return (int)v.size();
+    };
+    s.gcta[g + 1] = split(ctas, tn_apply_eb(N, few));
+    s.gadd[g + 1] = split(adds, tn_trace_add_eb(N));
     s.gN[g] = N;
     s.gcount[g] = (int)work.size() - w0;
     s.gpart_off[g] = w0;
@@ -826,8 +872,8 @@ static tn_status batch_finalize(tn_ctx *c) {
     s.gline[g] = reinterpret_cast<const int2 *>((size_t)l0);
   }
   std::vector<DevMesh> dms(b->n);
-  std::vector<long long> doff(b->n + 1), foff(b->n);
-  for (int i = 0; i < b->n; ++i) { dms[i] = b->inst[i].dm; doff[i] = b->inst[i].dof_off; foff[i] = b->inst[i].fac_off; }
+  std::vector<long long> doff(b->n + 1), foff(b->n), toff(b->n);
+  for (int i = 0; i < b->n; ++i) { dms[i] = b->inst[i].dm; doff[i] = b->inst[i].dof_off; foff[i] = b->inst[i].fac_off; toff[i] = b->inst[i].tr_off; }
   doff[b->n] = b->ndof;  // the last entry closes the last mirror (per-mirror norms)
   cudaError_t e = cudaSuccess;
   auto up = [&](void **dst, const void *src, size_t bytes) {
@@ -837,7 +883,12 @@ static tn_status batch_finalize(tn_ctx *c) {
   up((void **)&b->d_meshes, dms.data(), sizeof(DevMesh) * b->n);
   up((void **)&b->d_dof_off, doff.data(), sizeof(long long) * (b->n + 1));
   up((void **)&b->d_fac_off, foff.data(), sizeof(long long) * b->n);
+  up((void **)&b->d_tr_off, toff.data(), sizeof(long long) * b->n);
+  c->trace_entries = (size_t)tre;
   up((void **)&b->d_work, work.data(), sizeof(int2) * work.size());
+  const int nctas = (int)ctas.size();
+  ctas.insert(ctas.end(), adds.begin(), adds.end());
+  up((void **)&b->d_ctas, ctas.data(), sizeof(int4) * ctas.size());
   up((void **)&b->d_lines, lines.data(), sizeof(int2) * lines.size());
   if (e != cudaSuccess) return cuda_fail(e, "uploading the batch");
   for (int g = 0; g < s.ngroups; ++g) {
@@ -845,9 +896,13 @@ static tn_status batch_finalize(tn_ctx *c) {
     s.gline[g] = b->d_lines + (size_t)s.gline[g];
   }
   s.meshes = b->d_meshes;
+  s.work = b->d_work;
+  s.ctas = b->d_ctas;
+  s.adds = b->d_ctas + nctas;
   s.dof_off = b->d_dof_off;
   s.fac_off = b->d_fac_off;
-  s.n_apply_parts = elems;
+  s.tr_off = b->d_tr_off;
+  s.n_elems = elems;
   s.n_rz_parts = rz;
   b->h_work = new (std::nothrow) int2[work.size()];
   if (!b->h_work) return fail(TN_ENOMEM, "host allocation failed");
@@ -894,33 +949,21 @@ tn_status tn_batch_set(tn_ctx *c, int i, const tn_mesh_desc *d, int n_mat, const
   if (n_mat != hm.n_layers) { tn::free_host_mesh(&hm); return fail(TN_EINVAL, "instance %d: %d materials for %d layers", i, n_mat, hm.n_layers); }
   std::vector<double> h(3 * n_mat);
   if (!material_table(n_mat, mats, h.data(), msg, sizeof(msg))) { tn::free_host_mesh(&hm); return fail(TN_EINVAL, "instance %d: %s", i, msg); }
-  std::vector<float> h32(h.begin(), h.end());
   CU_TRY(cudaSetDevice(c->device), "cudaSetDevice");
   BatchInst &q = b->inst[i];
   q.hm = hm;
-  const int N2 = hm.N * hm.N;
-  const size_t ncg = (size_t)hm.ncol * CG_NF * N2, nsg = (size_t)hm.nslab * SG_NF * hm.N;
-  std::vector<float> cg32(hm.colgeo, hm.colgeo + ncg), sg32(hm.slabgeo, hm.slabgeo + nsg);
-  cudaError_t e = cudaSuccess;
-  auto up = [&](void **dst, const void *src, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(dst, bytes);
-    if (e == cudaSuccess) e = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
-  };
-  up((void **)&q.colgeo, hm.colgeo, sizeof(double) * ncg);
-  up((void **)&q.slabgeo, hm.slabgeo, sizeof(double) * nsg);
-  up((void **)&q.colgeo32, cg32.data(), sizeof(float) * ncg);
-  up((void **)&q.slabgeo32, sg32.data(), sizeof(float) * nsg);
-  up((void **)&q.colnb, hm.colnb, sizeof(int) * 4 * hm.ncol);
-  up((void **)&q.colnbf, hm.colnbf, sizeof(int) * 4 * hm.ncol);
-  up((void **)&q.slab_layer, hm.slab_layer, sizeof(int) * hm.nslab);
-  up((void **)&q.layer_c, h.data(), sizeof(double) * h.size());
-  up((void **)&q.layer_c32, h32.data(), sizeof(float) * h32.size());
+  TablePack pack;
+  MeshTables tab;
+  tab.pack(pack, hm);
+  const size_t lc = pack.add(h.data(), sizeof(double) * h.size()), lc32 = pack.add32(h.data(), h.size());
+  const cudaError_t e = pack.upload(&q.tables);
   if (e != cudaSuccess) return cuda_fail(e, "uploading a batch instance");
   DevMesh &m = q.dm;
   m.N = hm.N; m.p = hm.p; m.E = hm.E; m.ncol = hm.ncol; m.nslab = hm.nslab; m.n_layers = hm.n_layers;
   m.bc_side = hm.bc_side; m.bc_bottom = hm.bc_bottom; m.penC = hm.penC; m.penC32 = (float)hm.penC;
-  m.colgeo = q.colgeo; m.slabgeo = q.slabgeo; m.colnb = q.colnb; m.colnbf = q.colnbf; m.slab_layer = q.slab_layer;
-  m.layer_c = q.layer_c; m.colgeo32 = q.colgeo32; m.slabgeo32 = q.slabgeo32; m.layer_c32 = q.layer_c32;
+  tab.point(m, q.tables);
+  m.layer_c = (const double *)(q.tables + lc);
+  m.layer_c32 = (const float *)(q.tables + lc32);
   q.r0 = r0;
   q.F0 = F0;
   q.slab_z.assign(d->slab_z, d->slab_z + hm.nslab + 1);
@@ -960,6 +1003,18 @@ tn_status tn_apply_operator(tn_ctx *c, int precision, const void *u, void *y) {
   const char *a = (const char *)u, *b = (const char *)y;
   const size_t bytes = c->ndof * es;
   if (a < b + bytes && b < a + bytes) return fail(TN_EINVAL, "u and y overlap");
+  // a captured apply gets a traction scratch of its own, owned by the graph,
+  // so that a replay may overlap other work of the context
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  CU_TRY(cudaStreamIsCapturing(c->stream, &cs), "capture status");
+  if (cs != cudaStreamCaptureStatusNone) {
+    OpSys sys = make_sys(c);
+    CU_TRY(cudaMallocAsync(&sys.trace, c->trace_entries * es, c->stream), "traction scratch of a captured apply");
+    CU_TRY(sys.apply(precision, u, y, nullptr, c->stream), "apply launch");
+    CU_TRY(cudaFreeAsync(sys.trace, c->stream), "traction scratch of a captured apply");
+    return TN_OK;
+  }
+  if ((st = ensure_trace(c, precision))) return st;
   if (precision == TN_F32 && (st = ensure_tuned(c, (const float *)u, (float *)y, c->stream))) return st;
   CU_TRY(make_sys(c).apply(precision, u, y, nullptr, c->stream), "apply launch");
   return TN_OK;
@@ -1034,7 +1089,7 @@ static tn_status solve_impl(tn_ctx *c, const tn_solve_opts *o, const double *rhs
   if (o->mode == TN_SOLVE_MIXED_F32 && (!(o->inner_rtol > 0.0) || !(o->inner_rtol < 1.0) || o->max_outer < 1))
     return fail(TN_EINVAL, "mixed mode needs 0 < inner_rtol < 1 and max_outer >= 1");
   CU_TRY(cudaSetDevice(c->device), "cudaSetDevice");
-  if ((st = ensure_ws(c))) return st;
+  if ((st = ensure_ws(c)) || (st = ensure_trace(c, TN_F64))) return st;
   const int chunk = o->check_every > 0 ? o->check_every : 25;
   const auto t0 = std::chrono::steady_clock::now();
   tn::g_launches = 2;  // rhs and diagonal below

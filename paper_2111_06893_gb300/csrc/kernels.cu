@@ -11,36 +11,21 @@
 // Dirichlet faces (Eq. (bc), u_b = 0): u_ext = -u, T_ext = T, Y_* = Y.
 // Neumann faces: no term.
 //
-// One CTA per element, one thread per node.  The element's own field is
-// staged in shared memory; for each interior face the neighbour's face values
-// and its logical normal derivative are gathered (neighbour data are L2
-// hits), then the neighbour traction is formed at the face nodes, then every
-// node forms its strain, stress, face terms and fluxes, and finally the
-// transposed derivative contractions give y.  The FP32 kernel is built in two
-// occupancy variants (registers per thread against CTAs per SM) with
-// identical arithmetic; tn_tune_apply times both on the mesh at hand.
+// The FP64 / FP32 applies are in apply.cu; here is the dual-number form of
+// the gradients.  One CTA per element, one thread per node.  The element's own
+// field is staged in shared memory; for each interior face the neighbour's
+// face values and its logical normal derivative are gathered (neighbour data
+// are L2 hits), then the neighbour traction is formed at the face nodes, then
+// every node forms its strain, stress, face terms and fluxes, and finally the
+// transposed derivative contractions give A u.
 #include <cstdio>
 #include <type_traits>
 
 #include "tn_internal.h"
 
 __constant__ LglTables c_lgl;
-__constant__ float c_Df[TN_MAX_N + 1][TN_MAX_N * TN_MAX_N];
-__constant__ float c_wf[TN_MAX_N + 1][TN_MAX_N];
 
-cudaError_t tn_upload_lgl(const LglTables *t) {
-  cudaError_t err = cudaMemcpyToSymbol(c_lgl, t, sizeof(LglTables));
-  if (err != cudaSuccess) return err;
-  static float Df[TN_MAX_N + 1][TN_MAX_N * TN_MAX_N];
-  static float wf[TN_MAX_N + 1][TN_MAX_N];
-  for (int N = 0; N <= TN_MAX_N; ++N) {
-    for (int a = 0; a < TN_MAX_N * TN_MAX_N; ++a) Df[N][a] = (float)t->D[N][a];
-    for (int a = 0; a < TN_MAX_N; ++a) wf[N][a] = (float)t->w[N][a];
-  }
-  err = cudaMemcpyToSymbol(c_Df, Df, sizeof(Df));
-  if (err != cudaSuccess) return err;
-  return cudaMemcpyToSymbol(c_wf, wf, sizeof(wf));
-}
+cudaError_t tn_upload_lgl(const LglTables *t) { return cudaMemcpyToSymbol(c_lgl, t, sizeof(LglTables)); }
 
 namespace {
 
@@ -53,10 +38,6 @@ template <> struct Tab<Dual> {
   static __device__ __forceinline__ double D(int N, int a, int b) { return c_lgl.D[N][a * N + b]; }
   static __device__ __forceinline__ double w(int N, int a) { return c_lgl.w[N][a]; }
 };
-template <> struct Tab<float> {
-  static __device__ __forceinline__ float D(int N, int a, int b) { return c_Df[N][a * N + b]; }
-  static __device__ __forceinline__ float w(int N, int a) { return c_wf[N][a]; }
-};
 
 // geometry / material accessors: plain types round the FP64 tables, the dual
 // type also carries the derivative seed of the current direction
@@ -65,33 +46,12 @@ __device__ __forceinline__ T slab_dz(const DevMesh &m, int s, int k) {
   return (T)m.slabgeo[((size_t)s * SG_NF + SG_DZ) * m.N + k];
 }
 template <>
-__device__ __forceinline__ float slab_dz<float>(const DevMesh &m, int s, int k) {
-  return m.slabgeo32[((size_t)s * SG_NF + SG_DZ) * m.N + k];
-}
-template <>
 __device__ __forceinline__ Dual slab_dz<Dual>(const DevMesh &m, int s, int k) {
   return Dual(m.slabgeo[((size_t)s * SG_NF + SG_DZ) * m.N + k], m.d_slabdz ? m.d_slabdz[(size_t)s * m.N + k] : 0.0);
 }
 template <typename T>
 __device__ __forceinline__ T layer_coef(const DevMesh &m, int L, int q) {
   return (T)m.layer_c[3 * L + q];
-}
-template <>
-__device__ __forceinline__ float layer_coef<float>(const DevMesh &m, int L, int q) {
-  return m.layer_c32[3 * L + q];
-}
-// column geometry table in the kernel's precision
-template <typename T> struct ColGeo { using type = double; };
-template <> struct ColGeo<float> { using type = float; };
-template <typename T>
-__device__ __forceinline__ const typename ColGeo<T>::type *col_table(const DevMesh &m) {
-  if constexpr (std::is_same<T, float>::value) return m.colgeo32;
-  else return m.colgeo;
-}
-template <typename T>
-__device__ __forceinline__ T pen_const(const DevMesh &m) {
-  if constexpr (std::is_same<T, float>::value) return m.penC32;
-  else return T(m.penC);
 }
 template <>
 __device__ __forceinline__ Dual layer_coef<Dual>(const DevMesh &m, int L, int q) {
@@ -248,15 +208,14 @@ constexpr size_t apply_smem() {
   return sizeof(T) * (12 * N * N * N + 42 * N * N);
 }
 
-// T = double / float: y = A u (and optionally partial[e] = u_e . y_e).
-// T = Dual: derivative of A u along the seeded direction; partial[e] = lam_e . (dA u)_e, y unused.
-// work (optional, derivatives): CTA b contracts element work[b].y along
+// Derivative of A u along the seeded direction: partial[e] = lam_e . (dA u)_e.
+// work (optional): CTA b contracts element work[b].y along
 // parameter work[b].x, whose seeds are pseed[2 work[b].x] (d(dz/dzeta) per
 // slab node) and pseed[2 work[b].x + 1] (d(c11, c12, c44) per layer),
 // either may be nullptr; partial[b] as before.
-template <int N, typename T, typename TIO>
+template <int N, typename T>
 __global__ void __launch_bounds__(nthreads<N>())
-apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restrict__ y, double *__restrict__ partial,
+apply_kernel(const DevMesh m0, int e0, const double *__restrict__ u, double *__restrict__ partial,
              const double *__restrict__ lam, const int2 *__restrict__ work = nullptr,
              const double *const *__restrict__ pseed = nullptr) {
   DevMesh m = m0;
@@ -280,7 +239,7 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
 
   const int e = work ? ework : e0 + blockIdx.x, tid = threadIdx.x;
   const int s = e / m.ncol, c = e - s * m.ncol;
-  const TIO *ue = u + (size_t)e * 3 * n;
+  const double *ue = u + (size_t)e * 3 * n;
   for (int t = tid; t < 3 * n; t += NT) su[t] = T(ue[t]);
   if (tid < 6) {
     face_info(m, s, c, fi, tid);
@@ -304,7 +263,7 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
       k2 = t2;
       if (d2 == 0) { i2 = end; j2 = a; } else { i2 = a; j2 = end; }
     }
-    const TIO *u2 = u + (size_t)fi.nb[f] * 3 * n;
+    const double *u2 = u + (size_t)fi.nb[f] * 3 * n;
     const int stride = d2 == 0 ? 1 : (d2 == 1 ? N : N2);
     const int base = (k2 * N + j2) * N + i2 - end * stride;
 #pragma unroll
@@ -322,7 +281,7 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
     if (d2 == 2) {
       h2 = T(2) * slab_dz<T>(m, fi.nbslab[f], end);
     } else {
-      const auto *g2 = col_table<T>(m) + (size_t)fi.nbcol[f] * CG_NF * N2;
+      const auto *g2 = m.colgeo + (size_t)fi.nbcol[f] * CG_NF * N2;
       const int q2 = j2 * N + i2;
       const T rx = (T)g2[(d2 == 0 ? CG_IXX : CG_IEX) * N2 + q2];
       const T ry = (T)g2[(d2 == 0 ? CG_IXY : CG_IEY) * N2 + q2];
@@ -332,7 +291,7 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
   }
   __syncthreads();
 
-  const auto *cg = col_table<T>(m) + (size_t)c * CG_NF * N2;
+  const auto *cg = m.colgeo + (size_t)c * CG_NF * N2;
   const int Lown = m.slab_layer[s];
   const T c11 = layer_coef<T>(m, Lown, 0), c12 = layer_coef<T>(m, Lown, 1), c44 = layer_coef<T>(m, Lown, 2);
 
@@ -380,7 +339,7 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc) { deta[cc] = dn[cc]; dxi[cc] = sg1 * dt1[cc]; dzeta[cc] = dt2[cc]; }
       }
-      const auto *g2 = col_table<T>(m) + (size_t)fi.nbcol[f] * CG_NF * N2;
+      const auto *g2 = m.colgeo + (size_t)fi.nbcol[f] * CG_NF * N2;
       const int q2 = j2 * N + i2;
       jxx = (T)g2[CG_IXX * N2 + q2]; jxy = (T)g2[CG_IXY * N2 + q2];
       jex = (T)g2[CG_IEX * N2 + q2]; jey = (T)g2[CG_IEY * N2 + q2];
@@ -432,7 +391,7 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
     const bool onface = i == 0 || i == N - 1 || j == 0 || j == N - 1 || k == 0 || k == N - 1;
     if (onface) {
       const Sym<T> sig = stress(S, c11, c12, c44);
-      const T sp1 = T((float)((m.p + 1) * (m.p + 1))) * pen_const<T>(m);
+      const T sp1 = T((float)((m.p + 1) * (m.p + 1))) * T(m.penC);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         const int idx = d == 0 ? i : (d == 1 ? j : k);
@@ -491,7 +450,6 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
 
   // ---- weak divergence: y = sum_m D_m^T F^m
   double dot = 0.0;
-  T dott = T(0);
   if (active) {
 #pragma unroll
     for (int cc = 0; cc < 3; ++cc) {
@@ -503,582 +461,17 @@ apply_kernel(const DevMesh m0, int e0, const TIO *__restrict__ u, TIO *__restric
         acc += Tab<T>::D(N, mm, j) * F1[(k * N + mm) * N + i];
         acc += Tab<T>::D(N, mm, k) * F2[(mm * N + j) * N + i];
       }
-      if constexpr (std::is_same<T, Dual>::value) {
-        dot += acc.d * lam[(size_t)e * 3 * n + cc * n + p];
-      } else {
-        y[(size_t)e * 3 * n + cc * n + p] = acc;
-        dott += acc * su[cc * n + p];
-      }
+      dot += acc.d * lam[(size_t)e * 3 * n + cc * n + p];
     }
   }
-  if constexpr (!std::is_same<T, Dual>::value) dot = (double)dott;
-  if (partial) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    if ((tid & 31) == 0) red[tid >> 5] = dot;
-    __syncthreads();
-    if (tid == 0) {
-      double sum = 0.0;
-      for (int w = 0; w < NT / 32; ++w) sum += red[w];
-      partial[blockIdx.x] = sum;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Second form of the operator kernel for T = float / double.  Same arithmetic
-// as apply_kernel, reorganised so that every sum-factorised contraction is a
-// "line task": one thread owns a whole line of N nodes along one logical
-// direction, keeps it in registers and produces all N outputs with the
-// derivative matrix as compile-time (warp-uniform) constant operands.  This
-// removes the per-thread-indexed constant loads and cuts shared-memory traffic
-// about threefold.  Phases (one CTA per element, one thread per node):
-//   1  gather neighbour face values / normal derivatives  +  gradient lines
-//   2  neighbour tangential derivative lines on the face planes
-//   3  neighbour traction at the face nodes
-//   4  per node: strain, stress, face terms, lifted strain, fluxes
-//   5  weak-divergence lines (one partial sum per direction)
-//   6  per node: sum the three directions and the face terms, store y
-template <int N, typename T>
-constexpr size_t apply2_smem() {
-  return sizeof(T) * (3 * N * N * N + 9 * N * N * N + 9 * N * N * N + 18 * N * N * 4 + 6 * N * N);
-}
-
-// out[a'] = sum_a D[a'][a] v[a]   (derivative along the line)
-template <int N, typename T>
-__device__ __forceinline__ void line_diff(const T v[N], T out[N]) {
-#pragma unroll
-  for (int a2 = 0; a2 < N; ++a2) {
-    T acc = T(0);
-#pragma unroll
-    for (int a = 0; a < N; ++a) acc += Tab<T>::D(N, a2, a) * v[a];
-    out[a2] = acc;
-  }
-}
-// out[a'] = sum_a D[a][a'] v[a]   (transposed: weak divergence along the line)
-template <int N, typename T>
-__device__ __forceinline__ void line_difft(const T v[N], T out[N]) {
-#pragma unroll
-  for (int a2 = 0; a2 < N; ++a2) {
-    T acc = T(0);
-#pragma unroll
-    for (int a = 0; a < N; ++a) acc += Tab<T>::D(N, a, a2) * v[a];
-    out[a2] = acc;
-  }
-}
-
-// node index of position a on line l of direction d (l enumerates the N^2 lines)
-template <int N>
-__device__ __forceinline__ int line_node(int d, int l, int a) {
-  const int hi = l / N, lo = l - hi * N;
-  if (d == 0) return (hi * N + lo) * N + a;   // (k, j) fixed, i = a
-  if (d == 1) return (hi * N + a) * N + lo;   // (k, i) fixed, j = a
-  return (a * N + hi) * N + lo;               // (j, i) fixed, k = a
-}
-
-// u, y: the element's instance vectors; partial: this CTA's slot or nullptr
-template <int N, typename T>
-__device__ __forceinline__ void apply2_body(const DevMesh &m, const int e, const T *__restrict__ u,
-                                            T *__restrict__ y, double *__restrict__ partial,
-                                            unsigned char *smem_raw) {
-  constexpr int n = N * N * N, N2 = N * N, NT = nthreads<N>();
-  T *su = reinterpret_cast<T *>(smem_raw);  // [3][n]
-  T *sG = su + 3 * n;                        // [3 dir][3 comp][n] logical gradient, then fluxes F^m_j
-  T *sY = sG + 9 * n;                        // [3 dir][3 comp][n] divergence partial sums
-  T *nbv = sY + 9 * n;                       // [6][3][N2] neighbour face values
-  T *nbt = nbv + 18 * N2;                    // [6][3][N2] normal derivative, then traction
-  T *nbd = nbt + 18 * N2;                    // [2][6][3][N2] tangential derivatives
-  T *nbh = nbd + 36 * N2;                    // [6][N2]
-  __shared__ FaceInfo fi;
-  __shared__ T nbc[6][3];
-  __shared__ double red[NT / 32];
-
-  const int tid = threadIdx.x;
-  const int s = e / m.ncol, c = e - s * m.ncol;
-  const T *ue = u + (size_t)e * 3 * n;
-  for (int t = tid; t < 3 * n; t += NT) su[t] = ue[t];
-  if (tid < 6) {
-    face_info(m, s, c, fi, tid);
-    const int L = m.slab_layer[fi.nbslab[tid]];
-    nbc[tid][0] = layer_coef<T>(m, L, 0);
-    nbc[tid][1] = layer_coef<T>(m, L, 1);
-    nbc[tid][2] = layer_coef<T>(m, L, 2);
-  }
+  for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+  if ((tid & 31) == 0) red[tid >> 5] = dot;
   __syncthreads();
-
-  // ---- phase 1: neighbour gather tasks [0, 6 N2) and gradient line tasks [6 N2, 6 N2 + 9 N2)
-  for (int t = tid; t < 15 * N2; t += NT) {
-    if (t < 6 * N2) {
-      const int f = t / N2, q = t - f * N2;
-      if (fi.kind[f] != FK_INTERIOR) continue;
-      const int t1 = q % N, t2 = q / N;
-      const int f2 = fi.nbface[f], d2 = f2 >> 1, end = (f2 & 1) ? N - 1 : 0;
-      int i2, j2, k2;
-      if ((f >> 1) == 2) { i2 = t1; j2 = t2; k2 = end; }
-      else {
-        const int a = fi.flip[f] ? N - 1 - t1 : t1;
-        k2 = t2;
-        if (d2 == 0) { i2 = end; j2 = a; } else { i2 = a; j2 = end; }
-      }
-      const T *u2 = u + (size_t)fi.nb[f] * 3 * n;
-      const int stride = d2 == 0 ? 1 : (d2 == 1 ? N : N2);
-      const int base = (k2 * N + j2) * N + i2 - end * stride;
-#pragma unroll
-      for (int cc = 0; cc < 3; ++cc) {
-        T line[N];
-#pragma unroll
-        for (int mm = 0; mm < N; ++mm) line[mm] = u2[cc * n + base + mm * stride];
-        T dn = T(0);
-        if (end == 0) {
-#pragma unroll
-          for (int mm = 0; mm < N; ++mm) dn += Tab<T>::D(N, 0, mm) * line[mm];
-          nbv[(f * 3 + cc) * N2 + q] = line[0];
-        } else {
-#pragma unroll
-          for (int mm = 0; mm < N; ++mm) dn += Tab<T>::D(N, N - 1, mm) * line[mm];
-          nbv[(f * 3 + cc) * N2 + q] = line[N - 1];
-        }
-        nbt[(f * 3 + cc) * N2 + q] = dn;
-      }
-      T h2;
-      if (d2 == 2) {
-        h2 = T(2) * slab_dz<T>(m, fi.nbslab[f], end);
-      } else {
-        const auto *g2 = col_table<T>(m) + (size_t)fi.nbcol[f] * CG_NF * N2;
-        const int q2 = j2 * N + i2;
-        const T rx = (T)g2[(d2 == 0 ? CG_IXX : CG_IEX) * N2 + q2];
-        const T ry = (T)g2[(d2 == 0 ? CG_IXY : CG_IEY) * N2 + q2];
-        h2 = T(2) / sqrt(rx * rx + ry * ry);
-      }
-      nbh[f * N2 + q] = h2;
-    } else {
-      const int tt = t - 6 * N2, d = tt / (3 * N2), rem = tt - d * 3 * N2, cc = rem / N2, l = rem - cc * N2;
-      const T *v = su + cc * n;
-      T in[N], out[N];
-#pragma unroll
-      for (int a = 0; a < N; ++a) in[a] = v[line_node<N>(d, l, a)];
-      line_diff<N, T>(in, out);
-      T *g = sG + (d * 3 + cc) * n;
-#pragma unroll
-      for (int a = 0; a < N; ++a) g[line_node<N>(d, l, a)] = out[a];
-    }
-  }
-  __syncthreads();
-
-  // ---- phase 2: tangential derivatives of the neighbour face values
-  for (int t = tid; t < 36 * N; t += NT) {
-    const int f = t / (6 * N), rem = t - f * 6 * N, cc = rem / (2 * N), r2 = rem - cc * 2 * N;
-    const int dir = r2 / N, l = r2 - dir * N;
-    if (fi.kind[f] != FK_INTERIOR) continue;
-    const T *v = nbv + (f * 3 + cc) * N2;
-    T in[N], out[N];
-    if (dir == 0) {  // along t1, fixed t2 = l
-#pragma unroll
-      for (int a = 0; a < N; ++a) in[a] = v[l * N + a];
-    } else {         // along t2, fixed t1 = l
-#pragma unroll
-      for (int a = 0; a < N; ++a) in[a] = v[a * N + l];
-    }
-    line_diff<N, T>(in, out);
-    T *o = nbd + ((dir * 6 + f) * 3 + cc) * N2;
-    if (dir == 0) {
-#pragma unroll
-      for (int a = 0; a < N; ++a) o[l * N + a] = out[a];
-    } else {
-#pragma unroll
-      for (int a = 0; a < N; ++a) o[a * N + l] = out[a];
-    }
-  }
-  __syncthreads();
-
-  const auto *cg = col_table<T>(m) + (size_t)c * CG_NF * N2;
-  const int Lown = m.slab_layer[s];
-  const T c11 = layer_coef<T>(m, Lown, 0), c12 = layer_coef<T>(m, Lown, 1), c44 = layer_coef<T>(m, Lown, 2);
-
-  // ---- phase 3: neighbour traction n . Y_ext grad u_ext at the face nodes
-  for (int t = tid; t < 6 * N2; t += NT) {
-    const int f = t / N2, q = t - f * N2;
-    if (fi.kind[f] != FK_INTERIOR) continue;
-    const int t1 = q % N, t2 = q / N, d = f >> 1;
-    const int f2 = fi.nbface[f], d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0;
-    T dt1[3], dt2[3], dn[3];
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-      dt1[cc] = nbd[((0 * 6 + f) * 3 + cc) * N2 + q];
-      dt2[cc] = nbd[((1 * 6 + f) * 3 + cc) * N2 + q];
-      dn[cc] = nbt[(f * 3 + cc) * N2 + q];
-    }
-    T dxi[3], deta[3], dzeta[3];
-    T jxx, jxy, jex, jey, jdz;
-    int i, j, k;
-    face_node<N>(f, t1, t2, i, j, k);
-    if (d == 2) {
-#pragma unroll
-      for (int cc = 0; cc < 3; ++cc) { dxi[cc] = dt1[cc]; deta[cc] = dt2[cc]; dzeta[cc] = dn[cc]; }
-      const int qq = j * N + i;
-      jxx = (T)cg[CG_IXX * N2 + qq]; jxy = (T)cg[CG_IXY * N2 + qq];
-      jex = (T)cg[CG_IEX * N2 + qq]; jey = (T)cg[CG_IEY * N2 + qq];
-      jdz = T(1) / slab_dz<T>(m, fi.nbslab[f], end2);
-    } else {
-      const T sg1 = fi.flip[f] ? T(-1) : T(1);
-      const int a = fi.flip[f] ? N - 1 - t1 : t1;
-      int i2, j2;
-      if (d2 == 0) {
-        i2 = end2; j2 = a;
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) { dxi[cc] = dn[cc]; deta[cc] = sg1 * dt1[cc]; dzeta[cc] = dt2[cc]; }
-      } else {
-        i2 = a; j2 = end2;
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) { deta[cc] = dn[cc]; dxi[cc] = sg1 * dt1[cc]; dzeta[cc] = dt2[cc]; }
-      }
-      const auto *g2 = col_table<T>(m) + (size_t)fi.nbcol[f] * CG_NF * N2;
-      const int q2 = j2 * N + i2;
-      jxx = (T)g2[CG_IXX * N2 + q2]; jxy = (T)g2[CG_IXY * N2 + q2];
-      jex = (T)g2[CG_IEX * N2 + q2]; jey = (T)g2[CG_IEY * N2 + q2];
-      jdz = T(1) / slab_dz<T>(m, s, t2);
-    }
-    const Sym<T> S2 = strain(dxi, deta, dzeta, jxx, jxy, jex, jey, jdz);
-    const Sym<T> s2 = stress(S2, nbc[f][0], nbc[f][1], nbc[f][2]);
-    const int qq = j * N + i;
-    T nrm[3], W, h;
-    face_geom<T, N>(f, i, j, k, (T)cg[CG_IXX * N2 + qq], (T)cg[CG_IXY * N2 + qq],
-                    (T)cg[CG_IEX * N2 + qq], (T)cg[CG_IEY * N2 + qq], (T)cg[CG_DET * N2 + qq],
-                    slab_dz<T>(m, s, k), nrm, W, h);
-    T tr[3];
-    contract_n(s2, nrm, tr);
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) nbt[(f * 3 + cc) * N2 + q] = tr[cc];
-  }
-  __syncthreads();
-
-  // ---- phase 4: per node
-  T ysurf[3] = {T(0), T(0), T(0)};
-  T uown[3] = {T(0), T(0), T(0)};
-  const int p = tid;
-  const bool active = p < n;
-  const int i = p % N, j = (p / N) % N, k = p / N2;
-  if (active) {
-    T dxi[3], deta[3], dzeta[3];
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-      dxi[cc] = sG[(0 * 3 + cc) * n + p];
-      deta[cc] = sG[(1 * 3 + cc) * n + p];
-      dzeta[cc] = sG[(2 * 3 + cc) * n + p];
-      uown[cc] = su[cc * n + p];
-    }
-    const int qq = j * N + i;
-    const T ixx = (T)cg[CG_IXX * N2 + qq], ixy = (T)cg[CG_IXY * N2 + qq];
-    const T iex = (T)cg[CG_IEX * N2 + qq], iey = (T)cg[CG_IEY * N2 + qq];
-    const T det2 = (T)cg[CG_DET * N2 + qq], dz = slab_dz<T>(m, s, k);
-    const T idz = T(1) / dz;
-    const Sym<T> S = strain(dxi, deta, dzeta, ixx, ixy, iex, iey, idz);
-    const T wJ = Tab<T>::w(N, i) * Tab<T>::w(N, j) * Tab<T>::w(N, k) * det2 * dz;
-    Sym<T> Se = {wJ * S.xx, wJ * S.yy, wJ * S.zz, wJ * S.xy, wJ * S.xz, wJ * S.yz};
-    const bool onface = i == 0 || i == N - 1 || j == 0 || j == N - 1 || k == 0 || k == N - 1;
-    if (onface) {
-      const Sym<T> sig = stress(S, c11, c12, c44);
-      const T sp1 = T((float)((m.p + 1) * (m.p + 1))) * pen_const<T>(m);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const int idx = d == 0 ? i : (d == 1 ? j : k);
-        if (idx != 0 && idx != N - 1) continue;
-        const int f = 2 * d + (idx == N - 1 ? 1 : 0);
-        const int kind = fi.kind[f];
-        if (kind == FK_NEUMANN) continue;
-        T nrm[3], W, h;
-        face_geom<T, N>(f, i, j, k, ixx, ixy, iex, iey, det2, dz, nrm, W, h);
-        T tr[3];
-        contract_n(sig, nrm, tr);
-        const int t1 = d == 0 ? j : i, t2 = d == 2 ? j : k;
-        const int q = t2 * N + t1;
-        T jump[3], tr2[3], h2, y11, y12, y44;
-        if (kind == FK_INTERIOR) {
-#pragma unroll
-          for (int cc = 0; cc < 3; ++cc) {
-            jump[cc] = uown[cc] - nbv[(f * 3 + cc) * N2 + q];
-            tr2[cc] = nbt[(f * 3 + cc) * N2 + q];
-          }
-          h2 = nbh[f * N2 + q];
-          y11 = T(0.5) * (c11 + nbc[f][0]);
-          y12 = T(0.5) * (c12 + nbc[f][1]);
-          y44 = T(0.5) * (c44 + nbc[f][2]);
-        } else {
-#pragma unroll
-          for (int cc = 0; cc < 3; ++cc) { jump[cc] = uown[cc] + uown[cc]; tr2[cc] = tr[cc]; }
-          h2 = h; y11 = c11; y12 = c12; y44 = c44;
-        }
-        const T sigma = sp1 / hmin<T>(h, h2);
-        const Sym<T> Ej = sym_outer(nrm, jump);
-        const Sym<T> Sj = stress(Ej, y11, y12, y44);
-        T pen[3];
-        contract_n(Sj, nrm, pen);
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) ysurf[cc] -= W * (T(0.5) * (tr[cc] + tr2[cc]) - sigma * pen[cc]);
-        const T hw = T(-0.5) * W;
-        Se.xx += hw * Ej.xx; Se.yy += hw * Ej.yy; Se.zz += hw * Ej.zz;
-        Se.xy += hw * Ej.xy; Se.xz += hw * Ej.xz; Se.yz += hw * Ej.yz;
-      }
-    }
-    const Sym<T> se = stress(Se, c11, c12, c44);
-    // fluxes F^m_j overwrite the gradient at this node (read above by this thread only)
-    sG[(0 * 3 + 0) * n + p] = ixx * se.xx + ixy * se.xy;
-    sG[(0 * 3 + 1) * n + p] = ixx * se.xy + ixy * se.yy;
-    sG[(0 * 3 + 2) * n + p] = ixx * se.xz + ixy * se.yz;
-    sG[(1 * 3 + 0) * n + p] = iex * se.xx + iey * se.xy;
-    sG[(1 * 3 + 1) * n + p] = iex * se.xy + iey * se.yy;
-    sG[(1 * 3 + 2) * n + p] = iex * se.xz + iey * se.yz;
-    sG[(2 * 3 + 0) * n + p] = idz * se.xz;
-    sG[(2 * 3 + 1) * n + p] = idz * se.yz;
-    sG[(2 * 3 + 2) * n + p] = idz * se.zz;
-  }
-  __syncthreads();
-
-  // ---- phase 5: weak-divergence lines
-  for (int t = tid; t < 9 * N2; t += NT) {
-    const int d = t / (3 * N2), rem = t - d * 3 * N2, cc = rem / N2, l = rem - cc * N2;
-    const T *F = sG + (d * 3 + cc) * n;
-    T in[N], out[N];
-#pragma unroll
-    for (int a = 0; a < N; ++a) in[a] = F[line_node<N>(d, l, a)];
-    line_difft<N, T>(in, out);
-    T *o = sY + (d * 3 + cc) * n;
-#pragma unroll
-    for (int a = 0; a < N; ++a) o[line_node<N>(d, l, a)] = out[a];
-  }
-  __syncthreads();
-
-  // ---- phase 6: y = sum of the three directions + face terms
-  T dott = T(0);
-  if (active) {
-#pragma unroll
-    for (int cc = 0; cc < 3; ++cc) {
-      const T acc = ysurf[cc] + sY[(0 * 3 + cc) * n + p] + sY[(1 * 3 + cc) * n + p] + sY[(2 * 3 + cc) * n + p];
-      y[(size_t)e * 3 * n + cc * n + p] = acc;
-      dott += acc * uown[cc];
-    }
-  }
-  if (partial) {
-    double dot = (double)dott;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-    if ((tid & 31) == 0) red[tid >> 5] = dot;
-    __syncthreads();
-    if (tid == 0) {
-      double sum = 0.0;
-      for (int w = 0; w < NT / 32; ++w) sum += red[w];
-      *partial = sum;
-    }
-  }
-}
-
-// resident CTAs per SM requested from the register allocator for the
-// line-task kernel.  Variant 0: FP32, the CTAs per SM that fit ~60 registers
-// per thread (N = 7: three CTAs of 352 threads); FP64: one.  Variant 1
-// (FP32 only): one CTA more per SM than the registers of variant 0 allow,
-// within the shared-memory limit (N = 3: 32, 4: 16, 5: 8, 6: 5, 7: 4, 8: 3,
-// 9: 2), paid for with fewer registers per thread.  The two variants run the
-// same instructions in the same order, so their results are bit-identical;
-// the autotuner below times both on the mesh at hand.
-template <int N, typename T, int V>
-__host__ __device__ constexpr int apply2_min_blocks() {
-  if (sizeof(T) != 4) return 1;
-  if (V == 0) return N <= 4 ? 8 : (N == 5 ? 6 : (N == 6 ? 4 : (N == 7 ? 3 : (N == 8 ? 2 : 1))));
-  return N == 3 ? 32 : (N == 4 ? 16 : (N == 5 ? 8 : (N == 6 ? 5 : (N == 7 ? 4 : (N == 8 ? 3 : 2)))));
-}
-
-// The alpha step of a PCG iteration folded into the operator apply: once
-// every CTA of the step has written its p . Ap partial, the last reduces
-// all partials in a fixed order (0 .. nparts - 1) and sets alpha = rz / pAp
-// (breakdown if pAp <= 0 or not finite).  A run that has finished skips the
-// apply and marks the iteration inactive.
-__device__ __forceinline__ bool fold_skip(const PcgFold &f) {
-  if (!f.s || !f.s->done) return false;
-  if (blockIdx.x == 0 && threadIdx.x == 0) f.s->active = 0;
-  return true;
-}
-__device__ void fold_alpha(const PcgFold &f) {
-  const double *__restrict__ part = f.part;
-  __shared__ int last;
-  __shared__ double red[32];
-  __syncthreads();  // this CTA's partial is written
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last = atomicAdd(f.cnt, 1u) == (unsigned)(f.total - 1);
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double acc = 0.0;
-  for (int t = threadIdx.x; t < f.nparts; t += blockDim.x) acc += __ldcg(part + t);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double pq = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) pq += red[w];
-    tn_pcg_scalars *s = f.s;
-    s->active = 1;
-    s->pq = pq;
-    if (!(pq > 0.0) || !isfinite(pq)) {
-      s->breakdown = 1;
-      s->done = 1;
-      s->alpha = 0.0;
-    } else {
-      s->alpha = s->rz / pq;
-    }
-    *f.cnt = 0u;
-    __threadfence();
-  }
-}
-
-template <int N, typename T, int V>
-__global__ void __launch_bounds__(nthreads<N>(), (apply2_min_blocks<N, T, V>()))
-apply2_kernel(const DevMesh m, int e0, const T *__restrict__ u, T *__restrict__ y, double *__restrict__ partial,
-              const PcgFold fold) {
-  if (fold_skip(fold)) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  apply2_body<N, T>(m, e0 + blockIdx.x, u, y, partial ? partial + blockIdx.x : nullptr, smem_raw);
-  if (fold.s) fold_alpha(fold);
-}
-
-// a batch of meshes: CTA b works on element work[b].y of instance work[b].x
-template <int N, typename T, int V>
-__global__ void __launch_bounds__(nthreads<N>(), (apply2_min_blocks<N, T, V>()))
-apply2_batch_kernel(const DevMesh *__restrict__ meshes, const int2 *__restrict__ work,
-                    const long long *__restrict__ dof_off, const T *__restrict__ u, T *__restrict__ y,
-                    double *__restrict__ partial, const PcgFold fold) {
-  if (fold_skip(fold)) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ __align__(16) unsigned char sm_raw[sizeof(DevMesh)];
-  DevMesh &sm = *reinterpret_cast<DevMesh *>(sm_raw);
-  const int2 w = work[blockIdx.x];
-  if (threadIdx.x == 0) memcpy(sm_raw, &meshes[w.x], sizeof(DevMesh));
-  __syncthreads();
-  const long long off = dof_off[w.x];
-  apply2_body<N, T>(sm, w.y, u + off, y + off, partial ? partial + blockIdx.x : nullptr, smem_raw);
-  if (fold.s) fold_alpha(fold);
-}
-
-// the dynamic shared-memory opt-in of a kernel, once per device
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t bytes, int &configured_device) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (configured_device == dev) return cudaSuccess;
-  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (err == cudaSuccess) configured_device = dev;
-  return err;
-}
-
-// fold / fold_part: the alpha step (fold_part: the partials of all the
-// step's launches, of which this launch writes `partial` onwards)
-template <int N, typename T, int V>
-cudaError_t launch_apply2_batch_v(const DevMesh *meshes, const int2 *work, int nwork, const long long *dof_off,
-                                  const T *u, T *y, double *partial, cudaStream_t st, const PcgFold &fold) {
-  constexpr size_t sm = apply2_smem<N, T>();
-  static int configured_device = -1;
-  cudaError_t err = allow_smem(apply2_batch_kernel<N, T, V>, sm, configured_device);
-  if (err != cudaSuccess) return err;
-  if (nwork <= 0) return cudaSuccess;
-  apply2_batch_kernel<N, T, V><<<nwork, nthreads<N>(), sm, st>>>(meshes, work, dof_off, u, y, partial, fold);
-  return cudaGetLastError();
-}
-
-template <int N, typename T, int V>
-cudaError_t launch_apply2_v(const DevMesh &m, const T *u, T *y, double *partial, cudaStream_t st,
-                            const PcgFold &fold) {
-  constexpr size_t sm = apply2_smem<N, T>();
-  static int configured_device = -1;
-  cudaError_t err = allow_smem(apply2_kernel<N, T, V>, sm, configured_device);
-  if (err != cudaSuccess) return err;
-  apply2_kernel<N, T, V><<<m.E, nthreads<N>(), sm, st>>>(m, 0, u, y, partial, fold);
-  return cudaGetLastError();
-}
-
-// variant 1 exists for FP32 only
-template <int N, typename T>
-cudaError_t launch_apply2_batch(const DevMesh *meshes, const int2 *work, int nwork, const long long *dof_off,
-                                const T *u, T *y, double *partial, cudaStream_t st, int var,
-                                const PcgFold &fold = PcgFold()) {
-  if constexpr (sizeof(T) == 4) {
-    if (var == 1) return launch_apply2_batch_v<N, T, 1>(meshes, work, nwork, dof_off, u, y, partial, st, fold);
-  }
-  return launch_apply2_batch_v<N, T, 0>(meshes, work, nwork, dof_off, u, y, partial, st, fold);
-}
-
-template <int N, typename T>
-cudaError_t launch_apply2(const DevMesh &m, const T *u, T *y, double *partial, cudaStream_t st, int var,
-                          const PcgFold &fold = PcgFold()) {
-  if constexpr (sizeof(T) == 4) {
-    if (var == 1) return launch_apply2_v<N, T, 1>(m, u, y, partial, st, fold);
-  }
-  return launch_apply2_v<N, T, 0>(m, u, y, partial, st, fold);
-}
-
-// time per launch (us) of both FP32 variants on one mesh (m1) or one degree
-// group of a batch: 3 untimed launches, then 10 between CUDA events on st
-template <int N>
-cudaError_t tune_apply2(const DevMesh *m1, const DevMesh *meshes, const int2 *work, int nwork,
-                        const long long *dof_off, const float *u, float *y, cudaStream_t st, float us[2]) {
-  cudaEvent_t ev[2];
-  cudaError_t err = cudaEventCreate(&ev[0]);
-  if (err != cudaSuccess) return err;
-  err = cudaEventCreate(&ev[1]);
-  if (err != cudaSuccess) {
-    cudaEventDestroy(ev[0]);
-    return err;
-  }
-  for (int v = 0; v < 2 && err == cudaSuccess; ++v) {
-    for (int i = 0; i < 13 && err == cudaSuccess; ++i) {
-      if (i == 3) err = cudaEventRecord(ev[0], st);
-      if (err != cudaSuccess) break;
-      err = m1 ? launch_apply2<N, float>(*m1, u, y, nullptr, st, v)
-               : launch_apply2_batch<N, float>(meshes, work, nwork, dof_off, u, y, nullptr, st, v);
-    }
-    if (err == cudaSuccess) err = cudaEventRecord(ev[1], st);
-    if (err == cudaSuccess) err = cudaEventSynchronize(ev[1]);
-    float ms = 0.0f;
-    if (err == cudaSuccess) err = cudaEventElapsedTime(&ms, ev[0], ev[1]);
-    us[v] = ms * 100.0f;  // 10 launches: ms / 10 * 1000
-  }
-  cudaEventDestroy(ev[0]);
-  cudaEventDestroy(ev[1]);
-  return err;
-}
-
-template <int N, typename T, typename TIO>
-cudaError_t launch_apply_range(const DevMesh &m, int s0, int s1, const TIO *u, TIO *y, double *partial,
-                               const double *lam, cudaStream_t st) {
-  constexpr size_t sm = apply_smem<N, T>();
-  static int configured_device = -1;  // the attribute is per function and device
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (configured_device != dev) {
-    cudaError_t err = cudaFuncSetAttribute(apply_kernel<N, T, TIO>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (err != cudaSuccess) return err;
-    configured_device = dev;
-  }
-  const int nblk = (s1 - s0) * m.ncol;
-  if (nblk <= 0) return cudaSuccess;
-  apply_kernel<N, T, TIO><<<nblk, nthreads<N>(), sm, st>>>(m, s0 * m.ncol, u, y, partial, lam);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_apply_t(const DevMesh &m, const T *u, T *y, double *partial, cudaStream_t st, int var,
-                           const PcgFold &fold) {
-  switch (m.N) {
-    case 3: return launch_apply2<3, T>(m, u, y, partial, st, var, fold);
-    case 4: return launch_apply2<4, T>(m, u, y, partial, st, var, fold);
-    case 5: return launch_apply2<5, T>(m, u, y, partial, st, var, fold);
-    case 6: return launch_apply2<6, T>(m, u, y, partial, st, var, fold);
-    case 7: return launch_apply2<7, T>(m, u, y, partial, st, var, fold);
-    case 8: return launch_apply2<8, T>(m, u, y, partial, st, var, fold);
-    case 9: return launch_apply2<9, T>(m, u, y, partial, st, var, fold);
-    default: return cudaErrorInvalidValue;
+  if (tid == 0) {
+    double sum = 0.0;
+    for (int w = 0; w < NT / 32; ++w) sum += red[w];
+    partial[blockIdx.x] = sum;
   }
 }
 
@@ -1519,40 +912,7 @@ cudaError_t launch_energy_n(const DevMesh &m, const double *u, double *elem, cud
   return cudaGetLastError();
 }
 
-template <int N>
-cudaError_t launch_energy_dual_n(const DevMesh &m, int s0, int s1, const double *u, const double *w,
-                                 double *epart, cudaStream_t st) {
-  const int nblk = (s1 - s0) * m.ncol;
-  if (nblk <= 0) return cudaSuccess;
-  energy_kernel<N, Dual><<<nblk, nthreads<N>(), 0, st>>>(m, s0 * m.ncol, u, w, epart);
-  return cudaGetLastError();
-}
-
 }  // namespace
-
-cudaError_t tn_launch_apply(const DevMesh &m, int precision, const void *u, void *y,
-                            double *partial, int var, cudaStream_t st, const PcgFold *fold) {
-  const PcgFold f = fold ? *fold : PcgFold();
-  if (precision == TN_F64)
-    return launch_apply_t<double>(m, (const double *)u, (double *)y, partial, st, 0, f);
-  return launch_apply_t<float>(m, (const float *)u, (float *)y, partial, st, var, f);
-}
-
-int tn_apply_ctas(const DevMesh *m, int nwork) { return m ? m->E : nwork; }
-
-cudaError_t tn_tune_apply(const DevMesh *m1, int N, const DevMesh *meshes, const int2 *work, int nwork,
-                          const long long *dof_off, const float *u, float *y, cudaStream_t st, float us[2]) {
-  switch (N) {
-    case 3: return tune_apply2<3>(m1, meshes, work, nwork, dof_off, u, y, st, us);
-    case 4: return tune_apply2<4>(m1, meshes, work, nwork, dof_off, u, y, st, us);
-    case 5: return tune_apply2<5>(m1, meshes, work, nwork, dof_off, u, y, st, us);
-    case 6: return tune_apply2<6>(m1, meshes, work, nwork, dof_off, u, y, st, us);
-    case 7: return tune_apply2<7>(m1, meshes, work, nwork, dof_off, u, y, st, us);
-    case 8: return tune_apply2<8>(m1, meshes, work, nwork, dof_off, u, y, st, us);
-    case 9: return tune_apply2<9>(m1, meshes, work, nwork, dof_off, u, y, st, us);
-    default: return cudaErrorInvalidValue;
-  }
-}
 
 int tn_sm_count() {
   static int cache[64] = {0};
@@ -1616,16 +976,6 @@ cudaError_t tn_launch_energy_parts(const DevMesh &m, const double *u, double *pa
     default: return cudaErrorInvalidValue;  \
   }
 
-cudaError_t tn_launch_apply_dual(const DevMesh &m, int s0, int s1, const double *u, const double *lam,
-                                 double *part, cudaStream_t st) {
-  TN_DISPATCH_N(return launch_apply_range<NN, Dual, double>(m, s0, s1, u, nullptr, part, lam, st))
-}
-
-cudaError_t tn_launch_energy_dual(const DevMesh &m, int s0, int s1, const double *u, const double *w,
-                                  double *epart, cudaStream_t st) {
-  TN_DISPATCH_N(return launch_energy_dual_n<NN>(m, s0, s1, u, w, epart, st))
-}
-
 cudaError_t tn_launch_apply_dual_work(const DevMesh &m, const int2 *work, int nwork, const double *const *pseed,
                                       const double *u, const double *lam, double *part, cudaStream_t st) {
   if (nwork <= 0) return cudaSuccess;
@@ -1635,12 +985,12 @@ cudaError_t tn_launch_apply_dual_work(const DevMesh &m, const int2 *work, int nw
     int dev = 0;
     cudaGetDevice(&dev);
     if (configured_device != dev) {
-      cudaError_t err = cudaFuncSetAttribute(apply_kernel<NN, Dual, double>,
+      cudaError_t err = cudaFuncSetAttribute(apply_kernel<NN, Dual>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       if (err != cudaSuccess) return err;
       configured_device = dev;
     }
-    apply_kernel<NN, Dual, double><<<nwork, nthreads<NN>(), sm, st>>>(m, 0, u, nullptr, part, lam, work, pseed);
+    apply_kernel<NN, Dual><<<nwork, nthreads<NN>(), sm, st>>>(m, 0, u, part, lam, work, pseed);
     return cudaGetLastError();
   })
 }
@@ -1663,24 +1013,6 @@ cudaError_t tn_launch_rhs_dr0(const DevMesh &m, double r0, double F0, const doub
                               int nparts, cudaStream_t st) {
   rhs_dr0_kernel<<<nparts, 256, 0, st>>>(m, r0, F0, lam, part);
   return cudaGetLastError();
-}
-
-cudaError_t tn_launch_apply_batch(int N, int precision, const DevMesh *meshes, const int2 *work, int nwork,
-                                  const long long *dof_off, const void *u, void *y, double *partial,
-                                  int var, cudaStream_t st, const PcgFold *fold) {
-  const PcgFold f = fold ? *fold : PcgFold();
-  switch (N) {
-#define TN_CASE(NN)                                                                                    \
-  case NN:                                                                                            \
-    return precision == TN_F64                                                                        \
-               ? launch_apply2_batch<NN, double>(meshes, work, nwork, dof_off, (const double *)u,    \
-                                                 (double *)y, partial, st, 0, f)                      \
-               : launch_apply2_batch<NN, float>(meshes, work, nwork, dof_off, (const float *)u,      \
-                                                (float *)y, partial, st, var, f);
-    TN_CASE(3) TN_CASE(4) TN_CASE(5) TN_CASE(6) TN_CASE(7) TN_CASE(8) TN_CASE(9)
-#undef TN_CASE
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 cudaError_t tn_launch_energy_batch(int N, const DevMesh *meshes, const int2 *work, int nwork,

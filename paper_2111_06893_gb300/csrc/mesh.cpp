@@ -273,6 +273,27 @@ tn_status build_host_mesh(const tn_mesh_desc *d, HostMesh *out, char *msg, int m
       }
     }
   }
+  // ---- penalty scales of the lateral faces
+  for (int c = 0; c < ncol; ++c)
+    for (int f = 0; f < 4; ++f) {
+      const int nbc = m.colnb[4 * c + f], code = m.colnbf[4 * c + f];
+      const int dd = f >> 1, end = (f & 1) ? N - 1 : 0;
+      for (int t = 0; t < N; ++t) {
+        double *g = m.colgeo + (size_t)c * CG_NF * N2;
+        const int q = dd == 0 ? t * N + end : end * N + t;
+        double ratio = 1.0;
+        if (nbc >= 0) {
+          const int f2 = code & 3, d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0, a2 = (code >> 2) ? N - 1 - t : t;
+          const int q2 = d2 == 0 ? a2 * N + end2 : end2 * N + a2;
+          const double *g2 = m.colgeo + (size_t)nbc * CG_NF * N2;
+          const int bx = dd == 0 ? CG_IXX : CG_IEX, bx2 = d2 == 0 ? CG_IXX : CG_IEX;
+          const double mag = std::hypot(g[bx * N2 + q], g[(bx + 1) * N2 + q]);
+          const double mag2 = std::hypot(g2[bx2 * N2 + q2], g2[(bx2 + 1) * N2 + q2]);
+          if (mag2 > mag) ratio = mag2 / mag;
+        }
+        g[(dd == 0 ? CG_RXI : CG_RETA) * N2 + q] = 0.5 * ratio;
+      }
+    }
   // ---- slabs
   for (int s = 0; s < m.nslab; ++s) {
     double *g = m.slabgeo + (size_t)s * SG_NF * N;
@@ -290,8 +311,21 @@ tn_status build_host_mesh(const tn_mesh_desc *d, HostMesh *out, char *msg, int m
       }
       g[SG_DZ * N + k] = dz;
       g[SG_Z * N + k] = z;
+      g[SG_IDZ * N + k] = 1.0 / dz;
     }
     m.slab_layer[s] = d->slab_layer[s];
+  }
+  for (int s = 0; s < m.nslab; ++s) {
+    double *g = m.slabgeo + (size_t)s * SG_NF * N;
+    for (int e = 0; e < 2; ++e) {  // bottom (k = 0) and top (k = N - 1): the slab below / above
+      const int k = e ? N - 1 : 0, s2 = e ? s - 1 : s + 1;
+      double dz = g[SG_DZ * N + k];
+      if (s2 >= 0 && s2 < m.nslab) {
+        const double dz2 = m.slabgeo[((size_t)s2 * SG_NF + SG_DZ) * N + (e ? 0 : N - 1)];
+        dz = dz2 < dz ? dz2 : dz;
+      }
+      g[SG_HINV * N + k] = 0.5 / dz;
+    }
   }
   *out = m;
   return TN_OK;

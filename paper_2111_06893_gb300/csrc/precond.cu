@@ -1475,17 +1475,6 @@ cudaError_t zgroup_launch_n(const DevMesh &m, const ZGroupDev &gd, int k, int pr
   return zgroup_launch_t<N, float>(m, gd, k, fac, r, z, prz, prr, done, zerr, st, fold, grid_out);
 }
 
-// r -= alpha q ahead of the grouped-line solve (the PCG residual update; a
-// separate pass measured faster than the update fused into the line walk)
-template <typename T>
-__global__ void zgroup_rupdate_kernel(long long n, T *__restrict__ r, const T *__restrict__ q,
-                                      const double *__restrict__ alpha, const int *__restrict__ done) {
-  if (done && *done) return;
-  const T al = (T)*alpha;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    r[i] -= al * q[i];
-}
-
 }  // namespace
 
 // union-find over face matches of the lines (col * N^2 + j * N + i)
@@ -1636,9 +1625,8 @@ cudaError_t tn_zgroup_setup(const DevMesh &m, const ZGroupPlan &p, const ZGroupD
 // one launch per degree present (one for a single mesh): the first on st,
 // the others on side streams forked from and joined back into st (also
 // inside a capture)
-cudaError_t tn_zgroup_solve(const DevMesh *m, const ZGroupDev &gd, int prec, const void *fac, void *r,
-                            const void *q, void *z, const double *alpha, double *part_rz, double *part_rr,
-                            const int *done, TnWait *zerr, cudaStream_t st, const PcgFold *fold_in) {
+cudaError_t tn_zgroup_solve(const DevMesh *m, const ZGroupDev &gd, int prec, const void *fac, const void *r,
+                            void *z, double *part_rz, double *part_rr, const int *done, TnWait *zerr, cudaStream_t st, const PcgFold *fold_in) {
   const DevMesh one = m ? *m : DevMesh{};
   cudaError_t err = cudaSuccess;
   PcgFold fold = fold_in ? *fold_in : PcgFold();
@@ -1660,15 +1648,6 @@ cudaError_t tn_zgroup_solve(const DevMesh *m, const ZGroupDev &gd, int prec, con
       }
       fold.total += g;
     }
-    if (err != cudaSuccess) return err;
-  }
-  if (q) {  // the residual update, before every degree class reads r
-    const int blocks = 4 * tn_sm_count();
-    if (prec == TN_F64)
-      zgroup_rupdate_kernel<double><<<blocks, 256, 0, st>>>(gd.ndof, (double *)r, (const double *)q, alpha, done);
-    else
-      zgroup_rupdate_kernel<float><<<blocks, 256, 0, st>>>(gd.ndof, (float *)r, (const float *)q, alpha, done);
-    err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }
   if (gd.npk > 1) err = cudaEventRecord(gd.fork, st);

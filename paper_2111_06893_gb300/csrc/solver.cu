@@ -8,9 +8,9 @@
 // partial r.z and r.r), a one-block reduction for beta and the direction
 // update.  With the single-line preconditioner the residual update r -= alpha
 // q runs inside the line solve (which also returns partial r.z and r.r);
-// with grouped lines it is a launch of its own ahead of the solve (measured
-// faster than fused there), and alpha and beta fold into the apply and the
-// solve, four launches per iteration.  The solution update x += alpha p runs
+// with grouped lines the operator's second launch takes its place (it adds
+// the neighbours' traces on the way), and alpha and beta fold into the apply
+// and the solve, four launches per iteration.  The solution update x += alpha p runs
 // inside the direction update.  A chunk of
 // iterations is recorded once in a CUDA graph and replayed.  Krylov scalars
 // live on the device; once converged every kernel returns immediately, so a
@@ -407,7 +407,7 @@ template <typename T>
 static cudaError_t pcg_iteration(const OpSys &sys, int prec, size_t n, PcgVectors &v, tn_pcg_scalars *s,
                                  double *part_elem, double *part_red, cudaStream_t st) {
   TN_CU(sys.apply(prec, v.p, v.q, part_elem, st));
-  k_alpha<<<1, 1024, 0, st>>>(s, part_elem, sys.n_apply_parts);
+  k_alpha<<<1, 1024, 0, st>>>(s, part_elem, sys.apply_parts());
   TN_CU(cudaGetLastError());
   k_update<T><<<red_blocks(), kRedThreads, 0, st>>>(s, n, (T *)v.x, (T *)v.r, (T *)v.z, (const T *)v.p,
                                                   (const T *)v.q, (const T *)v.dinv, part_red);
@@ -421,25 +421,26 @@ static cudaError_t pcg_iteration(const OpSys &sys, int prec, size_t n, PcgVector
 template <typename T>
 static cudaError_t pcg_iteration_zline(const OpSys &sys, int prec, size_t n, PcgVectors &v, tn_pcg_scalars *s,
                                        double *part_elem, double *part_red, cudaStream_t st) {
-  if (sys.grouped && sys.fold_cnt) {
-    // four launches: the apply with the alpha step, the residual update,
-    // the grouped-line solve with the beta step, the direction update
+  if (sys.grouped) {
+    // four launches: the elements' own terms of the apply with the alpha
+    // step, the residual update with the traces, the grouped-line solve with
+    // the beta step, the direction update
     PcgFold fa;
     fa.s = s;
     fa.cnt = sys.fold_cnt;
-    fa.total = sys.n_apply_parts;  // one CTA per element
-    fa.nparts = sys.n_apply_parts;
+    fa.total = fa.nparts = sys.apply_parts();  // one partial per CTA
     fa.part = part_elem;
-    TN_CU(sys.apply(prec, v.p, v.q, part_elem, st, &fa));
+    TN_CU(sys.apply_own(prec, v.p, v.q, part_elem, st, &fa));
+    TN_CU(sys.apply_traces(prec, v.q, v.r, &s->alpha, &s->done, st));
     PcgFold fb;
     fb.s = s;
     fb.cnt = sys.fold_cnt + 1;
-    TN_CU(sys.zsolve(prec, v.zfac, v.r, v.q, v.z, &s->alpha, v.part_rz, &s->done, st, &fb));
+    TN_CU(sys.zsolve(prec, v.zfac, v.r, nullptr, v.z, nullptr, v.part_rz, &s->done, st, &fb));
     k_pupdate_x<T><<<red_blocks(), kRedThreads, 0, st>>>(s, n, (T *)v.x, (T *)v.p, (const T *)v.z);
     return cudaGetLastError();
   }
   TN_CU(sys.apply(prec, v.p, v.q, part_elem, st));
-  k_alpha<<<1, 1024, 0, st>>>(s, part_elem, sys.n_apply_parts);
+  k_alpha<<<1, 1024, 0, st>>>(s, part_elem, sys.apply_parts());
   TN_CU(cudaGetLastError());
   // r -= alpha q fused into the line solve (partials r.z and r.r)
   TN_CU(sys.zsolve(prec, v.zfac, v.r, v.q, v.z, &s->alpha, v.part_rz, &s->done, st));
@@ -484,7 +485,7 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
   TN_CU(cudaMemcpyAsync(s_host, s_dev, sizeof(tn_pcg_scalars), cudaMemcpyDeviceToHost, st));
   TN_CU(cudaStreamSynchronize(st));
   if (s_host->done) return cudaSuccess;
-  if (zl && sys.grouped && sys.fold_cnt) TN_CU(cudaMemsetAsync(sys.fold_cnt, 0, 2 * sizeof(unsigned), st));
+  if (zl && sys.grouped) TN_CU(cudaMemsetAsync(sys.fold_cnt, 0, 2 * sizeof(unsigned), st));
 
   // one graph of `chunk` iterations, cached while the run's buffers are unchanged
   struct Key {
@@ -502,7 +503,7 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
   std::memset(static_cast<void *>(&key), 0, sizeof(key));
   key.x = v.x; key.r = v.r; key.z = v.z; key.p = v.p; key.q = v.q; key.b = v.b; key.dinv = v.dinv;
   key.zfac = v.zfac; key.part_rz = v.part_rz; key.pe = part_elem; key.pr = part_red; key.s = s_dev;
-  key.n = n; key.chunk = chunk; key.prec = prec; key.E = sys.n_apply_parts;
+  key.n = n; key.chunk = chunk; key.prec = prec; key.E = sys.n_elems;
   key.geo = sys.m ? (const void *)sys.m->colgeo : (const void *)sys.meshes;
   if (sys.m) std::memcpy(static_cast<void *>(&key.dm), sys.m, sizeof(DevMesh));
   std::memcpy(static_cast<void *>(&key.sys), &sys, sizeof(OpSys));
@@ -534,7 +535,7 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
   double best = INFINITY;
   int stall = 0;
   for (;;) {
-    g_launches += (zl && sys.grouped && sys.fold_cnt ? 4LL : (zl && sys.grouped ? 6LL : 5LL)) * chunk;
+    g_launches += (zl && sys.grouped ? 4LL : 6LL) * chunk;
     err = cudaGraphLaunch(exec, st);
     if (err != cudaSuccess) break;
     err = cudaMemcpyAsync(s_host, s_dev, sizeof(tn_pcg_scalars), cudaMemcpyDeviceToHost, st);
@@ -633,21 +634,70 @@ int reduction_blocks() { return red_blocks(); }
 
 }  // namespace tn
 
-cudaError_t OpSys::apply(int prec, const void *u, void *y, double *part, cudaStream_t st,
-                         const PcgFold *fold) const {
-  if (m) return tn_launch_apply(*m, prec, u, y, part, mvar, st, fold);
-  for (int g = 0; g < ngroups; ++g) {
-    cudaError_t e = tn_launch_apply_batch(gN[g], prec, meshes, gwork[g], gcount[g], dof_off, u, y,
-                                          part ? part + gpart_off[g] : nullptr, gvar[g], st, fold);
+ApplyArgs OpSys::args(int g0, int g1, int prec, const void *u, void *y) const {
+  ApplyArgs a;
+  a.m = m;
+  a.prec = prec;
+  a.u = u;
+  a.y = y;
+  a.trace = trace;
+  if (m) {
+    a.var = mvar;
+    return a;
+  }
+  a.meshes = meshes;
+  a.work = work;
+  a.dof_off = dof_off;
+  a.tr_off = tr_off;
+  a.ctas = ctas + gcta[g0];
+  a.ncta = gcta[g1] - gcta[g0];
+  a.adds = adds + gadd[g0];
+  a.nadd = gadd[g1] - gadd[g0];
+  a.var = gvar[g0];
+  a.few = tn_apply_few(n_elems);
+  return a;
+}
+
+int OpSys::apply_parts() const { return m ? tn_apply_parts(m->N, m->E) : gcta[ngroups]; }
+
+cudaError_t OpSys::apply_own(int prec, const void *u, void *y, double *part, cudaStream_t st,
+                             const PcgFold *fold) const {
+  ApplyArgs a = args(0, ngroups, prec, u, y);
+  a.fold = fold;
+  a.partial = part;
+  if (m) return tn_launch_apply(a, st);
+  // neighbouring degrees of one variant in one launch (FP64 has one variant)
+  for (int g = 0; g < ngroups;) {
+    int h = g + 1;
+    while (h < ngroups && (prec == TN_F64 || a.few || gvar[h] == gvar[g])) ++h;
+    ApplyArgs b = args(g, h, prec, u, y);
+    b.fold = fold;
+    b.partial = part ? part + gcta[g] : nullptr;
+    const cudaError_t e = tn_launch_apply(b, st);
     if (e != cudaSuccess) return e;
+    g = h;
   }
   return cudaSuccess;
+}
+
+cudaError_t OpSys::apply_traces(int prec, void *y, void *r, const double *alpha, const int *done,
+                                cudaStream_t st) const {
+  ApplyArgs a = args(0, ngroups, prec, nullptr, y);
+  a.r = r;
+  a.alpha = alpha;
+  a.done = done;
+  return tn_launch_trace_add(a, st);
+}
+
+cudaError_t OpSys::apply(int prec, const void *u, void *y, double *part, cudaStream_t st) const {
+  const cudaError_t e = apply_own(prec, u, y, part, st);
+  return e != cudaSuccess ? e : apply_traces(prec, y, nullptr, nullptr, nullptr, st);
 }
 
 cudaError_t OpSys::zsolve(int prec, const void *fac, void *r, const void *q, void *z, const double *alpha,
                           double *part, const int *done, cudaStream_t st, const PcgFold *fold) const {
   double *prr = part ? part + n_rz_parts : nullptr;
-  if (grouped) return tn_zgroup_solve(m, zg, prec, fac, r, q, z, alpha, part, prr, done, zerr, st, fold);
+  if (grouped) return tn_zgroup_solve(m, zg, prec, fac, r, z, part, prr, done, zerr, st, fold);
   if (m) return tn_zline_solve(*m, prec, fac, r, q, z, alpha, part, prr, done, zerr, st);
   for (int g = 0; g < ngroups; ++g) {
     cudaError_t e = tn_zline_solve_batch(gN[g], prec, meshes, gline[g], glines[g], fac_off, dof_off, fac, r, q, z,

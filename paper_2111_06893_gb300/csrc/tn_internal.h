@@ -24,10 +24,17 @@ enum {
   CG_DET = 4,  // det of d(X, Y)/d(xi, eta)
   CG_X = 5,    // X
   CG_Y = 6,    // Y
-  CG_NF = 7
+  // penalty scale of the lateral faces, at the face nodes (xi faces: i = 0,
+  // N - 1; eta faces: j = 0, N - 1; zero elsewhere): 1/2 max(1, mag_ext / mag)
+  // with mag = |grad xi| (|grad eta|), so that W / min(h, h_ext) n n^T =
+  // w det2 dz (this value) r r^T with the unnormalised r = grad xi (grad eta)
+  CG_RXI = 7,
+  CG_RETA = 8,
+  CG_NF = 9
 };
-// slab geometry, per slab and per node k along zeta
-enum { SG_DZ = 0, SG_Z = 1, SG_NF = 2 };
+// slab geometry, per slab and per node k along zeta: dz/dzeta, z, its
+// inverse, and 1 / min(h, h_ext) of the zeta faces (entries 0 and N - 1)
+enum { SG_DZ = 0, SG_Z = 1, SG_IDZ = 2, SG_HINV = 3, SG_NF = 4 };
 
 struct DevMesh {
   int N;          // LGL points per dimension
@@ -156,14 +163,9 @@ int tn_sm_count();
 
 // kernels (kernels.cu) -- launchers return cudaError_t of the launch
 cudaError_t tn_upload_lgl(const LglTables *t);
-// derivative kernels: over the elements of slabs [s0, s1),
-//   part[e - s0*ncol] = lam_e . (dA/dtheta u)_e        (seeds in m.d_*)
-//   epart[e - s0*ncol] = w[layer(e)] dU_e/dtheta|_u
-cudaError_t tn_launch_apply_dual(const DevMesh &m, int s0, int s1, const double *u, const double *lam,
-                                 double *part, cudaStream_t st);
-cudaError_t tn_launch_energy_dual(const DevMesh &m, int s0, int s1, const double *u, const double *w,
-                                  double *epart, cudaStream_t st);
-// the same for many parameters in one launch each: CTA b contracts element
+// derivative kernels, many parameters in one launch each (seeds in m.d_*):
+//   part[b] = lam_e . (dA/dtheta u)_e,  epart[b] = w[layer(e)] dU_e/dtheta|_u;
+// CTA b contracts element
 // work[b].y along parameter work[b].x, seeded by pseed[2 p] (d_slabdz) and
 // pseed[2 p + 1] (d_layer_c), device arrays; part[b] / epart[b]
 cudaError_t tn_launch_apply_dual_work(const DevMesh &m, const int2 *work, int nwork, const double *const *pseed,
@@ -176,22 +178,45 @@ cudaError_t tn_launch_energy_source(const DevMesh &m, const double *u, const dou
 // part[b] = partial sums of lam . db/dr0 (beam width derivative of the load)
 cudaError_t tn_launch_rhs_dr0(const DevMesh &m, double r0, double F0, const double *lam, double *part,
                               int nparts, cudaStream_t st);
-// batches: one launch per polynomial degree; work[b] = (instance, element).
-// var: occupancy variant of the FP32 kernel (0 or 1, same results)
-cudaError_t tn_launch_apply_batch(int N, int precision, const DevMesh *meshes, const int2 *work, int nwork,
-                                  const long long *dof_off, const void *u, void *y, double *partial,
-                                  int var, cudaStream_t st, const PcgFold *fold = nullptr);
-// us[v]: time per launch of FP32 variant v on one mesh (m1) or on one degree
-// group of a batch (m1 = nullptr); y is overwritten
-cudaError_t tn_tune_apply(const DevMesh *m1, int N, const DevMesh *meshes, const int2 *work, int nwork,
-                          const long long *dof_off, const float *u, float *y, cudaStream_t st, float us[2]);
+// One operator apply (apply.cu): one mesh (m), or degree groups of a batch
+// (elements work[w] = (mirror, element), vectors at dof_off[mirror], traces at
+// tr_off[mirror]; CTA b works on ctas[b] = (N, first work item, count)).
+struct ApplyArgs {
+  const DevMesh *m = nullptr;       // one mesh (host copy of the struct); nullptr: a batch
+  const DevMesh *meshes = nullptr;  // batch: the mirrors' meshes (device)
+  const int2 *work = nullptr;
+  const long long *dof_off = nullptr, *tr_off = nullptr;
+  const int4 *ctas = nullptr, *adds = nullptr;  // batch: CTAs of the apply and of tn_launch_trace_add
+  int ncta = 0, nadd = 0;
+  bool few = false;                 // batch: tn_apply_few of its elements
+  int prec = TN_F64, var = 0;       // var: occupancy variant of the FP32 kernel (0 or 1, same results)
+  const void *u = nullptr;
+  void *y = nullptr, *trace = nullptr;  // trace: tn_trace_entries per element, of the vectors' precision
+  double *partial = nullptr;        // one partial of u . A u per CTA, or nullptr
+  const PcgFold *fold = nullptr;    // the alpha step of a PCG iteration (its partials: every launch's)
+  // tn_launch_trace_add: r != nullptr: r -= *alpha (A u) instead of
+  // completing y; *done != 0: returns at once
+  void *r = nullptr;
+  const double *alpha = nullptr;
+  const int *done = nullptr;
+};
+// traction values an apply keeps per element: 6 faces x 3 components x N^2
+constexpr long long tn_trace_entries(int N) { return 18LL * N * N; }
+cudaError_t tn_upload_lgl_apply(const LglTables *t);
+// the elements' own terms and their traces; once every degree has run,
+// tn_launch_trace_add completes y (or takes it into the residual)
+cudaError_t tn_launch_apply(const ApplyArgs &a, cudaStream_t st);
+cudaError_t tn_launch_trace_add(const ApplyArgs &a, cudaStream_t st);
+// CTAs (= partial sums) of the first launch over one mesh; elements per CTA
+// of a batch's launches
+int tn_apply_parts(int N, int E);
+bool tn_apply_few(int E);  // few elements: the form with three threads per pencil
+int tn_apply_eb(int N, bool few);
+int tn_trace_add_eb(int N);
+// us[v]: time per apply of FP32 variant v; y is overwritten
+cudaError_t tn_tune_apply(ApplyArgs a, cudaStream_t st, float us[2]);
 cudaError_t tn_launch_energy_batch(int N, const DevMesh *meshes, const int2 *work, int nwork,
                                    const long long *dof_off, const double *u, double *out, cudaStream_t st);
-// fold (optional): the alpha step of a PCG iteration (partial = p . Ap per CTA)
-cudaError_t tn_launch_apply(const DevMesh &m, int precision, const void *u, void *y,
-                            double *partial, int var, cudaStream_t st, const PcgFold *fold = nullptr);
-// CTAs one apply launches (one mesh, or one degree group of a batch)
-int tn_apply_ctas(const DevMesh *m, int nwork);
 cudaError_t tn_launch_rhs(const DevMesh &m, double r0, double F0, double *b, cudaStream_t st);
 cudaError_t tn_launch_diag(const DevMesh &m, double *d, cudaStream_t st);
 cudaError_t tn_launch_energy(const DevMesh &m, const double *u, double *elem_energy,

@@ -77,11 +77,9 @@ size_t tn_zgroup_work_bytes(const DevMesh &m, const ZGroupPlan &p, int inst);  /
 cudaError_t tn_zgroup_setup(const DevMesh &m, const ZGroupPlan &p, const ZGroupDev &gd, int inst,
                             const int4 *lines, const long long *fac_off, double *blk, double *xblk, double *work,
                             float *fac, double *fac64, int *status, cudaStream_t st);
-// as tn_zline_solve, over the groups (m: the mesh, nullptr for a batch);
-// partial sums: one per group.  q != nullptr: r -= alpha q first, as a
-// launch of its own over all gd.ndof unknowns
-// fold (optional): the beta step of a PCG iteration (s and cnt; the rest is
-// filled in here)
-cudaError_t tn_zgroup_solve(const DevMesh *m, const ZGroupDev &gd, int prec, const void *fac, void *r,
-                            const void *q, void *z, const double *alpha, double *part_rz, double *part_rr,
-                            const int *done, TnWait *zerr, cudaStream_t st, const PcgFold *fold = nullptr);
+// z = M^{-1} r over the groups (m: the mesh, nullptr for a batch); partial
+// sums: one per group.  fold (optional): the beta step of a PCG iteration (s
+// and cnt; the rest is filled in here)
+cudaError_t tn_zgroup_solve(const DevMesh *m, const ZGroupDev &gd, int prec, const void *fac, const void *r, void *z,
+                            double *part_rz, double *part_rr, const int *done, TnWait *zerr, cudaStream_t st,
+                            const PcgFold *fold = nullptr);

@@ -15,24 +15,36 @@ struct OpSys {
   const DevMesh *meshes = nullptr;  // batch: device array of the instances' meshes
   int ngroups = 0;
   int gN[8] = {0};
-  const int2 *gwork[8] = {nullptr};  // (instance, element) per CTA of the apply
+  const int2 *work = nullptr;        // all (instance, element) pairs, degree by degree
+  const int2 *gwork[8] = {nullptr};  // those of one degree
   int gcount[8] = {0};
-  int gpart_off[8] = {0};
+  int gpart_off[8] = {0};  // first element of the group
   const int2 *gline[8] = {nullptr};  // (instance, line) per warp of the z-line solve
   int glines[8] = {0};
   int grz_off[8] = {0};
   const long long *dof_off = nullptr, *fac_off = nullptr;
   int mvar = 0;           // occupancy variant of the FP32 operator kernel (single mesh)
   int gvar[8] = {0};      // the same per degree group of a batch
-  int n_apply_parts = 0;  // partial sums written by one apply
+  void *trace = nullptr;  // traction scratch of the operator (FP64-sized; FP32 applies use half of it)
+  const long long *tr_off = nullptr;  // batch: first trace entry of every mirror
+  int n_elems = 0;        // elements of the mesh or of the whole batch
   int n_rz_parts = 0;     // partial sums of r.z written by one z-line solve (r.r: as many, after them)
   TnWait *zerr = nullptr; // wait limit of the line solves; flag set by one whose staging wait ran out
   unsigned *fold_cnt = nullptr;  // grouped lines: 2 counters of the alpha / beta steps folded into
-                                 // the apply and the line solve (nullptr: separate scalar kernels)
+                                 // the apply and the line solve
   bool grouped = false;   // grouped lines (zg) instead of single lines
   ZGroupDev zg;
-  cudaError_t apply(int prec, const void *u, void *y, double *part, cudaStream_t st,
-                    const PcgFold *fold = nullptr) const;
+  const int4 *ctas = nullptr, *adds = nullptr;  // batch: CTAs of the operator's launches, degree by degree
+  int gcta[9] = {0}, gadd[9] = {0};             // first CTA of every degree group (and the total)
+  ApplyArgs args(int g0, int g1, int prec, const void *u, void *y) const;  // groups g0 .. g1 - 1 (one mesh: all)
+  int apply_parts() const;  // partial sums written by one apply (one per CTA)
+  // the two launches of y = A u: the elements' own terms (part: partial u . A u;
+  // fold: the alpha step), then the traces added to y, or r -= *alpha A u
+  // (y is left incomplete).  apply: both.
+  cudaError_t apply_own(int prec, const void *u, void *y, double *part, cudaStream_t st,
+                        const PcgFold *fold = nullptr) const;
+  cudaError_t apply_traces(int prec, void *y, void *r, const double *alpha, const int *done, cudaStream_t st) const;
+  cudaError_t apply(int prec, const void *u, void *y, double *part, cudaStream_t st) const;
   // z = M^{-1} r; q != nullptr: first r <- r - (*alpha) q.  part: n_rz_parts
   // partial r.z, then n_rz_parts partial r.r
   cudaError_t zsolve(int prec, const void *fac, void *r, const void *q, void *z, const double *alpha,
