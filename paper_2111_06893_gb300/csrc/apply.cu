@@ -37,6 +37,7 @@
 // overlap): 24 instead of 31 us per FP32 apply at 2.0 M unknowns.
 #include <initializer_list>
 
+#include "tn_device.h"
 #include "tn_internal.h"
 
 namespace {
@@ -718,13 +719,6 @@ __device__ void fold_alpha(const PcgFold &f) {
   }
 }
 
-// programmatic dependent launch: a kernel of the operator starts while the
-// one before it in the stream drains, reads only mesh tables until grid_wait
-// (which returns once every earlier kernel has completed), and lets the next
-// one start as early as it likes
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // FP32: variant 0 asks for three CTAs per SM (80 registers, some spilled at N
 // = 9), variant 1 for two (up to 128).  Both round alike (bit-identical
 // results); the autotuner times them on the mesh at hand (p = 6, 2.0 M
@@ -772,6 +766,7 @@ __device__ __forceinline__ void apply_cta(const DevMesh &m1, const DevMesh *__re
     }
   }
   grid_wait();
+  ue = after_wait(ue);
   if (fold_skip(fold)) return;
   const ElemI<T> &E = info[act ? el : 0];
   T dott;
@@ -888,8 +883,9 @@ __device__ __forceinline__ void trace_add_cta(const DevMesh &m1, const DevMesh *
   }
   __syncthreads();
   grid_wait();
+  done = after_wait(done);
   if (done && *done) return;
-  const T al = UPD ? (T)*alpha : T(0);
+  const T al = UPD ? (T)*after_wait(alpha) : T(0);
 #pragma unroll 4
   for (int id = tid; id < nw * SN; id += kAddThreads) {
     const int el = id / SN, rr0 = id - el * SN;
