@@ -166,11 +166,8 @@ struct tn_ctx {
   // grouped-line preconditioner (same validity)
   ZGroupPlan gplan;
   ZGroupDev zgd;
-  int4 *d_glines = nullptr;
-  long long *d_gfac_off = nullptr;
-  int *d_ginst = nullptr;
-  int4 *d_gpacks = nullptr;
-  int *d_gqueue = nullptr;
+  unsigned char *d_gplan = nullptr;  // the plan's tables, one block
+  double *gchain = nullptr;          // chain numbers of the solve
   float *gfac = nullptr;
   double *gfac64 = nullptr;
   double *gpart = nullptr;
@@ -197,11 +194,8 @@ static void free_zline(tn_ctx *c) {
 }
 
 static void free_zgroup(tn_ctx *c) {
-  dfree(c->d_glines);
-  dfree(c->d_gfac_off);
-  dfree(c->d_ginst);
-  dfree(c->d_gpacks);
-  dfree(c->d_gqueue);
+  dfree(c->d_gplan);
+  dfree(c->gchain);
   dfree(c->gfac);
   dfree(c->gfac64);
   dfree(c->gpart);
@@ -409,25 +403,32 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
     xb = x1 > xb ? x1 : xb;
     wb = w1 > wb ? w1 : wb;
   }
-  const size_t fb = (size_t)p.nfac * sizeof(float);
+  const size_t fb = (size_t)p.nfac * sizeof(float), fb64 = (size_t)p.nfac64 * sizeof(double);
   double *blk = nullptr, *xblk = nullptr, *work = nullptr;
   cudaError_t e = cudaMalloc((void **)&blk, bb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&xblk, xb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&work, wb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gfac, fb);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->gfac64, 2 * fb);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->gpart, sizeof(double) * 2 * p.ngroups);  // r.z, r.r
+  if (e == cudaSuccess) e = cudaMalloc((void **)&c->gfac64, fb64);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&c->gpart, sizeof(double) * 2 * std::max(p.ranges.size(), p.lines.size()));  // r.z, r.r
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gstatus, 2 * sizeof(int));  // factor status, solve timeout
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_glines, sizeof(int4) * p.ngroups);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_gfac_off, sizeof(long long) * p.ngroups);
-  if (e == cudaSuccess && is_batch(c)) e = cudaMalloc((void **)&c->d_ginst, sizeof(int) * p.ngroups);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_gpacks, sizeof(int4) * p.packs.size());
-  if (e == cudaSuccess) e = cudaMalloc((void **)&c->d_gqueue, sizeof(int) * 2 * kZgMaxPk);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&c->gchain, sizeof(double) * (size_t)p.nchain);
+  TablePack pack;
+  const size_t o_lines = pack.add(p.lines.data(), sizeof(int4) * p.lines.size());
+  const size_t o_fac = pack.add(p.fac_off.data(), sizeof(long long) * p.fac_off.size());
+  const size_t o_fac64 = pack.add(p.fac64_off.data(), sizeof(long long) * p.fac64_off.size());
+  const size_t o_chain = pack.add(p.chain_off.data(), sizeof(long long) * p.chain_off.size());
+  const size_t o_packs = pack.add(p.packs.data(), sizeof(int4) * p.packs.size());
+  const size_t o_ranges = pack.add(p.ranges.data(), sizeof(int4) * p.ranges.size());
+  const std::vector<int> zeros(2 * kZgMaxDg, 0);
+  const size_t o_queue = pack.add(zeros.data(), sizeof(int) * zeros.size());
+  const size_t o_inst = pack.add(p.inst.data(), sizeof(int) * p.inst.size());
+  if (e == cudaSuccess) e = pack.upload(&c->d_gplan);
   if (e != cudaSuccess) {
     dfree(blk); dfree(xblk); dfree(work);
     free_zgroup(c);
     cudaGetLastError();
-    return fail(TN_ENOMEM, "grouped-line preconditioner needs %.2f GB: %s", (bb + xb + wb + 3 * fb) / 1e9,
+    return fail(TN_ENOMEM, "grouped-line preconditioner needs %.2f GB: %s", (bb + xb + wb + fb + fb64) / 1e9,
                 cudaGetErrorString(e));
   }
   ZGroupDev &g = c->zgd;
@@ -436,34 +437,29 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g.join[k], cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming);
-  g.lines = c->d_glines;
-  g.fac_off = c->d_gfac_off;
-  g.inst = is_batch(c) ? c->d_ginst : nullptr;
+  const unsigned char *dp = c->d_gplan;
+  g.lines = (const int4 *)(dp + o_lines);
+  g.fac_off = (const long long *)(dp + o_fac);
+  g.fac64_off = (const long long *)(dp + o_fac64);
+  g.queue = (int *)(c->d_gplan + o_queue);
+  g.chain_off = (const long long *)(dp + o_chain);
+  g.packs = (const int4 *)(dp + o_packs);
+  g.ranges = (const int4 *)(dp + o_ranges);
+  g.inst = is_batch(c) ? (const int *)(dp + o_inst) : nullptr;
   g.meshes = is_batch(c) ? c->batch->d_meshes : nullptr;
   g.dof_off = is_batch(c) ? c->batch->d_dof_off : nullptr;
-  g.ndof = (long long)c->ndof;
   g.ngroups = p.ngroups;
-  g.ncls = p.ncls;
-  for (int k = 0; k < p.ncls; ++k) {
-    g.cls_N[k] = p.cls_N[k]; g.cls_G[k] = p.cls_G[k]; g.cls_start[k] = p.cls_start[k]; g.cls_n[k] = p.cls_n[k];
-  }
-  g.packs = c->d_gpacks;
-  g.queue = c->d_gqueue;
+  g.chain = c->gchain;
+  g.nranges = (int)p.ranges.size();
   g.npk = p.npk;
-  for (int k = 0; k < p.npk; ++k) { g.pk_N[k] = p.pk_N[k]; g.pk_start[k] = p.pk_start[k]; g.pk_n[k] = p.pk_n[k]; }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_gpacks, p.packs.data(), sizeof(int4) * p.packs.size(),
-                                            cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_gqueue, 0, sizeof(int) * 2 * kZgMaxPk, st);
+  for (int k = 0; k < p.npk; ++k) {
+    g.pk_N[k] = p.pk_N[k]; g.pk_start[k] = p.pk_start[k]; g.pk_n[k] = p.pk_n[k];
+    g.rg_start[k] = p.rg_start[k]; g.rg_n[k] = p.rg_n[k];
+  }
   int status = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_glines, p.lines.data(), sizeof(int4) * p.ngroups,
-                                            cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_gfac_off, p.fac_off.data(), sizeof(long long) * p.ngroups,
-                                            cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && is_batch(c))
-    e = cudaMemcpyAsync(c->d_ginst, p.inst.data(), sizeof(int) * p.ngroups, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->gstatus, 0, 2 * sizeof(int), st);
   for (int i = 0; i < n && e == cudaSuccess; ++i)  // one mirror after another (shared set-up scratch)
-    e = tn_zgroup_setup(dms[i], p, c->zgd, i, c->d_glines, c->d_gfac_off, blk, xblk, work, c->gfac, c->gfac64,
+    e = tn_zgroup_setup(dms[i], p, c->zgd, i, blk, xblk, work, c->gfac, c->gfac64,
                         c->gstatus, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&status, c->gstatus, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -479,7 +475,7 @@ static OpSys with_groups(OpSys s, const tn_ctx *c) {
   s.grouped = true;
   s.fold_cnt = c->fold_cnt;
   s.zg = c->zgd;
-  s.n_rz_parts = c->zgd.ngroups;
+  s.n_rz_parts = 0;  // by precision: rz_parts
   s.zerr = c->wctl;
   return s;
 }
@@ -661,6 +657,7 @@ tn_status tn_create(tn_ctx **out, int device, void *cuda_stream) {
     e = tn_upload_lgl(&tabs);
     if (e == cudaSuccess) e = tn_upload_lgl_apply(&tabs);
     if (e == cudaSuccess) e = tn_upload_lgl_precond(&tabs);
+    if (e == cudaSuccess) e = tn_upload_lgl_zgroup(&tabs);
   }
   if (e != cudaSuccess) {
     tn_destroy(c);

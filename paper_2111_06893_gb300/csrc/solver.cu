@@ -444,7 +444,7 @@ static cudaError_t pcg_iteration_zline(const OpSys &sys, int prec, size_t n, Pcg
   TN_CU(cudaGetLastError());
   // r -= alpha q fused into the line solve (partials r.z and r.r)
   TN_CU(sys.zsolve(prec, v.zfac, v.r, v.q, v.z, &s->alpha, v.part_rz, &s->done, st));
-  k_beta_split<<<1, 1024, 0, st>>>(s, v.part_rz, sys.n_rz_parts, v.part_rz + sys.n_rz_parts, sys.n_rz_parts);
+  k_beta_split<<<1, 1024, 0, st>>>(s, v.part_rz, sys.rz_parts(prec), v.part_rz + sys.rz_parts(prec), sys.rz_parts(prec));
   TN_CU(cudaGetLastError());
   k_pupdate_x<T><<<red_blocks(), kRedThreads, 0, st>>>(s, n, (T *)v.x, (T *)v.p, (const T *)v.z);
   return cudaGetLastError();
@@ -473,8 +473,8 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
     TN_CU(sys.zsolve(prec, v.zfac, v.r, nullptr, v.z, nullptr, v.part_rz, nullptr, st));
     k_copy<T><<<red_blocks(), kRedThreads, 0, st>>>(n, (T *)v.p, (const T *)v.z);
     TN_CU(cudaGetLastError());
-    k_init_scalars_split<<<1, 256, 0, st>>>(s_dev, v.part_rz, sys.n_rz_parts, v.part_rz + sys.n_rz_parts,
-                                            sys.n_rz_parts, rtol * rtol, max_iters);
+    k_init_scalars_split<<<1, 256, 0, st>>>(s_dev, v.part_rz, sys.rz_parts(prec), v.part_rz + sys.rz_parts(prec),
+                                            sys.rz_parts(prec), rtol * rtol, max_iters);
   } else {
     k_init<T><<<red_blocks(), kRedThreads, 0, st>>>(n, (const T *)v.b, Ax, (T *)v.r, (T *)v.z, (T *)v.p,
                                                   (const T *)v.dinv, part_red);
@@ -696,7 +696,7 @@ cudaError_t OpSys::apply(int prec, const void *u, void *y, double *part, cudaStr
 
 cudaError_t OpSys::zsolve(int prec, const void *fac, void *r, const void *q, void *z, const double *alpha,
                           double *part, const int *done, cudaStream_t st, const PcgFold *fold) const {
-  double *prr = part ? part + n_rz_parts : nullptr;
+  double *prr = part ? part + rz_parts(prec) : nullptr;
   if (grouped) return tn_zgroup_solve(m, zg, prec, fac, r, z, part, prr, done, zerr, st, fold);
   if (m) return tn_zline_solve(*m, prec, fac, r, q, z, alpha, part, prr, done, zerr, st);
   for (int g = 0; g < ngroups; ++g) {

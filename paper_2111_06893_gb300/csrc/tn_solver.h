@@ -28,7 +28,8 @@ struct OpSys {
   void *trace = nullptr;  // traction scratch of the operator (FP64-sized; FP32 applies use half of it)
   const long long *tr_off = nullptr;  // batch: first trace entry of every mirror
   int n_elems = 0;        // elements of the mesh or of the whole batch
-  int n_rz_parts = 0;     // partial sums of r.z written by one z-line solve (r.r: as many, after them)
+  int n_rz_parts = 0;     // single lines: partial sums of r.z written by one solve (r.r: as many, after them)
+  int rz_parts(int prec) const { return grouped ? tn_zgroup_partials(zg, prec) : n_rz_parts; }
   TnWait *zerr = nullptr; // wait limit of the line solves; flag set by one whose staging wait ran out
   unsigned *fold_cnt = nullptr;  // grouped lines: 2 counters of the alpha / beta steps folded into
                                  // the apply and the line solve
@@ -45,8 +46,8 @@ struct OpSys {
                         const PcgFold *fold = nullptr) const;
   cudaError_t apply_traces(int prec, void *y, void *r, const double *alpha, const int *done, cudaStream_t st) const;
   cudaError_t apply(int prec, const void *u, void *y, double *part, cudaStream_t st) const;
-  // z = M^{-1} r; q != nullptr: first r <- r - (*alpha) q.  part: n_rz_parts
-  // partial r.z, then n_rz_parts partial r.r
+  // z = M^{-1} r; q != nullptr: first r <- r - (*alpha) q.  part: rz_parts
+  // partial r.z, then rz_parts partial r.r
   cudaError_t zsolve(int prec, const void *fac, void *r, const void *q, void *z, const double *alpha,
                      double *part, const int *done, cudaStream_t st, const PcgFold *fold = nullptr) const;
 };
@@ -56,7 +57,7 @@ struct PcgVectors {
   void *x, *r, *z, *p, *q;
   const void *b, *dinv;
   const void *zfac = nullptr;   // z-line factors of the run's precision (nullptr: Jacobi)
-  double *part_rz = nullptr;    // partial r.z and r.r of the z-line solve (2 n_rz_parts)
+  double *part_rz = nullptr;    // partial r.z and r.r of the z-line solve (2 rz_parts)
 };
 
 cudaError_t tn_jacobi_apply(size_t n, int prec, const double *diag, const void *r, void *z, cudaStream_t st);

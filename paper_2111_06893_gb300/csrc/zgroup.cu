@@ -1,0 +1,1631 @@
+// Grouped-line block preconditioner (the default of the Krylov solves): plan,
+// set-up and solve.  See precond.cu for the single-line form it extends.
+#include <algorithm>
+#include <cstdio>
+#include <type_traits>
+#include <vector>
+
+#include "tn_device.h"
+#include "tn_internal.h"
+#include "tn_precond.h"
+
+// device constants are per translation unit (no relocatable device code):
+// this file keeps its own copy of the LGL tables
+__constant__ LglTables c_lgl_zg;
+
+cudaError_t tn_upload_lgl_zgroup(const LglTables *t) { return cudaMemcpyToSymbol(c_lgl_zg, t, sizeof(LglTables)); }
+
+namespace {
+
+#define LD(a, b) c_lgl_zg.D[N][(a) * N + (b)]
+#define LW(a) c_lgl_zg.w[N][(a)]
+
+// The lines through the matching nodes of two columns that share a lateral
+// face are coupled by that face's interior-penalty and flux terms (Eqs.
+// (numflux), (penalty)), which the single-line blocks leave out; with the
+// penalty ~ C (p + 1)^2 / h these are the stiffest couplings left.  A group
+// is a set of lines joined by such face matches (1 to 4 lines: a node inside
+// a column face, on a column edge or at a corner where up to four columns
+// meet); its block is the exact principal sub-matrix of A on all its lines,
+// again block tridiagonal over the slabs, with 3 g N unknowns per slab and
+// the cross-line face terms in the diagonal blocks.
+
+// Cross-line block of element e = (s, c), lateral face f and face position t:
+// rows = the line through the face node (this element), columns = the line
+// through the matching node of the neighbour column (same slab):
+//   -1/2 V^T W Tr_ext + 1/2 Tr^T W V_ext - V^T W Pen V_ext
+// restricted to the two lines (the neighbour's traction and this element's
+// test traction reduce to the zeta derivative and the diagonal xi / eta
+// derivative entries on a line).  Zero where f has no neighbour.
+template <int N>
+__global__ void zgroup_cross_kernel(const DevMesh m, double *__restrict__ xblk) {
+  constexpr int M = 3 * N, N2 = N * N;
+  const int e = blockIdx.x, t = threadIdx.x % N, f = threadIdx.x / N;
+  if (f >= 4) return;
+  const int s = e / m.ncol, c = e - s * m.ncol;
+  double *X = xblk + (((size_t)e * 4 + f) * N + t) * M * M;
+  for (int q = 0; q < M * M; ++q) X[q] = 0.0;
+  const int nbc = m.colnb[4 * c + f];
+  if (nbc < 0) return;
+  const int d = f >> 1, sd = f & 1, end = sd ? N - 1 : 0;
+  const int i = d == 0 ? end : t, j = d == 0 ? t : end;
+  const int code = m.colnbf[4 * c + f];
+  const int f2 = code & 3, d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0;
+  const int a2 = (code >> 2) ? N - 1 - t : t;
+  const int i2 = d2 == 0 ? end2 : a2, j2 = d2 == 0 ? a2 : end2;
+  const double *cg = m.colgeo + (size_t)c * CG_NF * N2;
+  const double *cg2 = m.colgeo + (size_t)nbc * CG_NF * N2;
+  const int q1 = j * N + i, q2 = j2 * N + i2;
+  const double ixx = cg[CG_IXX * N2 + q1], ixy = cg[CG_IXY * N2 + q1];
+  const double iex = cg[CG_IEX * N2 + q1], iey = cg[CG_IEY * N2 + q1], det2 = cg[CG_DET * N2 + q1];
+  const double jxx = cg2[CG_IXX * N2 + q2], jxy = cg2[CG_IXY * N2 + q2];
+  const double jex = cg2[CG_IEX * N2 + q2], jey = cg2[CG_IEY * N2 + q2];
+  const double *sg = m.slabgeo + (size_t)s * SG_NF * N;
+  double dz[N];
+  for (int k = 0; k < N; ++k) dz[k] = sg[SG_DZ * N + k];
+  const int L = m.slab_layer[s];  // both sides lie in slab s: one material
+  const double c11 = m.layer_c[3 * L], c12 = m.layer_c[3 * L + 1], c44 = m.layer_c[3 * L + 2];
+  const double rx = d == 0 ? ixx : iex, ry = d == 0 ? ixy : iey;
+  const double mag = sqrt(rx * rx + ry * ry);
+  const double n[3] = {(sd ? 1.0 : -1.0) * rx / mag, (sd ? 1.0 : -1.0) * ry / mag, 0.0};
+  const double sx = d2 == 0 ? jxx : jex, sy = d2 == 0 ? jxy : jey;
+  const double h = 2.0 / mag, h2 = 2.0 / sqrt(sx * sx + sy * sy);
+  const double sig = (double)((m.p + 1) * (m.p + 1)) * m.penC / (h < h2 ? h : h2);
+  const double Dii = LD(i, i), Djj = LD(j, j), Dii2 = LD(i2, i2), Djj2 = LD(j2, j2);
+  const double wt = d == 0 ? LW(j) : LW(i);
+  for (int k = 0; k < N; ++k) {
+    const double Wk = wt * LW(k) * det2 * dz[k] * mag;
+    for (int k2 = 0; k2 < N; ++k2) {
+      const double Wk2 = wt * LW(k2) * det2 * dz[k2] * mag;
+      // neighbour basis (i2, j2, k2) at its node (i2, j2, k); own basis (i, j, k) at (i, j, k2)
+      const double l2[3] = {k2 == k ? Dii2 : 0.0, k2 == k ? Djj2 : 0.0, LD(k, k2)};
+      const double l1[3] = {k == k2 ? Dii : 0.0, k == k2 ? Djj : 0.0, LD(k2, k)};
+      double g2[3], g1[3];
+      phys(l2, jxx, jxy, jex, jey, dz[k], g2);
+      phys(l1, ixx, ixy, iex, iey, dz[k2], g1);
+      for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b) {
+          double v = -0.5 * Wk * Qab(a, b, n, g2, c11, c12, c44) + 0.5 * Wk2 * Qab(b, a, n, g1, c11, c12, c44);
+          if (k == k2) v -= Wk * sig * Qab(a, b, n, n, c11, c12, c44);
+          X[(a * N + k) * M + b * N + k2] = v;
+        }
+    }
+  }
+}
+
+// FP32 record of slab s: [S_s^{-1} packed by columns (lower triangle,
+// zlp(MG)) | O_{s-1} in factored form (8 MG) | W_s], S_s = L_s L_s^T the
+// slab's Schur complement of the block Cholesky (S_s^{-1} = Linv_s^T
+// Linv_s).  The coupling block O_{s-1} (rows: slab s - 1,
+// columns: slab s, block diagonal over the lines) is nonzero only in the
+// rows of the bottom-face nodes (k = 0) and the columns of the top-face
+// nodes (k2 = N - 1) of each line (Eqs. (numflux), (penalty) on the zeta
+// face), so O = E_0 X^T + Y E_{N-1}^T with per row t: X[t][a] = O[(a, 0), t]
+// and Y[t][b] = O[t, (b, N - 1)] (Y zero on k = 0 rows).  Row t stores
+// X[t][0..2], 0, Y[t][0..2], 0.  The solve applies the coupling through
+// these factors instead of storing Z_s = Linv_{s-1} O_{s-1} densely.
+// The record ends with the backward sweep's coupling W_s = S_s^{-1} [Y_s | E_0]
+// (MG x 6G, rows padded to zp_ws(G)), S_s = L_s L_s^T the slab's Schur
+// complement and Y_s, E_0 of O_s (the coupling to slab s + 1): per line l,
+// column 6 l + b holds Y of component b and column 6 l + 3 + a the unit
+// vector of row (a, k = 0); zero for the last slab.  With it the backward
+// step x_s = Linv_s^T (y_s - Linv_s O_s x_{s+1}) = w_s - W_s v, v the six
+// numbers per line x_{s+1}(b, N - 1) and X^T x_{s+1}.
+__host__ __device__ constexpr int zp_ws(int G) { return pad4(6 * G); }
+__host__ __device__ constexpr int zp_rec(int MG, int G) { return zlp(MG) + 8 * MG + MG * zp_ws(G); }
+
+// FP64 solve.  The block O_{s-1} (rows: slab s - 1, columns: slab s, block
+// diagonal over the lines) is nonzero only in the rows of the bottom-face
+// nodes (k = 0) and the columns of the top-face nodes (k = N - 1) of each line
+// (Eqs. (numflux), (penalty) on the zeta face), so O_{s-1} = U_{s-1} V_s^T
+// with six columns per line l: U = [Y | E_0] (column 6 l + b: Y of component
+// b; 6 l + 3 + a: the unit vector of row (a, k = 0)) and V = [E_{N-1} | X]
+// (6 l + b: the unit vector of row (b, k = N - 1); 6 l + 3 + a: X of component
+// a).  Only the zeta derivative couples away from the face node, so with D
+// the derivative matrix
+//   Y[(b, k)][b] = y_b D(0, k), k != 0;      X[(a, k)][a] = x_a D(N-1, k), k != N-1
+// and X has a full 3 x 3 block in the rows k = N - 1 (all else zero): 15
+// numbers per line.
+//
+// Elimination, S_s the slab's Schur complement, W_s = S_s^{-1} U_s and Q_s =
+// S_s^{-1} V_s:
+//   w_s = S_s^{-1} (r_s - V_s g_{s-1}),   g_s = U_s^T w_s
+//   x_s = w_s - W_s f_{s+1},              f_s = V_s^T x_s
+// As written (the FP32 solve) each slab waits for the full solve of the one
+// above it (forward) or below it (backward): two chains of S dense products.
+// But only the 6 g numbers g and f cross an interface:
+//   a_s = S_s^{-1} r_s,   c_s = U_s^T a_s,   d_s = V_s^T a_s
+//   g_s = c_s - K_s g_{s-1},   f_s = d_s - H_s g_{s-1} - K_s^T f_{s+1}
+//   x_s = a_s - Q_s g_{s-1} - W_s f_{s+1}
+// with K_s = W_s^T V_s and H_s = V_s^T Q_s (6 g x 6 g).  The dense products of
+// all slabs are independent, and the chains run on 6 g numbers per step.
+// The factors grow (12 g entries more per row, 72 g^2 more per slab) and the
+// arithmetic shrinks: FP64 is bound by its arithmetic (an FP64 instruction
+// occupies the pipe for 16 cycles whether 6 or 32 lanes are on, and the chain
+// form spends most of them on packed triangles of few lanes), FP32 by the
+// latency and bytes of the factors, so FP64 takes this form and FP32 the one
+// above (FP64 | FP32, us: 2.0 M unknowns at p = 6: 669 -> 383 | 122 -> 176;
+// p = 7, 11 slabs: 173 -> 156 | 48 -> 68; p = 4 box, 12288: 30 -> 19 | 13 -> 11).
+//
+// Factors of a group, three arrays in turn, every record padded to 16 bytes:
+//   S_s^{-1}, s < S: by circulant diagonals, entry m MG + t = S^{-1}[t][(t + m)
+//        mod MG], m = 0 .. MG / 2 (each entry of the symmetric matrix once, the
+//        last diagonal of an even MG twice): a row reads two conflict-free
+//        entries per diagonal.  Then 16 numbers per line of the coupling:
+//        y_b of interface s, x_a of interface s - 1, X's 3 x 3 block [b][a]
+//   (Q_s | W_s)^T, s < S: 12 g rows of pad4(MG) (Q_0 and W_{S-1} zero)
+//   K_s | H_s, s < S: K by rows of odd stride 6 g + 1, H by rows of 6 g (used:
+//        K_1 .. K_{S-2}, H_1 .. H_{S-1})
+__host__ __device__ constexpr int zg_ld(int G) { return 6 * G + 1; }
+__host__ __device__ constexpr int zg_circ(int MG) { return MG * (MG / 2 + 1); }
+__host__ __device__ constexpr int zg_srec(int MG, int G) { return pad4(zg_circ(MG)) + 16 * G; }
+__host__ __device__ constexpr int zg_qrec(int MG, int G) { return 12 * G * pad4(MG); }
+__host__ __device__ constexpr int zg_kpart(int G) { return pad4(6 * G * zg_ld(G)); }
+__host__ __device__ constexpr int zg_krec(int G) { return zg_kpart(G) + 36 * G * G; }
+__host__ __device__ constexpr long long zg_qoff(int MG, int G, int S) { return (long long)S * zg_srec(MG, G); }
+__host__ __device__ constexpr long long zg_koff(int MG, int G, int S) {
+  return zg_qoff(MG, G, S) + (long long)S * zg_qrec(MG, G);
+}
+__host__ __device__ constexpr long long zg_entries(int MG, int G, int S) {
+  return zg_koff(MG, G, S) + (long long)S * zg_krec(G);
+}
+
+
+// block Cholesky along the slabs of one group (one CTA; FP64 working
+// matrices G and Linv of (3 g N)^2 entries each and the (6 g)^2 C in
+// `work`), then the FP32 records and the FP64 factors
+template <int N>
+__global__ void __launch_bounds__(128)
+zgroup_factor_kernel(const DevMesh m, const int4 *__restrict__ glines, const long long *__restrict__ gfac,
+                     int gbase, int g, const double *__restrict__ blk, const double *__restrict__ xblk,
+                     double *__restrict__ work, float *__restrict__ fac, const long long *__restrict__ gfac64,
+                     double *__restrict__ fac64, int *__restrict__ status) {
+  constexpr int M = 3 * N, N2 = N * N;
+  const int grp = gbase + blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
+  const int MG = g * M, S = m.nslab, MGP = pad4(MG), KS = zg_ld(g), G6 = 6 * g;
+  double *Gm = work + (size_t)blockIdx.x * 3 * MG * MG, *Li = Gm + MG * MG, *Cm = Li + MG * MG;
+  __shared__ int lid[4], xof[4][4];
+  if (tid < 4) {
+    const int4 L4 = glines[grp];
+    lid[tid] = tid == 0 ? L4.x : (tid == 1 ? L4.y : (tid == 2 ? L4.z : L4.w));
+  }
+  __syncthreads();
+  if (tid < 16) {  // which face block couples line t1 (rows) to line t2 (columns)
+    const int t1 = tid >> 2, t2 = tid & 3;
+    int x = -1;
+    if (t1 < g && t2 < g && t1 != t2) {
+      const int c1 = lid[t1] / N2, qq = lid[t1] - c1 * N2, i1 = qq % N, j1 = qq / N;
+      for (int f = 0; f < 4; ++f) {
+        const int nbc = m.colnb[4 * c1 + f];
+        const int d = f >> 1, end = (f & 1) ? N - 1 : 0;
+        if (nbc < 0 || (d == 0 ? i1 : j1) != end) continue;
+        const int tp = d == 0 ? j1 : i1;
+        const int code = m.colnbf[4 * c1 + f], f2 = code & 3, d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0;
+        const int a2 = (code >> 2) ? N - 1 - tp : tp;
+        const int i2 = d2 == 0 ? end2 : a2, j2 = d2 == 0 ? a2 : end2;
+        if (nbc * N2 + j2 * N + i2 == lid[t2]) x = f * N + tp;
+      }
+    }
+    xof[t1][t2] = x;
+  }
+  __syncthreads();
+  float *const f32 = fac + gfac[grp];
+  double *const f64 = fac64 + gfac64[grp];
+  const int RS = zp_rec(MG, g), LP = zlp(MG), WS = zp_ws(g);
+  const int SR = zg_srec(MG, g), QR = zg_qrec(MG, g), KR = zg_krec(g), KP = zg_kpart(g), LC = pad4(zg_circ(MG));
+  const long long qo = zg_qoff(MG, g, S), ko = zg_koff(MG, g, S);
+  // O_s of line l (rows: slab s)
+  auto Oblk = [&](int l, int s) { return blk + (((size_t)lid[l] * S + s) * 2 + 1) * M * M; };
+  // column j of V_s applied: sum_p V_s[p][j] f(p), f indexed by rows of the group
+  auto dotV = [&](int s, int j, auto f) {
+    const int l = j / 6, jj = j - l * 6;
+    if (jj < 3) return f(l * M + jj * N + N - 1);
+    const double *O = Oblk(l, s - 1) + ((jj - 3) * N) * M;
+    double acc = 0.0;
+    for (int k = 0; k < N - 1; ++k) acc += O[(jj - 3) * N + k] * f(l * M + (jj - 3) * N + k);
+    for (int b = 0; b < 3; ++b) acc += O[b * N + N - 1] * f(l * M + b * N + N - 1);
+    return acc;
+  };
+  // column j of U_s applied
+  auto dotU = [&](int s, int j, auto f) {
+    const int l = j / 6, jj = j - l * 6;
+    if (jj >= 3) return f(l * M + (jj - 3) * N);
+    const double *O = Oblk(l, s);
+    double acc = 0.0;
+    for (int k = 1; k < N; ++k) acc += O[(jj * N + k) * M + jj * N + N - 1] * f(l * M + jj * N + k);
+    return acc;
+  };
+  for (int s = 0; s < S; ++s) {
+    // Schur complement of slab s: the diagonal block (line blocks, cross-line
+    // face blocks) minus V_s C V_s^T, C = U_{s-1}^T W_{s-1} (6g x 6g); a row of
+    // V has at most four nonzeros
+    if (s > 0) {
+      const double *Wp = f64 + qo + (long long)(s - 1) * QR + G6 * MGP;
+      for (int q = tid; q < G6 * G6; q += nth) {
+        const int i = q / G6, j = q - i * G6;
+        Cm[q] = dotU(s - 1, i, [&](int p) { return Wp[(size_t)j * MGP + p]; });
+      }
+      __syncthreads();
+    }
+    for (int q = tid; q < MG * MG; q += nth) {
+      const int r = q / MG, cc = q - r * MG, t1 = r / M, t2 = cc / M, rr = r - t1 * M, c2 = cc - t2 * M;
+      double v = 0.0;
+      if (t1 == t2) {
+        v = blk[(((size_t)lid[t1] * S + s) * 2 + 0) * M * M + rr * M + c2];
+      } else if (xof[t1][t2] >= 0) {
+        const size_t e = (size_t)s * m.ncol + lid[t1] / N2;
+        v = xblk[(e * 4 * N + xof[t1][t2]) * M * M + rr * M + c2];
+      }
+      if (s > 0) {  // the nonzeros of V's rows r and cc: (column, value)
+        int ir[4], ic[4];
+        double vr[4], vc[4];
+        int nr = 0, nc = 0;
+        const double *Or = Oblk(t1, s - 1), *Oc = Oblk(t2, s - 1);
+        if (rr % N == N - 1) { ir[nr] = 6 * t1 + rr / N; vr[nr++] = 1.0; }
+        if (c2 % N == N - 1) { ic[nc] = 6 * t2 + c2 / N; vc[nc++] = 1.0; }
+        for (int a = 0; a < 3; ++a) {
+          if (a == rr / N || rr % N == N - 1) { ir[nr] = 6 * t1 + 3 + a; vr[nr++] = Or[(a * N) * M + rr]; }
+          if (a == c2 / N || c2 % N == N - 1) { ic[nc] = 6 * t2 + 3 + a; vc[nc++] = Oc[(a * N) * M + c2]; }
+        }
+        double sum = 0.0;
+        for (int x = 0; x < nr; ++x) {
+          double row = 0.0;
+          for (int y = 0; y < nc; ++y) row += Cm[ir[x] * G6 + ic[y]] * vc[y];
+          sum += vr[x] * row;
+        }
+        v -= sum;
+      }
+      Gm[q] = v;
+    }
+    __syncthreads();
+    // Cholesky, lower triangle in place
+    for (int col = 0; col < MG; ++col) {
+      if (tid == 0) {
+        double dv = Gm[col * MG + col];
+        if (!(dv > 0.0)) {
+          atomicExch(status, 1);
+          dv = 1e-300;
+        }
+        Gm[col * MG + col] = sqrt(dv);
+      }
+      __syncthreads();
+      const double piv = Gm[col * MG + col];
+      for (int r = col + 1 + tid; r < MG; r += nth) Gm[r * MG + col] /= piv;
+      __syncthreads();
+      const int w = MG - col - 1;
+      for (int q = tid; q < w * w; q += nth) {
+        const int r = col + 1 + q / w, c2 = col + 1 + q % w;
+        if (c2 <= r) Gm[r * MG + c2] -= Gm[r * MG + col] * Gm[c2 * MG + col];
+      }
+      __syncthreads();
+    }
+    // Linv = L^{-1}, one column per thread (forward substitution on the
+    // identity); its upper triangle is zero (read by the products below)
+    for (int cc = tid; cc < MG; cc += nth) {
+      for (int r = 0; r < cc; ++r) Li[r * MG + cc] = 0.0;
+      for (int r = cc; r < MG; ++r) {
+        double acc = r == cc ? 1.0 : 0.0;
+        for (int p = cc; p < r; ++p) acc -= Gm[r * MG + p] * Li[p * MG + cc];
+        Li[r * MG + cc] = acc / Gm[r * MG + r];
+      }
+    }
+    __syncthreads();
+    for (int q = tid; q < MG * MG; q += nth) {  // S^{-1} = Linv^T Linv, in place of L
+      const int r = q / MG, cc = q - r * MG;
+      if (r < cc) continue;
+      double acc = 0.0;
+      for (int p = r; p < MG; ++p) acc += Li[p * MG + r] * Li[p * MG + cc];
+      Gm[r * MG + cc] = acc;
+      Gm[cc * MG + r] = acc;
+    }
+    __syncthreads();
+    float *const R = f32 + (long long)s * RS;
+    for (int q = tid; q < MG * MG; q += nth) {  // S^{-1}, packed lower triangle
+      const int r = q / MG, cc = q - r * MG;
+      if (r >= cc) R[zcol(MG, cc) + r - cc] = (float)Gm[q];
+    }
+    for (int q = MG * (MG + 1) / 2 + tid; q < LP; q += nth) R[q] = 0.0f;
+    for (int q = tid; q < 8 * MG; q += nth) {  // factors of O_{s-1}
+      const int t = q >> 3, j = q & 7, l = t / M, tl = t - l * M, tk = tl % N;
+      double v = 0.0;
+      if (s > 0 && (j & 3) < 3) {
+        const double *O = Oblk(l, s - 1);
+        if (j < 4) v = O[(j * N) * M + tl];                        // X[t][a] = O[(a, 0), t]
+        else if (tk != 0) v = O[tl * M + (j - 4) * N + (N - 1)];  // Y[t][b] = O[t, (b, N - 1)]
+      }
+      R[LP + q] = (float)v;
+    }
+    double *Sd = f64 + (long long)s * SR;
+    for (int q = tid; q < SR; q += nth) {
+      double v = 0.0;
+      if (q < zg_circ(MG)) {
+        const int mm = q / MG, t = q - mm * MG, c = t + mm < MG ? t + mm : t + mm - MG;
+        v = Gm[t * MG + c];
+      } else if (q >= LC) {
+        const int l = (q - LC) / 16, i = (q - LC) - l * 16;
+        if (i < 3) {
+          if (s + 1 < S) v = Oblk(l, s)[(i * N + 1) * M + i * N + N - 1] / c_lgl_zg.D[N][1];  // Y[(b, 1)][b] / D(0, 1)
+        } else if (s > 0 && i < 6) {
+          const int a = i - 3;  // X[(a, 0)][a] / D(N-1, 0)
+          v = Oblk(l, s - 1)[(a * N) * M + a * N] / c_lgl_zg.D[N][(N - 1) * N];
+        } else if (s > 0 && i < 15) {
+          const int b = (i - 6) / 3, a = (i - 6) % 3;
+          v = Oblk(l, s - 1)[(a * N) * M + b * N + N - 1];
+        }
+      }
+      Sd[q] = v;
+    }
+    // (Q_s | W_s)^T = (V_s | U_s)^T S_s^{-1}
+    double *Qd = f64 + qo + (long long)s * QR;
+    for (int q = tid; q < QR; q += nth) {
+      const int j = q / MGP, t = q - j * MGP;
+      double v = 0.0;
+      if (t < MG) {
+        auto row = [&](int p) { return Gm[p * MG + t]; };
+        if (j < G6) {
+          if (s > 0) v = dotV(s, j, row);
+        } else if (s + 1 < S) {
+          v = dotU(s, j - G6, row);
+        }
+      }
+      Qd[q] = v;
+    }
+    __syncthreads();
+    for (int q = tid; q < MG * WS; q += nth) {  // W_s by rows
+      const int t = q / WS, j = q - t * WS;
+      R[LP + 8 * MG + q] = j < G6 ? (float)Qd[(G6 + j) * MGP + t] : 0.0f;
+    }
+    // K_s = W_s^T V_s, H_s = V_s^T Q_s
+    double *Kd = f64 + ko + (long long)s * KR;
+    for (int q = tid; q < KR; q += nth) {
+      double v = 0.0;
+      if (s > 0) {
+        if (q < KP) {
+          const int i = q / KS, j = q - i * KS;
+          if (i < G6 && j < G6) v = dotV(s, j, [&](int p) { return Qd[(G6 + i) * MGP + p]; });
+        } else {
+          const int i = (q - KP) / G6, j = (q - KP) - i * G6;
+          v = dotV(s, i, [&](int p) { return Qd[j * MGP + p]; });
+        }
+      }
+      Kd[q] = v;
+    }
+    __syncthreads();
+  }
+}
+
+// ---- the FP32 solve: packed slots, one launch per degree
+// A group of G lines (3 G N rows per slab) is solved by a slot of G warps,
+// one row per thread.  A CTA of four warps takes one pack at a time from a
+// queue: one group of 4 lines, 3 + 1, 2 + 2, 2 + 1 + 1 or 1 + 1 + 1 + 1
+// lines, largest packs first.  Each slot syncs with its own named barrier
+// (a warp with __syncwarp) and streams its factor records through a ring of
+// P stages in shared memory (bulk copies completing on one mbarrier per
+// stage), so that up to P - 1 copies are in flight while one stage is used:
+// small groups, whose per-slab work is short, get the deepest rings.
+constexpr int kZgThreads = 128;  // four warps per CTA
+constexpr int kZgMaxStages = 8;
+
+// floats of staging per warp: two records of the largest group
+// (4 lines) across the four warps of a CTA, so that six CTAs (FP32, N = 7)
+// share an SM; smaller groups fit more stages in the same room
+// stage buffer of a group of G lines: the larger of the forward stage
+// (S_s^{-1} and the O factors of record s) and the backward stage (W_s and
+// the O factors of record s + 1)
+template <int N, int G>
+__host__ __device__ constexpr int zp_stage() {
+  return (zlp(3 * G * N) > 3 * G * N * zp_ws(G) ? zlp(3 * G * N) : 3 * G * N * zp_ws(G)) + 8 * 3 * G * N;
+}
+template <int N>
+__host__ __device__ constexpr int zp_stage_per_warp() {
+  return pad4((zp_stage<N, 4>() * 2 + 3) / 4);
+}
+template <int N>
+constexpr size_t zp_smem() {
+  return (4 * (size_t)zp_stage_per_warp<N>() + 4 * kZgThreads) * sizeof(float) + 4 * kZgMaxStages * 8;
+}
+
+// barrier of a slot of G > 1 warps starting at warp w0 of its CTA.  Immediate
+// barrier numbers: a number in a register claims all 16 of the CTA.
+template <int G>
+__device__ __forceinline__ void slot_sync(int w0) {
+  if (G == 1) __syncwarp();
+  else if (w0 == 0) asm volatile("bar.sync 1, %0;\n" ::"n"(32 * G) : "memory");
+  else asm volatile("bar.sync 2, %0;\n" ::"n"(32 * G) : "memory");
+}
+// true if p holds on any thread of the slot (and a sync)
+template <int ID, int NT>
+__device__ __forceinline__ bool named_any(bool p) {
+  unsigned r;
+  asm volatile(
+      "{\n .reg .pred q, o;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred o, %2, %3, q;\n selp.u32 %0, 1, 0, o;\n}\n"
+      : "=r"(r)
+      : "r"((unsigned)p), "n"(ID), "n"(NT)
+      : "memory");
+  return r != 0;
+}
+template <int G>
+__device__ __forceinline__ bool slot_any(int w0, bool p) {
+  if (G == 1) return __any_sync(0xffffffffu, p);
+  return w0 == 0 ? named_any<1, 32 * G>(p) : named_any<2, 32 * G>(p);
+}
+__device__ __forceinline__ void mbar_inval(unsigned long long *bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// three warp-wide sums at once: the three butterflies interleaved level by
+// level, so that their shuffles overlap instead of running one sum after
+// the other (every lane gets the three sums)
+__device__ __forceinline__ void warp_allsum3(float &a, float &b, float &c) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float a2 = __shfl_xor_sync(0xffffffffu, a, o);
+    const float b2 = __shfl_xor_sync(0xffffffffu, b, o);
+    const float c2 = __shfl_xor_sync(0xffffffffu, c, o);
+    a += a2;
+    b += b2;
+    c += c2;
+  }
+}
+
+// z = A_GG^{-1} r on group grp by the slot of G warps starting at warp w0;
+// line li of the group is warp w0 + li, its rows (a, k) lanes a N + k < 3N:
+//   forward   y_s = Linv_s (r_s - O_{s-1}^float w_{s-1}),  w_s = Linv_s^float y_s
+//   backward  x_s = Linv_s^float (y_s - Linv_s O_s x_{s+1}) = w_s - W_s v_{s+1}
+// (v: six numbers per line, x_{s+1}(b, N - 1) and X^float x_{s+1}).  The forward
+// step forms w_s = S_s^{-1} b_s, b_s = r_s - O_{s-1}^float w_{s-1}, in one
+// symmetric product, and r.z = sum_s |y_s|^2 = sum_s b_s . w_s.  O in its
+// factored form acts line by line (it is block diagonal over the lines), so
+// its products are warp shuffles and warp sums; S_s^{-1} b_s and W_s v cross
+// lines, through broadcast vectors in shared memory (double-buffered by step
+// parity).  Stage u < S: S_u^{-1} and the O factors of record u; stage u >= S:
+// W_s of record s and the O factors of record s + 1, s = 2S - 2 - u.  Stage u
+// uses ring buffer u % P and mbarrier u % P with phase parity (u / P) & 1.
+// Writes the group's partial r.z (= |y|^2) and r.r.  A wait that runs
+// out sets err->flag and ends the slot after bounded waits for the copies in
+// flight.
+template <int N, int G>
+__device__ __forceinline__ void zp_slot(int grp, int w0, int mncol, int S, const float *__restrict__ r,
+                                        float *__restrict__ z, const int4 *__restrict__ glines,
+                                        const long long *__restrict__ gfac, const float *__restrict__ fac,
+                                        float *__restrict__ stage, int cap, float *__restrict__ vecs,
+                                        unsigned long long *__restrict__ bars, double *__restrict__ psum,
+                                        unsigned long long lim, TnWait *__restrict__ err, double *__restrict__ part_rz,
+                                        double *__restrict__ part_rr) {
+  constexpr int M = 3 * N, N2 = N * N, n = N * N * N, MG = G * M, NT = 32 * G;
+  constexpr int LP = zlp(MG), RS = zp_rec(MG, G), WS = zp_ws(G), RSS = zp_stage<N, G>();
+  constexpr int LPX = LP + 8 * MG;  // forward stage: S_s^{-1} and the O factors of record s
+  constexpr int BW = MG * WS;       // backward stage: W_s, then the O factors of record s + 1
+  const int lt = threadIdx.x - 32 * w0;
+  auto sync = [&]() { slot_sync<G>(w0); };
+  auto any = [&](bool p) { return slot_any<G>(w0, p); };
+  const int li = lt >> 5, lane = lt & 31;
+  const bool act = lane < M;
+  const int t = li * M + (act ? lane : 0);  // row of the group's blocks
+  const int a = (act ? lane : 0) / N, k = (act ? lane : 0) - a * N;
+  // broadcast vectors hold line lj's M entries at 32 lj (16-byte aligned)
+  float *const vbuf = vecs + 4 * 32 * w0;  // [2 parities][vb][32 G] (room for 2 x 2 x 32 G)
+  auto vb = [&](int par) { return vbuf + par * 2 * NT; };
+  const int4 L4 = glines[grp];
+  const int lid = li == 0 ? L4.x : (li == 1 ? L4.y : (li == 2 ? L4.z : L4.w));
+  const int c = lid / N2, qn = lid - c * N2;
+  // vector entry of this row in slab s: g0 + s * gs
+  const size_t gs = (size_t)mncol * 3 * n, g0 = ((size_t)c * 3 + a) * n + (size_t)k * N2 + qn;
+  auto gidx = [&](int s) { return g0 + (size_t)s * gs; };
+  const float *base = fac + gfac[grp];
+  const int total = 2 * S;
+  int P = cap / RSS;
+  P = P > kZgMaxStages ? kZgMaxStages : P;
+  P = P > total ? total : P;
+  // stage sources: forward stage u = S_u^{-1} and O factors of record u;
+  // backward stage u (slab s = 2S - 2 - u < S - 1) = W_s of record s and the
+  // O factors of record s + 1 (the last slab, s = S - 1, needs no stage)
+  const int total_st = 2 * S - 1;
+  int issued = 0, ib = 0;  // stages issued so far and the ring buffer of the next (same in every thread)
+  const float *src = base;     // lane 0: the next stage's (first) source
+  auto issue_next = [&]() {
+    if (issued >= total_st) return;
+    const int u = issued++, b = ib;
+    ib = ib + 1 == P ? 0 : ib + 1;
+    if (lt == 0) {
+      float *dst = stage + (size_t)b * RSS;
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      if (u < S) {
+        mbar_expect(bars + b, (unsigned)(LPX * sizeof(float)));
+        bulk_g2s(dst, src, (unsigned)(LPX * sizeof(float)), bars + b);
+        src = u + 1 < S ? src + RS : src - RS;  // then the backward stages from record S - 2 down
+      } else {
+        mbar_expect(bars + b, (unsigned)((BW + 8 * MG) * sizeof(float)));
+        bulk_g2s(dst, src + LPX, (unsigned)(BW * sizeof(float)), bars + b);
+        bulk_g2s(dst + BW, src + RS + LP, (unsigned)(8 * MG * sizeof(float)), bars + b);
+        src -= RS;
+      }
+    }
+  };
+  // the slot agrees on the outcome (a barrier of the slot): a stage counts
+  // as landed only if every thread saw it land.  wb / wpar: ring buffer and
+  // phase parity of the stage waited for next (stage u: u % P, (u / P) & 1)
+  int wb = 0;
+  unsigned wpar = 0u;
+  auto wait = [&]() {
+    const bool ok = !any(!mbar_wait(bars + wb, wpar, lim));
+    if (G == 1) __syncwarp();  // memory order across the warp, as the named barrier gives
+    return ok;
+  };
+  auto wait_done = [&]() {  // advance to the next stage
+    if (++wb == P) {
+      wb = 0;
+      wpar ^= 1u;
+    }
+  };
+  if (lt == 0) {
+    for (int b = 0; b < P; ++b) mbar_init(bars + b);
+    mbar_init_fence();
+  }
+  sync();
+  for (int u = 0; u + 1 < P; ++u) issue_next();
+  float rz = 0.0f, rr = 0.0f;
+  bool bad = false;
+  int at = 0;  // the stage being waited for
+  const int pl = zcol(MG, t) - t;
+  // w = S^{-1} v, line block by line block, the block index a compile-time
+  // constant so that every packed offset folds: row t of the symmetric
+  // S^{-1} is the stored lower triangle's row t (blocks before this thread's
+  // line, and its own block up to the diagonal) followed by its column t
+  // (its own block below the diagonal, and the blocks after it)
+  const int tl = act ? lane : 0;  // row within the line
+  auto lblock = [&](const float *Ls, const float *v, auto LJ) {
+    constexpr int c0 = decltype(LJ)::value * M;
+    return bcast_dot<M, float>(v + 32 * decltype(LJ)::value,
+                           [&](int cc) { return Ls[zcol(MG, c0 + cc) + t - c0 - cc]; });
+  };
+  auto ublock = [&](const float *Ls, const float *v, auto LJ) {
+    constexpr int c0 = decltype(LJ)::value * M;
+    return bcast_dot<M, float>(v + 32 * decltype(LJ)::value, [&](int cc) { return Ls[pl + c0 + cc]; });
+  };
+  auto dblock = [&](const float *Ls, const float *v, auto LJ) {
+    constexpr int c0 = decltype(LJ)::value * M;
+    return bcast_dot<M, float>(v + 32 * decltype(LJ)::value, [&](int cc) {
+      return cc <= tl ? Ls[zcol(MG, c0 + cc) + t - c0 - cc] : Ls[pl + c0 + cc];
+    });
+  };
+  auto symrow = [&](const float *Ls, const float *v) {
+    float acc = 0.0f;
+    auto part = [&](auto LJ) {
+      constexpr int J = decltype(LJ)::value;
+      if (J >= G) return;
+      if (J < li) acc += lblock(Ls, v, LJ);
+      else if (J == li) acc += dblock(Ls, v, LJ);
+      else acc += ublock(Ls, v, LJ);
+    };
+    part(std::integral_constant<int, 0>{});
+    part(std::integral_constant<int, 1>{});
+    part(std::integral_constant<int, 2>{});
+    part(std::integral_constant<int, 3>{});
+    return acc;
+  };
+  // forward sweep
+  float r0 = act ? r[gidx(0)] : 0.0f;
+  float r1 = (act && S > 1) ? r[gidx(1)] : 0.0f;
+  float w = 0.0f;
+  for (int s = 0; s < S; ++s, ++at) {
+    if (!wait()) { bad = true; break; }
+    const float *Ls = stage + (size_t)wb * RSS, *XY = Ls + LP + 8 * t;
+    wait_done();
+    issue_next();  // every thread is past step s - 1: its buffer is free
+    const int par = s & 1;
+    const float rv = r0;
+    r0 = r1;
+    if (act && s + 2 < S) r1 = r[gidx(s + 2)];
+    rr += rv * rv;
+    float bv = rv;
+    if (s > 0) {  // bv -= (O_{s-1}^float w_{s-1})_t, line by line
+      const float x0 = XY[0], x1 = XY[1], x2 = XY[2];
+      float s0 = act ? XY[4] * w : 0.0f, s1 = act ? XY[5] * w : 0.0f, s2 = act ? XY[6] * w : 0.0f;
+      warp_allsum3(s0, s1, s2);
+      float o = x0 * __shfl_sync(0xffffffffu, w, 0) + x1 * __shfl_sync(0xffffffffu, w, N) +
+            x2 * __shfl_sync(0xffffffffu, w, 2 * N);
+      if (k == N - 1) o += a == 0 ? s0 : (a == 1 ? s1 : s2);
+      bv -= o;
+    }
+    if (act) vb(par)[lt] = bv;
+    sync();
+    w = symrow(Ls, vb(par));  // w_s = S_s^{-1} bv = Linv_s^float y_s
+    if (!act) w = 0.0f;
+    rz += bv * w;             // |y_s|^2
+    if (act) z[gidx(s)] = w;  // read back by the backward sweep
+  }
+  // backward sweep: x_{S-1} = w_{S-1} (already in z), then
+  // x_s = w_s - W_s v_{s+1}, v per line: x_{s+1}(b, N - 1) and X^float x_{s+1}
+  if (!bad) {
+    float x = w;
+    float w1 = (act && S > 1) ? z[gidx(S - 2)] : 0.0f;
+    float w2 = (act && S > 2) ? z[gidx(S - 3)] : 0.0f;
+    for (int s = S - 2; s >= 0; --s, ++at) {
+      if (!wait()) { bad = true; break; }
+      const float *Ws = stage + (size_t)wb * RSS, *XY = Ws + BW + 8 * t;
+      wait_done();
+      issue_next();
+      const int par = s & 1;
+      const float wv = w1;
+      w1 = w2;
+      if (act && s >= 2) w2 = z[gidx(s - 2)];
+      const float e0 = __shfl_sync(0xffffffffu, x, N - 1);
+      const float e1 = __shfl_sync(0xffffffffu, x, 2 * N - 1);
+      const float e2 = __shfl_sync(0xffffffffu, x, 3 * N - 1);
+      float c0 = act ? XY[0] * x : 0.0f, c1 = act ? XY[1] * x : 0.0f, c2 = act ? XY[2] * x : 0.0f;
+      warp_allsum3(c0, c1, c2);
+      if (lane < 6) vb(par)[32 * li + lane] = lane < 3 ? (lane == 0 ? e0 : (lane == 1 ? e1 : e2))
+                                                      : (lane == 3 ? c0 : (lane == 4 ? c1 : c2));
+      sync();
+      const float *Wr = Ws + t * WS;
+      float acc = 0.0f;
+#pragma unroll
+      for (int l = 0; l < G; ++l) {
+        const float *vl = vb(par) + 32 * l;
+        acc += (Wr[6 * l] * vl[0] + Wr[6 * l + 1] * vl[1] + Wr[6 * l + 2] * vl[2]) +
+               (Wr[6 * l + 3] * vl[3] + Wr[6 * l + 4] * vl[4] + Wr[6 * l + 5] * vl[5]);
+      }
+      x = act ? wv - acc : 0.0f;
+      if (act) z[gidx(s)] = x;
+    }
+  }
+  if (bad) {  // a copy never landed: bounded waits for every copy in flight, then report
+    for (int u = at; u < issued; ++u) {
+      mbar_wait(bars + wb, wpar, kDrainNs);
+      wait_done();
+    }
+    if (lt == 0 && err) atomicExch(&err->flag, 1);
+  }
+  // the group's partial sums, in a fixed order
+  double vrz = (double)rz, vrr = (double)rr;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    vrz += __shfl_xor_sync(0xffffffffu, vrz, o);
+    vrr += __shfl_xor_sync(0xffffffffu, vrr, o);
+  }
+  if (lane == 0) {
+    psum[(w0 + li) * 2] = vrz;
+    psum[(w0 + li) * 2 + 1] = vrr;
+  }
+  sync();
+  if (lt == 0) {
+    double srz = 0.0, srr = 0.0;
+    for (int ww = 0; ww < G; ++ww) {
+      srz += psum[(w0 + ww) * 2];
+      srr += psum[(w0 + ww) * 2 + 1];
+    }
+    if (part_rz) part_rz[grp] = srz;
+    if (part_rr) part_rr[grp] = srr;
+    for (int b = 0; b < P; ++b) mbar_inval(bars + b);  // every phase issued has completed
+  }
+}
+
+// The beta step of a PCG iteration folded into the grouped-line solve: once
+// every CTA of all the step's launches has written its groups' r.z and r.r
+// partials, the last reduces them in a fixed order (group 0 .. ngroups - 1)
+// and updates beta and the stopping test.
+__device__ void fold_beta(const PcgFold &f) {
+  __shared__ int last;
+  __shared__ double red[2][kZgThreads / 32];
+  __syncthreads();  // every slot of this CTA has written its partials
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(f.cnt, 1u) == (unsigned)(f.total - 1);
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double rz = 0.0, rr = 0.0;
+  for (int t = threadIdx.x; t < f.nparts; t += blockDim.x) {
+    rz += __ldcg(f.part + t);
+    rr += __ldcg(f.part2 + t);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    rz += __shfl_xor_sync(0xffffffffu, rz, o);
+    rr += __shfl_xor_sync(0xffffffffu, rr, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = rz;
+    red[1][threadIdx.x >> 5] = rr;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0, b = 0.0;
+    for (int w = 0; w < kZgThreads / 32; ++w) {
+      a += red[0][w];
+      b += red[1][w];
+    }
+    pcg_finish_beta(f.s, a, b);
+    *f.cnt = 0u;
+    __threadfence();
+  }
+}
+
+// packs [pk0, pk0 + npk) of one degree; CTAs take packs from queue[0]
+// (largest first); the last CTA to finish resets queue[0..1] for the next
+// launch.  One mesh (ginst == nullptr) or a batch (per group: its mirror's
+// mesh and first unknown).
+template <int N>
+__global__ void __launch_bounds__(kZgThreads, 4)
+zgroup_packed_kernel(const DevMesh m1, const int *__restrict__ ginst, const DevMesh *__restrict__ meshes,
+                     const long long *__restrict__ dof_off, const int4 *__restrict__ glines,
+                     const long long *__restrict__ gfac, const int4 *__restrict__ packs, int pk0, int npk,
+                     int *__restrict__ queue, const float *__restrict__ fac, const float *__restrict__ r,
+                     float *__restrict__ z, double *__restrict__ part_rz, double *__restrict__ part_rr, const int *__restrict__ done,
+                     TnWait *__restrict__ err, const PcgFold fold) {
+  if (done && *done) return;
+  constexpr int SW = zp_stage_per_warp<N>();
+  extern __shared__ __align__(16) unsigned char zsm[];
+  float *const stage0 = reinterpret_cast<float *>(zsm);
+  float *const vecs = stage0 + 4 * SW;
+  unsigned long long *const bars = reinterpret_cast<unsigned long long *>(vecs + 4 * kZgThreads);
+  __shared__ int s_pk;
+  __shared__ double psum[8];
+  const int warp = threadIdx.x >> 5;
+  const unsigned long long lim = wait_limit(err);
+  for (;;) {
+    if (threadIdx.x == 0) s_pk = atomicAdd(queue, 1);
+    __syncthreads();
+    const int pk = s_pk;
+    __syncthreads();
+    if (pk >= npk) break;
+    const int4 P4 = packs[pk0 + pk];
+    const int ent[4] = {P4.x, P4.y, P4.z, P4.w};
+    int w0 = 0, grp = -1, G = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int g = ent[i];
+      if (g < 0 || grp >= 0) continue;
+      const int4 L = glines[g];
+      const int gs = 1 + (L.y >= 0) + (L.z >= 0) + (L.w >= 0);
+      if (warp >= w0 && warp < w0 + gs) {
+        grp = g;
+        G = gs;
+      } else {
+        w0 += gs;
+      }
+    }
+    if (grp >= 0) {
+      int mncol = m1.ncol, mslab = m1.nslab;
+      const float *rg = r;
+      float *zg = z;
+      if (ginst) {
+        const int in = ginst[grp];
+        mncol = meshes[in].ncol;
+        mslab = meshes[in].nslab;
+        const long long o = dof_off[in];
+        rg += o;
+        zg += o;
+      }
+      float *stg = stage0 + (size_t)w0 * SW;
+      unsigned long long *sb = bars + kZgMaxStages * w0;
+      const int cap = G * SW;
+      switch (G) {
+        case 1:
+          zp_slot<N, 1>(grp, w0, mncol, mslab, rg, zg, glines, gfac, fac, stg, cap, vecs, sb, psum,
+                                lim, err, part_rz, part_rr);
+          break;
+        case 2:
+          zp_slot<N, 2>(grp, w0, mncol, mslab, rg, zg, glines, gfac, fac, stg, cap, vecs, sb, psum,
+                                lim, err, part_rz, part_rr);
+          break;
+        case 3:
+          zp_slot<N, 3>(grp, w0, mncol, mslab, rg, zg, glines, gfac, fac, stg, cap, vecs, sb, psum,
+                                lim, err, part_rz, part_rr);
+          break;
+        default:
+          zp_slot<N, 4>(grp, w0, mncol, mslab, rg, zg, glines, gfac, fac, stg, cap, vecs, sb, psum,
+                                lim, err, part_rz, part_rr);
+          break;
+      }
+    }
+    __syncthreads();  // every slot of the pack is done with shared memory
+  }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {
+      queue[0] = 0;
+      queue[1] = 0;
+      __threadfence();
+    }
+  }
+  if (fold.s) fold_beta(fold);
+}
+
+// ---- the FP64 solve: three launches
+//   zg_slab_kernel   a_s = S_s^{-1} r_s (left in z), c_s and d_s, every slab of
+//                    every group on its own
+//   zg_chain_kernel  the two chains g and f of every group
+//   zg_final_kernel  x_s = a_s - Q_s g_{s-1} - W_s f_{s+1}, r.z and r.r, again
+//                    every slab on its own
+// All three are bound by the FP64 pipe (78, 80 and 88 % busy; 187 + 105 + 97 us
+// at 2.0 M unknowns, p = 6).  Loading the last launch's factors by bulk copies
+// through a ring, as the first does, was slower (441 against 383 us in all:
+// fewer CTAs per SM).
+// `chain` holds 12 g numbers per slab: c_s, then g_s; d_s, then f_s.
+constexpr int kZgChunks = 4;   // stages of slabs per CTA of the first and last launch, at most
+constexpr int kZgFill = 1024;  // CTAs the first launch aims at before a CTA takes more than one stage
+constexpr int kZgBlock = 32;   // slabs the chain kernel holds at a time, however many there are
+constexpr int kZgKWarp = 640;  // K entries a warp stages at a time (one record of the largest group: 600)
+
+// what the kernels need of the groups; one degree's packs and slab ranges
+struct ZgView {
+  const int *inst;             // batch: mirror of every group (nullptr: one mesh)
+  const DevMesh *meshes;
+  const long long *dof_off;
+  const int4 *lines;
+  const long long *fac, *chain;  // first factor and chain entry of every group
+  const int4 *packs;
+  const int4 *ranges;            // (group, first slab, end slab, partial sum)
+};
+
+struct ZgGroup {
+  int ncol, S;
+  long long off;  // first unknown of the mirror
+};
+__device__ __forceinline__ ZgGroup zg_where(const DevMesh &m1, const ZgView &v, int grp) {
+  if (!v.inst) return {m1.ncol, m1.nslab, 0};
+  const int in = v.inst[grp];
+  return {v.meshes[in].ncol, v.meshes[in].nslab, v.dof_off[in]};
+}
+__device__ __forceinline__ int zg_line(const int4 &L, int li) { return li == 0 ? L.x : (li == 1 ? L.y : (li == 2 ? L.z : L.w)); }
+__device__ __forceinline__ int zg_size(const int4 &L) { return 1 + (L.y >= 0) + (L.z >= 0) + (L.w >= 0); }
+
+// ---- the slabs
+template <int N, int G>
+struct ZgSlab {
+  static constexpr int M = 3 * N, MG = G * M, C6 = 6 * G, SREC = zg_srec(MG, G), QREC = zg_qrec(MG, G), MGP = pad4(MG);
+  // slabs per stage: rows on the CTA's threads, room of one slab of the largest group
+  static constexpr int by_rows = kZgThreads / MG, by_room = zg_srec(12 * N, 4) / SREC;
+  static constexpr int SL = by_rows < 1 ? 1 : (by_rows < by_room ? by_rows : by_room);
+};
+int zg_slabs(int N, int G) {
+  const int MG = 3 * N * G, by_rows = kZgThreads / MG, by_room = zg_srec(12 * N, 4) / zg_srec(MG, G);
+  return by_rows < 1 ? 1 : std::min(by_rows, by_room);
+}
+// two stages, the vector twice over (rows read it at t + m), the products, two rows of D
+template <int N, typename T>
+constexpr size_t zg_slab_smem() { return sizeof(T) * (size_t)(2 * zg_srec(12 * N, 4) + 3 * kZgThreads + 2 * N); }
+
+// row t of S^{-1} v from the circulant diagonals; v repeated: v[MG + i] = v[i]
+template <int MG, typename T>
+__device__ __forceinline__ T circ_row(const T *__restrict__ A, const T *__restrict__ v, int t) {
+  constexpr int H = (MG - 1) / 2;
+  const T *const At = A + t, *const vt = v + t;
+  T a0 = At[0] * vt[0], a1 = T(0), a2 = T(0), a3 = T(0);
+#pragma unroll
+  for (int m = 1; m <= H; ++m) {
+    const int back = t < m ? MG : 0;
+    const T f = At[m * MG], b = At[m * MG - m + back];
+    if (m & 1) {
+      a1 += f * vt[m];
+      a2 += b * vt[MG - m];
+    } else {
+      a3 += f * vt[m];
+      a0 += b * vt[MG - m];
+    }
+  }
+  if (MG % 2 == 0) a1 += At[(MG / 2) * MG] * vt[MG / 2];
+  return (a0 + a1) + (a2 + a3);
+}
+
+template <int N, int G, typename T>
+__device__ __forceinline__ void zg_slab(const DevMesh &m1, const ZgView &v, const int4 &rg, const T *__restrict__ fac,
+                                        const T *r0, T *__restrict__ z0, T *__restrict__ chain,
+                                        T *__restrict__ stage, unsigned long long *bars, const int *done,
+                                        TnWait *__restrict__ err) {
+  using Z = ZgSlab<N, G>;
+  constexpr int M = Z::M, MG = Z::MG, C6 = Z::C6, SREC = Z::SREC, SL = Z::SL, LC = pad4(zg_circ(MG));
+  constexpr int N2 = N * N, n = N * N2, ROOM = zg_srec(12 * N, 4);
+  static_assert(SL * MG <= kZgThreads, "rows");
+  T *const vb = stage + 2 * ROOM, *const av = vb + 2 * kZgThreads, *const dl = av + kZgThreads;
+  const int tid = threadIdx.x, grp = rg.x, s0 = rg.y, s1 = rg.z;
+  const ZgGroup q = zg_where(m1, v, grp);
+  const T *const src = fac + v.fac[grp];
+  auto issue = [&](int s) {  // the stage of slabs s ..: thread 0
+    const int i = (s - s0) / SL, b = i & 1;
+    const unsigned bytes = (unsigned)(min(SL, s1 - s) * SREC * sizeof(T));
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    mbar_expect(bars + b, bytes);
+    bulk_g2s(stage + b * ROOM, src + (size_t)s * SREC, bytes, bars + b);
+  };
+  if (tid == 0) {  // the factors do not depend on the launch before this one
+    mbar_init(bars);
+    mbar_init(bars + 1);
+    mbar_init_fence();
+    issue(s0);
+  }
+  const int sl = tid / MG, t = tid - sl * MG, li = t / M, tl = t - li * M, a = tl / N, k = tl - a * N;
+  const int lid = zg_line(v.lines[grp], li), col = lid / N2, qn = lid - col * N2;
+  const bool row = sl < SL;
+  const size_t gs = (size_t)q.ncol * 3 * n, g0 = q.off + ((size_t)col * 3 + a) * n + (size_t)k * N2 + qn;
+  T *const ch = chain + v.chain[grp];
+  const unsigned long long lim = wait_limit(err);
+  if (tid < 2 * N) {  // D(0, k), k != 0, and D(N-1, k), k != N - 1; zero at the face node itself
+    const int kk = tid < N ? tid : tid - N;
+    dl[tid] = tid == 0 || tid == 2 * N - 1 ? T(0) : (T)c_lgl_zg.D[N][(tid < N ? 0 : (N - 1) * N) + kk];
+  }
+  __syncthreads();  // the barriers are initialised
+  grid_wait();
+  r0 = after_wait(r0);
+  done = after_wait(done);
+  const bool skip = done && *done;
+  T rn = row && !skip && s0 + sl < s1 ? r0[g0 + (size_t)(s0 + sl) * gs] : T(0);
+  for (int s = s0; s < s1; s += SL) {
+    const int i = (s - s0) / SL, b = i & 1;
+    const bool on = row && s + sl < s1;
+    const bool ok = mbar_wait(bars + b, (i >> 1) & 1, lim);
+    if (on) vb[sl * 2 * MG + t] = vb[sl * 2 * MG + MG + t] = rn;
+    // the stage has landed, the vector is complete, the other stage is free
+    if (__syncthreads_or(!ok)) {  // a copy did not land in time: a bounded wait for it, then report
+      mbar_wait(bars + b, (i >> 1) & 1, kDrainNs);
+      if (tid == 0 && err) atomicExch(&err->flag, 1);
+      return;
+    }
+    if (skip) return;
+    if (tid == 0 && s + SL < s1) issue(s + SL);
+    if (s + SL >= s1) grid_trigger();
+    rn = row && s + SL + sl < s1 ? r0[g0 + (size_t)(s + SL + sl) * gs] : T(0);
+    const T *A = stage + b * ROOM;
+    if (on) {
+      const T w = circ_row<MG, T>(A + sl * SREC, vb + sl * 2 * MG, t);
+      z0[g0 + (size_t)(s + sl) * gs] = w;
+      av[tid] = w;
+    }
+    __syncthreads();
+    // c_s = U_s^T a_s and d_s = V_s^T a_s: one thread per slab, line, component and side
+    constexpr int NT6 = SL * 6 * G;
+    static_assert(NT6 <= kZgThreads, "one task per thread");
+    if (tid < NT6) {
+      const int es = tid / (6 * G), ea = tid - es * (6 * G), el = ea / 6, e6 = ea - el * 6;
+      const bool bottom = e6 >= 3;  // d (the top face) or c (the bottom face, k = 0)
+      const int ec = bottom ? e6 - 3 : e6;
+      if (s + es < s1) {
+        const T *w = av + es * MG + el * M, *C = A + es * SREC + LC + 16 * el, *wc = w + ec * N;
+        const T *D = dl + (bottom ? 0 : N), *X3 = C + 6 + ec;
+        T e = T(0);
+#pragma unroll
+        for (int kk = 0; kk < N; ++kk) e += D[kk] * wc[kk];
+        T *const o = ch + (size_t)(s + es) * 2 * C6 + 6 * el + (bottom ? 0 : C6) + ec;
+        if (bottom) {
+          o[0] = C[ec] * e;
+          o[3] = wc[0];
+        } else {
+          o[0] = wc[N - 1];
+          o[3] = C[3 + ec] * e + ((X3[0] * w[N - 1] + X3[3] * w[2 * N - 1]) + X3[6] * w[3 * N - 1]);
+        }
+      }
+    }
+  }
+}
+
+template <int N, typename T>
+__global__ void __launch_bounds__(kZgThreads, sizeof(T) == 4 ? 7 : 3)
+zg_slab_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, const T *__restrict__ r,
+               T *__restrict__ z, T *__restrict__ chain, const int *__restrict__ done, TnWait *__restrict__ err) {
+  extern __shared__ __align__(16) unsigned char zsm[];
+  __shared__ __align__(8) unsigned long long bars[2];
+  T *const stage = reinterpret_cast<T *>(zsm);
+  const int4 rg = v.ranges[blockIdx.x];
+  switch (zg_size(v.lines[rg.x])) {
+#define TN_CASE(GG) case GG: zg_slab<N, GG, T>(m1, v, rg, fac, r, z, chain, stage, bars, done, err); break;
+    TN_CASE(1) TN_CASE(2) TN_CASE(3) TN_CASE(4)
+#undef TN_CASE
+  }
+}
+
+// ---- the chains: a group of G lines on G warps of a CTA of four, which takes
+// a pack of groups: 4, 3 + 1, 2 + 2, 2 + 1 + 1 or 1 + 1 + 1 + 1 lines.  Slabs
+// go by blocks of kZgBlock, so that shared memory does not depend on their
+// number.  One warp runs the chains, the others bring K.
+constexpr int kZgChLine = pad4(12 * (kZgBlock + 1));  // chain entries of a block and the slab before or after it, per line
+template <typename T>
+constexpr size_t zg_chain_smem() { return sizeof(T) * 4 * (size_t)(kZgChLine + kZgKWarp); }
+
+// the group this warp works on: its first warp w0 in the CTA, its size (0: idle)
+__device__ __forceinline__ int zg_slot(const ZgView &v, int &w0, int &G) {
+  const int4 P4 = v.packs[blockIdx.x];
+  const int ent[4] = {P4.x, P4.y, P4.z, P4.w}, warp = threadIdx.x >> 5;
+  int at = 0;
+  w0 = 0;
+  G = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (ent[i] < 0) continue;
+    const int gs = zg_size(v.lines[ent[i]]);
+    if (warp >= at && warp < at + gs) {
+      w0 = at;
+      G = gs;
+      return ent[i];
+    }
+    at += gs;
+  }
+  return -1;
+}
+
+// K records brought through registers: load issues, store lands them
+template <int G, typename T>
+struct KStage {
+  static constexpr int KP = zg_kpart(G), KREC = zg_krec(G), SLK = G * kZgKWarp / KP;  // slabs per stage
+  static constexpr int PER = (SLK * KP + 32 * G - 1) / (32 * G);
+  T v[PER];
+  __device__ __forceinline__ void load(const T *__restrict__ k, int cnt, int lt) {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int at = i * 32 * G + lt, s = at / KP;
+      v[i] = at < cnt * KP ? k[(size_t)s * KREC + (at - s * KP)] : T(0);
+    }
+  }
+  __device__ __forceinline__ void store(T *__restrict__ ks, int cnt, int lt) const {
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+      const int at = i * 32 * G + lt;
+      if (at < cnt * KP) ks[at] = v[i];
+    }
+  }
+};
+
+// lanes per row of a chain step (112 -> 105 us at 2.0 M unknowns, p = 6): the six or twelve rows of small groups leave
+// lanes over, and an FP64 instruction costs the same with a few lanes on
+__host__ __device__ constexpr int chain_parts(int G) { return G == 1 ? 4 : (G == 2 ? 2 : 1); }
+template <int G, typename T, typename KF, typename VF>
+__device__ __forceinline__ T chain_dot(T a0, KF k, VF v, int part) {
+  constexpr int P = chain_parts(G), C6 = 6 * G, STEPS = (C6 + P - 1) / P;
+  T a1 = T(0), a2 = T(0);
+#pragma unroll
+  for (int i = 0; i < STEPS; ++i) {
+    const int j = i * P + part;
+    if (C6 % P != 0 && j >= C6) break;
+    (i % 3 == 0 ? a0 : (i % 3 == 1 ? a1 : a2)) -= k(j) * v(j);
+  }
+  a0 += a1 + a2;
+#pragma unroll
+  for (int o = P / 2; o > 0; o >>= 1) a0 += __shfl_xor_sync(0x00ffffffu, a0, o);  // 6 x 4 or 12 x 2 lanes
+  return a0;
+}
+
+template <int G, typename T>
+__device__ __forceinline__ void zg_chain(int S, int w0, const T *__restrict__ fk, T *chain,
+                                         T *__restrict__ sm) {
+  constexpr int C6 = 6 * G, C12 = 12 * G, LD = zg_ld(G), NT = 32 * G;
+  constexpr int KP = zg_kpart(G), KREC = zg_krec(G), SLK = KStage<G, T>::SLK;
+  const int lt = threadIdx.x - 32 * w0, row = lt / chain_parts(G), part = lt % chain_parts(G);
+  T *const ch = sm, *const ks = ch + G * kZgChLine;
+  const int nblk = (S + kZgBlock - 1) / kZgBlock;
+  KStage<G, T> K;
+  // forward: slabs b0 .. b0 + nb - 1 at ch[(1 + i) C12], slab b0 - 1 at ch[0]
+  for (int b0 = 0; b0 < S; b0 += kZgBlock) {
+    const int nb = min(kZgBlock, S - b0), k0 = max(1, b0), k1 = min(b0 + nb, S - 1);  // steps k0 .. k1 - 1
+    K.load(fk + (size_t)k0 * KREC, min(SLK, k1 - k0), lt);
+    if (b0 > 0) {  // the last slab of the block before
+      slot_sync<G>(w0);
+      if (lt < C6) ch[lt] = ch[kZgBlock * C12 + lt];
+      slot_sync<G>(w0);
+    }
+    for (int id = lt; id < nb * C12; id += NT) ch[C12 + id] = chain[(size_t)b0 * C12 + id];
+    for (int s0 = k0; s0 < k1; s0 += SLK) {
+      const int cnt = min(SLK, k1 - s0);
+      slot_sync<G>(w0);
+      K.store(ks, cnt, lt);
+      if (s0 + SLK < k1) K.load(fk + (size_t)(s0 + SLK) * KREC, min(SLK, k1 - s0 - SLK), lt);
+      slot_sync<G>(w0);
+      if (lt < 32)
+        for (int i = 0; i < cnt; ++i) {  // g_s = c_s - K_s g_{s-1}
+          T *const g = ch + (s0 + i - b0) * C12;
+          if (row < C6) {
+            const T *Kr = ks + i * KP + row * LD;
+            const T w = chain_dot<G, T>(part == 0 ? g[C12 + row] : T(0), [&](int j) { return Kr[j]; },
+                                        [&](int j) { return g[j]; }, part);
+            if (part == 0) g[C12 + row] = w;
+          }
+          __syncwarp();
+        }
+    }
+    slot_sync<G>(w0);
+    // d_s - H_s g_{s-1}, in place of d_s
+    for (int id = lt; id < nb * C6; id += NT) {
+      const int i = id / C6, j = id - i * C6, s = b0 + i;
+      if (s == 0) continue;
+      const T *H = fk + (size_t)s * KREC + KP + j, *g = ch + i * C12;
+      T a0 = ch[(1 + i) * C12 + C6 + j], a1 = T(0), a2 = T(0);
+#pragma unroll
+      for (int p = 0; p < C6; p += 3) {
+        a0 -= H[p * C6] * g[p];
+        a1 -= H[(p + 1) * C6] * g[p + 1];
+        a2 -= H[(p + 2) * C6] * g[p + 2];
+      }
+      ch[(1 + i) * C12 + C6 + j] = a0 + (a1 + a2);
+    }
+    if (nblk > 1) {
+      slot_sync<G>(w0);
+      for (int id = lt; id < nb * C12; id += NT) chain[(size_t)b0 * C12 + id] = ch[C12 + id];
+    }
+  }
+  grid_trigger();
+  // backward: slabs b0 .. at ch[(1 + i) C12] (the last block is there), the
+  // first f of the block below kept aside
+  for (int blk = nblk - 1; blk >= 0; --blk) {
+    const int b0 = blk * kZgBlock, nb = min(kZgBlock, S - b0);
+    const int k1 = blk == nblk - 1 ? S - 2 : b0 + nb - 1, k0 = max(1, b0);  // steps k1 down to k0
+    if (blk < nblk - 1) {
+      slot_sync<G>(w0);
+      const T f = lt < C6 ? ch[C12 + C6 + lt] : T(0);
+      slot_sync<G>(w0);
+      for (int id = lt; id < nb * C12; id += NT) ch[C12 + id] = chain[(size_t)b0 * C12 + id];
+      slot_sync<G>(w0);
+      // f_{b0 + nb}: the block is full, so it goes to slab b0 - 1's place
+      if (lt < C6) ch[C6 + lt] = f;
+    }
+    K.load(fk + (size_t)max(k0, k1 - SLK + 1) * KREC, min(SLK, k1 - k0 + 1), lt);
+    for (int hi = k1; hi >= k0; hi -= SLK) {
+      const int lo = max(k0, hi - SLK + 1);
+      slot_sync<G>(w0);
+      K.store(ks, hi - lo + 1, lt);
+      if (lo > k0) K.load(fk + (size_t)max(k0, lo - SLK) * KREC, min(SLK, lo - k0), lt);
+      slot_sync<G>(w0);
+      if (lt < 32)
+        for (int s = hi; s >= lo; --s) {  // f_s = e_s - K_s^T f_{s+1}
+          const T *f = s + 1 == b0 + nb ? ch + C6 : ch + (s - b0 + 2) * C12 + C6;
+          if (row < C6) {
+            T *const o = ch + (s - b0 + 1) * C12 + C6 + row;
+            const T *Kc = ks + (s - lo) * KP + row;
+            const T w = chain_dot<G, T>(part == 0 ? *o : T(0), [&](int j) { return Kc[j * LD]; },
+                                        [&](int j) { return f[j]; }, part);
+            if (part == 0) *o = w;
+          }
+          __syncwarp();
+        }
+    }
+    slot_sync<G>(w0);
+    for (int id = lt; id < nb * C12; id += NT) chain[(size_t)b0 * C12 + id] = ch[C12 + id];
+  }
+}
+
+template <int N, typename T>
+__global__ void __launch_bounds__(kZgThreads)
+zg_chain_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, T *__restrict__ chain,
+                const int *__restrict__ done) {
+  extern __shared__ __align__(16) unsigned char zsm[];
+  int w0, G;
+  const int grp = zg_slot(v, w0, G);
+  grid_wait();
+  done = after_wait(done);
+  chain = after_wait(chain);
+  if ((done && *done) || grp < 0) return;
+  T *const sm = reinterpret_cast<T *>(zsm) + (size_t)w0 * (kZgChLine + kZgKWarp);
+  const int S = zg_where(m1, v, grp).S;
+  const T *const f = fac + v.fac[grp];
+  T *const c = chain + v.chain[grp];
+  switch (G) {
+#define TN_CASE(GG) case GG: zg_chain<GG, T>(S, w0, f + zg_koff(3 * N * GG, GG, S), c, sm); break;
+    TN_CASE(1) TN_CASE(2) TN_CASE(3) TN_CASE(4)
+#undef TN_CASE
+  }
+}
+
+// ---- the correction of every slab, r.z and r.r
+template <int N, int G, typename T>
+__device__ __forceinline__ void zg_final(const DevMesh &m1, const ZgView &v, const int4 &rg, const T *__restrict__ fac,
+                                         const T *r0, T *z0, const T *chain,
+                                         T *__restrict__ qv, T &rz, T &rr) {
+  using Z = ZgSlab<N, G>;
+  constexpr int M = Z::M, MG = Z::MG, MGP = Z::MGP, C6 = Z::C6, C12 = 2 * C6, SL = Z::SL, N2 = N * N, n = N * N2;
+  const int tid = threadIdx.x, grp = rg.x, s0 = rg.y, s1 = rg.z;
+  const ZgGroup q = zg_where(m1, v, grp);
+  const int S = q.S;
+  const T *const qw = fac + v.fac[grp] + zg_qoff(MG, G, S);
+  const T *const ch = chain + v.chain[grp];
+  for (int id = tid; id < (s1 - s0) * C12; id += kZgThreads) {  // g_{s-1} | f_{s+1}
+    const int i = id / C12, j = id - i * C12, s = s0 + i;
+    qv[id] = j < C6 ? (s > 0 ? ch[(size_t)(s - 1) * C12 + j] : T(0)) : (s + 1 < S ? ch[(size_t)(s + 1) * C12 + j] : T(0));
+  }
+  __syncthreads();
+  const int sl = tid / MG, t = tid - sl * MG, li = t / M, tl = t - li * M, a = tl / N, k = tl - a * N;
+  if (sl >= SL) return;
+  const int lid = zg_line(v.lines[grp], li), col = lid / N2, qn = lid - col * N2;
+  const size_t gs = (size_t)q.ncol * 3 * n, g0 = q.off + ((size_t)col * 3 + a) * n + (size_t)k * N2 + qn;
+  for (int s = s0 + sl; s < s1; s += SL) {
+    const size_t at = g0 + (size_t)s * gs;
+    const T *w = qw + (size_t)s * Z::QREC + t, *f = qv + (s - s0) * C12;
+    const T rv = r0[at];
+    T a0 = z0[at], a1 = T(0), a2 = T(0);
+#pragma unroll
+    for (int j = 0; j < C12; j += 3) {
+      a0 -= w[j * MGP] * f[j];
+      a1 -= w[(j + 1) * MGP] * f[j + 1];
+      a2 -= w[(j + 2) * MGP] * f[j + 2];
+    }
+    const T x = a0 + (a1 + a2);
+    z0[at] = x;
+    rz += rv * x;
+    rr += rv * rv;
+  }
+}
+
+template <int N, typename T>
+__global__ void __launch_bounds__(kZgThreads, sizeof(T) == 4 ? 8 : 4)
+zg_final_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, const T *__restrict__ r,
+                T *__restrict__ z, const T *__restrict__ chain, double *__restrict__ part_rz,
+                double *__restrict__ part_rr, const int *__restrict__ done, const PcgFold fold) {
+  constexpr int QV = 12 * kZgChunks * kZgThreads / (3 * N);  // 12 g numbers of at most kZgChunks kZgThreads / (3 g N) slabs
+  __shared__ T qv[QV > 48 * kZgChunks ? QV : 48 * kZgChunks];
+  const int4 rg = v.ranges[blockIdx.x];
+  const int G = zg_size(v.lines[rg.x]);
+  grid_wait();
+  done = after_wait(done);
+  r = after_wait(r);
+  z = after_wait(z);
+  chain = after_wait(chain);
+  if (done && *done) return;
+  T rz = T(0), rr = T(0);
+  switch (G) {
+#define TN_CASE(GG) case GG: zg_final<N, GG, T>(m1, v, rg, fac, r, z, chain, qv, rz, rr); break;
+    TN_CASE(1) TN_CASE(2) TN_CASE(3) TN_CASE(4)
+#undef TN_CASE
+  }
+  if (part_rz) {  // FP64 sums of the rows' sums: warp 0 for r.z, warp 1 for r.r
+    __shared__ T ps[2][kZgThreads];
+    ps[0][threadIdx.x] = rz;
+    ps[1][threadIdx.x] = rr;
+    __syncthreads();
+    const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
+    if (w < 2) {
+      double x = 0.0;
+#pragma unroll
+      for (int i = 0; i < kZgThreads / 32; ++i) x += (double)ps[w][32 * i + ln];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      double *const dst = w == 0 ? part_rz : part_rr;
+      if (ln == 0 && dst) dst[rg.w] = x;
+    }
+    if (fold.s) fold_beta(fold);
+  }
+}
+
+template <int N>
+cudaError_t zgroup_setup_n(const DevMesh &m, const ZGroupPlan &p, const ZGroupDev &gd, int inst,
+                           double *blk, double *xblk, double *work, float *fac, double *fac64, int *status,
+                           cudaStream_t st) {
+  cudaError_t err = tn_zline_blocks(m, blk, st);
+  if (err != cudaSuccess) return err;
+  zgroup_cross_kernel<N><<<m.E, ((4 * N + 31) / 32) * 32, 0, st>>>(m, xblk);
+  err = cudaGetLastError();
+  // the four group sizes at once, each with its own scratch: the 4-line
+  // groups (few, long) on st, the others on side streams forked from it
+  if (err == cudaSuccess) err = cudaEventRecord(gd.fork, st);
+  size_t off = 0;
+  bool used[3] = {false, false, false};
+  for (int g = 1; g <= 4 && err == cudaSuccess; ++g) {
+    const int cnt = p.inst_n[(size_t)inst * 5 + g];
+    if (!cnt) continue;
+    cudaStream_t sg = st;
+    if (g < 4) {
+      sg = gd.side[g - 1];
+      err = cudaStreamWaitEvent(sg, gd.fork, 0);
+      used[g - 1] = true;
+      if (err != cudaSuccess) break;
+    }
+    zgroup_factor_kernel<N><<<cnt, 128, 0, sg>>>(m, gd.lines, gd.fac_off, p.inst_start[(size_t)inst * 5 + g], g,
+                                                 blk, xblk, work + off, fac, gd.fac64_off, fac64, status);
+    err = cudaGetLastError();
+    const size_t MG = (size_t)g * 3 * N;
+    off += (size_t)cnt * 3 * MG * MG;
+  }
+  for (int k = 0; k < 3 && err == cudaSuccess; ++k) {
+    if (!used[k]) continue;
+    err = cudaEventRecord(gd.join[k], gd.side[k]);
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(st, gd.join[k], 0);
+  }
+  return err;
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_zg(void (*kernel)(P...), int grid, size_t smem, bool dependent, cudaStream_t st, A... args) {
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kZgThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <int N>
+cudaError_t launch_f64(const DevMesh &m, const ZGroupDev &gd, int k, const double *fac, const double *r, double *z,
+                       double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, bool first,
+                       const PcgFold &fold) {
+  const ZgView v{gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac64_off, gd.chain_off,
+                 gd.packs + gd.pk_start[k], gd.ranges + gd.rg_start[k]};
+  cudaError_t e = launch_zg(zg_slab_kernel<N, double>, gd.rg_n[k], zg_slab_smem<N, double>(), first, st, m, v, fac, r,
+                            z, gd.chain, done, zerr);
+  if (e != cudaSuccess) return e;
+  e = launch_zg(zg_chain_kernel<N, double>, gd.pk_n[k], zg_chain_smem<double>(), true, st, m, v, fac, gd.chain, done);
+  if (e != cudaSuccess) return e;
+  return launch_zg(zg_final_kernel<N, double>, gd.rg_n[k], 0, true, st, m, v, fac, r, z, (const double *)gd.chain, prz,
+                   prr, done, fold);
+}
+
+// the FP32 kernel is persistent: as many CTAs as fit at once, never more than
+// packs.  grid_out: only compute the grid; else launch with it.
+template <int N>
+cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float *fac, const float *r, float *z,
+                       double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, const PcgFold &fold,
+                       int *grid_out) {
+  constexpr size_t sm = zp_smem<N>();
+  auto kern = zgroup_packed_kernel<N>;
+  cudaError_t err = sm > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
+                                   : cudaSuccess;
+  if (err != cudaSuccess) return err;
+  static int per_sm[64] = {0};
+  int dev = 0;
+  err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!per_sm[dev]) {
+    // shared memory before L1: the CTAs per SM are limited by the staging rings
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (err != cudaSuccess) return err;
+    int b = 0;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kZgThreads, sm);
+    if (err != cudaSuccess) return err;
+    per_sm[dev] = b > 0 ? b : 1;
+  }
+  int grid = per_sm[dev] * tn_sm_count();
+  grid = grid < gd.pk_n[k] ? grid : gd.pk_n[k];
+  if (grid_out) {
+    *grid_out = grid;
+    return cudaSuccess;
+  }
+  kern<<<grid, kZgThreads, sm, st>>>(m, gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac_off, gd.packs,
+                                     gd.pk_start[k], gd.pk_n[k], gd.queue + 2 * k, fac, r, z, prz, prr, done, zerr,
+                                     fold);
+  return cudaGetLastError();
+}
+
+cudaError_t zgroup_launch(const DevMesh &m, const ZGroupDev &gd, int k, int prec, const void *fac, const void *r,
+                          void *z, double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, bool first,
+                          const PcgFold &fold, int *grid_out) {
+  if (prec == TN_F64 && grid_out) {
+    *grid_out = gd.rg_n[k];
+    return cudaSuccess;
+  }
+  switch (gd.pk_N[k]) {
+#define TN_CASE(NN)                                                                                              \
+  case NN:                                                                                                       \
+    return prec == TN_F64 ? launch_f64<NN>(m, gd, k, (const double *)fac, (const double *)r, (double *)z, prz,   \
+                                           prr, done, zerr, st, first, fold)                                     \
+                          : launch_f32<NN>(m, gd, k, (const float *)fac, (const float *)r, (float *)z, prz, prr, \
+                                           done, zerr, st, fold, grid_out);
+    TN_CASE(3) TN_CASE(4) TN_CASE(5) TN_CASE(6) TN_CASE(7) TN_CASE(8) TN_CASE(9)
+#undef TN_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace
+
+// union-find over face matches of the lines (col * N^2 + j * N + i)
+static int uf_find(std::vector<int> &p, int x) {
+  while (p[x] != x) {
+    p[x] = p[p[x]];
+    x = p[x];
+  }
+  return x;
+}
+
+// the groups of one mesh (members ascending), or false if a node is shared
+// by more than 4 columns
+static bool mesh_groups(const tn::HostMesh &hm, std::vector<std::vector<int>> &out, char *msg, int msglen) {
+  const int N = hm.N, N2 = N * N, nl = hm.ncol * N2;
+  std::vector<int> par(nl);
+  for (int x = 0; x < nl; ++x) par[x] = x;
+  for (int c = 0; c < hm.ncol; ++c)
+    for (int f = 0; f < 4; ++f) {
+      const int nbc = hm.colnb[4 * c + f];
+      if (nbc < 0) continue;
+      const int d = f >> 1, end = (f & 1) ? N - 1 : 0;
+      const int code = hm.colnbf[4 * c + f], f2 = code & 3, d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0;
+      for (int t = 0; t < N; ++t) {
+        const int i = d == 0 ? end : t, j = d == 0 ? t : end;
+        const int a2 = (code >> 2) ? N - 1 - t : t;
+        const int i2 = d2 == 0 ? end2 : a2, j2 = d2 == 0 ? a2 : end2;
+        const int ra = uf_find(par, c * N2 + j * N + i), rb = uf_find(par, nbc * N2 + j2 * N + i2);
+        if (ra != rb) par[ra < rb ? rb : ra] = ra < rb ? ra : rb;
+      }
+    }
+  std::vector<std::vector<int>> comp(nl);
+  for (int x = 0; x < nl; ++x) comp[uf_find(par, x)].push_back(x);
+  out.clear();
+  for (int x = 0; x < nl; ++x) {
+    if (comp[x].empty()) continue;
+    if (comp[x].size() > 4) {
+      std::snprintf(msg, msglen, "a cross-section node is shared by %d columns (line groups hold at most 4)",
+                    (int)comp[x].size());
+      return false;
+    }
+    out.push_back(comp[x]);
+  }
+  return true;
+}
+
+bool tn_zgroup_plan(const tn::HostMesh *const *hms, int n, ZGroupPlan *p, char *msg, int msglen) {
+  std::vector<std::vector<std::vector<int>>> per(n);
+  for (int i = 0; i < n; ++i)
+    if (!mesh_groups(*hms[i], per[i], msg, msglen)) return false;
+  *p = ZGroupPlan();
+  p->inst_start.assign((size_t)n * 5, 0);
+  p->inst_n.assign((size_t)n * 5, 0);
+  // order: group size (largest first), degree, mirror -- one class per (size, degree)
+  for (int g = 4; g >= 1; --g)
+    for (int N = TN_MIN_N; N <= TN_MAX_N; ++N) {
+      const int start = p->ngroups;
+      for (int i = 0; i < n; ++i) {
+        if (hms[i]->N != N) continue;
+        p->inst_start[(size_t)i * 5 + g] = p->ngroups;
+        for (const auto &mm : per[i]) {
+          if ((int)mm.size() != g) continue;
+          p->lines.push_back(make_int4(mm[0], g > 1 ? mm[1] : -1, g > 2 ? mm[2] : -1, g > 3 ? mm[3] : -1));
+          p->inst.push_back(i);
+          p->fac_off.push_back(p->nfac);
+          p->nfac += (long long)hms[i]->nslab * zp_rec(g * 3 * N, g);
+          p->fac64_off.push_back(p->nfac64);
+          p->nfac64 += zg_entries(g * 3 * N, g, hms[i]->nslab);
+          p->chain_off.push_back(p->nchain);
+          p->nchain += (long long)hms[i]->nslab * 12 * g;
+          p->ncompact += (long long)hms[i]->nslab * (zlp(g * 3 * N) + 8 * g * 3 * N);
+          ++p->inst_n[(size_t)i * 5 + g];
+          ++p->ngroups;
+        }
+      }
+      if (p->ngroups == start) continue;
+      if (p->ncls >= kZgMaxCls) {
+        std::snprintf(msg, msglen, "too many line-group classes");
+        return false;
+      }
+      p->cls_N[p->ncls] = N;
+      p->cls_G[p->ncls] = g;
+      p->cls_start[p->ncls] = start;
+      p->cls_n[p->ncls] = p->ngroups - start;
+      ++p->ncls;
+    }
+  // packs of groups filling the four warps of a CTA, per degree, largest
+  // first: 4, 3 + 1, 2 + 2, 2 + 1 + 1, 1 + 1 + 1 + 1 lines
+  for (int N = TN_MIN_N; N <= TN_MAX_N; ++N) {
+    std::vector<int> by[5];
+    for (int k = 0; k < p->ncls; ++k)
+      if (p->cls_N[k] == N)
+        for (int i = 0; i < p->cls_n[k]; ++i) by[p->cls_G[k]].push_back(p->cls_start[k] + i);
+    if (by[1].empty() && by[2].empty() && by[3].empty() && by[4].empty()) continue;
+    const int start = (int)p->packs.size();
+    size_t i1 = 0;
+    auto one = [&]() { return i1 < by[1].size() ? by[1][i1++] : -1; };
+    for (int g4 : by[4]) p->packs.push_back(make_int4(g4, -1, -1, -1));
+    for (int g3 : by[3]) p->packs.push_back(make_int4(g3, one(), -1, -1));
+    for (size_t i = 0; i < by[2].size(); i += 2) {
+      if (i + 1 < by[2].size()) {
+        p->packs.push_back(make_int4(by[2][i], by[2][i + 1], -1, -1));
+      } else {
+        const int a = one();
+        const int b = a >= 0 ? one() : -1;
+        p->packs.push_back(make_int4(by[2][i], a, b, -1));
+      }
+    }
+    while (i1 < by[1].size()) {
+      const int a = one(), b = one(), c = one(), d = one();
+      p->packs.push_back(make_int4(a, b, c, d));
+    }
+    if (p->npk >= kZgMaxDg) {
+      std::snprintf(msg, msglen, "too many degrees for the grouped-line solve");
+      return false;
+    }
+    p->pk_N[p->npk] = N;
+    p->pk_start[p->npk] = start;
+    p->pk_n[p->npk] = (int)p->packs.size() - start;
+    // slab ranges of the first and last launch, in the order of the groups:
+    // as many stages each as leave every SM its CTAs
+    auto stages = [&](int k, int i) {
+      const int sl = zg_slabs(N, p->cls_G[k]);
+      return (hms[p->inst[i]]->nslab + sl - 1) / sl;
+    };
+    long long all = 0;
+    for (int k = 0; k < p->ncls; ++k)
+      if (p->cls_N[k] == N)
+        for (int i = p->cls_start[k]; i < p->cls_start[k] + p->cls_n[k]; ++i) all += stages(k, i);
+    const int per = (int)std::min<long long>(std::max<long long>(all / kZgFill, 1), kZgChunks);
+    p->rg_start[p->npk] = (int)p->ranges.size();
+    for (int k = 0; k < p->ncls; ++k) {
+      if (p->cls_N[k] != N) continue;
+      const int sl = zg_slabs(N, p->cls_G[k]) * per;
+      for (int i = p->cls_start[k]; i < p->cls_start[k] + p->cls_n[k]; ++i) {
+        const int S = hms[p->inst[i]]->nslab;
+        for (int s = 0; s < S; s += sl)
+          p->ranges.push_back(make_int4(i, s, std::min(S, s + sl), (int)p->ranges.size()));
+      }
+    }
+    p->rg_n[p->npk] = (int)p->ranges.size() - p->rg_start[p->npk];
+    ++p->npk;
+  }
+  return true;
+}
+
+size_t tn_zgroup_cross_bytes(const DevMesh &m) {
+  const size_t M = 3 * m.N;
+  return (size_t)m.E * 4 * m.N * M * M * sizeof(double);
+}
+
+size_t tn_zgroup_work_bytes(const DevMesh &m, const ZGroupPlan &p, int inst) {
+  size_t sum = 0;
+  for (int g = 1; g <= 4; ++g) {
+    const size_t MG = (size_t)g * 3 * m.N;
+    sum += (size_t)p.inst_n[(size_t)inst * 5 + g] * 3 * MG * MG * sizeof(double);
+  }
+  return sum;
+}
+
+cudaError_t tn_zgroup_setup(const DevMesh &m, const ZGroupPlan &p, const ZGroupDev &gd, int inst,
+                            double *blk, double *xblk, double *work, float *fac, double *fac64, int *status,
+                            cudaStream_t st) {
+  switch (m.N) {
+#define TN_CASE(NN) \
+    case NN: return zgroup_setup_n<NN>(m, p, gd, inst, blk, xblk, work, fac, fac64, status, st);
+    TN_CASE(3) TN_CASE(4) TN_CASE(5) TN_CASE(6) TN_CASE(7) TN_CASE(8) TN_CASE(9)
+#undef TN_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// per degree present (one for a single mesh) one launch (FP32) or three
+// (FP64): the first degree on st, the others on side streams forked from and
+// joined back into st (also inside a capture)
+cudaError_t tn_zgroup_solve(const DevMesh *m, const ZGroupDev &gd, int prec, const void *fac, const void *r, void *z,
+                            double *part_rz, double *part_rr, const int *done, TnWait *zerr, cudaStream_t st,
+                            const PcgFold *fold_in) {
+  const DevMesh one = m ? *m : DevMesh{};
+  cudaError_t err = cudaSuccess;
+  PcgFold fold = fold_in ? *fold_in : PcgFold();
+  if (fold.s) {  // the grids of the launches that fold, for the last-CTA count
+    fold.total = 0;
+    fold.nparts = tn_zgroup_partials(gd, prec);
+    fold.part = part_rz;
+    fold.part2 = part_rr;
+    for (int k = 0; k < gd.npk && err == cudaSuccess; ++k) {
+      int g = 0;
+      err = zgroup_launch(one, gd, k, prec, fac, r, z, part_rz, part_rr, done, zerr, st, false, fold, &g);
+      fold.total += g;
+    }
+    if (err != cudaSuccess) return err;
+  }
+  if (gd.npk > 1) err = cudaEventRecord(gd.fork, st);
+  bool used[kZgSide] = {false};
+  for (int k = 0; k < gd.npk && err == cudaSuccess; ++k) {
+    cudaStream_t sk = st;
+    if (k > 0) {
+      const int sd = (k - 1) % kZgSide;
+      sk = gd.side[sd];
+      if (!used[sd]) {
+        err = cudaStreamWaitEvent(sk, gd.fork, 0);
+        used[sd] = true;
+        if (err != cudaSuccess) break;
+      }
+    }
+    // (a launch behind an event is not a programmatic dependent)
+    err = zgroup_launch(one, gd, k, prec, fac, r, z, part_rz, part_rr, done, zerr, sk, gd.npk == 1, fold,
+                        nullptr);
+  }
+  for (int sd = 0; sd < kZgSide && err == cudaSuccess; ++sd) {
+    if (!used[sd]) continue;
+    err = cudaEventRecord(gd.join[sd], gd.side[sd]);
+    if (err == cudaSuccess) err = cudaStreamWaitEvent(st, gd.join[sd], 0);
+  }
+  return err;
+}
