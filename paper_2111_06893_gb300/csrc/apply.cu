@@ -1051,6 +1051,203 @@ cudaError_t launch_batch(const ApplyArgs &a, cudaStream_t st) {
 
 #define TN_FOR_N(CASE) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8) CASE(9)
 
+// ------------------------------------------------------------- energies
+// Energy of an element, 1/2 sum_p w_p detJ_p S_p : Y : S_p with S = sym grad u
+// (unlifted), by pencils as the operator: thread q keeps the zeta line of its
+// node (i, j) in registers, lines along xi and eta go through shared memory.
+// With G_ij = 2 S_ij (i != j), T = tr S, D = sum S_ii^2, O = sum G_ij^2 the
+// density is c12 T^2 + (c11 - c12) D + c44 O, so three sums per element do
+// (parts != 0: their split along the stiffness's eigen-modes, dilatational
+// (c11 + 2 c12) / 3 T^2, tetragonal (c11 - c12) (D - T^2 / 3) and shear
+// c44 O).  Bound by the FP64 pipe.  One thread per node with whole rows of D
+// serialised on the constant cache (a row per lane) and divided by dz at
+// every node: 549 -> 419 us at 8.0 M unknowns, p = 5 (FP64 pipe 35 -> 84 %).
+// SPLIT (few elements, one per CTA): three threads per pencil, one per
+// component, and every third node of the pencil, for latency.
+constexpr int kEnergyThreads = 256;
+template <int N>
+constexpr int energy_eb() { return kEnergyThreads / (N * N); }
+template <int N, bool SPLIT>
+constexpr size_t energy_smem(int eb) { return sizeof(double) * (size_t)eb * (SPLIT ? 9 : 6) * N * N * N; }
+
+// elements w0 .. of one mesh (meshes == nullptr: m1, element w) or of a batch
+// (element work[w].y of mirror work[w].x); out: 1 or 3 numbers per element
+template <int N, bool SPLIT>
+__global__ void __launch_bounds__(kEnergyThreads)
+energy_pencil_kernel(const DevMesh m1, const DevMesh *__restrict__ meshes, const int2 *__restrict__ work,
+                     const long long *__restrict__ dof_off, int nwork, int eb, const double *__restrict__ u,
+                     double *__restrict__ out, int parts) {
+  constexpr int N2 = N * N, n = N * N2, PT = SPLIT ? 3 * N2 : N2;  // threads per element
+  constexpr int NC = SPLIT ? 1 : 3, NK = SPLIT ? (N + 2) / 3 : N;     // components and nodes per thread
+  extern __shared__ __align__(16) double esm[];
+  grid_trigger();
+  const int tid = threadIdx.x, el = tid / PT, r = tid - el * PT, c0 = r / N2, q = r - c0 * N2, wi = blockIdx.x * eb + el;
+  const bool act = el < eb && wi < nwork;
+  double *const A = esm + (size_t)(act ? el : 0) * (SPLIT ? 9 : 6) * n, *const B = A + 3 * n;
+  const int2 wk = act && meshes ? work[wi] : make_int2(0, act ? wi : 0);
+  const DevMesh &m = meshes ? meshes[wk.x] : m1;
+  const int e = wk.y, s = e / m.ncol, col = e - s * m.ncol;
+  grid_wait();
+  const double *const ue = after_wait(u) + (meshes ? dof_off[wk.x] : 0) + (size_t)e * 3 * n + q;
+  double z[NC][N];
+  if (act) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int k = 0; k < N; ++k) B[(c0 + c) * n + k * N2 + q] = z[c][k] = ue[(c0 + c) * n + k * N2];
+  }
+  __syncthreads();
+  if (act) {  // xi lines: thread q has (j, k) = (q % N, q / N)
+#pragma unroll
+    for (int c = c0; c < c0 + NC; ++c) {
+      double v[N], o[N];
+#pragma unroll
+      for (int i = 0; i < N; ++i) v[i] = B[c * n + q * N + i];
+      line_eo<N, 0>(v, o);
+#pragma unroll
+      for (int i = 0; i < N; ++i) A[c * n + q * N + i] = o[i];
+    }
+  }
+  __syncthreads();
+  if (act) {  // eta lines, in place: (i, k) = (q % N, q / N)
+    const int at = (q / N) * N2 + q % N;
+#pragma unroll
+    for (int c = c0; c < c0 + NC; ++c) {
+      double v[N], o[N];
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j] = B[c * n + at + j * N];
+      line_eo<N, 0>(v, o);
+#pragma unroll
+      for (int j = 0; j < N; ++j) B[c * n + at + j * N] = o[j];
+    }
+  }
+  __syncthreads();
+  double sT = 0.0, sD = 0.0, sO = 0.0;
+  if (act) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) line_eo<N, 0>(z[c], z[c]);
+    if constexpr (SPLIT) {
+#pragma unroll
+      for (int k = 0; k < N; ++k) A[(6 + c0) * n + k * N2 + q] = z[0][k];
+    }
+  }
+  if constexpr (SPLIT) __syncthreads();
+  if (act) {
+    const double *cg = m.colgeo + (size_t)col * CG_NF * N2 + q, *sg = m.slabgeo + (size_t)s * SG_NF * N;
+    const double ixx = cg[CG_IXX * N2], ixy = cg[CG_IXY * N2], iex = cg[CG_IEX * N2], iey = cg[CG_IEY * N2];
+#pragma unroll
+    for (int kk = 0; kk < NK; ++kk) {
+      const int k = SPLIT ? 3 * kk + c0 : kk;
+      if (SPLIT && k >= N) break;
+      const double id = sg[SG_IDZ * N + k], wz = tabs<double>(N).w[k] * sg[SG_DZ * N + k];
+      const double *a = A + k * N2 + q, *b = B + k * N2 + q;
+      const double a0 = a[0], a1 = a[n], a2 = a[2 * n], b0 = b[0], b1 = b[n], b2 = b[2 * n];
+      const double z0 = SPLIT ? a[6 * n] : z[0][kk], z1 = SPLIT ? a[7 * n] : z[NC / 2][kk], z2 = SPLIT ? a[8 * n] : z[NC - 1][kk];
+      const double gxx = fm(ixx, a0, iex * b0), gyy = fm(ixy, a1, iey * b1), gzz = id * z2;
+      const double gxy = fm(ixx, a1, fm(iex, b1, fm(ixy, a0, iey * b0)));
+      const double gxz = fm(id, z0, fm(ixx, a2, iex * b2)), gyz = fm(id, z1, fm(ixy, a2, iey * b2));
+      const double t = (gxx + gyy) + gzz;
+      sT = fm(wz, t * t, sT);
+      sD = fm(wz, fm(gxx, gxx, fm(gyy, gyy, gzz * gzz)), sD);
+      sO = fm(wz, fm(gxy, gxy, fm(gxz, gxz, gyz * gyz)), sO);
+    }
+    const double w2 = 0.5 * tabs<double>(N).w[q % N] * tabs<double>(N).w[q / N] * cg[CG_DET * N2];
+    sT *= w2;
+    sD *= w2;
+    sO *= w2;
+  }
+  __syncthreads();
+  // the element's sums in a fixed order: rows of N threads, then the rows
+  if (act) {
+    A[r] = sT;
+    A[PT + r] = sD;
+    A[2 * PT + r] = sO;
+  }
+  __syncthreads();
+  constexpr int RW = PT / N;  // rows per sum
+  if (act && r < 3 * RW) {
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) t += A[r * N + i];
+    B[r] = t;
+  }
+  __syncthreads();
+  if (act && r == 0) {
+    double t[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < RW; ++i) {
+      t[0] += B[i];
+      t[1] += B[RW + i];
+      t[2] += B[2 * RW + i];
+    }
+    const double *lay = m.layer_c + 3 * m.slab_layer[s];
+    const double c11 = lay[0], c12 = lay[1], c44 = lay[2];
+    if (parts) {
+      out[3 * (size_t)wi] = (c11 + 2.0 * c12) / 3.0 * t[0];
+      out[3 * (size_t)wi + 1] = (c11 - c12) * (t[1] - t[0] / 3.0);
+      out[3 * (size_t)wi + 2] = c44 * t[2];
+    } else {
+      out[wi] = fm(c12, t[0], fm(c11 - c12, t[1], c44 * t[2]));
+    }
+  }
+}
+
+// layer blockIdx.x: the sum of its element energies, slab by slab in a fixed
+// order.  A block per layer: one block for all 41 layers of a mesh took 205 us,
+// more than the other 20 us of the call together.
+__global__ void layer_sum_kernel(const DevMesh m, const double *__restrict__ elem, double *__restrict__ out) {
+  __shared__ double red[8];
+  const int L = blockIdx.x;
+  grid_wait();
+  elem = after_wait(elem);
+  double acc = 0.0;
+  for (int s = 0; s < m.nslab; ++s) {
+    if (m.slab_layer[s] != L) continue;
+    for (int c = threadIdx.x; c < m.ncol; c += blockDim.x) acc += elem[(size_t)s * m.ncol + c];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
+    out[L] = sum;
+  }
+}
+
+// few elements (below 8 per SM, as for the operator): split pencils, one
+// element per CTA (64 elements, p = 3: 32 us a call, 37 with whole pencils);
+// else as many per CTA as its threads hold
+template <int N>
+cudaError_t launch_energy(const DevMesh &m, const DevMesh *meshes, const int2 *work, int nwork,
+                          const long long *dof_off, const double *u, double *out, int parts, cudaStream_t st) {
+  constexpr int EB = energy_eb<N>();
+  if (apply_small(nwork)) {
+    static int few_device = -1;
+    const cudaError_t err = allow_smem(energy_pencil_kernel<N, true>, energy_smem<N, true>(1), few_device);
+    if (err != cudaSuccess) return err;
+    return launch_pdl(energy_pencil_kernel<N, true>, nwork, (3 * N * N + 31) / 32 * 32, energy_smem<N, true>(1), st, m,
+                      meshes, work, dof_off, nwork, 1, u, out, parts);
+  }
+  static int configured_device = -1;
+  const cudaError_t err = allow_smem(energy_pencil_kernel<N, false>, energy_smem<N, false>(EB), configured_device);
+  if (err != cudaSuccess) return err;
+  return launch_pdl(energy_pencil_kernel<N, false>, (nwork + EB - 1) / EB, (EB * N * N + 31) / 32 * 32,
+                    energy_smem<N, false>(EB), st, m, meshes, work, dof_off, nwork, EB, u, out, parts);
+}
+
+cudaError_t energies(int N, const DevMesh &m, const DevMesh *meshes, const int2 *work, int nwork,
+                     const long long *dof_off, const double *u, double *out, int parts, cudaStream_t st) {
+  if (nwork <= 0) return cudaSuccess;
+  switch (N) {
+#define TN_CASE(NN) case NN: return launch_energy<NN>(m, meshes, work, nwork, dof_off, u, out, parts, st);
+    TN_FOR_N(TN_CASE)
+#undef TN_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 template <typename T>
 void fill_tabs(const LglTables *t, ApplyTabs<T> *out) {
   for (int N = TN_MIN_N; N <= TN_MAX_N; ++N) {
@@ -1159,4 +1356,19 @@ cudaError_t tn_tune_apply(ApplyArgs a, cudaStream_t st, float us[2]) {
   cudaEventDestroy(ev[0]);
   cudaEventDestroy(ev[1]);
   return err;
+}
+
+cudaError_t tn_launch_energy(const DevMesh &m, const double *u, double *elem, double *layer, cudaStream_t st) {
+  const cudaError_t err = energies(m.N, m, nullptr, nullptr, m.E, nullptr, u, elem, 0, st);
+  if (err != cudaSuccess) return err;
+  return launch_pdl(layer_sum_kernel, m.n_layers, 256, 0, st, m, (const double *)elem, layer);
+}
+
+cudaError_t tn_launch_energy_parts(const DevMesh &m, const double *u, double *parts, cudaStream_t st) {
+  return energies(m.N, m, nullptr, nullptr, m.E, nullptr, u, parts, 1, st);
+}
+
+cudaError_t tn_launch_energy_batch(int N, const DevMesh *meshes, const int2 *work, int nwork, const long long *dof_off,
+                                   const double *u, double *out, cudaStream_t st) {
+  return energies(N, DevMesh{}, meshes, work, nwork, dof_off, u, out, 0, st);
 }

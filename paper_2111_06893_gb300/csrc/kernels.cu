@@ -1,5 +1,5 @@
-// sm_103a kernels of the DG elasticity operator (Sec. 2.2), its right-hand
-// side, diagonal and per-layer energies.
+// sm_103a kernels of the DG elasticity operator (Sec. 2.2): its right-hand
+// side and diagonal, and the dual-number forms of the gradients.
 //
 // Operator (weak form of Eq. (dg_residuals), LGL quadrature, M = w detJ):
 //   y = sum_m D_m^T F^m  -  sum_faces W ( 1/2 (T + T_ext) - sigma P[[u]] )
@@ -11,7 +11,7 @@
 // Dirichlet faces (Eq. (bc), u_b = 0): u_ext = -u, T_ext = T, Y_* = Y.
 // Neumann faces: no term.
 //
-// The FP64 / FP32 applies are in apply.cu; here is the dual-number form of
+// The FP64 / FP32 applies and the energies are in apply.cu; here is the dual-number form of
 // the gradients.  One CTA per element, one thread per node.  The element's own
 // field is staged in shared memory; for each interior face the neighbour's
 // face values and its logical normal derivative are gathered (neighbour data
@@ -19,7 +19,6 @@
 // every node forms its strain, stress, face terms and fluxes, and finally the
 // transposed derivative contractions give A u.
 #include <cstdio>
-#include <type_traits>
 
 #include "tn_internal.h"
 
@@ -604,36 +603,32 @@ __global__ void diag_kernel(const DevMesh m, double *__restrict__ dg) {
 }
 
 // ------------------------------------------------------------- energies
-// elem[blockIdx.x] = 1/2 sum_p w_p detJ_p S_p : Y : S_p, S = sym grad u
-// (unlifted), for the elements e0 + blockIdx.x; T = Dual gives the derivative
-// along the seeded direction instead; scaled by w[layer] if w is given.
-template <int N, typename T>
+// elem[blockIdx.x] = derivative of 1/2 sum_p w_p detJ_p S_p : Y : S_p, S = sym
+// grad u (unlifted), of element work[blockIdx.x].y along the direction of seed
+// work[blockIdx.x].x, scaled by w[layer]
+template <int N>
 __global__ void __launch_bounds__(nthreads<N>())
-energy_kernel(const DevMesh m0, int e0, const double *__restrict__ u, const double *__restrict__ w,
-              double *__restrict__ elem, const int2 *__restrict__ work = nullptr,
-              const double *const *__restrict__ pseed = nullptr) {
-  DevMesh m = m0;  // work: as for apply_kernel
-  int ework = -1;
-  if (work) {
-    const int2 wk = work[blockIdx.x];
-    ework = wk.y;
-    m.d_slabdz = pseed[2 * wk.x];
-    m.d_layer_c = pseed[2 * wk.x + 1];
-  }
+energy_dual_kernel(const DevMesh m0, const double *__restrict__ u, const double *__restrict__ w,
+                   double *__restrict__ elem, const int2 *__restrict__ work,
+                   const double *const *__restrict__ pseed) {
+  const int2 wk = work[blockIdx.x];
+  DevMesh m = m0;
+  m.d_slabdz = pseed[2 * wk.x];
+  m.d_layer_c = pseed[2 * wk.x + 1];
   constexpr int n = N * N * N, N2 = N * N, NT = nthreads<N>();
   __shared__ double su[3 * n];
   __shared__ double red[NT / 32];
-  const int e = work ? ework : e0 + blockIdx.x, tid = threadIdx.x;
+  const int e = wk.y, tid = threadIdx.x;
   const int s = e / m.ncol, c = e - s * m.ncol;
   for (int t = tid; t < 3 * n; t += NT) su[t] = u[(size_t)e * 3 * n + t];
   __syncthreads();
   const double *cg = m.colgeo + (size_t)c * CG_NF * N2;
   const int L = m.slab_layer[s];
-  const T c11 = layer_coef<T>(m, L, 0), c12 = layer_coef<T>(m, L, 1), c44 = layer_coef<T>(m, L, 2);
+  const Dual c11 = layer_coef<Dual>(m, L, 0), c12 = layer_coef<Dual>(m, L, 1), c44 = layer_coef<Dual>(m, L, 2);
   double en = 0.0;
   if (tid < n) {
     const int p = tid, i = p % N, j = (p / N) % N, k = p / N2;
-    T dxi[3], deta[3], dzeta[3];
+    Dual dxi[3], deta[3], dzeta[3];
     for (int cc = 0; cc < 3; ++cc) {
       const double *v = su + cc * n;
       double a0 = 0, a1 = 0, a2 = 0;
@@ -643,20 +638,18 @@ energy_kernel(const DevMesh m0, int e0, const double *__restrict__ u, const doub
         a1 += Tab<double>::D(N, j, mm) * v[(k * N + mm) * N + i];
         a2 += Tab<double>::D(N, k, mm) * v[(mm * N + j) * N + i];
       }
-      dxi[cc] = T(a0); deta[cc] = T(a1); dzeta[cc] = T(a2);
+      dxi[cc] = Dual(a0); deta[cc] = Dual(a1); dzeta[cc] = Dual(a2);
     }
     const int q = j * N + i;
-    const T dz = slab_dz<T>(m, s, k);
-    const Sym<T> S = strain<T>(dxi, deta, dzeta, T(cg[CG_IXX * N2 + q]), T(cg[CG_IXY * N2 + q]),
-                               T(cg[CG_IEX * N2 + q]), T(cg[CG_IEY * N2 + q]), T(1.0) / dz);
-    const Sym<T> sg2 = stress(S, c11, c12, c44);
-    const T dens = S.xx * sg2.xx + S.yy * sg2.yy + S.zz * sg2.zz +
-                   T(2.0) * (S.xy * sg2.xy + S.xz * sg2.xz + S.yz * sg2.yz);
-    const T val = T(0.5 * Tab<double>::w(N, i) * Tab<double>::w(N, j) * Tab<double>::w(N, k) *
+    const Dual dz = slab_dz<Dual>(m, s, k);
+    const Sym<Dual> S = strain<Dual>(dxi, deta, dzeta, Dual(cg[CG_IXX * N2 + q]), Dual(cg[CG_IXY * N2 + q]),
+                               Dual(cg[CG_IEX * N2 + q]), Dual(cg[CG_IEY * N2 + q]), Dual(1.0) / dz);
+    const Sym<Dual> sg2 = stress(S, c11, c12, c44);
+    const Dual dens = S.xx * sg2.xx + S.yy * sg2.yy + S.zz * sg2.zz +
+                   Dual(2.0) * (S.xy * sg2.xy + S.xz * sg2.xz + S.yz * sg2.yz);
+    const Dual val = Dual(0.5 * Tab<double>::w(N, i) * Tab<double>::w(N, j) * Tab<double>::w(N, k) *
                     cg[CG_DET * N2 + q]) * dz * dens;
-    if constexpr (std::is_same<T, Dual>::value) en = val.d;
-    else en = val;
-    if (w) en *= w[L];
+    en = val.d * w[L];
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
@@ -666,127 +659,6 @@ energy_kernel(const DevMesh m0, int e0, const double *__restrict__ u, const doub
     double sum = 0.0;
     for (int ww = 0; ww < NT / 32; ++ww) sum += red[ww];
     elem[blockIdx.x] = sum;
-  }
-}
-
-// The layer energy split along the eigen-modes of the (cubic-aligned)
-// stiffness, for separate loss angles per modulus (Sec. 2.1): with
-// T = tr S, D = sum_i S_ii^2, O = S_xy^2 + S_xz^2 + S_yz^2,
-//   dilatational   1/2 (c11 + 2 c12) / 3 T^2
-//   tetragonal     1/2 (c11 - c12) (D - T^2 / 3)
-//   shear          1/2 4 c44 O
-// (they sum to 1/2 S : Y : S; isotropic: bulk K T^2 / 2 and shear
-// mu S_dev : S_dev = tetragonal + shear).  parts[3 e + j], element e.
-template <int N>
-__global__ void __launch_bounds__(nthreads<N>())
-energy_parts_kernel(const DevMesh m, const double *__restrict__ u, double *__restrict__ parts) {
-  constexpr int n = N * N * N, N2 = N * N, NT = nthreads<N>();
-  __shared__ double su[3 * n];
-  __shared__ double red[3][NT / 32];
-  const int e = blockIdx.x, tid = threadIdx.x;
-  const int s = e / m.ncol, c = e - s * m.ncol;
-  for (int t = tid; t < 3 * n; t += NT) su[t] = u[(size_t)e * 3 * n + t];
-  __syncthreads();
-  const double *cg = m.colgeo + (size_t)c * CG_NF * N2;
-  const int L = m.slab_layer[s];
-  const double c11 = m.layer_c[3 * L], c12 = m.layer_c[3 * L + 1], c44 = m.layer_c[3 * L + 2];
-  double pe[3] = {0.0, 0.0, 0.0};
-  if (tid < n) {
-    const int p = tid, i = p % N, j = (p / N) % N, k = p / N2;
-    double dxi[3], deta[3], dzeta[3];
-    for (int cc = 0; cc < 3; ++cc) {
-      const double *v = su + cc * n;
-      double a0 = 0, a1 = 0, a2 = 0;
-#pragma unroll
-      for (int mm = 0; mm < N; ++mm) {
-        a0 += Tab<double>::D(N, i, mm) * v[(k * N + j) * N + mm];
-        a1 += Tab<double>::D(N, j, mm) * v[(k * N + mm) * N + i];
-        a2 += Tab<double>::D(N, k, mm) * v[(mm * N + j) * N + i];
-      }
-      dxi[cc] = a0; deta[cc] = a1; dzeta[cc] = a2;
-    }
-    const int q = j * N + i;
-    const double dz = slab_dz<double>(m, s, k);
-    const Sym<double> S = strain<double>(dxi, deta, dzeta, cg[CG_IXX * N2 + q], cg[CG_IXY * N2 + q],
-                                         cg[CG_IEX * N2 + q], cg[CG_IEY * N2 + q], 1.0 / dz);
-    const double wJ = 0.5 * Tab<double>::w(N, i) * Tab<double>::w(N, j) * Tab<double>::w(N, k) *
-                      cg[CG_DET * N2 + q] * dz;
-    const double T = S.xx + S.yy + S.zz, D = S.xx * S.xx + S.yy * S.yy + S.zz * S.zz;
-    const double O = S.xy * S.xy + S.xz * S.xz + S.yz * S.yz;
-    pe[0] = wJ * (c11 + 2.0 * c12) / 3.0 * T * T;
-    pe[1] = wJ * (c11 - c12) * (D - T * T / 3.0);
-    pe[2] = wJ * 4.0 * c44 * O;
-  }
-#pragma unroll
-  for (int jj = 0; jj < 3; ++jj) {
-    double v = pe[jj];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((tid & 31) == 0) red[jj][tid >> 5] = v;
-  }
-  __syncthreads();
-  if (tid < 3) {
-    double sum = 0.0;
-    for (int ww = 0; ww < NT / 32; ++ww) sum += red[tid][ww];
-    parts[(size_t)e * 3 + tid] = sum;
-  }
-}
-
-// element energies of a batch: out[b] = energy of element work[b].y of
-// instance work[b].x (FP64)
-template <int N>
-__global__ void __launch_bounds__(nthreads<N>())
-energy_batch_kernel(const DevMesh *__restrict__ meshes, const int2 *__restrict__ work,
-                    const long long *__restrict__ dof_off, const double *__restrict__ u, double *__restrict__ out) {
-  constexpr int n = N * N * N, N2 = N * N, NT = nthreads<N>();
-  __shared__ double su[3 * n];
-  __shared__ double red[NT / 32];
-  __shared__ __align__(16) unsigned char m_raw[sizeof(DevMesh)];
-  DevMesh &m = *reinterpret_cast<DevMesh *>(m_raw);
-  const int2 w = work[blockIdx.x];
-  const int tid = threadIdx.x;
-  if (tid == 0) memcpy(m_raw, &meshes[w.x], sizeof(DevMesh));
-  __syncthreads();
-  const int e = w.y;
-  const int s = e / m.ncol, c = e - s * m.ncol;
-  const double *ue = u + dof_off[w.x] + (size_t)e * 3 * n;
-  for (int t = tid; t < 3 * n; t += NT) su[t] = ue[t];
-  __syncthreads();
-  const double *cg = m.colgeo + (size_t)c * CG_NF * N2;
-  const int L = m.slab_layer[s];
-  const double c11 = m.layer_c[3 * L], c12 = m.layer_c[3 * L + 1], c44 = m.layer_c[3 * L + 2];
-  double en = 0.0;
-  if (tid < n) {
-    const int p = tid, i = p % N, j = (p / N) % N, k = p / N2;
-    double dxi[3], deta[3], dzeta[3];
-    for (int cc = 0; cc < 3; ++cc) {
-      const double *v = su + cc * n;
-      double a0 = 0, a1 = 0, a2 = 0;
-#pragma unroll
-      for (int mm = 0; mm < N; ++mm) {
-        a0 += Tab<double>::D(N, i, mm) * v[(k * N + j) * N + mm];
-        a1 += Tab<double>::D(N, j, mm) * v[(k * N + mm) * N + i];
-        a2 += Tab<double>::D(N, k, mm) * v[(mm * N + j) * N + i];
-      }
-      dxi[cc] = a0; deta[cc] = a1; dzeta[cc] = a2;
-    }
-    const int q = j * N + i;
-    const double dz = m.slabgeo[((size_t)s * SG_NF + SG_DZ) * N + k];
-    const Sym<double> S = strain<double>(dxi, deta, dzeta, cg[CG_IXX * N2 + q], cg[CG_IXY * N2 + q],
-                                         cg[CG_IEX * N2 + q], cg[CG_IEY * N2 + q], 1.0 / dz);
-    const Sym<double> sg2 = stress(S, c11, c12, c44);
-    const double dens = S.xx * sg2.xx + S.yy * sg2.yy + S.zz * sg2.zz +
-                        2.0 * (S.xy * sg2.xy + S.xz * sg2.xz + S.yz * sg2.yz);
-    en = 0.5 * Tab<double>::w(N, i) * Tab<double>::w(N, j) * Tab<double>::w(N, k) * cg[CG_DET * N2 + q] * dz * dens;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) en += __shfl_xor_sync(0xffffffffu, en, o);
-  if ((tid & 31) == 0) red[tid >> 5] = en;
-  __syncthreads();
-  if (tid == 0) {
-    double sum = 0.0;
-    for (int ww = 0; ww < NT / 32; ++ww) sum += red[ww];
-    out[blockIdx.x] = sum;
   }
 }
 
@@ -884,34 +756,6 @@ __global__ void rhs_dr0_kernel(const DevMesh m, double r0, double F0, const doub
   }
 }
 
-// one block: per layer, sum the element energies slab by slab in a fixed order
-__global__ void layer_sum_kernel(const DevMesh m, const double *__restrict__ elem, double *__restrict__ out) {
-  __shared__ double red[32];
-  for (int L = 0; L < m.n_layers; ++L) {
-    double acc = 0.0;
-    for (int s = 0; s < m.nslab; ++s) {
-      if (m.slab_layer[s] != L) continue;
-      for (int c = threadIdx.x; c < m.ncol; c += blockDim.x) acc += elem[(size_t)s * m.ncol + c];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double sum = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
-      out[L] = sum;
-    }
-    __syncthreads();
-  }
-}
-
-template <int N>
-cudaError_t launch_energy_n(const DevMesh &m, const double *u, double *elem, cudaStream_t st) {
-  energy_kernel<N, double><<<m.E, nthreads<N>(), 0, st>>>(m, 0, u, nullptr, elem);
-  return cudaGetLastError();
-}
-
 }  // namespace
 
 int tn_sm_count() {
@@ -934,34 +778,6 @@ cudaError_t tn_launch_rhs(const DevMesh &m, double r0, double F0, double *b, cud
 cudaError_t tn_launch_diag(const DevMesh &m, double *d, cudaStream_t st) {
   diag_kernel<<<m.E, 128, 0, st>>>(m, d);
   return cudaGetLastError();
-}
-
-cudaError_t tn_launch_energy(const DevMesh &m, const double *u, double *elem, double *layer,
-                             cudaStream_t st) {
-  cudaError_t err;
-  switch (m.N) {
-    case 3: err = launch_energy_n<3>(m, u, elem, st); break;
-    case 4: err = launch_energy_n<4>(m, u, elem, st); break;
-    case 5: err = launch_energy_n<5>(m, u, elem, st); break;
-    case 6: err = launch_energy_n<6>(m, u, elem, st); break;
-    case 7: err = launch_energy_n<7>(m, u, elem, st); break;
-    case 8: err = launch_energy_n<8>(m, u, elem, st); break;
-    case 9: err = launch_energy_n<9>(m, u, elem, st); break;
-    default: return cudaErrorInvalidValue;
-  }
-  if (err != cudaSuccess) return err;
-  layer_sum_kernel<<<1, 256, 0, st>>>(m, elem, layer);
-  return cudaGetLastError();
-}
-
-cudaError_t tn_launch_energy_parts(const DevMesh &m, const double *u, double *parts, cudaStream_t st) {
-  switch (m.N) {
-#define TN_CASE(NN) \
-    case NN: energy_parts_kernel<NN><<<m.E, nthreads<NN>(), 0, st>>>(m, u, parts); return cudaGetLastError();
-    TN_CASE(3) TN_CASE(4) TN_CASE(5) TN_CASE(6) TN_CASE(7) TN_CASE(8) TN_CASE(9)
-#undef TN_CASE
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 #define TN_DISPATCH_N(...)                  \
@@ -999,7 +815,7 @@ cudaError_t tn_launch_energy_dual_work(const DevMesh &m, const int2 *work, int n
                                        const double *u, const double *w, double *epart, cudaStream_t st) {
   if (nwork <= 0) return cudaSuccess;
   TN_DISPATCH_N({
-    energy_kernel<NN, Dual><<<nwork, nthreads<NN>(), 0, st>>>(m, 0, u, w, epart, work, pseed);
+    energy_dual_kernel<NN><<<nwork, nthreads<NN>(), 0, st>>>(m, u, w, epart, work, pseed);
     return cudaGetLastError();
   })
 }
@@ -1013,18 +829,4 @@ cudaError_t tn_launch_rhs_dr0(const DevMesh &m, double r0, double F0, const doub
                               int nparts, cudaStream_t st) {
   rhs_dr0_kernel<<<nparts, 256, 0, st>>>(m, r0, F0, lam, part);
   return cudaGetLastError();
-}
-
-cudaError_t tn_launch_energy_batch(int N, const DevMesh *meshes, const int2 *work, int nwork,
-                                   const long long *dof_off, const double *u, double *out, cudaStream_t st) {
-  if (nwork <= 0) return cudaSuccess;
-  switch (N) {
-#define TN_CASE(NN)                                                                                    \
-  case NN:                                                                                            \
-    energy_batch_kernel<NN><<<nwork, nthreads<NN>(), 0, st>>>(meshes, work, dof_off, u, out);          \
-    return cudaGetLastError();
-    TN_CASE(3) TN_CASE(4) TN_CASE(5) TN_CASE(6) TN_CASE(7) TN_CASE(8) TN_CASE(9)
-#undef TN_CASE
-    default: return cudaErrorInvalidValue;
-  }
 }
