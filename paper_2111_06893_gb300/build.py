@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libthermonoise.so")
-SOURCES = ["apply.cu", "kernels.cu", "precond.cu", "zgroup.cu", "solver.cu", "capi.cu", "peak.cu", "mesh.cpp"]
+SOURCES = ["apply.cu", "kernels.cu", "precond.cu", "zgfactor.cu", "zgroup.cu", "solver.cu", "capi.cu", "peak.cu", "mesh.cpp"]
 # the operator's kernels round alike in all their forms: fused operations are written out there
 NO_CONTRACT = ["apply.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

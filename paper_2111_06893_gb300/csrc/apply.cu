@@ -1059,9 +1059,10 @@ cudaError_t launch_batch(const ApplyArgs &a, cudaStream_t st) {
 // density is c12 T^2 + (c11 - c12) D + c44 O, so three sums per element do
 // (parts != 0: their split along the stiffness's eigen-modes, dilatational
 // (c11 + 2 c12) / 3 T^2, tetragonal (c11 - c12) (D - T^2 / 3) and shear
-// c44 O).  Bound by the FP64 pipe.  One thread per node with whole rows of D
-// serialised on the constant cache (a row per lane) and divided by dz at
-// every node: 549 -> 419 us at 8.0 M unknowns, p = 5 (FP64 pipe 35 -> 84 %).
+// c44 O).  Bound by the FP64 pipe (84 % busy; 77 operations per node).  One
+// thread per node with whole rows of D, the stress and a division by dz at
+// every node kept the pipe as busy with more: 549 -> 419 us at 8.0 M unknowns,
+// p = 5.
 // SPLIT (few elements, one per CTA): three threads per pencil, one per
 // component, and every third node of the pencil, for latency.
 constexpr int kEnergyThreads = 256;

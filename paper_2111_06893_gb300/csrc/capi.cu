@@ -395,19 +395,16 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   char msg[160];
   if (!tn_zgroup_plan(hms.data(), n, &c->gplan, msg, sizeof(msg))) return fail(TN_EINVAL, "%s", msg);
   const ZGroupPlan &p = c->gplan;
-  size_t bb = 0, xb = 0, wb = 0;
+  size_t bb = 0, xb = 0;
   for (int i = 0; i < n; ++i) {
-    const size_t b1 = tn_zline_block_bytes(dms[i]), x1 = tn_zgroup_cross_bytes(dms[i]),
-                 w1 = tn_zgroup_work_bytes(dms[i], p, i);
+    const size_t b1 = tn_zline_block_bytes(dms[i]), x1 = tn_zgroup_cross_bytes(dms[i]);
     bb = b1 > bb ? b1 : bb;
     xb = x1 > xb ? x1 : xb;
-    wb = w1 > wb ? w1 : wb;
   }
   const size_t fb = (size_t)p.nfac * sizeof(float), fb64 = (size_t)p.nfac64 * sizeof(double);
-  double *blk = nullptr, *xblk = nullptr, *work = nullptr;
+  double *blk = nullptr, *xblk = nullptr;
   cudaError_t e = cudaMalloc((void **)&blk, bb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&xblk, xb);
-  if (e == cudaSuccess) e = cudaMalloc((void **)&work, wb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gfac, fb);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gfac64, fb64);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gpart, sizeof(double) * 2 * std::max(p.ranges.size(), p.lines.size()));  // r.z, r.r
@@ -425,10 +422,10 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   const size_t o_inst = pack.add(p.inst.data(), sizeof(int) * p.inst.size());
   if (e == cudaSuccess) e = pack.upload(&c->d_gplan);
   if (e != cudaSuccess) {
-    dfree(blk); dfree(xblk); dfree(work);
+    dfree(blk); dfree(xblk);
     free_zgroup(c);
     cudaGetLastError();
-    return fail(TN_ENOMEM, "grouped-line preconditioner needs %.2f GB: %s", (bb + xb + wb + fb + fb64) / 1e9,
+    return fail(TN_ENOMEM, "grouped-line preconditioner needs %.2f GB: %s", (bb + xb + fb + fb64) / 1e9,
                 cudaGetErrorString(e));
   }
   ZGroupDev &g = c->zgd;
@@ -459,11 +456,11 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   int status = 0;
   if (e == cudaSuccess) e = cudaMemsetAsync(c->gstatus, 0, 2 * sizeof(int), st);
   for (int i = 0; i < n && e == cudaSuccess; ++i)  // one mirror after another (shared set-up scratch)
-    e = tn_zgroup_setup(dms[i], p, c->zgd, i, blk, xblk, work, c->gfac, c->gfac64,
+    e = tn_zgroup_setup(dms[i], p, c->zgd, i, blk, xblk, c->gfac, c->gfac64,
                         c->gstatus, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&status, c->gstatus, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  dfree(blk); dfree(xblk); dfree(work);
+  dfree(blk); dfree(xblk);
   if (e != cudaSuccess) { free_zgroup(c); return cuda_fail(e, "grouped-line set-up"); }
   if (status) { free_zgroup(c); return fail(TN_EBREAKDOWN, "grouped-line block not positive definite"); }
   c->gready = true;
@@ -658,6 +655,7 @@ tn_status tn_create(tn_ctx **out, int device, void *cuda_stream) {
     if (e == cudaSuccess) e = tn_upload_lgl_apply(&tabs);
     if (e == cudaSuccess) e = tn_upload_lgl_precond(&tabs);
     if (e == cudaSuccess) e = tn_upload_lgl_zgroup(&tabs);
+    if (e == cudaSuccess) e = tn_upload_lgl_zgfactor(&tabs);
   }
   if (e != cudaSuccess) {
     tn_destroy(c);

@@ -1,4 +1,4 @@
-// Column-line (precond.cu) and grouped-line (zgroup.cu) block preconditioners.
+// Column-line (precond.cu) and grouped-line (zgroup.cu, zgfactor.cu) block preconditioners.
 #pragma once
 
 #include <cstddef>
@@ -22,6 +22,7 @@ cudaError_t tn_zline_solve(const DevMesh &m, int prec, const void *fac, void *r,
                            cudaStream_t st);
 cudaError_t tn_upload_lgl_precond(const LglTables *t);
 cudaError_t tn_upload_lgl_zgroup(const LglTables *t);
+cudaError_t tn_upload_lgl_zgfactor(const LglTables *t);
 // the FP64 line blocks (tn_zline_block_bytes(m) at blk)
 cudaError_t tn_zline_blocks(const DevMesh &m, double *blk, cudaStream_t st);
 // batch: warp w of block b solves line work[4 b + w] = (instance, line); factors of
@@ -82,14 +83,12 @@ struct ZGroupDev {
 };
 bool tn_zgroup_plan(const tn::HostMesh *const *hms, int n, ZGroupPlan *plan, char *msg, int msglen);
 size_t tn_zgroup_cross_bytes(const DevMesh &m);                                // FP64 cross-line blocks (set-up)
-size_t tn_zgroup_work_bytes(const DevMesh &m, const ZGroupPlan &p, int inst);  // FP64 scratch (set-up)
 // factors of mirror `inst` (its mesh m); blk: tn_zline_block_bytes(m);
 // fac / fac64: plan.nfac / nfac64 entries; *status = 1 on a non-positive pivot.  The
 // group sizes factor at once on st and gd's first three side streams
 // (forked from and joined back into st with gd's events).
 cudaError_t tn_zgroup_setup(const DevMesh &m, const ZGroupPlan &p, const ZGroupDev &gd, int inst,
-                            double *blk, double *xblk, double *work, float *fac, double *fac64, int *status,
-                            cudaStream_t st);
+                            double *blk, double *xblk, float *fac, double *fac64, int *status, cudaStream_t st);
 // partial sums of r.z (and of r.r) of one solve: one per group (FP32) or slab range (FP64)
 inline int tn_zgroup_partials(const ZGroupDev &gd, int prec) { return prec == TN_F64 ? gd.nranges : gd.ngroups; }
 // z = M^{-1} r over the groups (m: the mesh, nullptr for a batch); partial

@@ -1,5 +1,6 @@
-// Grouped-line block preconditioner (the default of the Krylov solves): plan,
-// set-up and solve.  See precond.cu for the single-line form it extends.
+// Grouped-line block preconditioner (the default of the Krylov solves): plan
+// and solve; zgfactor.cu is its set-up.  See precond.cu for the single-line
+// form it extends.
 #include <algorithm>
 #include <cstdio>
 #include <type_traits>
@@ -8,6 +9,7 @@
 #include "tn_device.h"
 #include "tn_internal.h"
 #include "tn_precond.h"
+#include "tn_zgroup.h"
 
 // device constants are per translation unit (no relocatable device code):
 // this file keeps its own copy of the LGL tables
@@ -16,383 +18,6 @@ __constant__ LglTables c_lgl_zg;
 cudaError_t tn_upload_lgl_zgroup(const LglTables *t) { return cudaMemcpyToSymbol(c_lgl_zg, t, sizeof(LglTables)); }
 
 namespace {
-
-#define LD(a, b) c_lgl_zg.D[N][(a) * N + (b)]
-#define LW(a) c_lgl_zg.w[N][(a)]
-
-// The lines through the matching nodes of two columns that share a lateral
-// face are coupled by that face's interior-penalty and flux terms (Eqs.
-// (numflux), (penalty)), which the single-line blocks leave out; with the
-// penalty ~ C (p + 1)^2 / h these are the stiffest couplings left.  A group
-// is a set of lines joined by such face matches (1 to 4 lines: a node inside
-// a column face, on a column edge or at a corner where up to four columns
-// meet); its block is the exact principal sub-matrix of A on all its lines,
-// again block tridiagonal over the slabs, with 3 g N unknowns per slab and
-// the cross-line face terms in the diagonal blocks.
-
-// Cross-line block of element e = (s, c), lateral face f and face position t:
-// rows = the line through the face node (this element), columns = the line
-// through the matching node of the neighbour column (same slab):
-//   -1/2 V^T W Tr_ext + 1/2 Tr^T W V_ext - V^T W Pen V_ext
-// restricted to the two lines (the neighbour's traction and this element's
-// test traction reduce to the zeta derivative and the diagonal xi / eta
-// derivative entries on a line).  Zero where f has no neighbour.
-template <int N>
-__global__ void zgroup_cross_kernel(const DevMesh m, double *__restrict__ xblk) {
-  constexpr int M = 3 * N, N2 = N * N;
-  const int e = blockIdx.x, t = threadIdx.x % N, f = threadIdx.x / N;
-  if (f >= 4) return;
-  const int s = e / m.ncol, c = e - s * m.ncol;
-  double *X = xblk + (((size_t)e * 4 + f) * N + t) * M * M;
-  for (int q = 0; q < M * M; ++q) X[q] = 0.0;
-  const int nbc = m.colnb[4 * c + f];
-  if (nbc < 0) return;
-  const int d = f >> 1, sd = f & 1, end = sd ? N - 1 : 0;
-  const int i = d == 0 ? end : t, j = d == 0 ? t : end;
-  const int code = m.colnbf[4 * c + f];
-  const int f2 = code & 3, d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0;
-  const int a2 = (code >> 2) ? N - 1 - t : t;
-  const int i2 = d2 == 0 ? end2 : a2, j2 = d2 == 0 ? a2 : end2;
-  const double *cg = m.colgeo + (size_t)c * CG_NF * N2;
-  const double *cg2 = m.colgeo + (size_t)nbc * CG_NF * N2;
-  const int q1 = j * N + i, q2 = j2 * N + i2;
-  const double ixx = cg[CG_IXX * N2 + q1], ixy = cg[CG_IXY * N2 + q1];
-  const double iex = cg[CG_IEX * N2 + q1], iey = cg[CG_IEY * N2 + q1], det2 = cg[CG_DET * N2 + q1];
-  const double jxx = cg2[CG_IXX * N2 + q2], jxy = cg2[CG_IXY * N2 + q2];
-  const double jex = cg2[CG_IEX * N2 + q2], jey = cg2[CG_IEY * N2 + q2];
-  const double *sg = m.slabgeo + (size_t)s * SG_NF * N;
-  double dz[N];
-  for (int k = 0; k < N; ++k) dz[k] = sg[SG_DZ * N + k];
-  const int L = m.slab_layer[s];  // both sides lie in slab s: one material
-  const double c11 = m.layer_c[3 * L], c12 = m.layer_c[3 * L + 1], c44 = m.layer_c[3 * L + 2];
-  const double rx = d == 0 ? ixx : iex, ry = d == 0 ? ixy : iey;
-  const double mag = sqrt(rx * rx + ry * ry);
-  const double n[3] = {(sd ? 1.0 : -1.0) * rx / mag, (sd ? 1.0 : -1.0) * ry / mag, 0.0};
-  const double sx = d2 == 0 ? jxx : jex, sy = d2 == 0 ? jxy : jey;
-  const double h = 2.0 / mag, h2 = 2.0 / sqrt(sx * sx + sy * sy);
-  const double sig = (double)((m.p + 1) * (m.p + 1)) * m.penC / (h < h2 ? h : h2);
-  const double Dii = LD(i, i), Djj = LD(j, j), Dii2 = LD(i2, i2), Djj2 = LD(j2, j2);
-  const double wt = d == 0 ? LW(j) : LW(i);
-  for (int k = 0; k < N; ++k) {
-    const double Wk = wt * LW(k) * det2 * dz[k] * mag;
-    for (int k2 = 0; k2 < N; ++k2) {
-      const double Wk2 = wt * LW(k2) * det2 * dz[k2] * mag;
-      // neighbour basis (i2, j2, k2) at its node (i2, j2, k); own basis (i, j, k) at (i, j, k2)
-      const double l2[3] = {k2 == k ? Dii2 : 0.0, k2 == k ? Djj2 : 0.0, LD(k, k2)};
-      const double l1[3] = {k == k2 ? Dii : 0.0, k == k2 ? Djj : 0.0, LD(k2, k)};
-      double g2[3], g1[3];
-      phys(l2, jxx, jxy, jex, jey, dz[k], g2);
-      phys(l1, ixx, ixy, iex, iey, dz[k2], g1);
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-          double v = -0.5 * Wk * Qab(a, b, n, g2, c11, c12, c44) + 0.5 * Wk2 * Qab(b, a, n, g1, c11, c12, c44);
-          if (k == k2) v -= Wk * sig * Qab(a, b, n, n, c11, c12, c44);
-          X[(a * N + k) * M + b * N + k2] = v;
-        }
-    }
-  }
-}
-
-// FP32 record of slab s: [S_s^{-1} packed by columns (lower triangle,
-// zlp(MG)) | O_{s-1} in factored form (8 MG) | W_s], S_s = L_s L_s^T the
-// slab's Schur complement of the block Cholesky (S_s^{-1} = Linv_s^T
-// Linv_s).  The coupling block O_{s-1} (rows: slab s - 1,
-// columns: slab s, block diagonal over the lines) is nonzero only in the
-// rows of the bottom-face nodes (k = 0) and the columns of the top-face
-// nodes (k2 = N - 1) of each line (Eqs. (numflux), (penalty) on the zeta
-// face), so O = E_0 X^T + Y E_{N-1}^T with per row t: X[t][a] = O[(a, 0), t]
-// and Y[t][b] = O[t, (b, N - 1)] (Y zero on k = 0 rows).  Row t stores
-// X[t][0..2], 0, Y[t][0..2], 0.  The solve applies the coupling through
-// these factors instead of storing Z_s = Linv_{s-1} O_{s-1} densely.
-// The record ends with the backward sweep's coupling W_s = S_s^{-1} [Y_s | E_0]
-// (MG x 6G, rows padded to zp_ws(G)), S_s = L_s L_s^T the slab's Schur
-// complement and Y_s, E_0 of O_s (the coupling to slab s + 1): per line l,
-// column 6 l + b holds Y of component b and column 6 l + 3 + a the unit
-// vector of row (a, k = 0); zero for the last slab.  With it the backward
-// step x_s = Linv_s^T (y_s - Linv_s O_s x_{s+1}) = w_s - W_s v, v the six
-// numbers per line x_{s+1}(b, N - 1) and X^T x_{s+1}.
-__host__ __device__ constexpr int zp_ws(int G) { return pad4(6 * G); }
-__host__ __device__ constexpr int zp_rec(int MG, int G) { return zlp(MG) + 8 * MG + MG * zp_ws(G); }
-
-// FP64 solve.  The block O_{s-1} (rows: slab s - 1, columns: slab s, block
-// diagonal over the lines) is nonzero only in the rows of the bottom-face
-// nodes (k = 0) and the columns of the top-face nodes (k = N - 1) of each line
-// (Eqs. (numflux), (penalty) on the zeta face), so O_{s-1} = U_{s-1} V_s^T
-// with six columns per line l: U = [Y | E_0] (column 6 l + b: Y of component
-// b; 6 l + 3 + a: the unit vector of row (a, k = 0)) and V = [E_{N-1} | X]
-// (6 l + b: the unit vector of row (b, k = N - 1); 6 l + 3 + a: X of component
-// a).  Only the zeta derivative couples away from the face node, so with D
-// the derivative matrix
-//   Y[(b, k)][b] = y_b D(0, k), k != 0;      X[(a, k)][a] = x_a D(N-1, k), k != N-1
-// and X has a full 3 x 3 block in the rows k = N - 1 (all else zero): 15
-// numbers per line.
-//
-// Elimination, S_s the slab's Schur complement, W_s = S_s^{-1} U_s and Q_s =
-// S_s^{-1} V_s:
-//   w_s = S_s^{-1} (r_s - V_s g_{s-1}),   g_s = U_s^T w_s
-//   x_s = w_s - W_s f_{s+1},              f_s = V_s^T x_s
-// As written (the FP32 solve) each slab waits for the full solve of the one
-// above it (forward) or below it (backward): two chains of S dense products.
-// But only the 6 g numbers g and f cross an interface:
-//   a_s = S_s^{-1} r_s,   c_s = U_s^T a_s,   d_s = V_s^T a_s
-//   g_s = c_s - K_s g_{s-1},   f_s = d_s - H_s g_{s-1} - K_s^T f_{s+1}
-//   x_s = a_s - Q_s g_{s-1} - W_s f_{s+1}
-// with K_s = W_s^T V_s and H_s = V_s^T Q_s (6 g x 6 g).  The dense products of
-// all slabs are independent, and the chains run on 6 g numbers per step.
-// The factors grow (12 g entries more per row, 72 g^2 more per slab) and the
-// arithmetic shrinks: FP64 is bound by its arithmetic (an FP64 instruction
-// occupies the pipe for 16 cycles whether 6 or 32 lanes are on, and the chain
-// form spends most of them on packed triangles of few lanes), FP32 by the
-// latency and bytes of the factors, so FP64 takes this form and FP32 the one
-// above (FP64 | FP32, us: 2.0 M unknowns at p = 6: 669 -> 383 | 122 -> 176;
-// p = 7, 11 slabs: 173 -> 156 | 48 -> 68; p = 4 box, 12288: 30 -> 19 | 13 -> 11).
-//
-// Factors of a group, three arrays in turn, every record padded to 16 bytes:
-//   S_s^{-1}, s < S: by circulant diagonals, entry m MG + t = S^{-1}[t][(t + m)
-//        mod MG], m = 0 .. MG / 2 (each entry of the symmetric matrix once, the
-//        last diagonal of an even MG twice): a row reads two conflict-free
-//        entries per diagonal.  Then 16 numbers per line of the coupling:
-//        y_b of interface s, x_a of interface s - 1, X's 3 x 3 block [b][a]
-//   (Q_s | W_s)^T, s < S: 12 g rows of pad4(MG) (Q_0 and W_{S-1} zero)
-//   K_s | H_s, s < S: K by rows of odd stride 6 g + 1, H by rows of 6 g (used:
-//        K_1 .. K_{S-2}, H_1 .. H_{S-1})
-__host__ __device__ constexpr int zg_ld(int G) { return 6 * G + 1; }
-__host__ __device__ constexpr int zg_circ(int MG) { return MG * (MG / 2 + 1); }
-__host__ __device__ constexpr int zg_srec(int MG, int G) { return pad4(zg_circ(MG)) + 16 * G; }
-__host__ __device__ constexpr int zg_qrec(int MG, int G) { return 12 * G * pad4(MG); }
-__host__ __device__ constexpr int zg_kpart(int G) { return pad4(6 * G * zg_ld(G)); }
-__host__ __device__ constexpr int zg_krec(int G) { return zg_kpart(G) + 36 * G * G; }
-__host__ __device__ constexpr long long zg_qoff(int MG, int G, int S) { return (long long)S * zg_srec(MG, G); }
-__host__ __device__ constexpr long long zg_koff(int MG, int G, int S) {
-  return zg_qoff(MG, G, S) + (long long)S * zg_qrec(MG, G);
-}
-__host__ __device__ constexpr long long zg_entries(int MG, int G, int S) {
-  return zg_koff(MG, G, S) + (long long)S * zg_krec(G);
-}
-
-
-// block Cholesky along the slabs of one group (one CTA; FP64 working
-// matrices G and Linv of (3 g N)^2 entries each and the (6 g)^2 C in
-// `work`), then the FP32 records and the FP64 factors
-template <int N>
-__global__ void __launch_bounds__(128)
-zgroup_factor_kernel(const DevMesh m, const int4 *__restrict__ glines, const long long *__restrict__ gfac,
-                     int gbase, int g, const double *__restrict__ blk, const double *__restrict__ xblk,
-                     double *__restrict__ work, float *__restrict__ fac, const long long *__restrict__ gfac64,
-                     double *__restrict__ fac64, int *__restrict__ status) {
-  constexpr int M = 3 * N, N2 = N * N;
-  const int grp = gbase + blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
-  const int MG = g * M, S = m.nslab, MGP = pad4(MG), KS = zg_ld(g), G6 = 6 * g;
-  double *Gm = work + (size_t)blockIdx.x * 3 * MG * MG, *Li = Gm + MG * MG, *Cm = Li + MG * MG;
-  __shared__ int lid[4], xof[4][4];
-  if (tid < 4) {
-    const int4 L4 = glines[grp];
-    lid[tid] = tid == 0 ? L4.x : (tid == 1 ? L4.y : (tid == 2 ? L4.z : L4.w));
-  }
-  __syncthreads();
-  if (tid < 16) {  // which face block couples line t1 (rows) to line t2 (columns)
-    const int t1 = tid >> 2, t2 = tid & 3;
-    int x = -1;
-    if (t1 < g && t2 < g && t1 != t2) {
-      const int c1 = lid[t1] / N2, qq = lid[t1] - c1 * N2, i1 = qq % N, j1 = qq / N;
-      for (int f = 0; f < 4; ++f) {
-        const int nbc = m.colnb[4 * c1 + f];
-        const int d = f >> 1, end = (f & 1) ? N - 1 : 0;
-        if (nbc < 0 || (d == 0 ? i1 : j1) != end) continue;
-        const int tp = d == 0 ? j1 : i1;
-        const int code = m.colnbf[4 * c1 + f], f2 = code & 3, d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0;
-        const int a2 = (code >> 2) ? N - 1 - tp : tp;
-        const int i2 = d2 == 0 ? end2 : a2, j2 = d2 == 0 ? a2 : end2;
-        if (nbc * N2 + j2 * N + i2 == lid[t2]) x = f * N + tp;
-      }
-    }
-    xof[t1][t2] = x;
-  }
-  __syncthreads();
-  float *const f32 = fac + gfac[grp];
-  double *const f64 = fac64 + gfac64[grp];
-  const int RS = zp_rec(MG, g), LP = zlp(MG), WS = zp_ws(g);
-  const int SR = zg_srec(MG, g), QR = zg_qrec(MG, g), KR = zg_krec(g), KP = zg_kpart(g), LC = pad4(zg_circ(MG));
-  const long long qo = zg_qoff(MG, g, S), ko = zg_koff(MG, g, S);
-  // O_s of line l (rows: slab s)
-  auto Oblk = [&](int l, int s) { return blk + (((size_t)lid[l] * S + s) * 2 + 1) * M * M; };
-  // column j of V_s applied: sum_p V_s[p][j] f(p), f indexed by rows of the group
-  auto dotV = [&](int s, int j, auto f) {
-    const int l = j / 6, jj = j - l * 6;
-    if (jj < 3) return f(l * M + jj * N + N - 1);
-    const double *O = Oblk(l, s - 1) + ((jj - 3) * N) * M;
-    double acc = 0.0;
-    for (int k = 0; k < N - 1; ++k) acc += O[(jj - 3) * N + k] * f(l * M + (jj - 3) * N + k);
-    for (int b = 0; b < 3; ++b) acc += O[b * N + N - 1] * f(l * M + b * N + N - 1);
-    return acc;
-  };
-  // column j of U_s applied
-  auto dotU = [&](int s, int j, auto f) {
-    const int l = j / 6, jj = j - l * 6;
-    if (jj >= 3) return f(l * M + (jj - 3) * N);
-    const double *O = Oblk(l, s);
-    double acc = 0.0;
-    for (int k = 1; k < N; ++k) acc += O[(jj * N + k) * M + jj * N + N - 1] * f(l * M + jj * N + k);
-    return acc;
-  };
-  for (int s = 0; s < S; ++s) {
-    // Schur complement of slab s: the diagonal block (line blocks, cross-line
-    // face blocks) minus V_s C V_s^T, C = U_{s-1}^T W_{s-1} (6g x 6g); a row of
-    // V has at most four nonzeros
-    if (s > 0) {
-      const double *Wp = f64 + qo + (long long)(s - 1) * QR + G6 * MGP;
-      for (int q = tid; q < G6 * G6; q += nth) {
-        const int i = q / G6, j = q - i * G6;
-        Cm[q] = dotU(s - 1, i, [&](int p) { return Wp[(size_t)j * MGP + p]; });
-      }
-      __syncthreads();
-    }
-    for (int q = tid; q < MG * MG; q += nth) {
-      const int r = q / MG, cc = q - r * MG, t1 = r / M, t2 = cc / M, rr = r - t1 * M, c2 = cc - t2 * M;
-      double v = 0.0;
-      if (t1 == t2) {
-        v = blk[(((size_t)lid[t1] * S + s) * 2 + 0) * M * M + rr * M + c2];
-      } else if (xof[t1][t2] >= 0) {
-        const size_t e = (size_t)s * m.ncol + lid[t1] / N2;
-        v = xblk[(e * 4 * N + xof[t1][t2]) * M * M + rr * M + c2];
-      }
-      if (s > 0) {  // the nonzeros of V's rows r and cc: (column, value)
-        int ir[4], ic[4];
-        double vr[4], vc[4];
-        int nr = 0, nc = 0;
-        const double *Or = Oblk(t1, s - 1), *Oc = Oblk(t2, s - 1);
-        if (rr % N == N - 1) { ir[nr] = 6 * t1 + rr / N; vr[nr++] = 1.0; }
-        if (c2 % N == N - 1) { ic[nc] = 6 * t2 + c2 / N; vc[nc++] = 1.0; }
-        for (int a = 0; a < 3; ++a) {
-          if (a == rr / N || rr % N == N - 1) { ir[nr] = 6 * t1 + 3 + a; vr[nr++] = Or[(a * N) * M + rr]; }
-          if (a == c2 / N || c2 % N == N - 1) { ic[nc] = 6 * t2 + 3 + a; vc[nc++] = Oc[(a * N) * M + c2]; }
-        }
-        double sum = 0.0;
-        for (int x = 0; x < nr; ++x) {
-          double row = 0.0;
-          for (int y = 0; y < nc; ++y) row += Cm[ir[x] * G6 + ic[y]] * vc[y];
-          sum += vr[x] * row;
-        }
-        v -= sum;
-      }
-      Gm[q] = v;
-    }
-    __syncthreads();
-    // Cholesky, lower triangle in place
-    for (int col = 0; col < MG; ++col) {
-      if (tid == 0) {
-        double dv = Gm[col * MG + col];
-        if (!(dv > 0.0)) {
-          atomicExch(status, 1);
-          dv = 1e-300;
-        }
-        Gm[col * MG + col] = sqrt(dv);
-      }
-      __syncthreads();
-      const double piv = Gm[col * MG + col];
-      for (int r = col + 1 + tid; r < MG; r += nth) Gm[r * MG + col] /= piv;
-      __syncthreads();
-      const int w = MG - col - 1;
-      for (int q = tid; q < w * w; q += nth) {
-        const int r = col + 1 + q / w, c2 = col + 1 + q % w;
-        if (c2 <= r) Gm[r * MG + c2] -= Gm[r * MG + col] * Gm[c2 * MG + col];
-      }
-      __syncthreads();
-    }
-    // Linv = L^{-1}, one column per thread (forward substitution on the
-    // identity); its upper triangle is zero (read by the products below)
-    for (int cc = tid; cc < MG; cc += nth) {
-      for (int r = 0; r < cc; ++r) Li[r * MG + cc] = 0.0;
-      for (int r = cc; r < MG; ++r) {
-        double acc = r == cc ? 1.0 : 0.0;
-        for (int p = cc; p < r; ++p) acc -= Gm[r * MG + p] * Li[p * MG + cc];
-        Li[r * MG + cc] = acc / Gm[r * MG + r];
-      }
-    }
-    __syncthreads();
-    for (int q = tid; q < MG * MG; q += nth) {  // S^{-1} = Linv^T Linv, in place of L
-      const int r = q / MG, cc = q - r * MG;
-      if (r < cc) continue;
-      double acc = 0.0;
-      for (int p = r; p < MG; ++p) acc += Li[p * MG + r] * Li[p * MG + cc];
-      Gm[r * MG + cc] = acc;
-      Gm[cc * MG + r] = acc;
-    }
-    __syncthreads();
-    float *const R = f32 + (long long)s * RS;
-    for (int q = tid; q < MG * MG; q += nth) {  // S^{-1}, packed lower triangle
-      const int r = q / MG, cc = q - r * MG;
-      if (r >= cc) R[zcol(MG, cc) + r - cc] = (float)Gm[q];
-    }
-    for (int q = MG * (MG + 1) / 2 + tid; q < LP; q += nth) R[q] = 0.0f;
-    for (int q = tid; q < 8 * MG; q += nth) {  // factors of O_{s-1}
-      const int t = q >> 3, j = q & 7, l = t / M, tl = t - l * M, tk = tl % N;
-      double v = 0.0;
-      if (s > 0 && (j & 3) < 3) {
-        const double *O = Oblk(l, s - 1);
-        if (j < 4) v = O[(j * N) * M + tl];                        // X[t][a] = O[(a, 0), t]
-        else if (tk != 0) v = O[tl * M + (j - 4) * N + (N - 1)];  // Y[t][b] = O[t, (b, N - 1)]
-      }
-      R[LP + q] = (float)v;
-    }
-    double *Sd = f64 + (long long)s * SR;
-    for (int q = tid; q < SR; q += nth) {
-      double v = 0.0;
-      if (q < zg_circ(MG)) {
-        const int mm = q / MG, t = q - mm * MG, c = t + mm < MG ? t + mm : t + mm - MG;
-        v = Gm[t * MG + c];
-      } else if (q >= LC) {
-        const int l = (q - LC) / 16, i = (q - LC) - l * 16;
-        if (i < 3) {
-          if (s + 1 < S) v = Oblk(l, s)[(i * N + 1) * M + i * N + N - 1] / c_lgl_zg.D[N][1];  // Y[(b, 1)][b] / D(0, 1)
-        } else if (s > 0 && i < 6) {
-          const int a = i - 3;  // X[(a, 0)][a] / D(N-1, 0)
-          v = Oblk(l, s - 1)[(a * N) * M + a * N] / c_lgl_zg.D[N][(N - 1) * N];
-        } else if (s > 0 && i < 15) {
-          const int b = (i - 6) / 3, a = (i - 6) % 3;
-          v = Oblk(l, s - 1)[(a * N) * M + b * N + N - 1];
-        }
-      }
-      Sd[q] = v;
-    }
-    // (Q_s | W_s)^T = (V_s | U_s)^T S_s^{-1}
-    double *Qd = f64 + qo + (long long)s * QR;
-    for (int q = tid; q < QR; q += nth) {
-      const int j = q / MGP, t = q - j * MGP;
-      double v = 0.0;
-      if (t < MG) {
-        auto row = [&](int p) { return Gm[p * MG + t]; };
-        if (j < G6) {
-          if (s > 0) v = dotV(s, j, row);
-        } else if (s + 1 < S) {
-          v = dotU(s, j - G6, row);
-        }
-      }
-      Qd[q] = v;
-    }
-    __syncthreads();
-    for (int q = tid; q < MG * WS; q += nth) {  // W_s by rows
-      const int t = q / WS, j = q - t * WS;
-      R[LP + 8 * MG + q] = j < G6 ? (float)Qd[(G6 + j) * MGP + t] : 0.0f;
-    }
-    // K_s = W_s^T V_s, H_s = V_s^T Q_s
-    double *Kd = f64 + ko + (long long)s * KR;
-    for (int q = tid; q < KR; q += nth) {
-      double v = 0.0;
-      if (s > 0) {
-        if (q < KP) {
-          const int i = q / KS, j = q - i * KS;
-          if (i < G6 && j < G6) v = dotV(s, j, [&](int p) { return Qd[(G6 + i) * MGP + p]; });
-        } else {
-          const int i = (q - KP) / G6, j = (q - KP) - i * G6;
-          v = dotV(s, i, [&](int p) { return Qd[j * MGP + p]; });
-        }
-      }
-      Kd[q] = v;
-    }
-    __syncthreads();
-  }
-}
 
 // ---- the FP32 solve: packed slots, one launch per degree
 // A group of G lines (3 G N rows per slab) is solved by a slot of G warps,
@@ -1284,43 +909,6 @@ zg_final_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, con
   }
 }
 
-template <int N>
-cudaError_t zgroup_setup_n(const DevMesh &m, const ZGroupPlan &p, const ZGroupDev &gd, int inst,
-                           double *blk, double *xblk, double *work, float *fac, double *fac64, int *status,
-                           cudaStream_t st) {
-  cudaError_t err = tn_zline_blocks(m, blk, st);
-  if (err != cudaSuccess) return err;
-  zgroup_cross_kernel<N><<<m.E, ((4 * N + 31) / 32) * 32, 0, st>>>(m, xblk);
-  err = cudaGetLastError();
-  // the four group sizes at once, each with its own scratch: the 4-line
-  // groups (few, long) on st, the others on side streams forked from it
-  if (err == cudaSuccess) err = cudaEventRecord(gd.fork, st);
-  size_t off = 0;
-  bool used[3] = {false, false, false};
-  for (int g = 1; g <= 4 && err == cudaSuccess; ++g) {
-    const int cnt = p.inst_n[(size_t)inst * 5 + g];
-    if (!cnt) continue;
-    cudaStream_t sg = st;
-    if (g < 4) {
-      sg = gd.side[g - 1];
-      err = cudaStreamWaitEvent(sg, gd.fork, 0);
-      used[g - 1] = true;
-      if (err != cudaSuccess) break;
-    }
-    zgroup_factor_kernel<N><<<cnt, 128, 0, sg>>>(m, gd.lines, gd.fac_off, p.inst_start[(size_t)inst * 5 + g], g,
-                                                 blk, xblk, work + off, fac, gd.fac64_off, fac64, status);
-    err = cudaGetLastError();
-    const size_t MG = (size_t)g * 3 * N;
-    off += (size_t)cnt * 3 * MG * MG;
-  }
-  for (int k = 0; k < 3 && err == cudaSuccess; ++k) {
-    if (!used[k]) continue;
-    err = cudaEventRecord(gd.join[k], gd.side[k]);
-    if (err == cudaSuccess) err = cudaStreamWaitEvent(st, gd.join[k], 0);
-  }
-  return err;
-}
-
 template <typename... P, typename... A>
 cudaError_t launch_zg(void (*kernel)(P...), int grid, size_t smem, bool dependent, cudaStream_t st, A... args) {
   if (smem > 48 * 1024) {
@@ -1556,32 +1144,6 @@ bool tn_zgroup_plan(const tn::HostMesh *const *hms, int n, ZGroupPlan *p, char *
     ++p->npk;
   }
   return true;
-}
-
-size_t tn_zgroup_cross_bytes(const DevMesh &m) {
-  const size_t M = 3 * m.N;
-  return (size_t)m.E * 4 * m.N * M * M * sizeof(double);
-}
-
-size_t tn_zgroup_work_bytes(const DevMesh &m, const ZGroupPlan &p, int inst) {
-  size_t sum = 0;
-  for (int g = 1; g <= 4; ++g) {
-    const size_t MG = (size_t)g * 3 * m.N;
-    sum += (size_t)p.inst_n[(size_t)inst * 5 + g] * 3 * MG * MG * sizeof(double);
-  }
-  return sum;
-}
-
-cudaError_t tn_zgroup_setup(const DevMesh &m, const ZGroupPlan &p, const ZGroupDev &gd, int inst,
-                            double *blk, double *xblk, double *work, float *fac, double *fac64, int *status,
-                            cudaStream_t st) {
-  switch (m.N) {
-#define TN_CASE(NN) \
-    case NN: return zgroup_setup_n<NN>(m, p, gd, inst, blk, xblk, work, fac, fac64, status, st);
-    TN_CASE(3) TN_CASE(4) TN_CASE(5) TN_CASE(6) TN_CASE(7) TN_CASE(8) TN_CASE(9)
-#undef TN_CASE
-    default: return cudaErrorInvalidValue;
-  }
 }
 
 // per degree present (one for a single mesh) one launch (FP32) or three
