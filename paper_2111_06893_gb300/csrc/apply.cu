@@ -989,21 +989,6 @@ cudaError_t allow_smem(K kernel, size_t bytes, int &configured_device) {
   return err;
 }
 
-template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-
 template <int N, typename T, int V, int MODE>
 cudaError_t launch_elem(const ApplyArgs &a, cudaStream_t st) {
   constexpr size_t sm = apply_smem<N, T, MODE>();

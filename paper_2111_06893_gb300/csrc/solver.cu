@@ -24,6 +24,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "tn_device.h"
 #include "tn_internal.h"
 #include "tn_precond.h"
 #include "tn_solver.h"
@@ -330,6 +331,10 @@ __global__ void k_beta_split(tn_pcg_scalars *s, const double *rzp, int nrz, cons
 template <typename T>
 __global__ void k_pupdate_x(const tn_pcg_scalars *s, size_t n, T *__restrict__ x, T *__restrict__ p,
                             const T *__restrict__ z) {
+  grid_trigger();
+  grid_wait();
+  s = after_wait(s);
+  z = after_wait(z);
   if (!s->active) return;
   const T alpha = (T)s->alpha, beta = (T)s->beta;
   const bool more = !s->done;
@@ -436,8 +441,8 @@ static cudaError_t pcg_iteration_zline(const OpSys &sys, int prec, size_t n, Pcg
     fb.s = s;
     fb.cnt = sys.fold_cnt + 1;
     TN_CU(sys.zsolve(prec, v.zfac, v.r, nullptr, v.z, nullptr, v.part_rz, &s->done, st, &fb));
-    k_pupdate_x<T><<<red_blocks(), kRedThreads, 0, st>>>(s, n, (T *)v.x, (T *)v.p, (const T *)v.z);
-    return cudaGetLastError();
+    return launch_pdl(k_pupdate_x<T>, red_blocks(), kRedThreads, 0, st, (const tn_pcg_scalars *)s, n, (T *)v.x,
+                      (T *)v.p, (const T *)v.z);
   }
   TN_CU(sys.apply(prec, v.p, v.q, part_elem, st));
   k_alpha<<<1, 1024, 0, st>>>(s, part_elem, sys.apply_parts());

@@ -111,6 +111,22 @@ __device__ __forceinline__ P *after_wait(P *p) {
   return p;
 }
 
+// launch that may start before the kernel ahead of it in st has ended
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // 16-byte broadcast read of entries c4 .. c4 + 16/sizeof(T) - 1 of a vector
 // that every lane of the warp reads at once
 template <typename T> struct Vec16;

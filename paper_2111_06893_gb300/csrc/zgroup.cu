@@ -380,6 +380,10 @@ zgroup_packed_kernel(const DevMesh m1, const int *__restrict__ ginst, const DevM
                      int *__restrict__ queue, const float *__restrict__ fac, const float *__restrict__ r,
                      float *__restrict__ z, double *__restrict__ part_rz, double *__restrict__ part_rr, const int *__restrict__ done,
                      TnWait *__restrict__ err, const PcgFold fold) {
+  grid_wait();
+  done = after_wait(done);
+  r = after_wait(r);
+  queue = after_wait(queue);
   if (done && *done) return;
   constexpr int SW = zp_stage_per_warp<N>();
   extern __shared__ __align__(16) unsigned char zsm[];
@@ -448,6 +452,7 @@ zgroup_packed_kernel(const DevMesh m1, const int *__restrict__ ginst, const DevM
     }
     __syncthreads();  // every slot of the pack is done with shared memory
   }
+  grid_trigger();
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(queue + 1, 1) == (int)gridDim.x - 1) {
@@ -947,21 +952,20 @@ cudaError_t launch_f64(const DevMesh &m, const ZGroupDev &gd, int k, const doubl
 // packs.  grid_out: only compute the grid; else launch with it.
 template <int N>
 cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float *fac, const float *r, float *z,
-                       double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, const PcgFold &fold,
-                       int *grid_out) {
+                       double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, bool first,
+                       const PcgFold &fold, int *grid_out) {
   constexpr size_t sm = zp_smem<N>();
   auto kern = zgroup_packed_kernel<N>;
-  cudaError_t err = sm > 48 * 1024 ? cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                                   : cudaSuccess;
-  if (err != cudaSuccess) return err;
   static int per_sm[64] = {0};
   int dev = 0;
-  err = cudaGetDevice(&dev);
+  cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   if (!per_sm[dev]) {
     // shared memory before L1: the CTAs per SM are limited by the staging rings
     err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (err == cudaSuccess && sm > 48 * 1024)
+      err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (err != cudaSuccess) return err;
     int b = 0;
     err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, kZgThreads, sm);
@@ -974,10 +978,8 @@ cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float
     *grid_out = grid;
     return cudaSuccess;
   }
-  kern<<<grid, kZgThreads, sm, st>>>(m, gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac_off, gd.packs,
-                                     gd.pk_start[k], gd.pk_n[k], gd.queue + 2 * k, fac, r, z, prz, prr, done, zerr,
-                                     fold);
-  return cudaGetLastError();
+  return launch_zg(kern, grid, sm, first, st, m, gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac_off, gd.packs,
+                   gd.pk_start[k], gd.pk_n[k], gd.queue + 2 * k, fac, r, z, prz, prr, done, zerr, fold);
 }
 
 cudaError_t zgroup_launch(const DevMesh &m, const ZGroupDev &gd, int k, int prec, const void *fac, const void *r,
@@ -993,7 +995,7 @@ cudaError_t zgroup_launch(const DevMesh &m, const ZGroupDev &gd, int k, int prec
     return prec == TN_F64 ? launch_f64<NN>(m, gd, k, (const double *)fac, (const double *)r, (double *)z, prz,   \
                                            prr, done, zerr, st, first, fold)                                     \
                           : launch_f32<NN>(m, gd, k, (const float *)fac, (const float *)r, (float *)z, prz, prr, \
-                                           done, zerr, st, fold, grid_out);
+                                           done, zerr, st, first, fold, grid_out);
     TN_CASE(3) TN_CASE(4) TN_CASE(5) TN_CASE(6) TN_CASE(7) TN_CASE(8) TN_CASE(9)
 #undef TN_CASE
     default: return cudaErrorInvalidValue;
