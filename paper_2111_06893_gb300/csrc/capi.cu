@@ -168,6 +168,7 @@ struct tn_ctx {
   ZGroupDev zgd;
   unsigned char *d_gplan = nullptr;  // the plan's tables, one block
   double *gchain = nullptr;          // chain numbers of the solve
+  int *gqueue = nullptr;             // work queues of the FP32 solve (not among the tables: they are written all along)
   float *gfac = nullptr;
   double *gfac64 = nullptr;
   double *gpart = nullptr;
@@ -196,6 +197,7 @@ static void free_zline(tn_ctx *c) {
 static void free_zgroup(tn_ctx *c) {
   dfree(c->d_gplan);
   dfree(c->gchain);
+  dfree(c->gqueue);
   dfree(c->gfac);
   dfree(c->gfac64);
   dfree(c->gpart);
@@ -410,6 +412,7 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gpart, sizeof(double) * 2 * std::max(p.ranges.size(), p.lines.size()));  // r.z, r.r
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gstatus, 2 * sizeof(int));  // factor status, solve timeout
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gchain, sizeof(double) * (size_t)p.nchain);
+  if (e == cudaSuccess) e = cudaMalloc((void **)&c->gqueue, sizeof(int) * kZgQueue * kZgMaxDg);
   TablePack pack;
   const size_t o_lines = pack.add(p.lines.data(), sizeof(int4) * p.lines.size());
   const size_t o_fac = pack.add(p.fac_off.data(), sizeof(long long) * p.fac_off.size());
@@ -417,8 +420,6 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   const size_t o_chain = pack.add(p.chain_off.data(), sizeof(long long) * p.chain_off.size());
   const size_t o_packs = pack.add(p.packs.data(), sizeof(int4) * p.packs.size());
   const size_t o_ranges = pack.add(p.ranges.data(), sizeof(int4) * p.ranges.size());
-  const std::vector<int> zeros(2 * kZgMaxDg, 0);
-  const size_t o_queue = pack.add(zeros.data(), sizeof(int) * zeros.size());
   const size_t o_inst = pack.add(p.inst.data(), sizeof(int) * p.inst.size());
   if (e == cudaSuccess) e = pack.upload(&c->d_gplan);
   if (e != cudaSuccess) {
@@ -438,7 +439,7 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   g.lines = (const int4 *)(dp + o_lines);
   g.fac_off = (const long long *)(dp + o_fac);
   g.fac64_off = (const long long *)(dp + o_fac64);
-  g.queue = (int *)(c->d_gplan + o_queue);
+  g.queue = c->gqueue;
   g.chain_off = (const long long *)(dp + o_chain);
   g.packs = (const int4 *)(dp + o_packs);
   g.ranges = (const int4 *)(dp + o_ranges);
@@ -455,6 +456,7 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   }
   int status = 0;
   if (e == cudaSuccess) e = cudaMemsetAsync(c->gstatus, 0, 2 * sizeof(int), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->gqueue, 0, sizeof(int) * kZgQueue * kZgMaxDg, st);
   for (int i = 0; i < n && e == cudaSuccess; ++i)  // one mirror after another (shared set-up scratch)
     e = tn_zgroup_setup(dms[i], p, c->zgd, i, blk, xblk, c->gfac, c->gfac64,
                         c->gstatus, st);

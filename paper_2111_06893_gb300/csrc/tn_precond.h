@@ -35,6 +35,7 @@ cudaError_t tn_zline_solve_batch(int N, int prec, const DevMesh *meshes, const i
 // ---- line groups: lines joined by matching nodes of lateral faces
 constexpr int kZgMaxCls = 28;  // classes: (group size 1..4) x (N = 3..9)
 constexpr int kZgMaxDg = 7;    // degrees (N = 3..9), one launch (FP32) or three (FP64) each
+constexpr int kZgQueue = 64;   // ints from one work queue to the next (lines of their own)
 constexpr int kZgSide = 6;     // side streams the launches of a batch run on
 // the groups of one mesh or of every mirror of a batch, ordered by class
 // (group size, largest first; then N; then mirror)

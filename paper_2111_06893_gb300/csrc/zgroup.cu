@@ -978,8 +978,14 @@ cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float
     *grid_out = grid;
     return cudaSuccess;
   }
-  return launch_zg(kern, grid, sm, first, st, m, gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac_off, gd.packs,
-                   gd.pk_start[k], gd.pk_n[k], gd.queue + 2 * k, fac, r, z, prz, prr, done, zerr, fold);
+  if (first)
+    return launch_pdl(kern, grid, kZgThreads, sm, st, m, gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac_off,
+                      gd.packs, gd.pk_start[k], gd.pk_n[k], gd.queue + kZgQueue * k, fac, r, z, prz, prr, done, zerr,
+                      fold);
+  kern<<<grid, kZgThreads, sm, st>>>(m, gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac_off, gd.packs,
+                                     gd.pk_start[k], gd.pk_n[k], gd.queue + kZgQueue * k, fac, r, z, prz, prr, done,
+                                     zerr, fold);
+  return cudaGetLastError();
 }
 
 cudaError_t zgroup_launch(const DevMesh &m, const ZGroupDev &gd, int k, int prec, const void *fac, const void *r,
