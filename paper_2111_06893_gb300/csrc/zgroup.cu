@@ -372,8 +372,8 @@ __device__ void fold_beta(const PcgFold &f) {
 // (largest first); the last CTA to finish resets queue[0..1] for the next
 // launch.  One mesh (ginst == nullptr) or a batch (per group: its mirror's
 // mesh and first unknown).
-template <int N>
-__global__ void __launch_bounds__(kZgThreads, 4)
+template <int N, int B>
+__global__ void __launch_bounds__(kZgThreads, B)
 zgroup_packed_kernel(const DevMesh m1, const int *__restrict__ ginst, const DevMesh *__restrict__ meshes,
                      const long long *__restrict__ dof_off, const int4 *__restrict__ glines,
                      const long long *__restrict__ gfac, const int4 *__restrict__ packs, int pk0, int npk,
@@ -948,14 +948,10 @@ cudaError_t launch_f64(const DevMesh &m, const ZGroupDev &gd, int k, const doubl
                    prr, done, fold);
 }
 
-// the FP32 kernel is persistent: as many CTAs as fit at once, never more than
-// packs.  grid_out: only compute the grid; else launch with it.
-template <int N>
-cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float *fac, const float *r, float *z,
-                       double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, bool first,
-                       const PcgFold &fold, int *grid_out) {
-  constexpr size_t sm = zp_smem<N>();
-  auto kern = zgroup_packed_kernel<N>;
+// CTAs of the FP32 kernel for B CTAs per SM (registers) that an SM holds
+template <int N, int B>
+cudaError_t packed_per_sm(size_t sm, int *out) {
+  auto kern = zgroup_packed_kernel<N, B>;
   static int per_sm[64] = {0};
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
@@ -972,12 +968,15 @@ cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float
     if (err != cudaSuccess) return err;
     per_sm[dev] = b > 0 ? b : 1;
   }
-  int grid = per_sm[dev] * tn_sm_count();
-  grid = grid < gd.pk_n[k] ? grid : gd.pk_n[k];
-  if (grid_out) {
-    *grid_out = grid;
-    return cudaSuccess;
-  }
+  *out = per_sm[dev];
+  return cudaSuccess;
+}
+
+template <int N, int B>
+cudaError_t launch_packed(const DevMesh &m, const ZGroupDev &gd, int k, int grid, size_t sm, const float *fac,
+                          const float *r, float *z, double *prz, double *prr, const int *done, TnWait *zerr,
+                          cudaStream_t st, bool first, const PcgFold &fold) {
+  auto kern = zgroup_packed_kernel<N, B>;
   if (first)
     return launch_pdl(kern, grid, kZgThreads, sm, st, m, gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac_off,
                       gd.packs, gd.pk_start[k], gd.pk_n[k], gd.queue + kZgQueue * k, fac, r, z, prz, prr, done, zerr,
@@ -986,6 +985,35 @@ cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float
                                      gd.pk_start[k], gd.pk_n[k], gd.queue + kZgQueue * k, fac, r, z, prz, prr, done,
                                      zerr, fold);
   return cudaGetLastError();
+}
+
+// The FP32 kernel is persistent: as many CTAs as fit at once, never more than
+// packs.  Four CTAs per SM run a pack fastest; seven (72 registers) take more
+// packs at once, which pays from three rounds of packs where it saves a third
+// of them (crystalline stack, p = 5, 4 -> 2 rounds: 442 -> 368 us; p = 5 at 324
+// columns, 5 -> 3: 174 -> 153).  Below that it is not worth it (p = 6, 993
+// packs, 2 -> 2 rounds: 116 -> 132; p = 5 at 81 columns, 2 -> 1: 62 -> 67), nor
+// with kernels of several degrees side by side (24 mirrors: 268 -> 276).
+// grid_out: only compute the grid; else launch with it.
+template <int N>
+cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float *fac, const float *r, float *z,
+                       double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, bool first,
+                       const PcgFold &fold, int *grid_out) {
+  constexpr size_t sm = zp_smem<N>();
+  int four = 0, seven = 0;
+  cudaError_t err = packed_per_sm<N, 4>(sm, &four);
+  if (err == cudaSuccess) err = packed_per_sm<N, 7>(sm, &seven);
+  if (err != cudaSuccess) return err;
+  const int npk = gd.pk_n[k], sms = tn_sm_count();
+  auto rounds = [&](int per_sm) { return (npk + per_sm * sms - 1) / (per_sm * sms); };
+  const bool more = gd.npk == 1 && rounds(four) >= 3 && 3 * rounds(seven) <= 2 * rounds(four);
+  const int grid = std::min((more ? seven : four) * sms, npk);
+  if (grid_out) {
+    *grid_out = grid;
+    return cudaSuccess;
+  }
+  if (more) return launch_packed<N, 7>(m, gd, k, grid, sm, fac, r, z, prz, prr, done, zerr, st, first, fold);
+  return launch_packed<N, 4>(m, gd, k, grid, sm, fac, r, z, prz, prr, done, zerr, st, first, fold);
 }
 
 cudaError_t zgroup_launch(const DevMesh &m, const ZGroupDev &gd, int k, int prec, const void *fac, const void *r,
