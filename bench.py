@@ -60,14 +60,13 @@ def fp32_apply_flops_per_dof(N):
 # from `ncu --set full -k regex:zgroup_packed_kernel` of `bench.py --mode
 # apply --workload single_coating`; absent where no capture of the current
 # kernel exists
-ZLINE_TRAFFIC = {("single_coating", "zgroup_packed_kernel<7,float>"): 342619136.0 + 10593280.0}
+ZLINE_TRAFFIC = {("single_coating", "zgroup_packed_kernel<7>"): 342619136.0 + 10593280.0}
 
 
-# DRAM bytes (read + write) of one FP32 apply per occupancy variant, from
-# `ncu --set full -k regex:apply2_kernel` of `bench.py --mode apply --workload
-# single_coating` (variant 0 captured; variant 1's register spills add
-# local-memory traffic, not captured for the current kernel)
-APPLY_TRAFFIC = {("single_coating", "apply2_kernel<7,float,0>"): 8148736.0}
+# DRAM bytes (read + write) of one FP32 apply (both launches), from ncu on the
+# single-coating mesh (variant 1 captured; the variants move the same bytes)
+APPLY_TRAFFIC = {("single_coating", f"apply_elem_kernel<7,float,{v}> + trace_add_kernel<7,float>"): 22863872.0
+                 for v in (0, 1)}
 
 
 def measured_peaks():
@@ -535,8 +534,8 @@ def main():
 
     t32 = time_apply(x32, y32, 200)
     tuning = ctx.apply_tuning()  # FP32 operator variant per degree, timed by the first FP32 call
-    akernel = ("apply2_batch_kernel<N,float,V>" if batched
-               else f"apply2_kernel<{N},float,{tuning.get(N - 1, {}).get('variant', 0)}>")
+    akernel = ("apply_batch_kernel<float,V> + trace_add_batch_kernel<float>" if batched
+               else f"apply_elem_kernel<{N},float,{tuning.get(N - 1, {}).get('variant', 0)}> + trace_add_kernel<{N},float>")
     t64 = time_apply(x64, y64, 20)
 
     # the dominant kernel of the step: the FP32 preconditioner solve (column lines)
@@ -658,7 +657,7 @@ def main():
     hbm_peak = peaks.get("hbm_gbs") or 6800.0
     peak_src = "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks.get("hbm_gbs") else "fallback 6.8 TB/s"
     if pc == "zgroup":
-        zkernel = (f"zgroup_packed_kernel<{'N' if batched else N},float>"
+        zkernel = (f"zgroup_packed_kernel<{'N' if batched else N}>"
                    + (", one launch per degree" if batched else ""))
     else:
         zkernel = ("zline_solve_batch_kernel<N,float,float,0>" if batched
@@ -697,7 +696,8 @@ def main():
                            "peak_source": "measured: tn_fma_peak FP32 (FMA chains, CUDA events)"},
         "roofline_apply_f64": {"bound": "alu", "achieved": flops / t64 / 1e12, "peak": peak_fp64,
                                "unit": "TFLOP/s", "frac": flops / t64 / 1e12 / peak_fp64,
-                               "kernel": f"apply2_kernel<{N},double,0>" if not batched else "apply2_batch_kernel<N,double,0>",
+                               "kernel": (f"apply_elem_kernel<{N},double,0> + trace_add_kernel<{N},double>" if not batched
+                                          else "apply_batch_kernel<double,0> + trace_add_batch_kernel<double>"),
                                "peak_source": "measured: tn_fma_peak FP64 (FMA chains, CUDA events)"},
         "gradient": grad,
         "e2e": {"value": e2e_value, "unit": "GDOF/s", "h2d_bytes_per_step": h2d,
