@@ -540,7 +540,7 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
   double best = INFINITY;
   int stall = 0;
   for (;;) {
-    g_launches += (zl && sys.grouped ? 4LL : 6LL) * chunk;
+    g_launches += (zl && sys.grouped && prec == TN_F32 ? 4LL : 6LL) * chunk;
     err = cudaGraphLaunch(exec, st);
     if (err != cudaSuccess) break;
     err = cudaMemcpyAsync(s_host, s_dev, sizeof(tn_pcg_scalars), cudaMemcpyDeviceToHost, st);

@@ -72,3 +72,19 @@ def test_chain_solve_of_a_batch_is_the_single_solves():
         lo, hi = batch.dof_off[i], batch.dof_off[i + 1]
         zi = thermonoise.setup(d).precond_apply(r[lo:hi].clone(), precond="zgroup")
         assert torch.equal(z[lo:hi], zi), i
+
+
+@pytest.mark.parametrize("nx", [30, 40])
+def test_fp32_solve_of_many_packs(nx):
+    """More packs of line groups than the GPU holds at once, several times over
+    (nx = 40: the build with seven CTAs per SM; 30: four), against the FP64
+    solve; 2e-5 as above.  Repeated, the work queue starts empty again."""
+    from paper_2111_06893_gb300 import thermonoise
+    br = [0.25 * i for i in range(nx + 1)]
+    desc = W.box(br, br, [0.0, -0.3, -0.7], 2, W.FUSED_SILICA)
+    ctx = thermonoise.setup(desc)
+    r = torch.tensor(np.random.default_rng(nx).uniform(-1, 1, ctx.ndof), dtype=torch.float64, device="cuda")
+    z = ctx.precond_apply(r, precond="zgroup")
+    first = ctx.precond_apply(r.float(), precond="zgroup")
+    assert float((first.double() - z).norm() / z.norm()) < 2e-5
+    assert torch.equal(first, ctx.precond_apply(r.float(), precond="zgroup"))
