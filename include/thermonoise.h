@@ -135,7 +135,15 @@ tn_status tn_set_beam(tn_ctx *ctx, double r0, double F0);
  * form, homogeneous boundary data).  precision TN_F64: u, y are double;
  * TN_F32: float (geometry is kept in FP64 and rounded per node).  u and y
  * are caller-owned device buffers of tn_ndof() elements, must not overlap,
- * and must be 16-byte aligned. */
+ * and must be 16-byte aligned.
+ * Two launches, with 18 N^2 numbers of scratch per element between them (N =
+ * p + 1; a quotient 6 / N of a field), kept by the context until its mesh
+ * goes.  The first apply allocates it in its own precision; a first FP64 apply
+ * after FP32 ones, and every tn_solve, has it in FP64 (TN_ENOMEM if that fails).
+ * Under stream capture the apply records kernel nodes only, and a capture has
+ * scratch of its own, so that its replays may overlap other work of the
+ * context: it is given back once the graph and every instance of it are
+ * destroyed, and freed, like the mesh's tables, when the mesh is replaced. */
 tn_status tn_apply_operator(tn_ctx *ctx, int precision, const void *u_dev, void *y_dev);
 
 /* Autotuning of the FP32 operator kernel (the element-wise apply of

@@ -119,6 +119,128 @@ struct MeshTables {
   }
 };
 
+// cudaMalloc and cudaFree that may run while this thread, or another, captures
+// a stream (they touch no captured stream)
+static cudaError_t malloc_any(void **p, size_t bytes) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) return e;
+  e = cudaMalloc(p, bytes);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
+}
+static void free_any(void *p) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  const cudaError_t e = cudaThreadExchangeStreamCaptureMode(&mode);
+  if (p) cudaFree(p);
+  if (e == cudaSuccess) cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+// Traction scratch of captured applies.  A capture gets a block of its own, so
+// that replays may overlap each other and other work of the context, and the
+// graph stays one of kernel nodes only (memory nodes would bar clones, child
+// graphs, a second instance and conditional bodies).  The applies of one
+// capture follow one another on the context's stream and share its block.
+// The graph and what is instantiated from it hold a user object that gives
+// the block back for the next capture: as many blocks as graphs in use at
+// once.  All are freed with the mesh, on whose tables the graphs rely too.
+struct TraceBlocks {
+  struct Block {
+    void *p = nullptr;
+    size_t bytes = 0;
+    bool used = false;
+    bool kept = false;  // no graph could hold its user object: in use until the mesh goes
+    TraceBlocks *owner = nullptr;
+    Block *next = nullptr;
+  };
+  std::mutex lock;  // blocks come back on a thread of the CUDA runtime
+  Block *blocks = nullptr;
+  int refs = 1;     // the context, and every user object
+  unsigned long long capture = 0;  // id of the last capture served, and its block
+  Block *last = nullptr;
+
+  ~TraceBlocks() {
+    while (Block *b = blocks) {
+      blocks = b->next;
+      delete b;
+    }
+  }
+  static void drop(TraceBlocks *t) {
+    bool dead;
+    {
+      std::lock_guard<std::mutex> g(t->lock);
+      dead = --t->refs == 0;
+    }
+    if (dead) delete t;
+  }
+  static void CUDART_CB give_back(void *arg) {
+    Block *b = (Block *)arg;
+    TraceBlocks *t = b->owner;
+    {
+      std::lock_guard<std::mutex> g(t->lock);
+      if (!b->kept) b->used = false;
+    }
+    drop(t);
+  }
+  // a block of `bytes` for the capture `id` into `graph`
+  cudaError_t take(unsigned long long id, cudaGraph_t graph, size_t bytes, void **out) {
+    cudaUserObject_t unheld = nullptr;
+    {
+      std::lock_guard<std::mutex> g(lock);
+      if (last && capture == id && last->bytes >= bytes) {
+        *out = last->p;
+        return cudaSuccess;
+      }
+      Block *b = blocks;
+      while (b && (b->used || b->bytes < bytes)) b = b->next;
+      if (!b) {
+        b = new (std::nothrow) Block();
+        if (!b) return cudaErrorMemoryAllocation;
+        const cudaError_t e = malloc_any(&b->p, bytes);
+        if (e != cudaSuccess) {
+          delete b;
+          return e;
+        }
+        b->bytes = bytes;
+        b->owner = this;
+        b->next = blocks;
+        blocks = b;
+      }
+      b->used = true;
+      cudaUserObject_t obj = nullptr;
+      if (cudaUserObjectCreate(&obj, b, give_back, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+        b->kept = true;
+      } else {
+        ++refs;
+        if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+          b->kept = true;
+          unheld = obj;
+        }
+      }
+      if (b->kept) cudaGetLastError();
+      capture = id;
+      last = b;
+      *out = b->p;
+    }
+    if (unheld) cudaUserObjectRelease(unheld, 1);
+    return cudaSuccess;
+  }
+  // the mesh goes: frees the memory; the struct lives on for the user objects
+  static void release(TraceBlocks *&t) {
+    if (!t) return;
+    {
+      std::lock_guard<std::mutex> g(t->lock);
+      for (Block *b = t->blocks; b; b = b->next) {
+        free_any(b->p);
+        b->p = nullptr;
+        b->bytes = 0;
+      }
+    }
+    drop(t);
+    t = nullptr;
+  }
+};
+
 struct tn_ctx {
   int device = 0;
   Batch *batch = nullptr;
@@ -139,6 +261,7 @@ struct tn_ctx {
   // precision asked for (an FP64 one serves FP32 applies too)
   void *trace = nullptr;
   size_t trace_entries = 0, trace_bytes = 0;
+  TraceBlocks *trace_blocks = nullptr;  // of captured applies
   // workspace
   size_t ws_ndof = 0;
   double *b64 = nullptr, *diag64 = nullptr, *dinv64 = nullptr, *r64 = nullptr, *z64 = nullptr,
@@ -235,6 +358,7 @@ static void free_mesh(tn_ctx *c) {
   dfree(c->d_tables);
   dfree(c->trace);
   c->trace_bytes = 0;
+  TraceBlocks::release(c->trace_blocks);
   tn::free_host_mesh(&c->hm);
   std::free(c->slab_z_host);
   std::free(c->slab_log_host);
@@ -1000,15 +1124,17 @@ tn_status tn_apply_operator(tn_ctx *c, int precision, const void *u, void *y) {
   const char *a = (const char *)u, *b = (const char *)y;
   const size_t bytes = c->ndof * es;
   if (a < b + bytes && b < a + bytes) return fail(TN_EINVAL, "u and y overlap");
-  // a captured apply gets a traction scratch of its own, owned by the graph,
-  // so that a replay may overlap other work of the context
+  // a captured apply takes its traction scratch from the blocks of captures
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  CU_TRY(cudaStreamIsCapturing(c->stream, &cs), "capture status");
-  if (cs != cudaStreamCaptureStatusNone) {
+  unsigned long long id = 0;
+  cudaGraph_t graph = nullptr;
+  CU_TRY(cudaStreamGetCaptureInfo(c->stream, &cs, &id, &graph, nullptr, nullptr, nullptr), "capture status");
+  if (cs == cudaStreamCaptureStatusActive) {
     OpSys sys = make_sys(c);
-    CU_TRY(cudaMallocAsync(&sys.trace, c->trace_entries * es, c->stream), "traction scratch of a captured apply");
+    if (!c->trace_blocks && !(c->trace_blocks = new (std::nothrow) TraceBlocks()))
+      return fail(TN_ENOMEM, "host allocation failed");
+    CU_TRY(c->trace_blocks->take(id, graph, c->trace_entries * es, &sys.trace), "traction scratch of a captured apply");
     CU_TRY(sys.apply(precision, u, y, nullptr, c->stream), "apply launch");
-    CU_TRY(cudaFreeAsync(sys.trace, c->stream), "traction scratch of a captured apply");
     return TN_OK;
   }
   if ((st = ensure_trace(c, precision))) return st;
