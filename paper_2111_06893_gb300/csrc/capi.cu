@@ -417,9 +417,10 @@ static tn_status ensure_ws(tn_ctx *c) {
 static tn_status ensure_trace(tn_ctx *c, int prec) {
   const size_t bytes = c->trace_entries * (prec == TN_F64 ? sizeof(double) : sizeof(float));
   if (c->trace_bytes >= bytes) return TN_OK;
-  dfree(c->trace);
+  free_any(c->trace);
+  c->trace = nullptr;
   c->trace_bytes = 0;
-  const cudaError_t e = cudaMalloc(&c->trace, bytes);
+  const cudaError_t e = malloc_any(&c->trace, bytes);
   if (e != cudaSuccess) {
     c->trace = nullptr;
     cudaGetLastError();

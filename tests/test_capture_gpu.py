@@ -37,9 +37,11 @@ def ptr(v=None):
 def capture(stream, calls):
     g = ptr()
     cu("cuStreamBeginCapture_v2", ptr(stream.cuda_stream), 0)
-    for c in calls:
-        c()
-    cu("cuStreamEndCapture", ptr(stream.cuda_stream), C.byref(g))
+    try:
+        for c in calls:
+            c()
+    finally:
+        cu("cuStreamEndCapture", ptr(stream.cuda_stream), C.byref(g))
     return g
 
 
@@ -56,6 +58,8 @@ def launch(e, stream):
 def node_types(g):
     n = C.c_size_t(0)
     cu("cuGraphGetNodes", g, None, C.byref(n))
+    if n.value == 0:
+        return []
     nodes = (C.c_void_p * n.value)()
     cu("cuGraphGetNodes", g, nodes, C.byref(n))
     out = []
@@ -168,3 +172,18 @@ def test_captures_give_their_scratch_back():
             st.synchronize()
             left.append(torch.cuda.mem_get_info()[0])
         assert left[0] - left[-1] < 10 * block
+
+
+def test_first_fp64_apply_beside_a_capture_of_another_stream():
+    """The scratch is allocated without disturbing a capture in progress (the
+    kernels have run before, on another context: loading them would)."""
+    st, other = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        warm, ctx = context("mesh", st), context("mesh", st)
+        u = field(ctx.ndof, torch.float64, 4)
+        ref, y = warm.apply_operator(u), torch.zeros_like(u)
+        st.synchronize()
+        g = capture(other, [lambda: ctx.apply_operator(u, y)])
+        assert node_types(g) == []
+        cu("cuGraphDestroy", g)
+        assert torch.equal(y, ref)
