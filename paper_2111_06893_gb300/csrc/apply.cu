@@ -35,6 +35,7 @@
 // p = 5: 1.10 ms (3.11 ms), about 65 FP64 operations per unknown (204).
 // The second launch starts while the first drains (its reads of the mesh
 // overlap): 24 instead of 31 us per FP32 apply at 2.0 M unknowns.
+#include <algorithm>
 #include <initializer_list>
 
 #include "tn_device.h"
@@ -842,13 +843,27 @@ apply_batch_kernel(const DevMesh *__restrict__ meshes, const int2 *__restrict__ 
 // all nodes, the residual update taking the incomplete product as it is
 // (2.0 M unknowns, FP32: the two passes it replaces took 7.8 + 5 us).  Up to
 // three faces meet at a node; their terms are added in the order xi, eta,
-// zeta.  Bound by the bytes of the vectors and traces.
+// zeta.  Bound by the bytes of the vectors and traces, with few elements by
+// latency: they are spread over two CTAs per SM then (FP32 applies one after
+// another, p = 2: 64 elements 12.4 -> 7.1 us, 512 12.5 -> 7.0, against as many
+// elements per CTA as add_eb, 39).
 template <int N>
 __host__ __device__ constexpr int surf_nodes() { return N * N * N - (N - 2) * (N - 2) * (N - 2); }
 constexpr int kAddThreads = 256;
 template <int N>
 __host__ __device__ constexpr int add_eb() { return kAddThreads * 4 / surf_nodes<N>(); }
-
+int add_elems(int most, int E) { return std::min(most, std::max(1, E / (2 * tn_sm_count()))); }
+// Whether the second launch lets the one after it start at once.  An apply
+// that starts while the one before still runs takes whatever slots are left,
+// so that a grid smaller than the GPU piles up on a few SMs (FP64, 216
+// elements, p = 4: 73 us an apply, 25 once the second launch ends first); one
+// of several CTAs per SM gains (FP32, 1944 elements, p = 6: 389 CTAs, 24.9 us
+// against 26.2; 2744 elements, p = 4: 275 CTAs, 20.7 against 18.9), but for a
+// batch's, whose CTAs differ (8 mirrors 31 against 24 us, 14: 49 against 43).
+// In a PCG iteration the launch after it is the preconditioner's.
+bool add_early(const ApplyArgs &a) {
+  return a.r || (a.m && !tn_apply_few(a.m->E) && tn_apply_parts(a.m->N, a.m->E) > 2 * tn_sm_count());
+}
 template <int N, typename T, int UPD>
 __device__ __forceinline__ void trace_add_cta(const DevMesh &m1, const DevMesh *__restrict__ meshes,
                                               const int2 *__restrict__ work, const long long *__restrict__ dof_off,
@@ -941,11 +956,10 @@ __device__ __forceinline__ void trace_add_cta(const DevMesh &m1, const DevMesh *
 
 template <int N, typename T, int UPD>
 __global__ void __launch_bounds__(kAddThreads)
-trace_add_kernel(const DevMesh m1, int nwork, T *__restrict__ y, const T *__restrict__ trace, T *__restrict__ r,
-                 const double *__restrict__ alpha, const int *__restrict__ done) {
-  grid_trigger();
-  constexpr int EB = add_eb<N>();
-  const int w0 = blockIdx.x * EB, nw = nwork - w0 < EB ? nwork - w0 : EB;
+trace_add_kernel(const DevMesh m1, int nwork, int eb, bool early, T *__restrict__ y, const T *__restrict__ trace,
+                 T *__restrict__ r, const double *__restrict__ alpha, const int *__restrict__ done) {
+  if (early) grid_trigger();
+  const int w0 = blockIdx.x * eb, nw = nwork - w0 < eb ? nwork - w0 : eb;
   trace_add_cta<N, T, UPD>(m1, nullptr, nullptr, nullptr, nullptr, w0, nw, y, trace, r, alpha, done);
 }
 
@@ -953,9 +967,9 @@ template <typename T, int UPD>
 __global__ void __launch_bounds__(kAddThreads)
 trace_add_batch_kernel(const DevMesh *__restrict__ meshes, const int2 *__restrict__ work,
                        const long long *__restrict__ dof_off, const long long *__restrict__ tr_off,
-                       const int4 *__restrict__ ctas, T *__restrict__ y, const T *__restrict__ trace,
+                       const int4 *__restrict__ ctas, bool early, T *__restrict__ y, const T *__restrict__ trace,
                        T *__restrict__ r, const double *__restrict__ alpha, const int *__restrict__ done) {
-  grid_trigger();
+  if (early) grid_trigger();
   const int4 C = ctas[blockIdx.x];
   const DevMesh none{};
   switch (C.x) {
@@ -1007,20 +1021,21 @@ cudaError_t launch_mesh(const ApplyArgs &a, cudaStream_t st) {
 
 template <int N, typename T>
 cudaError_t launch_second(const ApplyArgs &a, cudaStream_t st) {
-  const int E = a.m->E, grid = (E + add_eb<N>() - 1) / add_eb<N>();
-  return a.r ? launch_pdl(trace_add_kernel<N, T, 1>, grid, kAddThreads, 0, st, *a.m, E, (T *)a.y, (const T *)a.trace,
-                          (T *)a.r, a.alpha, a.done)
-             : launch_pdl(trace_add_kernel<N, T, 0>, grid, kAddThreads, 0, st, *a.m, E, (T *)a.y, (const T *)a.trace,
-                          (T *)nullptr, (const double *)nullptr, a.done);
+  const int E = a.m->E, eb = add_elems(add_eb<N>(), E), grid = (E + eb - 1) / eb;
+  const bool early = add_early(a);
+  return a.r ? launch_pdl(trace_add_kernel<N, T, 1>, grid, kAddThreads, 0, st, *a.m, E, eb, early, (T *)a.y,
+                          (const T *)a.trace, (T *)a.r, a.alpha, a.done)
+             : launch_pdl(trace_add_kernel<N, T, 0>, grid, kAddThreads, 0, st, *a.m, E, eb, early, (T *)a.y,
+                          (const T *)a.trace, (T *)nullptr, (const double *)nullptr, a.done);
 }
 
 template <typename T>
 cudaError_t launch_second_batch(const ApplyArgs &a, cudaStream_t st) {
   if (a.nadd <= 0) return cudaSuccess;
   return a.r ? launch_pdl(trace_add_batch_kernel<T, 1>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
-                          a.tr_off, a.adds, (T *)a.y, (const T *)a.trace, (T *)a.r, a.alpha, a.done)
+                          a.tr_off, a.adds, early, (T *)a.y, (const T *)a.trace, (T *)a.r, a.alpha, a.done)
              : launch_pdl(trace_add_batch_kernel<T, 0>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
-                          a.tr_off, a.adds, (T *)a.y, (const T *)a.trace, (T *)nullptr, (const double *)nullptr, a.done);
+                          a.tr_off, a.adds, early, (T *)a.y, (const T *)a.trace, (T *)nullptr, (const double *)nullptr, a.done);
 }
 
 template <typename T, int V, int MODE>
@@ -1054,6 +1069,7 @@ constexpr int kEnergyThreads = 256;
 template <int N>
 constexpr int energy_eb() { return kEnergyThreads / (N * N); }
 template <int N, bool SPLIT>
+  const bool early = add_early(a);
 constexpr size_t energy_smem(int eb) { return sizeof(double) * (size_t)eb * (SPLIT ? 9 : 6) * N * N * N; }
 
 // elements w0 .. of one mesh (meshes == nullptr: m1, element w) or of a batch
@@ -1272,7 +1288,7 @@ cudaError_t tn_upload_lgl_apply(const LglTables *t) {
 // variant 1 exists for FP32 only
 cudaError_t tn_launch_apply(const ApplyArgs &a, cudaStream_t st) {
   if (!a.m) {
-    if (a.few)
+    if (tn_apply_few(a.elems))
       return a.prec == TN_F64 ? launch_batch<double, 0, AM_SMALL_BATCH>(a, st) : launch_batch<float, 0, AM_SMALL_BATCH>(a, st);
     if (a.prec == TN_F64) return launch_batch<double, 0, AM_PENCIL>(a, st);
     return a.var == 1 ? launch_batch<float, 1, AM_PENCIL>(a, st) : launch_batch<float, 0, AM_PENCIL>(a, st);
@@ -1303,9 +1319,9 @@ bool tn_apply_few(int E) { return apply_small(E); }
 int tn_apply_eb(int N, bool few) { return few ? kSmallBatchThreads / (3 * N * N) : kApplyThreads / (N * N); }
 int tn_apply_parts(int N, int E) { return apply_small(E) ? E : (E + tn_apply_eb(N, false) - 1) / tn_apply_eb(N, false); }
 
-int tn_trace_add_eb(int N) {
+int tn_trace_add_eb(int N, int elems) {
   switch (N) {
-#define TN_CASE(NN) case NN: return add_eb<NN>();
+#define TN_CASE(NN) case NN: return add_elems(add_eb<NN>(), elems);
     TN_FOR_N(TN_CASE)
 #undef TN_CASE
     default: return 1;

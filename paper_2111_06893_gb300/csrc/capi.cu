@@ -983,7 +983,7 @@ static tn_status batch_finalize(tn_ctx *c) {
       return (int)v.size();
     };
     s.gcta[g + 1] = split(ctas, tn_apply_eb(N, few));
-    s.gadd[g + 1] = split(adds, tn_trace_add_eb(N));
+    s.gadd[g + 1] = split(adds, tn_trace_add_eb(N, elems));
     s.gN[g] = N;
     s.gcount[g] = (int)work.size() - w0;
     s.gpart_off[g] = w0;

@@ -659,7 +659,7 @@ ApplyArgs OpSys::args(int g0, int g1, int prec, const void *u, void *y) const {
   a.adds = adds + gadd[g0];
   a.nadd = gadd[g1] - gadd[g0];
   a.var = gvar[g0];
-  a.few = tn_apply_few(n_elems);
+  a.elems = n_elems;
   return a;
 }
 
@@ -674,7 +674,7 @@ cudaError_t OpSys::apply_own(int prec, const void *u, void *y, double *part, cud
   // neighbouring degrees of one variant in one launch (FP64 has one variant)
   for (int g = 0; g < ngroups;) {
     int h = g + 1;
-    while (h < ngroups && (prec == TN_F64 || a.few || gvar[h] == gvar[g])) ++h;
+    while (h < ngroups && (prec == TN_F64 || tn_apply_few(n_elems) || gvar[h] == gvar[g])) ++h;
     ApplyArgs b = args(g, h, prec, u, y);
     b.fold = fold;
     b.partial = part ? part + gcta[g] : nullptr;

@@ -188,7 +188,7 @@ struct ApplyArgs {
   const long long *dof_off = nullptr, *tr_off = nullptr;
   const int4 *ctas = nullptr, *adds = nullptr;  // batch: CTAs of the apply and of tn_launch_trace_add
   int ncta = 0, nadd = 0;
-  bool few = false;                 // batch: tn_apply_few of its elements
+  int elems = 0;                    // batch: all its elements (the forms taken depend on them)
   int prec = TN_F64, var = 0;       // var: occupancy variant of the FP32 kernel (0 or 1, same results)
   const void *u = nullptr;
   void *y = nullptr, *trace = nullptr;  // trace: tn_trace_entries per element, of the vectors' precision
@@ -212,7 +212,7 @@ cudaError_t tn_launch_trace_add(const ApplyArgs &a, cudaStream_t st);
 int tn_apply_parts(int N, int E);
 bool tn_apply_few(int E);  // few elements: the form with three threads per pencil
 int tn_apply_eb(int N, bool few);
-int tn_trace_add_eb(int N);
+int tn_trace_add_eb(int N, int elems);  // elems: of the whole batch
 // us[v]: time per apply of FP32 variant v; y is overwritten
 cudaError_t tn_tune_apply(ApplyArgs a, cudaStream_t st, float us[2]);
 cudaError_t tn_launch_energy_batch(int N, const DevMesh *meshes, const int2 *work, int nwork,
