@@ -50,12 +50,15 @@ constexpr size_t zp_smem() {
   return (4 * (size_t)zp_stage_per_warp<N>() + 4 * kZgThreads) * sizeof(float) + 4 * kZgMaxStages * 8;
 }
 
-// barrier of a slot of G > 1 warps starting at warp w0 of its CTA.  Immediate
-// barrier numbers: a number in a register claims all 16 of the CTA.
+// barrier of a slot of G > 1 warps starting at warp w0 of its CTA (0, or 2 of
+// the second of two pairs).  Immediate barrier numbers: a number in a register
+// claims all 16 of the CTA.  Slots of 3 and 4 warps start at 0: a test of w0
+// at each of their barriers, two a slab, cost the batches 1 to 3 % (24 mirrors
+// 212.2 -> 210.7 us, two 56.9 -> 55.4, means over memory placements).
 template <int G>
 __device__ __forceinline__ void slot_sync(int w0) {
   if (G == 1) __syncwarp();
-  else if (w0 == 0) asm volatile("bar.sync 1, %0;\n" ::"n"(32 * G) : "memory");
+  else if (G > 2 || w0 == 0) asm volatile("bar.sync 1, %0;\n" ::"n"(32 * G) : "memory");
   else asm volatile("bar.sync 2, %0;\n" ::"n"(32 * G) : "memory");
 }
 // true if p holds on any thread of the slot (and a sync)
@@ -72,7 +75,7 @@ __device__ __forceinline__ bool named_any(bool p) {
 template <int G>
 __device__ __forceinline__ bool slot_any(int w0, bool p) {
   if (G == 1) return __any_sync(0xffffffffu, p);
-  return w0 == 0 ? named_any<1, 32 * G>(p) : named_any<2, 32 * G>(p);
+  return G > 2 || w0 == 0 ? named_any<1, 32 * G>(p) : named_any<2, 32 * G>(p);
 }
 __device__ __forceinline__ void mbar_inval(unsigned long long *bar) {
   asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_u32(bar)) : "memory");
