@@ -98,7 +98,7 @@ static void rotate(int r, double *X, double *Y) {
   }
 }
 
-static void cyl_block_map(int blk, double xb, double eb, double a, double R1, double R,
+static void cyl_block_map(int blk, double xb, double eb, double ct, double st, double a, double R1, double R,
                           double *X, double *Y, double J[4]) {
   if (blk == 0) {
     *X = a * xb;
@@ -106,7 +106,7 @@ static void cyl_block_map(int blk, double xb, double eb, double a, double R1, do
     J[0] = a; J[1] = 0.0; J[2] = 0.0; J[3] = a;
     return;
   }
-  const double t = M_PI * eb / 4.0, ct = std::cos(t), st = std::sin(t), dt = M_PI / 4.0;
+  const double dt = M_PI / 4.0;
   double X0, Y0, j0, j1, j2, j3;
   if (blk <= 4) {
     X0 = 0.5 * (1 - xb) * a + 0.5 * (1 + xb) * R1 * ct;
@@ -199,7 +199,15 @@ tn_status build_host_mesh(const tn_mesh_desc *d, HostMesh *out, char *msg, int m
   // ---- columns: geometry and neighbours
   for (int c = 0; c < ncol; ++c) {
     double *g = m.colgeo + (size_t)c * CG_NF * N2;
-    for (int j = 0; j < N; ++j)
+    for (int j = 0; j < N; ++j) {
+      double eb = 0.0, ct = 1.0, st = 0.0;  // cylinder: eta on the block, and the cosine and sine of its angle
+      if (d->kind != TN_MESH_BOX) {
+        const int k = d->k, bi = c % (k * k) / k;
+        eb = -1.0 + (2.0 * bi + 1.0 + x[j]) / k;
+        const double t = M_PI * eb / 4.0;
+        ct = std::cos(t);
+        st = std::sin(t);
+      }
       for (int i = 0; i < N; ++i) {
         double X, Y, J[4];
         if (d->kind == TN_MESH_BOX) {
@@ -210,10 +218,9 @@ tn_status build_host_mesh(const tn_mesh_desc *d, HostMesh *out, char *msg, int m
           Y = y0 + 0.5 * (1 + x[j]) * (y1 - y0);
           J[0] = 0.5 * (x1 - x0); J[1] = 0.0; J[2] = 0.0; J[3] = 0.5 * (y1 - y0);
         } else {
-          const int k = d->k, blk = c / (k * k), cl = c % (k * k), bi = cl / k, ai = cl % k;
+          const int k = d->k, blk = c / (k * k), ai = c % k;
           const double xb = -1.0 + (2.0 * ai + 1.0 + x[i]) / k;
-          const double eb = -1.0 + (2.0 * bi + 1.0 + x[j]) / k;
-          cyl_block_map(blk, xb, eb, d->a, d->R1, d->R, &X, &Y, J);
+          cyl_block_map(blk, xb, eb, ct, st, d->a, d->R1, d->R, &X, &Y, J);
           for (int t = 0; t < 4; ++t) J[t] /= k;
         }
         const double det = J[0] * J[3] - J[1] * J[2];
@@ -231,6 +238,7 @@ tn_status build_host_mesh(const tn_mesh_desc *d, HostMesh *out, char *msg, int m
         g[CG_X * N2 + q] = X;
         g[CG_Y * N2 + q] = Y;
       }
+    }
     int *nb = m.colnb + 4 * c, *nf = m.colnbf + 4 * c;
     if (d->kind == TN_MESH_BOX) {
       const int ix = c % d->nx, jy = c / d->nx;
@@ -273,27 +281,39 @@ tn_status build_host_mesh(const tn_mesh_desc *d, HostMesh *out, char *msg, int m
       }
     }
   }
-  // ---- penalty scales of the lateral faces
+  // ---- penalty scales of the lateral faces, from |grad xi|^2 (|grad eta|^2) at
+  // the face nodes: one square root where the neighbour's is the larger
+  double *const mag2 = (double *)std::malloc(sizeof(double) * ncol * 4 * N);
+  if (!mag2) {
+    free_host_mesh(&m);
+    set_err(msg, msglen, "host allocation failed");
+    return TN_ENOMEM;
+  }
+  for (int c = 0; c < ncol; ++c)
+    for (int f = 0; f < 4; ++f) {
+      const int dd = f >> 1, end = (f & 1) ? N - 1 : 0;
+      const double *r = m.colgeo + ((size_t)c * CG_NF + (dd == 0 ? CG_IXX : CG_IEX)) * N2;
+      for (int t = 0; t < N; ++t) {
+        const int q = dd == 0 ? t * N + end : end * N + t;
+        mag2[((size_t)c * 4 + f) * N + t] = r[q] * r[q] + r[N2 + q] * r[N2 + q];
+      }
+    }
   for (int c = 0; c < ncol; ++c)
     for (int f = 0; f < 4; ++f) {
       const int nbc = m.colnb[4 * c + f], code = m.colnbf[4 * c + f];
       const int dd = f >> 1, end = (f & 1) ? N - 1 : 0;
+      const double *own = mag2 + ((size_t)c * 4 + f) * N, *ext = mag2 + ((size_t)(nbc < 0 ? c : nbc) * 4 + (code & 3)) * N;
+      double *g = m.colgeo + ((size_t)c * CG_NF + (dd == 0 ? CG_RXI : CG_RETA)) * N2;
       for (int t = 0; t < N; ++t) {
-        double *g = m.colgeo + (size_t)c * CG_NF * N2;
-        const int q = dd == 0 ? t * N + end : end * N + t;
         double ratio = 1.0;
         if (nbc >= 0) {
-          const int f2 = code & 3, d2 = f2 >> 1, end2 = (f2 & 1) ? N - 1 : 0, a2 = (code >> 2) ? N - 1 - t : t;
-          const int q2 = d2 == 0 ? a2 * N + end2 : end2 * N + a2;
-          const double *g2 = m.colgeo + (size_t)nbc * CG_NF * N2;
-          const int bx = dd == 0 ? CG_IXX : CG_IEX, bx2 = d2 == 0 ? CG_IXX : CG_IEX;
-          const double mag = std::hypot(g[bx * N2 + q], g[(bx + 1) * N2 + q]);
-          const double mag2 = std::hypot(g2[bx2 * N2 + q2], g2[(bx2 + 1) * N2 + q2]);
-          if (mag2 > mag) ratio = mag2 / mag;
+          const double e = ext[(code >> 2) ? N - 1 - t : t];
+          if (e > own[t]) ratio = std::sqrt(e / own[t]);
         }
-        g[(dd == 0 ? CG_RXI : CG_RETA) * N2 + q] = 0.5 * ratio;
+        g[dd == 0 ? t * N + end : end * N + t] = 0.5 * ratio;
       }
     }
+  std::free(mag2);
   // ---- slabs
   for (int s = 0; s < m.nslab; ++s) {
     double *g = m.slabgeo + (size_t)s * SG_NF * N;
