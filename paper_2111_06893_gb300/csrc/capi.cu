@@ -74,23 +74,38 @@ struct Batch {
 
 // host tables gathered into one block, for one allocation and one copy
 struct TablePack {
-  std::vector<unsigned char> host;
-  size_t add(const void *src, size_t bytes) {  // offset of the copy (256-byte aligned)
-    const size_t off = (host.size() + 255) / 256 * 256;
-    host.resize(off + bytes);
-    std::memcpy(host.data() + off, src, bytes);
+  static constexpr size_t kAlign = 256;
+  unsigned char *host;
+  size_t room, size = 0;
+  TablePack(size_t bytes, int tables) : room(bytes + kAlign * tables) { host = (unsigned char *)std::malloc(room); }
+  ~TablePack() { std::free(host); }
+  TablePack(const TablePack &) = delete;
+  TablePack &operator=(const TablePack &) = delete;
+  // offset of the next table, of `bytes` bytes; at: its place (nullptr: no memory, or more than announced)
+  size_t next(size_t bytes, void **at) {
+    const size_t off = (size + kAlign - 1) / kAlign * kAlign;
+    size = off + bytes;
+    *at = host && size <= room ? host + off : nullptr;
+    return off;
+  }
+  size_t add(const void *src, size_t bytes) {
+    void *at;
+    const size_t off = next(bytes, &at);
+    if (at && bytes) std::memcpy(at, src, bytes);
     return off;
   }
   size_t add32(const double *src, size_t n) {  // rounded to FP32
-    const size_t off = (host.size() + 255) / 256 * 256;
-    host.resize(off + n * sizeof(float));
-    float *d = reinterpret_cast<float *>(host.data() + off);
-    for (size_t i = 0; i < n; ++i) d[i] = (float)src[i];
+    void *at;
+    const size_t off = next(n * sizeof(float), &at);
+    if (float *d = (float *)at)
+      for (size_t i = 0; i < n; ++i) d[i] = (float)src[i];
     return off;
   }
   cudaError_t upload(unsigned char **dev) const {
-    cudaError_t e = cudaMalloc((void **)dev, host.size());
-    if (e == cudaSuccess) e = cudaMemcpy(*dev, host.data(), host.size(), cudaMemcpyHostToDevice);
+    if (!host) return cudaErrorMemoryAllocation;
+    if (size > room) return cudaErrorInvalidValue;
+    cudaError_t e = cudaMalloc((void **)dev, size);
+    if (e == cudaSuccess) e = cudaMemcpy(*dev, host, size, cudaMemcpyHostToDevice);
     return e;
   }
 };
@@ -98,6 +113,11 @@ struct TablePack {
 // the tables of a mesh and their places in the block
 struct MeshTables {
   size_t cg, sg, cg32, sg32, nb, nbf, sl;
+  static constexpr int kTables = 7;
+  static size_t bytes(const tn::HostMesh &hm) {
+    const size_t ncg = (size_t)hm.ncol * CG_NF * hm.N * hm.N, nsg = (size_t)hm.nslab * SG_NF * hm.N;
+    return (ncg + nsg) * (sizeof(double) + sizeof(float)) + sizeof(int) * (8 * (size_t)hm.ncol + hm.nslab);
+  }
   void pack(TablePack &p, const tn::HostMesh &hm) {
     const size_t ncg = (size_t)hm.ncol * CG_NF * hm.N * hm.N, nsg = (size_t)hm.nslab * SG_NF * hm.N;
     cg = p.add(hm.colgeo, sizeof(double) * ncg);
@@ -538,7 +558,8 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gstatus, 2 * sizeof(int));  // factor status, solve timeout
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gchain, sizeof(double) * (size_t)p.nchain);
   if (e == cudaSuccess) e = cudaMalloc((void **)&c->gqueue, sizeof(int) * kZgQueue * kZgMaxDg);
-  TablePack pack;
+  TablePack pack(sizeof(int4) * (p.lines.size() + p.packs.size() + p.ranges.size()) + sizeof(int) * p.inst.size() +
+                     sizeof(long long) * (p.fac_off.size() + p.fac64_off.size() + p.chain_off.size()), 7);
   const size_t o_lines = pack.add(p.lines.data(), sizeof(int4) * p.lines.size());
   const size_t o_fac = pack.add(p.fac_off.data(), sizeof(long long) * p.fac_off.size());
   const size_t o_fac64 = pack.add(p.fac64_off.data(), sizeof(long long) * p.fac64_off.size());
@@ -823,7 +844,7 @@ tn_status tn_build_mesh(tn_ctx *c, const tn_mesh_desc *d) {
   dfree(c->d_layer_c32);
   c->have_mat = false;
   c->hm = hm;
-  TablePack pack;
+  TablePack pack(MeshTables::bytes(hm), MeshTables::kTables);
   MeshTables tab;
   tab.pack(pack, hm);
   const cudaError_t e = pack.upload(&c->d_tables);
@@ -1074,7 +1095,7 @@ tn_status tn_batch_set(tn_ctx *c, int i, const tn_mesh_desc *d, int n_mat, const
   CU_TRY(cudaSetDevice(c->device), "cudaSetDevice");
   BatchInst &q = b->inst[i];
   q.hm = hm;
-  TablePack pack;
+  TablePack pack(MeshTables::bytes(hm) + (sizeof(double) + sizeof(float)) * h.size(), MeshTables::kTables + 2);
   MeshTables tab;
   tab.pack(pack, hm);
   const size_t lc = pack.add(h.data(), sizeof(double) * h.size()), lc32 = pack.add32(h.data(), h.size());
