@@ -456,11 +456,12 @@ static cudaError_t pcg_iteration_zline(const OpSys &sys, int prec, size_t n, Pcg
 }
 
 // PCG on A x = b in precision T; x holds the initial guess (x0_zero: x = 0).
-// Records `chunk` iterations in a graph and replays it until done.
+// Records `chunk` iterations in a graph and replays it until done, or, if
+// patience > 0, until the recursive residual has not halved for that many chunks.
 template <typename T>
 static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, bool x0_zero, double rtol,
                            int max_iters, int chunk, tn_pcg_scalars *s_dev, tn_pcg_scalars *s_host,
-                           double *part_elem, double *part_red, cudaStream_t st, int *applies,
+                           double *part_elem, double *part_red, cudaStream_t st, int *applies, int patience,
                            ChunkHook hook = ChunkHook()) {
   const bool zl = v.zfac != nullptr;
   g_launches += zl ? 5 : 3;
@@ -556,9 +557,8 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
     }
     if (s_host->done) break;
     if (hook.fn && hook.fn(hook.user)) break;
-    // stagnation: the recursive residual has not halved for 40 chunks
     if (s_host->rr < 0.5 * best) { best = s_host->rr; stall = 0; }
-    else if (++stall >= 40) break;
+    else if (++stall == patience) break;
   }
   *applies += s_host->iters;
   return err;
@@ -568,14 +568,15 @@ cudaError_t pcg_f64(const OpSys &sys, size_t n, PcgVectors &v, bool x0_zero, dou
                     int chunk, tn_pcg_scalars *s_dev, tn_pcg_scalars *s_host, double *part_elem,
                     double *part_red, cudaStream_t st, int *applies, ChunkHook hook) {
   return pcg_run<double>(sys, TN_F64, n, v, x0_zero, rtol, max_iters, chunk, s_dev, s_host, part_elem,
-                         part_red, st, applies, hook);
+                         part_red, st, applies, 40, hook);
 }
 
 cudaError_t pcg_f32(const OpSys &sys, size_t n, PcgVectors &v, bool x0_zero, double rtol, int max_iters,
                     int chunk, tn_pcg_scalars *s_dev, tn_pcg_scalars *s_host, double *part_elem,
                     double *part_red, cudaStream_t st, int *applies) {
   return pcg_run<float>(sys, TN_F32, n, v, x0_zero, rtol, max_iters, chunk, s_dev, s_host, part_elem,
-                        part_red, st, applies);
+                        part_red, st, applies, 0);
+  // the inner run of a mixed solve goes to rtol or max_iters, in whatever chunks
 }
 
 // r = b - A x in FP64; returns ||r||^2 in *rr_host (synchronises)
