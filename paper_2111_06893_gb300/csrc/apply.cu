@@ -934,6 +934,8 @@ __device__ __forceinline__ void trace_add_cta(const DevMesh &m1, const DevMesh *
   __syncthreads();
   grid_wait();
   done = after_wait(done);
+  y = after_wait(y);
+  r = after_wait(r);
   if (done && *done) return;
   const T al = UPD ? (T)*after_wait(alpha) : T(0);
 #pragma unroll 4
@@ -1067,9 +1069,9 @@ cudaError_t launch_second(const ApplyArgs &a, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_second_batch(const ApplyArgs &a, cudaStream_t st) {
   if (a.nadd <= 0) return cudaSuccess;
+  const bool early = add_early(a);
   return a.r ? launch_pdl(trace_add_batch_kernel<T, 1>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
                           a.tr_off, a.adds, early, (T *)a.y, (const T *)a.trace, (T *)a.r, a.alpha, a.done)
-  const bool early = add_early(a);
              : launch_pdl(trace_add_batch_kernel<T, 0>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
                           a.tr_off, a.adds, early, (T *)a.y, (const T *)a.trace, (T *)nullptr, (const double *)nullptr, a.done);
 }

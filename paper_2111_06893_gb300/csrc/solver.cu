@@ -335,6 +335,8 @@ __global__ void k_pupdate_x(const tn_pcg_scalars *s, size_t n, T *__restrict__ x
   grid_wait();
   s = after_wait(s);
   z = after_wait(z);
+  x = after_wait(x);
+  p = after_wait(p);
   if (!s->active) return;
   const T alpha = (T)s->alpha, beta = (T)s->beta;
   const bool more = !s->done;
@@ -574,9 +576,9 @@ cudaError_t pcg_f64(const OpSys &sys, size_t n, PcgVectors &v, bool x0_zero, dou
 cudaError_t pcg_f32(const OpSys &sys, size_t n, PcgVectors &v, bool x0_zero, double rtol, int max_iters,
                     int chunk, tn_pcg_scalars *s_dev, tn_pcg_scalars *s_host, double *part_elem,
                     double *part_red, cudaStream_t st, int *applies) {
+  // the inner run of a mixed solve goes to rtol or max_iters, in whatever chunks
   return pcg_run<float>(sys, TN_F32, n, v, x0_zero, rtol, max_iters, chunk, s_dev, s_host, part_elem,
                         part_red, st, applies, 0);
-  // the inner run of a mixed solve goes to rtol or max_iters, in whatever chunks
 }
 
 // r = b - A x in FP64; returns ||r||^2 in *rr_host (synchronises)
