@@ -437,6 +437,7 @@ static tn_status ensure_ws(tn_ctx *c) {
 static tn_status ensure_trace(tn_ctx *c, int prec) {
   const size_t bytes = c->trace_entries * (prec == TN_F64 ? sizeof(double) : sizeof(float));
   if (c->trace_bytes >= bytes) return TN_OK;
+  CU_TRY(cudaSetDevice(c->device), "cudaSetDevice");
   free_any(c->trace);
   c->trace = nullptr;
   c->trace_bytes = 0;
@@ -1152,6 +1153,7 @@ tn_status tn_apply_operator(tn_ctx *c, int precision, const void *u, void *y) {
   cudaGraph_t graph = nullptr;
   CU_TRY(cudaStreamGetCaptureInfo(c->stream, &cs, &id, &graph, nullptr, nullptr, nullptr), "capture status");
   if (cs == cudaStreamCaptureStatusActive) {
+    CU_TRY(cudaSetDevice(c->device), "cudaSetDevice");
     OpSys sys = make_sys(c);
     if (!c->trace_blocks && !(c->trace_blocks = new (std::nothrow) TraceBlocks()))
       return fail(TN_ENOMEM, "host allocation failed");
