@@ -46,8 +46,10 @@ struct OpSys {
                         const PcgFold *fold = nullptr) const;
   cudaError_t apply_traces(int prec, void *y, void *r, const double *alpha, const int *done, cudaStream_t st) const;
   cudaError_t apply(int prec, const void *u, void *y, double *part, cudaStream_t st) const;
-  // z = M^{-1} r; q != nullptr: first r <- r - (*alpha) q.  part: rz_parts
-  // partial r.z, then rz_parts partial r.r
+  // z = M^{-1} r.  Single lines: q != nullptr: first r <- r - (*alpha) q.
+  // Grouped lines: q and alpha null (apply_traces updates r), fold the beta
+  // step.  What a form does not do is refused.  part: rz_parts partial r.z,
+  // then rz_parts partial r.r
   cudaError_t zsolve(int prec, const void *fac, void *r, const void *q, void *z, const double *alpha,
                      double *part, const int *done, cudaStream_t st, const PcgFold *fold = nullptr) const;
 };
