@@ -1239,7 +1239,7 @@ static tn_status solve_impl(tn_ctx *c, const tn_solve_opts *o, const double *rhs
   if ((st = ensure_ws(c)) || (st = ensure_trace(c, TN_F64))) return st;
   const int chunk = o->check_every > 0 ? o->check_every : 25;
   const auto t0 = std::chrono::steady_clock::now();
-  tn::g_launches = 2;  // rhs and diagonal below
+  tn::g_launches = (rhs ? 0 : is_batch(c) ? c->batch->n : 1) + (is_batch(c) ? 0 : 1);  // right-hand side, diagonal
   tn::g_timed_out = false;
   cudaStream_t s = c->sstream;
   CU_TRY(cudaEventRecord(c->ev_in, c->stream), "event");
@@ -1402,7 +1402,7 @@ static tn_status solve_impl(tn_ctx *c, const tn_solve_opts *o, const double *rhs
       // z = |r| d (FP64), q = A z
       CU_TRY(tn::upcast(n, c->d32, rn, c->z64, s), "upcast");
       CU_TRY(sys.apply(TN_F64, c->z64, c->q64, nullptr, s), "apply f64");
-      tn::g_launches += 1;
+      tn::g_launches += sys.apply_launches(TN_F64);
       r.applies_f64 += 1;
       // keep the new direction A-orthogonal to the last nb ones
       const int nb = k < m ? k : m, slot = k % m;

@@ -2,7 +2,7 @@
 //
 // The paper solves with GMRES; the weak-form DG operator built here is
 // symmetric positive definite, so the solver is preconditioned conjugate
-// gradients.  With the Jacobi preconditioner an iteration is five launches:
+// gradients.  With the Jacobi preconditioner an iteration is six launches:
 // the fused operator apply (which also returns p.Ap per element), a
 // one-block reduction for alpha, a fused vector update (x, r, z = D^-1 r,
 // partial r.z and r.r), a one-block reduction for beta and the direction
@@ -10,7 +10,8 @@
 // q runs inside the line solve (which also returns partial r.z and r.r);
 // with grouped lines the operator's second launch takes its place (it adds
 // the neighbours' traces on the way), and alpha and beta fold into the apply
-// and the solve, four launches per iteration.  The solution update x += alpha p runs
+// and the solve, four launches per iteration (FP64, whose line solve takes
+// three: six).  The solution update x += alpha p runs
 // inside the direction update.  A chunk of
 // iterations is recorded once in a CUDA graph and replayed.  Krylov scalars
 // live on the device; once converged every kernel returns immediately, so a
@@ -409,7 +410,7 @@ cudaError_t pcg_setup_dinv(size_t n, const double *diag, void *dinv, int prec, c
   return cudaGetLastError();
 }
 
-// one PCG iteration (five launches), all on stream st
+// one PCG iteration (six launches), all on stream st
 template <typename T>
 static cudaError_t pcg_iteration(const OpSys &sys, int prec, size_t n, PcgVectors &v, tn_pcg_scalars *s,
                                  double *part_elem, double *part_red, cudaStream_t st) {
@@ -429,7 +430,7 @@ template <typename T>
 static cudaError_t pcg_iteration_zline(const OpSys &sys, int prec, size_t n, PcgVectors &v, tn_pcg_scalars *s,
                                        double *part_elem, double *part_red, cudaStream_t st) {
   if (sys.grouped) {
-    // four launches: the elements' own terms of the apply with the alpha
+    // four launches (FP64: six): the elements' own terms of the apply with the alpha
     // step, the residual update with the traces, the grouped-line solve with
     // the beta step, the direction update
     PcgFold fa;
@@ -466,7 +467,7 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
                            double *part_elem, double *part_red, cudaStream_t st, int *applies, int patience,
                            ChunkHook hook = ChunkHook()) {
   const bool zl = v.zfac != nullptr;
-  g_launches += zl ? 5 : 3;
+  g_launches += (x0_zero ? 1 : sys.apply_launches(prec)) + (zl ? 3 + sys.zsolve_launches(prec) : 2);
   if (x0_zero) {
     k_fill<T><<<red_blocks(), kRedThreads, 0, st>>>(n, (T *)v.x, T(0));
     TN_CU(cudaGetLastError());
@@ -542,8 +543,10 @@ static cudaError_t pcg_run(const OpSys &sys, int prec, size_t n, PcgVectors &v, 
   }
   double best = INFINITY;
   int stall = 0;
+  const long long per_iter =
+      sys.apply_launches(prec) + (zl ? sys.zsolve_launches(prec) + (sys.grouped ? 1 : 3) : 4);
   for (;;) {
-    g_launches += (zl && sys.grouped && prec == TN_F32 ? 4LL : 6LL) * chunk;
+    g_launches += per_iter * chunk;
     err = cudaGraphLaunch(exec, st);
     if (err != cudaSuccess) break;
     err = cudaMemcpyAsync(s_host, s_dev, sizeof(tn_pcg_scalars), cudaMemcpyDeviceToHost, st);
@@ -584,7 +587,7 @@ cudaError_t pcg_f32(const OpSys &sys, size_t n, PcgVectors &v, bool x0_zero, dou
 // r = b - A x in FP64; returns ||r||^2 in *rr_host (synchronises)
 cudaError_t residual_f64(const OpSys &sys, size_t n, const double *b, const double *x, double *Ax, double *r,
                          double *part_red, double *sum_dev, double *rr_host, cudaStream_t st) {
-  g_launches += 3;
+  g_launches += sys.apply_launches(TN_F64) + 2;
   TN_CU(sys.apply(TN_F64, x, Ax, nullptr, st));
   k_residual<<<red_blocks(), kRedThreads, 0, st>>>(n, b, Ax, r, part_red);
   TN_CU(cudaGetLastError());
@@ -668,16 +671,32 @@ ApplyArgs OpSys::args(int g0, int g1, int prec, const void *u, void *y) const {
 
 int OpSys::apply_parts() const { return m ? tn_apply_parts(m->N, m->E) : gcta[ngroups]; }
 
+// neighbouring degrees of one variant go in one launch (FP64 has one variant)
+int OpSys::launch_end(int g, int prec) const {
+  int h = g + 1;
+  while (h < ngroups && (prec == TN_F64 || tn_apply_few(n_elems) || gvar[h] == gvar[g])) ++h;
+  return h;
+}
+
+int OpSys::apply_launches(int prec) const {
+  if (m) return 2;
+  int n = 1;  // the traces
+  for (int g = 0; g < ngroups; g = launch_end(g, prec)) ++n;
+  return n;
+}
+
+int OpSys::zsolve_launches(int prec) const {
+  return grouped ? zg.npk * (prec == TN_F64 ? 3 : 1) : (m ? 1 : ngroups);
+}
+
 cudaError_t OpSys::apply_own(int prec, const void *u, void *y, double *part, cudaStream_t st,
                              const PcgFold *fold) const {
   ApplyArgs a = args(0, ngroups, prec, u, y);
   a.fold = fold;
   a.partial = part;
   if (m) return tn_launch_apply(a, st);
-  // neighbouring degrees of one variant in one launch (FP64 has one variant)
   for (int g = 0; g < ngroups;) {
-    int h = g + 1;
-    while (h < ngroups && (prec == TN_F64 || tn_apply_few(n_elems) || gvar[h] == gvar[g])) ++h;
+    const int h = launch_end(g, prec);
     ApplyArgs b = args(g, h, prec, u, y);
     b.fold = fold;
     b.partial = part ? part + gcta[g] : nullptr;

@@ -39,6 +39,9 @@ struct OpSys {
   int gcta[9] = {0}, gadd[9] = {0};             // first CTA of every degree group (and the total)
   ApplyArgs args(int g0, int g1, int prec, const void *u, void *y) const;  // groups g0 .. g1 - 1 (one mesh: all)
   int apply_parts() const;  // partial sums written by one apply (one per CTA)
+  int launch_end(int g, int prec) const;  // batch: the degree group after those launched with group g
+  int apply_launches(int prec) const;     // launches of one apply, of one line solve
+  int zsolve_launches(int prec) const;
   // the two launches of y = A u: the elements' own terms (part: partial u . A u;
   // fold: the alpha step), then the traces added to y, or r -= *alpha A u
   // (y is left incomplete).  apply: both.
