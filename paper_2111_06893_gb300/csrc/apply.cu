@@ -1029,17 +1029,6 @@ constexpr size_t max_smem() {
   return m;
 }
 
-// the dynamic shared-memory opt-in of a kernel, once per device
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t bytes, int &configured_device) {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (configured_device == dev) return cudaSuccess;
-  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (err == cudaSuccess) configured_device = dev;
-  return err;
-}
-
 template <int N, typename T, int V, int MODE>
 cudaError_t launch_elem(const ApplyArgs &a, cudaStream_t st) {
   constexpr size_t sm = apply_smem<N, T, MODE>();

@@ -111,6 +111,17 @@ __device__ __forceinline__ P *after_wait(P *p) {
   return p;
 }
 
+// the dynamic shared-memory opt-in of a kernel, once per device
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t bytes, int &configured_device) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (configured_device == dev) return cudaSuccess;
+  cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (err == cudaSuccess) configured_device = dev;
+  return err;
+}
+
 // launch that may start before the kernel ahead of it in st has ended
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {

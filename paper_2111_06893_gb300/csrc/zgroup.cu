@@ -919,10 +919,6 @@ zg_final_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, con
 
 template <typename... P, typename... A>
 cudaError_t launch_zg(void (*kernel)(P...), int grid, size_t smem, bool dependent, cudaStream_t st, A... args) {
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kZgThreads);
@@ -942,7 +938,11 @@ cudaError_t launch_f64(const DevMesh &m, const ZGroupDev &gd, int k, const doubl
                        const PcgFold &fold) {
   const ZgView v{gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac64_off, gd.chain_off,
                  gd.packs + gd.pk_start[k], gd.ranges + gd.rg_start[k]};
-  cudaError_t e = launch_zg(zg_slab_kernel<N, double>, gd.rg_n[k], zg_slab_smem<N, double>(), first, st, m, v, fac, r,
+  static int slab_device = -1, chain_device = -1;
+  cudaError_t e = allow_smem(zg_slab_kernel<N, double>, zg_slab_smem<N, double>(), slab_device);
+  if (e == cudaSuccess) e = allow_smem(zg_chain_kernel<N, double>, zg_chain_smem<double>(), chain_device);
+  if (e != cudaSuccess) return e;
+  e = launch_zg(zg_slab_kernel<N, double>, gd.rg_n[k], zg_slab_smem<N, double>(), first, st, m, v, fac, r,
                             z, gd.chain, done, zerr);
   if (e != cudaSuccess) return e;
   e = launch_zg(zg_chain_kernel<N, double>, gd.pk_n[k], zg_chain_smem<double>(), true, st, m, v, fac, gd.chain, done);
