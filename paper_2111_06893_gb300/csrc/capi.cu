@@ -868,7 +868,6 @@ tn_status tn_build_mesh(tn_ctx *c, const tn_mesh_desc *d) {
   m.layer_c = nullptr;
   m.layer_c32 = nullptr;
   c->trace_entries = (size_t)tn_trace_entries(hm.N) * hm.E;
-  m.penC32 = (float)hm.penC;
   c->ndof = (size_t)3 * hm.N * hm.N * hm.N * hm.E;
   c->have_mesh = true;
   return TN_OK;
@@ -1104,7 +1103,7 @@ tn_status tn_batch_set(tn_ctx *c, int i, const tn_mesh_desc *d, int n_mat, const
   if (e != cudaSuccess) return cuda_fail(e, "uploading a batch instance");
   DevMesh &m = q.dm;
   m.N = hm.N; m.p = hm.p; m.E = hm.E; m.ncol = hm.ncol; m.nslab = hm.nslab; m.n_layers = hm.n_layers;
-  m.bc_side = hm.bc_side; m.bc_bottom = hm.bc_bottom; m.penC = hm.penC; m.penC32 = (float)hm.penC;
+  m.bc_side = hm.bc_side; m.bc_bottom = hm.bc_bottom; m.penC = hm.penC;
   tab.point(m, q.tables);
   m.layer_c = (const double *)(q.tables + lc);
   m.layer_c32 = (const float *)(q.tables + lc32);

@@ -57,7 +57,6 @@ struct DevMesh {
   const float *colgeo32 = nullptr;
   const float *slabgeo32 = nullptr;
   const float *layer_c32 = nullptr;
-  float penC32 = 0.0f;
   // forward-mode seeds for derivative kernels (nullptr: no dependence)
   const double *d_slabdz = nullptr;  // [nslab][N]: d(dz/dzeta)/dtheta at each node
   const double *d_layer_c = nullptr;  // [n_layers][3]: d(c11, c12, c44)/dtheta

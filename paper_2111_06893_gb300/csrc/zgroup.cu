@@ -98,10 +98,10 @@ __device__ __forceinline__ void warp_allsum3(float &a, float &b, float &c) {
 
 // z = A_GG^{-1} r on group grp by the slot of G warps starting at warp w0;
 // line li of the group is warp w0 + li, its rows (a, k) lanes a N + k < 3N:
-//   forward   y_s = Linv_s (r_s - O_{s-1}^float w_{s-1}),  w_s = Linv_s^float y_s
-//   backward  x_s = Linv_s^float (y_s - Linv_s O_s x_{s+1}) = w_s - W_s v_{s+1}
-// (v: six numbers per line, x_{s+1}(b, N - 1) and X^float x_{s+1}).  The forward
-// step forms w_s = S_s^{-1} b_s, b_s = r_s - O_{s-1}^float w_{s-1}, in one
+//   forward   y_s = Linv_s (r_s - O_{s-1}^T w_{s-1}),  w_s = Linv_s^T y_s
+//   backward  x_s = Linv_s^T (y_s - Linv_s O_s x_{s+1}) = w_s - W_s v_{s+1}
+// (v: six numbers per line, x_{s+1}(b, N - 1) and X^T x_{s+1}).  The forward
+// step forms w_s = S_s^{-1} b_s, b_s = r_s - O_{s-1}^T w_{s-1}, in one
 // symmetric product, and r.z = sum_s |y_s|^2 = sum_s b_s . w_s.  O in its
 // factored form acts line by line (it is block diagonal over the lines), so
 // its products are warp shuffles and warp sums; S_s^{-1} b_s and W_s v cross
@@ -247,7 +247,7 @@ __device__ __forceinline__ void zp_slot(int grp, int w0, int mncol, int S, const
     if (act && s + 2 < S) r1 = r[gidx(s + 2)];
     rr += rv * rv;
     float bv = rv;
-    if (s > 0) {  // bv -= (O_{s-1}^float w_{s-1})_t, line by line
+    if (s > 0) {  // bv -= (O_{s-1}^T w_{s-1})_t, line by line
       const float x0 = XY[0], x1 = XY[1], x2 = XY[2];
       float s0 = act ? XY[4] * w : 0.0f, s1 = act ? XY[5] * w : 0.0f, s2 = act ? XY[6] * w : 0.0f;
       warp_allsum3(s0, s1, s2);
@@ -258,13 +258,13 @@ __device__ __forceinline__ void zp_slot(int grp, int w0, int mncol, int S, const
     }
     if (act) vb(par)[lt] = bv;
     sync();
-    w = symrow(Ls, vb(par));  // w_s = S_s^{-1} bv = Linv_s^float y_s
+    w = symrow(Ls, vb(par));  // w_s = S_s^{-1} bv = Linv_s^T y_s
     if (!act) w = 0.0f;
     rz += bv * w;             // |y_s|^2
     if (act) z[gidx(s)] = w;  // read back by the backward sweep
   }
   // backward sweep: x_{S-1} = w_{S-1} (already in z), then
-  // x_s = w_s - W_s v_{s+1}, v per line: x_{s+1}(b, N - 1) and X^float x_{s+1}
+  // x_s = w_s - W_s v_{s+1}, v per line: x_{s+1}(b, N - 1) and X^T x_{s+1}
   if (!bad) {
     float x = w;
     float w1 = (act && S > 1) ? z[gidx(S - 2)] : 0.0f;
@@ -519,19 +519,19 @@ int zg_slabs(int N, int G) {
   return by_rows < 1 ? 1 : std::min(by_rows, by_room);
 }
 // two stages, the vector twice over (rows read it at t + m), the products, two rows of D
-template <int N, typename T>
-constexpr size_t zg_slab_smem() { return sizeof(T) * (size_t)(2 * zg_srec(12 * N, 4) + 3 * kZgThreads + 2 * N); }
+template <int N>
+constexpr size_t zg_slab_smem() { return sizeof(double) * (size_t)(2 * zg_srec(12 * N, 4) + 3 * kZgThreads + 2 * N); }
 
 // row t of S^{-1} v from the circulant diagonals; v repeated: v[MG + i] = v[i]
-template <int MG, typename T>
-__device__ __forceinline__ T circ_row(const T *__restrict__ A, const T *__restrict__ v, int t) {
+template <int MG>
+__device__ __forceinline__ double circ_row(const double *__restrict__ A, const double *__restrict__ v, int t) {
   constexpr int H = (MG - 1) / 2;
-  const T *const At = A + t, *const vt = v + t;
-  T a0 = At[0] * vt[0], a1 = T(0), a2 = T(0), a3 = T(0);
+  const double *const At = A + t, *const vt = v + t;
+  double a0 = At[0] * vt[0], a1 = 0.0, a2 = 0.0, a3 = 0.0;
 #pragma unroll
   for (int m = 1; m <= H; ++m) {
     const int back = t < m ? MG : 0;
-    const T f = At[m * MG], b = At[m * MG - m + back];
+    const double f = At[m * MG], b = At[m * MG - m + back];
     if (m & 1) {
       a1 += f * vt[m];
       a2 += b * vt[MG - m];
@@ -544,22 +544,22 @@ __device__ __forceinline__ T circ_row(const T *__restrict__ A, const T *__restri
   return (a0 + a1) + (a2 + a3);
 }
 
-template <int N, int G, typename T>
-__device__ __forceinline__ void zg_slab(const DevMesh &m1, const ZgView &v, const int4 &rg, const T *__restrict__ fac,
-                                        const T *r0, T *__restrict__ z0, T *__restrict__ chain,
-                                        T *__restrict__ stage, unsigned long long *bars, const int *done,
+template <int N, int G>
+__device__ __forceinline__ void zg_slab(const DevMesh &m1, const ZgView &v, const int4 &rg,
+                                        const double *__restrict__ fac, const double *r0, double *__restrict__ z0, double *__restrict__ chain,
+                                        double *__restrict__ stage, unsigned long long *bars, const int *done,
                                         TnWait *__restrict__ err) {
   using Z = ZgSlab<N, G>;
   constexpr int M = Z::M, MG = Z::MG, C6 = Z::C6, SREC = Z::SREC, SL = Z::SL, LC = pad4(zg_circ(MG));
   constexpr int N2 = N * N, n = N * N2, ROOM = zg_srec(12 * N, 4);
   static_assert(SL * MG <= kZgThreads, "rows");
-  T *const vb = stage + 2 * ROOM, *const av = vb + 2 * kZgThreads, *const dl = av + kZgThreads;
+  double *const vb = stage + 2 * ROOM, *const av = vb + 2 * kZgThreads, *const dl = av + kZgThreads;
   const int tid = threadIdx.x, grp = rg.x, s0 = rg.y, s1 = rg.z;
   const ZgGroup q = zg_where(m1, v, grp);
-  const T *const src = fac + v.fac[grp];
+  const double *const src = fac + v.fac[grp];
   auto issue = [&](int s) {  // the stage of slabs s ..: thread 0
     const int i = (s - s0) / SL, b = i & 1;
-    const unsigned bytes = (unsigned)(min(SL, s1 - s) * SREC * sizeof(T));
+    const unsigned bytes = (unsigned)(min(SL, s1 - s) * SREC * sizeof(double));
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     mbar_expect(bars + b, bytes);
     bulk_g2s(stage + b * ROOM, src + (size_t)s * SREC, bytes, bars + b);
@@ -574,18 +574,18 @@ __device__ __forceinline__ void zg_slab(const DevMesh &m1, const ZgView &v, cons
   const int lid = zg_line(v.lines[grp], li), col = lid / N2, qn = lid - col * N2;
   const bool row = sl < SL;
   const size_t gs = (size_t)q.ncol * 3 * n, g0 = q.off + ((size_t)col * 3 + a) * n + (size_t)k * N2 + qn;
-  T *const ch = chain + v.chain[grp];
+  double *const ch = chain + v.chain[grp];
   const unsigned long long lim = wait_limit(err);
   if (tid < 2 * N) {  // D(0, k), k != 0, and D(N-1, k), k != N - 1; zero at the face node itself
     const int kk = tid < N ? tid : tid - N;
-    dl[tid] = tid == 0 || tid == 2 * N - 1 ? T(0) : (T)c_lgl_zg.D[N][(tid < N ? 0 : (N - 1) * N) + kk];
+    dl[tid] = tid == 0 || tid == 2 * N - 1 ? 0.0 : c_lgl_zg.D[N][(tid < N ? 0 : (N - 1) * N) + kk];
   }
   __syncthreads();  // the barriers are initialised
   grid_wait();
   r0 = after_wait(r0);
   done = after_wait(done);
   const bool skip = done && *done;
-  T rn = row && !skip && s0 + sl < s1 ? r0[g0 + (size_t)(s0 + sl) * gs] : T(0);
+  double rn = row && !skip && s0 + sl < s1 ? r0[g0 + (size_t)(s0 + sl) * gs] : 0.0;
   for (int s = s0; s < s1; s += SL) {
     const int i = (s - s0) / SL, b = i & 1;
     const bool on = row && s + sl < s1;
@@ -600,10 +600,10 @@ __device__ __forceinline__ void zg_slab(const DevMesh &m1, const ZgView &v, cons
     if (skip) return;
     if (tid == 0 && s + SL < s1) issue(s + SL);
     if (s + SL >= s1) grid_trigger();
-    rn = row && s + SL + sl < s1 ? r0[g0 + (size_t)(s + SL + sl) * gs] : T(0);
-    const T *A = stage + b * ROOM;
+    rn = row && s + SL + sl < s1 ? r0[g0 + (size_t)(s + SL + sl) * gs] : 0.0;
+    const double *A = stage + b * ROOM;
     if (on) {
-      const T w = circ_row<MG, T>(A + sl * SREC, vb + sl * 2 * MG, t);
+      const double w = circ_row<MG>(A + sl * SREC, vb + sl * 2 * MG, t);
       z0[g0 + (size_t)(s + sl) * gs] = w;
       av[tid] = w;
     }
@@ -616,12 +616,12 @@ __device__ __forceinline__ void zg_slab(const DevMesh &m1, const ZgView &v, cons
       const bool bottom = e6 >= 3;  // d (the top face) or c (the bottom face, k = 0)
       const int ec = bottom ? e6 - 3 : e6;
       if (s + es < s1) {
-        const T *w = av + es * MG + el * M, *C = A + es * SREC + LC + 16 * el, *wc = w + ec * N;
-        const T *D = dl + (bottom ? 0 : N), *X3 = C + 6 + ec;
-        T e = T(0);
+        const double *w = av + es * MG + el * M, *C = A + es * SREC + LC + 16 * el, *wc = w + ec * N;
+        const double *D = dl + (bottom ? 0 : N), *X3 = C + 6 + ec;
+        double e = 0.0;
 #pragma unroll
         for (int kk = 0; kk < N; ++kk) e += D[kk] * wc[kk];
-        T *const o = ch + (size_t)(s + es) * 2 * C6 + 6 * el + (bottom ? 0 : C6) + ec;
+        double *const o = ch + (size_t)(s + es) * 2 * C6 + 6 * el + (bottom ? 0 : C6) + ec;
         if (bottom) {
           o[0] = C[ec] * e;
           o[3] = wc[0];
@@ -634,16 +634,17 @@ __device__ __forceinline__ void zg_slab(const DevMesh &m1, const ZgView &v, cons
   }
 }
 
-template <int N, typename T>
-__global__ void __launch_bounds__(kZgThreads, sizeof(T) == 4 ? 7 : 3)
-zg_slab_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, const T *__restrict__ r,
-               T *__restrict__ z, T *__restrict__ chain, const int *__restrict__ done, TnWait *__restrict__ err) {
+template <int N>
+__global__ void __launch_bounds__(kZgThreads, 3)
+zg_slab_kernel(const DevMesh m1, const ZgView v, const double *__restrict__ fac, const double *__restrict__ r,
+               double *__restrict__ z, double *__restrict__ chain, const int *__restrict__ done,
+               TnWait *__restrict__ err) {
   extern __shared__ __align__(16) unsigned char zsm[];
   __shared__ __align__(8) unsigned long long bars[2];
-  T *const stage = reinterpret_cast<T *>(zsm);
+  double *const stage = reinterpret_cast<double *>(zsm);
   const int4 rg = v.ranges[blockIdx.x];
   switch (zg_size(v.lines[rg.x])) {
-#define TN_CASE(GG) case GG: zg_slab<N, GG, T>(m1, v, rg, fac, r, z, chain, stage, bars, done, err); break;
+#define TN_CASE(GG) case GG: zg_slab<N, GG>(m1, v, rg, fac, r, z, chain, stage, bars, done, err); break;
     TN_CASE(1) TN_CASE(2) TN_CASE(3) TN_CASE(4)
 #undef TN_CASE
   }
@@ -654,8 +655,7 @@ zg_slab_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, cons
 // go by blocks of kZgBlock, so that shared memory does not depend on their
 // number.  One warp runs the chains, the others bring K.
 constexpr int kZgChLine = pad4(12 * (kZgBlock + 1));  // chain entries of a block and the slab before or after it, per line
-template <typename T>
-constexpr size_t zg_chain_smem() { return sizeof(T) * 4 * (size_t)(kZgChLine + kZgKWarp); }
+constexpr size_t zg_chain_smem() { return sizeof(double) * 4 * (size_t)(kZgChLine + kZgKWarp); }
 
 // the group this warp works on: its first warp w0 in the CTA, its size (0: idle)
 __device__ __forceinline__ int zg_slot(const ZgView &v, int &w0, int &G) {
@@ -679,19 +679,19 @@ __device__ __forceinline__ int zg_slot(const ZgView &v, int &w0, int &G) {
 }
 
 // K records brought through registers: load issues, store lands them
-template <int G, typename T>
+template <int G>
 struct KStage {
   static constexpr int KP = zg_kpart(G), KREC = zg_krec(G), SLK = G * kZgKWarp / KP;  // slabs per stage
   static constexpr int PER = (SLK * KP + 32 * G - 1) / (32 * G);
-  T v[PER];
-  __device__ __forceinline__ void load(const T *__restrict__ k, int cnt, int lt) {
+  double v[PER];
+  __device__ __forceinline__ void load(const double *__restrict__ k, int cnt, int lt) {
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
       const int at = i * 32 * G + lt, s = at / KP;
-      v[i] = at < cnt * KP ? k[(size_t)s * KREC + (at - s * KP)] : T(0);
+      v[i] = at < cnt * KP ? k[(size_t)s * KREC + (at - s * KP)] : 0.0;
     }
   }
-  __device__ __forceinline__ void store(T *__restrict__ ks, int cnt, int lt) const {
+  __device__ __forceinline__ void store(double *__restrict__ ks, int cnt, int lt) const {
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
       const int at = i * 32 * G + lt;
@@ -703,10 +703,10 @@ struct KStage {
 // lanes per row of a chain step (112 -> 105 us at 2.0 M unknowns, p = 6): the six or twelve rows of small groups leave
 // lanes over, and an FP64 instruction costs the same with a few lanes on
 __host__ __device__ constexpr int chain_parts(int G) { return G == 1 ? 4 : (G == 2 ? 2 : 1); }
-template <int G, typename T, typename KF, typename VF>
-__device__ __forceinline__ T chain_dot(T a0, KF k, VF v, int part) {
+template <int G, typename KF, typename VF>
+__device__ __forceinline__ double chain_dot(double a0, KF k, VF v, int part) {
   constexpr int P = chain_parts(G), C6 = 6 * G, STEPS = (C6 + P - 1) / P;
-  T a1 = T(0), a2 = T(0);
+  double a1 = 0.0, a2 = 0.0;
 #pragma unroll
   for (int i = 0; i < STEPS; ++i) {
     const int j = i * P + part;
@@ -719,15 +719,15 @@ __device__ __forceinline__ T chain_dot(T a0, KF k, VF v, int part) {
   return a0;
 }
 
-template <int G, typename T>
-__device__ __forceinline__ void zg_chain(int S, int w0, const T *__restrict__ fk, T *chain,
-                                         T *__restrict__ sm) {
+template <int G>
+__device__ __forceinline__ void zg_chain(int S, int w0, const double *__restrict__ fk, double *chain,
+                                         double *__restrict__ sm) {
   constexpr int C6 = 6 * G, C12 = 12 * G, LD = zg_ld(G), NT = 32 * G;
-  constexpr int KP = zg_kpart(G), KREC = zg_krec(G), SLK = KStage<G, T>::SLK;
+  constexpr int KP = zg_kpart(G), KREC = zg_krec(G), SLK = KStage<G>::SLK;
   const int lt = threadIdx.x - 32 * w0, row = lt / chain_parts(G), part = lt % chain_parts(G);
-  T *const ch = sm, *const ks = ch + G * kZgChLine;
+  double *const ch = sm, *const ks = ch + G * kZgChLine;
   const int nblk = (S + kZgBlock - 1) / kZgBlock;
-  KStage<G, T> K;
+  KStage<G> K;
   // forward: slabs b0 .. b0 + nb - 1 at ch[(1 + i) C12], slab b0 - 1 at ch[0]
   for (int b0 = 0; b0 < S; b0 += kZgBlock) {
     const int nb = min(kZgBlock, S - b0), k0 = max(1, b0), k1 = min(b0 + nb, S - 1);  // steps k0 .. k1 - 1
@@ -746,10 +746,10 @@ __device__ __forceinline__ void zg_chain(int S, int w0, const T *__restrict__ fk
       slot_sync<G>(w0);
       if (lt < 32)
         for (int i = 0; i < cnt; ++i) {  // g_s = c_s - K_s g_{s-1}
-          T *const g = ch + (s0 + i - b0) * C12;
+          double *const g = ch + (s0 + i - b0) * C12;
           if (row < C6) {
-            const T *Kr = ks + i * KP + row * LD;
-            const T w = chain_dot<G, T>(part == 0 ? g[C12 + row] : T(0), [&](int j) { return Kr[j]; },
+            const double *Kr = ks + i * KP + row * LD;
+            const double w = chain_dot<G>(part == 0 ? g[C12 + row] : 0.0, [&](int j) { return Kr[j]; },
                                         [&](int j) { return g[j]; }, part);
             if (part == 0) g[C12 + row] = w;
           }
@@ -761,8 +761,8 @@ __device__ __forceinline__ void zg_chain(int S, int w0, const T *__restrict__ fk
     for (int id = lt; id < nb * C6; id += NT) {
       const int i = id / C6, j = id - i * C6, s = b0 + i;
       if (s == 0) continue;
-      const T *H = fk + (size_t)s * KREC + KP + j, *g = ch + i * C12;
-      T a0 = ch[(1 + i) * C12 + C6 + j], a1 = T(0), a2 = T(0);
+      const double *H = fk + (size_t)s * KREC + KP + j, *g = ch + i * C12;
+      double a0 = ch[(1 + i) * C12 + C6 + j], a1 = 0.0, a2 = 0.0;
 #pragma unroll
       for (int p = 0; p < C6; p += 3) {
         a0 -= H[p * C6] * g[p];
@@ -784,7 +784,7 @@ __device__ __forceinline__ void zg_chain(int S, int w0, const T *__restrict__ fk
     const int k1 = blk == nblk - 1 ? S - 2 : b0 + nb - 1, k0 = max(1, b0);  // steps k1 down to k0
     if (blk < nblk - 1) {
       slot_sync<G>(w0);
-      const T f = lt < C6 ? ch[C12 + C6 + lt] : T(0);
+      const double f = lt < C6 ? ch[C12 + C6 + lt] : 0.0;
       slot_sync<G>(w0);
       for (int id = lt; id < nb * C12; id += NT) ch[C12 + id] = chain[(size_t)b0 * C12 + id];
       slot_sync<G>(w0);
@@ -800,11 +800,11 @@ __device__ __forceinline__ void zg_chain(int S, int w0, const T *__restrict__ fk
       slot_sync<G>(w0);
       if (lt < 32)
         for (int s = hi; s >= lo; --s) {  // f_s = e_s - K_s^T f_{s+1}
-          const T *f = s + 1 == b0 + nb ? ch + C6 : ch + (s - b0 + 2) * C12 + C6;
+          const double *f = s + 1 == b0 + nb ? ch + C6 : ch + (s - b0 + 2) * C12 + C6;
           if (row < C6) {
-            T *const o = ch + (s - b0 + 1) * C12 + C6 + row;
-            const T *Kc = ks + (s - lo) * KP + row;
-            const T w = chain_dot<G, T>(part == 0 ? *o : T(0), [&](int j) { return Kc[j * LD]; },
+            double *const o = ch + (s - b0 + 1) * C12 + C6 + row;
+            const double *Kc = ks + (s - lo) * KP + row;
+            const double w = chain_dot<G>(part == 0 ? *o : 0.0, [&](int j) { return Kc[j * LD]; },
                                         [&](int j) { return f[j]; }, part);
             if (part == 0) *o = w;
           }
@@ -816,9 +816,9 @@ __device__ __forceinline__ void zg_chain(int S, int w0, const T *__restrict__ fk
   }
 }
 
-template <int N, typename T>
+template <int N>
 __global__ void __launch_bounds__(kZgThreads)
-zg_chain_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, T *__restrict__ chain,
+zg_chain_kernel(const DevMesh m1, const ZgView v, const double *__restrict__ fac, double *__restrict__ chain,
                 const int *__restrict__ done) {
   extern __shared__ __align__(16) unsigned char zsm[];
   int w0, G;
@@ -827,32 +827,32 @@ zg_chain_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, T *
   done = after_wait(done);
   chain = after_wait(chain);
   if ((done && *done) || grp < 0) return;
-  T *const sm = reinterpret_cast<T *>(zsm) + (size_t)w0 * (kZgChLine + kZgKWarp);
+  double *const sm = reinterpret_cast<double *>(zsm) + (size_t)w0 * (kZgChLine + kZgKWarp);
   const int S = zg_where(m1, v, grp).S;
-  const T *const f = fac + v.fac[grp];
-  T *const c = chain + v.chain[grp];
+  const double *const f = fac + v.fac[grp];
+  double *const c = chain + v.chain[grp];
   switch (G) {
-#define TN_CASE(GG) case GG: zg_chain<GG, T>(S, w0, f + zg_koff(3 * N * GG, GG, S), c, sm); break;
+#define TN_CASE(GG) case GG: zg_chain<GG>(S, w0, f + zg_koff(3 * N * GG, GG, S), c, sm); break;
     TN_CASE(1) TN_CASE(2) TN_CASE(3) TN_CASE(4)
 #undef TN_CASE
   }
 }
 
 // ---- the correction of every slab, r.z and r.r
-template <int N, int G, typename T>
-__device__ __forceinline__ void zg_final(const DevMesh &m1, const ZgView &v, const int4 &rg, const T *__restrict__ fac,
-                                         const T *r0, T *z0, const T *chain,
-                                         T *__restrict__ qv, T &rz, T &rr) {
+template <int N, int G>
+__device__ __forceinline__ void zg_final(const DevMesh &m1, const ZgView &v, const int4 &rg,
+                                         const double *__restrict__ fac, const double *r0, double *z0, const double *chain,
+                                         double *__restrict__ qv, double &rz, double &rr) {
   using Z = ZgSlab<N, G>;
   constexpr int M = Z::M, MG = Z::MG, MGP = Z::MGP, C6 = Z::C6, C12 = 2 * C6, SL = Z::SL, N2 = N * N, n = N * N2;
   const int tid = threadIdx.x, grp = rg.x, s0 = rg.y, s1 = rg.z;
   const ZgGroup q = zg_where(m1, v, grp);
   const int S = q.S;
-  const T *const qw = fac + v.fac[grp] + zg_qoff(MG, G, S);
-  const T *const ch = chain + v.chain[grp];
+  const double *const qw = fac + v.fac[grp] + zg_qoff(MG, G, S);
+  const double *const ch = chain + v.chain[grp];
   for (int id = tid; id < (s1 - s0) * C12; id += kZgThreads) {  // g_{s-1} | f_{s+1}
     const int i = id / C12, j = id - i * C12, s = s0 + i;
-    qv[id] = j < C6 ? (s > 0 ? ch[(size_t)(s - 1) * C12 + j] : T(0)) : (s + 1 < S ? ch[(size_t)(s + 1) * C12 + j] : T(0));
+    qv[id] = j < C6 ? (s > 0 ? ch[(size_t)(s - 1) * C12 + j] : 0.0) : (s + 1 < S ? ch[(size_t)(s + 1) * C12 + j] : 0.0);
   }
   __syncthreads();
   const int sl = tid / MG, t = tid - sl * MG, li = t / M, tl = t - li * M, a = tl / N, k = tl - a * N;
@@ -861,29 +861,29 @@ __device__ __forceinline__ void zg_final(const DevMesh &m1, const ZgView &v, con
   const size_t gs = (size_t)q.ncol * 3 * n, g0 = q.off + ((size_t)col * 3 + a) * n + (size_t)k * N2 + qn;
   for (int s = s0 + sl; s < s1; s += SL) {
     const size_t at = g0 + (size_t)s * gs;
-    const T *w = qw + (size_t)s * Z::QREC + t, *f = qv + (s - s0) * C12;
-    const T rv = r0[at];
-    T a0 = z0[at], a1 = T(0), a2 = T(0);
+    const double *w = qw + (size_t)s * Z::QREC + t, *f = qv + (s - s0) * C12;
+    const double rv = r0[at];
+    double a0 = z0[at], a1 = 0.0, a2 = 0.0;
 #pragma unroll
     for (int j = 0; j < C12; j += 3) {
       a0 -= w[j * MGP] * f[j];
       a1 -= w[(j + 1) * MGP] * f[j + 1];
       a2 -= w[(j + 2) * MGP] * f[j + 2];
     }
-    const T x = a0 + (a1 + a2);
+    const double x = a0 + (a1 + a2);
     z0[at] = x;
     rz += rv * x;
     rr += rv * rv;
   }
 }
 
-template <int N, typename T>
-__global__ void __launch_bounds__(kZgThreads, sizeof(T) == 4 ? 8 : 4)
-zg_final_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, const T *__restrict__ r,
-                T *__restrict__ z, const T *__restrict__ chain, double *__restrict__ part_rz,
+template <int N>
+__global__ void __launch_bounds__(kZgThreads, 4)
+zg_final_kernel(const DevMesh m1, const ZgView v, const double *__restrict__ fac, const double *__restrict__ r,
+                double *__restrict__ z, const double *__restrict__ chain, double *__restrict__ part_rz,
                 double *__restrict__ part_rr, const int *__restrict__ done, const PcgFold fold) {
   constexpr int QV = 12 * kZgChunks * kZgThreads / (3 * N);  // 12 g numbers of at most kZgChunks kZgThreads / (3 g N) slabs
-  __shared__ T qv[QV > 48 * kZgChunks ? QV : 48 * kZgChunks];
+  __shared__ double qv[QV > 48 * kZgChunks ? QV : 48 * kZgChunks];
   const int4 rg = v.ranges[blockIdx.x];
   const int G = zg_size(v.lines[rg.x]);
   grid_wait();
@@ -892,14 +892,14 @@ zg_final_kernel(const DevMesh m1, const ZgView v, const T *__restrict__ fac, con
   z = after_wait(z);
   chain = after_wait(chain);
   if (done && *done) return;
-  T rz = T(0), rr = T(0);
+  double rz = 0.0, rr = 0.0;
   switch (G) {
-#define TN_CASE(GG) case GG: zg_final<N, GG, T>(m1, v, rg, fac, r, z, chain, qv, rz, rr); break;
+#define TN_CASE(GG) case GG: zg_final<N, GG>(m1, v, rg, fac, r, z, chain, qv, rz, rr); break;
     TN_CASE(1) TN_CASE(2) TN_CASE(3) TN_CASE(4)
 #undef TN_CASE
   }
   if (part_rz) {  // FP64 sums of the rows' sums: warp 0 for r.z, warp 1 for r.r
-    __shared__ T ps[2][kZgThreads];
+    __shared__ double ps[2][kZgThreads];
     ps[0][threadIdx.x] = rz;
     ps[1][threadIdx.x] = rr;
     __syncthreads();
@@ -939,15 +939,15 @@ cudaError_t launch_f64(const DevMesh &m, const ZGroupDev &gd, int k, const doubl
   const ZgView v{gd.inst, gd.meshes, gd.dof_off, gd.lines, gd.fac64_off, gd.chain_off,
                  gd.packs + gd.pk_start[k], gd.ranges + gd.rg_start[k]};
   static int slab_device = -1, chain_device = -1;
-  cudaError_t e = allow_smem(zg_slab_kernel<N, double>, zg_slab_smem<N, double>(), slab_device);
-  if (e == cudaSuccess) e = allow_smem(zg_chain_kernel<N, double>, zg_chain_smem<double>(), chain_device);
+  cudaError_t e = allow_smem(zg_slab_kernel<N>, zg_slab_smem<N>(), slab_device);
+  if (e == cudaSuccess) e = allow_smem(zg_chain_kernel<N>, zg_chain_smem(), chain_device);
   if (e != cudaSuccess) return e;
-  e = launch_zg(zg_slab_kernel<N, double>, gd.rg_n[k], zg_slab_smem<N, double>(), first, st, m, v, fac, r,
+  e = launch_zg(zg_slab_kernel<N>, gd.rg_n[k], zg_slab_smem<N>(), first, st, m, v, fac, r,
                             z, gd.chain, done, zerr);
   if (e != cudaSuccess) return e;
-  e = launch_zg(zg_chain_kernel<N, double>, gd.pk_n[k], zg_chain_smem<double>(), true, st, m, v, fac, gd.chain, done);
+  e = launch_zg(zg_chain_kernel<N>, gd.pk_n[k], zg_chain_smem(), true, st, m, v, fac, gd.chain, done);
   if (e != cudaSuccess) return e;
-  return launch_zg(zg_final_kernel<N, double>, gd.rg_n[k], 0, true, st, m, v, fac, r, z, (const double *)gd.chain, prz,
+  return launch_zg(zg_final_kernel<N>, gd.rg_n[k], 0, true, st, m, v, fac, r, z, (const double *)gd.chain, prz,
                    prr, done, fold);
 }
 
@@ -993,29 +993,43 @@ cudaError_t launch_packed(const DevMesh &m, const ZGroupDev &gd, int k, int grid
 // The FP32 kernel is persistent: as many CTAs as fit at once, never more than
 // packs.  Four CTAs per SM run a pack fastest; seven (72 registers) take more
 // packs at once, which pays from three rounds of packs where it saves a third
-// of them (crystalline stack, p = 5, 4 -> 2 rounds: 442 -> 368 us; p = 5 at 324
-// columns, 5 -> 3: 174 -> 153).  Below that it is not worth it (p = 6, 993
-// packs, 2 -> 2 rounds: 116 -> 132; p = 5 at 81 columns, 2 -> 1: 62 -> 67), nor
-// with kernels of several degrees side by side (24 mirrors: 268 -> 276).
+// of them: with four against so, us: crystalline stack, p = 5, 4 -> 2 rounds
+// 442 -> 368; 12 slabs, p = 2, 576 columns, 3 -> 2 68 -> 52; p = 3, 900, 6 -> 4
+// 150 -> 120; p = 4, 324, 4 -> 2 98 -> 77; p = 5, 576, 9 -> 5 254 -> 214; p = 6,
+// whose shared memory holds six, 441, 9 -> 6 287 -> 260, 576, 12 -> 8 375 -> 343.
+// Below that it is not worth it (p = 6, 993 packs, 2 -> 2 rounds: 116 -> 132; p
+// = 5 at 81 columns, 2 -> 1: 62 -> 67), nor with kernels of several degrees
+// side by side (24 mirrors: 268 -> 276).  In rounds rather than packs the rule
+// turns off again where a round is left over (p = 6, 900 columns, 19 -> 13: 577
+// us with four, as before).  From p = 7 shared memory holds four.
 // grid_out: only compute the grid; else launch with it.
+template <int N>
+constexpr bool zp_more() { return 5 * (zp_smem<N>() + 1024) <= 228 * 1024; }
 template <int N>
 cudaError_t launch_f32(const DevMesh &m, const ZGroupDev &gd, int k, const float *fac, const float *r, float *z,
                        double *prz, double *prr, const int *done, TnWait *zerr, cudaStream_t st, bool first,
                        const PcgFold &fold, int *grid_out) {
   constexpr size_t sm = zp_smem<N>();
-  int four = 0, seven = 0;
-  cudaError_t err = packed_per_sm<N, 4>(sm, &four);
-  if (err == cudaSuccess) err = packed_per_sm<N, 7>(sm, &seven);
+  int per_sm = 0;
+  cudaError_t err = packed_per_sm<N, 4>(sm, &per_sm);
   if (err != cudaSuccess) return err;
   const int npk = gd.pk_n[k], sms = tn_sm_count();
-  auto rounds = [&](int per_sm) { return (npk + per_sm * sms - 1) / (per_sm * sms); };
-  const bool more = gd.npk == 1 && rounds(four) >= 3 && 3 * rounds(seven) <= 2 * rounds(four);
-  const int grid = std::min((more ? seven : four) * sms, npk);
+  bool more = false;
+  if constexpr (zp_more<N>()) {
+    int seven = 0;
+    err = packed_per_sm<N, 7>(sm, &seven);
+    if (err != cudaSuccess) return err;
+    auto rounds = [&](int per) { return (npk + per * sms - 1) / (per * sms); };
+    more = gd.npk == 1 && rounds(per_sm) >= 3 && 3 * rounds(seven) <= 2 * rounds(per_sm);
+    if (more) per_sm = seven;
+  }
+  const int grid = std::min(per_sm * sms, npk);
   if (grid_out) {
     *grid_out = grid;
     return cudaSuccess;
   }
-  if (more) return launch_packed<N, 7>(m, gd, k, grid, sm, fac, r, z, prz, prr, done, zerr, st, first, fold);
+  if constexpr (zp_more<N>())
+    if (more) return launch_packed<N, 7>(m, gd, k, grid, sm, fac, r, z, prz, prr, done, zerr, st, first, fold);
   return launch_packed<N, 4>(m, gd, k, grid, sm, fac, r, z, prz, prr, done, zerr, st, first, fold);
 }
 
