@@ -72,25 +72,6 @@ template <typename T> __device__ __forceinline__ T fm(T a, T b, T c);
 template <> __device__ __forceinline__ double fm(double a, double b, double c) { return fma(a, b, c); }
 template <> __device__ __forceinline__ float fm(float a, float b, float c) { return fmaf(a, b, c); }
 
-// a thread's part of u . A u: its products in threes (one node, one face
-// position), the threes summed with the rounding errors kept (Knuth's two-sum)
-// in FP32, so that single precision adds no more than the three products it
-// always did; per node 6 additions, nothing beside the node's work
-template <typename T> struct DotSum {
-  T sum = T(0);
-  __device__ __forceinline__ void add(T v) { sum += v; }
-  __device__ __forceinline__ double value() const { return (double)sum; }
-};
-template <> struct DotSum<float> {
-  float sum = 0.0f, err = 0.0f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = sum + v, b = t - sum;
-    err += (sum - (t - b)) + (v - b);
-    sum = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)sum + (double)err; }
-};
-
 // out = D v (TR = 0) or D^T v (TR = 1) along one line of N nodes
 template <int N, int TR, typename T>
 __device__ __forceinline__ void line_eo(const T v[N], T out[N]) {
@@ -281,8 +262,8 @@ __host__ __device__ constexpr size_t apply_smem() {
 // face position (t1, t2) = (a, b) of all six faces -- the two ends of its
 // own lines -- so that jumps and face terms stay in registers.
 template <int N, typename T>
-__device__ __forceinline__ double apply_body(const ElemI<T> &E, T *__restrict__ sm, int q, bool act, bool want_dot,
-                                             T (&z)[3][N]) {
+__device__ __forceinline__ T apply_body(const ElemI<T> &E, T *__restrict__ sm, int q, bool act, bool want_dot,
+                                        T (&z)[3][N]) {
   constexpr int N2 = N * N, n = N * N2, NP = N | 1, PL = N * NP, CN = N * PL;
   T *const g0 = sm, *const g1 = sm + 3 * CN, *const sf = sm + 6 * CN, *const sc = sf + 12 * N2;
   const int a = q % N, b = q / N;
@@ -368,8 +349,7 @@ __device__ __forceinline__ double apply_body(const ElemI<T> &E, T *__restrict__ 
   // ---- faces: traction and penalty at position (t1, t2) = (a, b)
   const ApplyTabs<T> &tb = tabs<T>(N);
   const T lf = tb.whalf;
-  T surf[6][3];
-  DotSum<T> dot;
+  T surf[6][3], dot = T(0);
   const T *const dzs = E.sg + SG_DZ * N, *const idzs = E.sg + SG_IDZ * N;
   const Moduli<T> C = E.C;
   Map2<T> J = {T(0), T(0), T(0), T(0)};  // of the pencil's node
@@ -398,10 +378,8 @@ __device__ __forceinline__ double apply_body(const ElemI<T> &E, T *__restrict__ 
 #pragma unroll
         for (int c = 0; c < 3; ++c) E.tr[(f * 3 + c) * N2 + q] = tw[c];
         if (want_dot) {
-          T d = T(0);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) d = fm(tw[c], E.u[c * n + b * N2 + qf] - jump[f][c], d);
-          dot.add(d);
+          for (int c = 0; c < 3; ++c) dot = fm(tw[c], E.u[c * n + b * N2 + qf] - jump[f][c], dot);
         }
       }
     }
@@ -426,10 +404,8 @@ __device__ __forceinline__ double apply_body(const ElemI<T> &E, T *__restrict__ 
 #pragma unroll
         for (int c = 0; c < 3; ++c) E.tr[(f * 3 + c) * N2 + q] = tw[c];
         if (want_dot) {
-          T d = T(0);
 #pragma unroll
-          for (int c = 0; c < 3; ++c) d = fm(tw[c], E.u[c * n + k * N2 + q] - jump[f][c], d);
-          dot.add(d);
+          for (int c = 0; c < 3; ++c) dot = fm(tw[c], E.u[c * n + k * N2 + q] - jump[f][c], dot);
         }
       }
 #pragma unroll
@@ -499,7 +475,6 @@ __device__ __forceinline__ double apply_body(const ElemI<T> &E, T *__restrict__ 
   }
   __syncthreads();
   if (act) {
-    T d[N];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -507,14 +482,10 @@ __device__ __forceinline__ double apply_body(const ElemI<T> &E, T *__restrict__ 
         const int at = c * CN + k * PL + row;
         const T yv = z[c][k] + (g0[at] + g1[at]);
         E.y[c * n + k * N2 + q] = yv;
-        if (want_dot) d[k] = fm(yv, E.u[c * n + k * N2 + q], c == 0 ? T(0) : d[k]);
+        if (want_dot) dot = fm(yv, E.u[c * n + k * N2 + q], dot);
       }
-    if (want_dot) {
-#pragma unroll
-      for (int k = 0; k < N; ++k) dot.add(d[k]);
-    }
   }
-  return dot.value();
+  return dot;
 }
 
 // ---- few elements: three threads per pencil, one per component
@@ -531,8 +502,8 @@ __device__ __forceinline__ double apply_body(const ElemI<T> &E, T *__restrict__ 
 // (a, b, k = c, c + 3, ..).  z: the zeta line of u.  Returns this thread's
 // part of u . A u.
 template <int N, typename T>
-__device__ __forceinline__ double apply_body_small(const ElemI<T> &E, T *__restrict__ sm, int c, int q, bool act,
-                                                   bool want_dot, T (&z)[N]) {
+__device__ __forceinline__ T apply_body_small(const ElemI<T> &E, T *__restrict__ sm, int c, int q, bool act, bool want_dot,
+                                        T (&z)[N]) {
   constexpr int N2 = N * N, n = N * N2, NP = N | 1, PL = N * NP, CN = N * PL;
   T *const g0 = sm, *const g1 = sm + 3 * CN, *const g2 = sm + 6 * CN, *const js = sm + 9 * CN, *const sc = js + 18 * N2;
   const int a = q % N, b = q / N;
@@ -586,8 +557,7 @@ __device__ __forceinline__ double apply_body_small(const ElemI<T> &E, T *__restr
   // ---- the two faces across direction c: traction and penalty at (a, b)
   const ApplyTabs<T> &tb = tabs<T>(N);
   const T lf = tb.whalf;
-  DotSum<T> dot;
-  T jf[2][3], wab = T(0);
+  T dot = T(0), jf[2][3], wab = T(0);
   const T *const dzs = E.sg + SG_DZ * N, *const idzs = E.sg + SG_IDZ * N;
   const Moduli<T> C = E.C;
   if (act) {
@@ -624,10 +594,8 @@ __device__ __forceinline__ double apply_body_small(const ElemI<T> &E, T *__restr
 #pragma unroll
         for (int l = 0; l < 3; ++l) E.tr[(f * 3 + l) * N2 + q] = tw[l];
         if (want_dot) {
-          T d = T(0);
 #pragma unroll
-          for (int l = 0; l < 3; ++l) d = fm(tw[l], E.u[l * n + kf * N2 + qf] - jf[e][l], d);
-          dot.add(d);
+          for (int l = 0; l < 3; ++l) dot = fm(tw[l], E.u[l * n + kf * N2 + qf] - jf[e][l], dot);
         }
       }
     }
@@ -695,19 +663,15 @@ __device__ __forceinline__ double apply_body_small(const ElemI<T> &E, T *__restr
   }
   __syncthreads();
   if (act) {
-    T d = T(0);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
       const int at = row + k * PL;
       const T yv = z[k] + (g0[at] + g1[at]);
       E.y[c * n + k * N2 + q] = yv;
-      if (want_dot) {
-        d = fm(yv, E.u[c * n + k * N2 + q], k % 3 == 0 ? T(0) : d);
-        if (k % 3 == 2 || k == N - 1) dot.add(d);
-      }
+      if (want_dot) dot = fm(yv, E.u[c * n + k * N2 + q], dot);
     }
   }
-  return dot.value();
+  return dot;
 }
 
 // The alpha step of a PCG iteration folded into the operator apply: once
@@ -806,7 +770,7 @@ __device__ __forceinline__ void apply_cta(const DevMesh &m1, const DevMesh *__re
   ue = after_wait(ue);
   if (fold_skip(fold)) return;
   const ElemI<T> &E = info[act ? el : 0];
-  double dot;
+  T dott;
   if constexpr (MODE != AM_PENCIL) {
     T z[N];
     if (act) {
@@ -814,7 +778,7 @@ __device__ __forceinline__ void apply_cta(const DevMesh &m1, const DevMesh *__re
       for (int k = 0; k < N; ++k) z[k] = ue[k * N2];
     }
     __syncthreads();
-    dot = apply_body_small<N, T>(E, reinterpret_cast<T *>(info + EB) + (size_t)(act ? el : 0) * apply_small_words<N>(),
+    dott = apply_body_small<N, T>(E, reinterpret_cast<T *>(info + EB) + (size_t)(act ? el : 0) * apply_small_words<N>(),
                                   cc, q, act, partial != nullptr, z);
   } else {
     T z[3][N];
@@ -826,10 +790,11 @@ __device__ __forceinline__ void apply_cta(const DevMesh &m1, const DevMesh *__re
     }
     __syncthreads();
     T *sm = reinterpret_cast<T *>(info + EB) + (size_t)(act ? el : 0) * apply_elem_words<N>();
-    dot = apply_body<N, T>(E, sm, q, act, partial != nullptr, z);
+    dott = apply_body<N, T>(E, sm, q, act, partial != nullptr, z);
   }
   if (partial) {
     __shared__ double red[NT / 32];
+    double dot = (double)dott;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
     if ((tid & 31) == 0) red[tid >> 5] = dot;
@@ -1096,6 +1061,7 @@ constexpr int kEnergyThreads = 256;
 template <int N>
 constexpr int energy_eb() { return kEnergyThreads / (N * N); }
 template <int N, bool SPLIT>
+  const bool early = add_early(a);
 constexpr size_t energy_smem(int eb) { return sizeof(double) * (size_t)eb * (SPLIT ? 9 : 6) * N * N * N; }
 
 // elements w0 .. of one mesh (meshes == nullptr: m1, element w) or of a batch
