@@ -1061,7 +1061,6 @@ constexpr int kEnergyThreads = 256;
 template <int N>
 constexpr int energy_eb() { return kEnergyThreads / (N * N); }
 template <int N, bool SPLIT>
-  const bool early = add_early(a);
 constexpr size_t energy_smem(int eb) { return sizeof(double) * (size_t)eb * (SPLIT ? 9 : 6) * N * N * N; }
 
 // elements w0 .. of one mesh (meshes == nullptr: m1, element w) or of a batch
