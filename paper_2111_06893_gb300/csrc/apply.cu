@@ -239,7 +239,8 @@ template <int N, int MODE>
 __host__ __device__ constexpr int apply_threads() {
   return MODE == AM_PENCIL ? kApplyThreads : (MODE == AM_SMALL ? (3 * N * N + 31) / 32 * 32 : kSmallBatchThreads);
 }
-bool apply_small(int E) { return E <= 8 * tn_sm_count(); }
+bool apply_small(int E, int sms) { return E <= 8 * sms; }
+bool apply_small(int E) { return apply_small(E, tn_sm_count()); }
 // shared memory of one element: the two lateral derivatives (the field is
 // staged where the xi derivatives go), rows of i padded to an odd pitch, the
 // zeta derivative at the lateral faces, and seven column tables
@@ -852,17 +853,26 @@ __host__ __device__ constexpr int surf_nodes() { return N * N * N - (N - 2) * (N
 constexpr int kAddThreads = 256;
 template <int N>
 __host__ __device__ constexpr int add_eb() { return kAddThreads * 4 / surf_nodes<N>(); }
-int add_elems(int most, int E) { return std::min(most, std::max(1, E / (2 * tn_sm_count()))); }
-// Whether the second launch lets the one after it start at once.  An apply
-// that starts while the one before still runs takes whatever slots are left,
-// so that a grid smaller than the GPU piles up on a few SMs (FP64, 216
-// elements, p = 4: 73 us an apply, 25 once the second launch ends first); one
-// of several CTAs per SM gains (FP32, 1944 elements, p = 6: 389 CTAs, 24.9 us
-// against 26.2; 2744 elements, p = 4: 275 CTAs, 20.7 against 18.9), but for a
-// batch's, whose CTAs differ (8 mirrors 31 against 24 us, 14: 49 against 43).
-// In a PCG iteration the launch after it is the preconditioner's.
-bool add_early(const ApplyArgs &a) {
-  return a.r || (a.m && !tn_apply_few(a.m->E) && tn_apply_parts(a.m->N, a.m->E) > 2 * tn_sm_count());
+int add_elems(int most, int E, int sms) { return std::min(most, std::max(1, E / (2 * sms))); }
+// Whether the second launch lets the one after it start at once (in a PCG
+// iteration, the preconditioner's: yes).  An apply that starts while the one
+// before still runs takes whatever slots are left: a grid that would spread over
+// the GPU piles up on a few SMs, one that fills it, or leaves most of it empty,
+// gains the start.  us an apply, FP64 / FP32 by itself, early against late:
+//   one element per CTA: 216 elements, p = 4: 56 / 7.0 against 25 / 7.2; 343 to
+//   512, p = 2, 3: 42 to 59 against 16 to 27; 8, p = 2: 14.6 against 15.6; 729,
+//   p = 8 (1165 threads per SM): 252.5 / 21.2 against 253.3 / 22.1
+//   pencils: 98 CTAs (p = 2, 2744 elements) 54.2 / 14.0 against 53.7 / 9.1; 275
+//   CTAs, p = 4: 164.7 / 20.6 against 165.6 / 19.4; 389, p = 6: 24.9 against 26.2
+//   batches (FP32, means over placements): 2 to 6 mirrors, few elements: 10.1 to
+//   22.7 against 10.3 to 24.5; 8 to 14, 283 to 501 CTAs: 40 to 54 against 31 to
+//   44; 24, 799 and 833 CTAs: 64.5 and 65.0 against 67.2 and 67.4
+bool add_early(const ApplyArgs &a, int sms) {
+  if (a.r) return true;
+  if (!a.m) return apply_small(a.elems, sms) || a.ncta > 5 * sms;
+  const int E = a.m->E, N = a.m->N;
+  if (apply_small(E, sms)) return E <= sms / 8 || 3 * N * N * E > 600 * sms;
+  return E / tn_apply_eb(N, false) > 2 * sms;
 }
 template <int N, typename T, int UPD>
 __device__ __forceinline__ void trace_add_cta(const DevMesh &m1, const DevMesh *__restrict__ meshes,
@@ -1012,8 +1022,8 @@ cudaError_t launch_mesh(const ApplyArgs &a, cudaStream_t st) {
 
 template <int N, typename T>
 cudaError_t launch_second(const ApplyArgs &a, cudaStream_t st) {
-  const int E = a.m->E, eb = add_elems(add_eb<N>(), E), grid = (E + eb - 1) / eb;
-  const bool early = add_early(a);
+  const int E = a.m->E, sms = tn_sm_count(), eb = add_elems(add_eb<N>(), E, sms), grid = (E + eb - 1) / eb;
+  const bool early = add_early(a, sms);
   return a.r ? launch_pdl(trace_add_kernel<N, T, 1>, grid, kAddThreads, 0, st, *a.m, E, eb, early, (T *)a.y,
                           (const T *)a.trace, (T *)a.r, a.alpha, a.done)
              : launch_pdl(trace_add_kernel<N, T, 0>, grid, kAddThreads, 0, st, *a.m, E, eb, early, (T *)a.y,
@@ -1023,7 +1033,7 @@ cudaError_t launch_second(const ApplyArgs &a, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_second_batch(const ApplyArgs &a, cudaStream_t st) {
   if (a.nadd <= 0) return cudaSuccess;
-  const bool early = add_early(a);
+  const bool early = add_early(a, tn_sm_count());
   return a.r ? launch_pdl(trace_add_batch_kernel<T, 1>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
                           a.tr_off, a.adds, early, (T *)a.y, (const T *)a.trace, (T *)a.r, a.alpha, a.done)
              : launch_pdl(trace_add_batch_kernel<T, 0>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
@@ -1312,7 +1322,7 @@ int tn_apply_parts(int N, int E) { return apply_small(E) ? E : (E + tn_apply_eb(
 
 int tn_trace_add_eb(int N, int elems) {
   switch (N) {
-#define TN_CASE(NN) case NN: return add_elems(add_eb<NN>(), elems);
+#define TN_CASE(NN) case NN: return add_elems(add_eb<NN>(), elems, tn_sm_count());
     TN_FOR_N(TN_CASE)
 #undef TN_CASE
     default: return 1;
