@@ -1148,10 +1148,11 @@ tn_status tn_apply_operator(tn_ctx *c, int precision, const void *u, void *y) {
   if (a < b + bytes && b < a + bytes) return fail(TN_EINVAL, "u and y overlap");
   // a captured apply takes its traction scratch from the blocks of captures
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  unsigned long long id = 0;
-  cudaGraph_t graph = nullptr;
-  CU_TRY(cudaStreamGetCaptureInfo(c->stream, &cs, &id, &graph, nullptr, nullptr, nullptr), "capture status");
+  CU_TRY(cudaStreamIsCapturing(c->stream, &cs), "capture status");
   if (cs == cudaStreamCaptureStatusActive) {
+    unsigned long long id = 0;
+    cudaGraph_t graph = nullptr;
+    CU_TRY(cudaStreamGetCaptureInfo(c->stream, &cs, &id, &graph, nullptr, nullptr, nullptr), "capture status");
     CU_TRY(cudaSetDevice(c->device), "cudaSetDevice");
     OpSys sys = make_sys(c);
     if (!c->trace_blocks && !(c->trace_blocks = new (std::nothrow) TraceBlocks()))
