@@ -854,11 +854,14 @@ constexpr int kAddThreads = 256;
 template <int N>
 __host__ __device__ constexpr int add_eb() { return kAddThreads * 4 / surf_nodes<N>(); }
 int add_elems(int most, int E, int sms) { return std::min(most, std::max(1, E / (2 * sms))); }
-// Whether the second launch lets the one after it start at once (in a PCG
-// iteration, the preconditioner's: yes).  An apply that starts while the one
-// before still runs takes whatever slots are left: a grid that would spread over
-// the GPU piles up on a few SMs, one that fills it, or leaves most of it empty,
-// gains the start.  us an apply, FP64 / FP32 by itself, early against late:
+// Whether the second launch lets the one after it start at once.  A launch that
+// starts while the operator still runs takes whatever slots are left: a grid that
+// would spread over the GPU piles up on a few SMs, one that fills it, or leaves
+// most of it empty, gains the start.  In a PCG iteration it is the
+// preconditioner's (mixed solves, early against late: 153 elements, p = 7, 58.6
+// against 45.3 ms; 396, p = 5, 49.4 against 47.6; 1944, p = 6, 200 against 207;
+// FP64, 8 elements, p = 3, 1.87 against 1.92), else the next apply (us an apply,
+// FP64 / FP32):
 //   one element per CTA: 216 elements, p = 4: 56 / 7.0 against 25 / 7.2; 343 to
 //   512, p = 2, 3: 42 to 59 against 16 to 27; 8, p = 2: 14.6 against 15.6; 729,
 //   p = 8 (1165 threads per SM): 252.5 / 21.2 against 253.3 / 22.1
@@ -868,9 +871,10 @@ int add_elems(int most, int E, int sms) { return std::min(most, std::max(1, E / 
 //   22.7 against 10.3 to 24.5; 8 to 14, 283 to 501 CTAs: 40 to 54 against 31 to
 //   44; 24, 799 and 833 CTAs: 64.5 and 65.0 against 67.2 and 67.4
 bool add_early(const ApplyArgs &a, int sms) {
-  if (a.r) return true;
-  if (!a.m) return apply_small(a.elems, sms) || a.ncta > 5 * sms;
-  const int E = a.m->E, N = a.m->N;
+  const int E = a.m ? a.m->E : a.elems;
+  if (a.r) return !apply_small(E, sms) || E <= sms / 8;
+  if (!a.m) return apply_small(E, sms) || a.ncta > 5 * sms;
+  const int N = a.m->N;
   if (apply_small(E, sms)) return E <= sms / 8 || 3 * N * N * E > 600 * sms;
   return E / tn_apply_eb(N, false) > 2 * sms;
 }
