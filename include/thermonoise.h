@@ -190,9 +190,11 @@ tn_status tn_diagonal(tn_ctx *ctx, double *d_dev);
  * the interior-penalty and flux coupling across the vertical element faces
  * (Eqs. (numflux), (penalty)) that single lines leave out; TN_EINVAL if a
  * node is shared by more than 4 columns.  The first call after
- * tn_build_mesh / tn_set_materials builds the factors (FP64 set-up, about
- * (3 g N)^2 / 2 + 3 g N (8 + 6 g) FP32 and FP64 entries per group of g
- * lines and slab).
+ * tn_build_mesh / tn_set_materials builds the factors in FP64 and keeps, with
+ * M = 3 g N unknowns of a group of g lines and one slab, about
+ * M^2 / 2 + M (8 + 6 g) FP32 and M^2 / 2 + 12 g M + 72 g^2 + 16 g FP64 entries
+ * per group and slab, and 12 g FP64 numbers of solve scratch (2.0 M unknowns,
+ * p = 6: 0.29 and 0.72 GB, and 0.01).
  * precision TN_F64 / TN_F32 selects double / float vectors r, z
  * (caller-owned device buffers of tn_ndof() values, 16-byte aligned, not
  * overlapping). */
@@ -316,8 +318,8 @@ tn_status tn_energy_grad(tn_ctx *ctx, const tn_solve_opts *opts, const double *u
  *     above); tn_batch_offsets gives the first unknown and the first layer of
  *     every mirror (n + 1 entries each) and tn_ndof the total;
  *   - tn_apply_operator applies the block-diagonal operator of all mirrors:
- *     one launch per polynomial degree present, each CTA working on one
- *     element of one mirror;
+ *     neighbouring degrees of one occupancy variant in one launch, each CTA
+ *     working on elements of one degree, then one launch for the traces;
  *   - tn_precond_apply (TN_PC_ZLINE, TN_PC_ZGROUP) and tn_solve solve all mirrors at
  *     once (one Krylov iteration serves every mirror; the energy test covers
  *     every layer of every mirror);

@@ -573,8 +573,8 @@ static tn_status ensure_zgroup(tn_ctx *c, cudaStream_t st) {
     dfree(blk); dfree(xblk);
     free_zgroup(c);
     cudaGetLastError();
-    return fail(TN_ENOMEM, "grouped-line preconditioner needs %.2f GB: %s", (bb + xb + fb + fb64) / 1e9,
-                cudaGetErrorString(e));
+    return fail(TN_ENOMEM, "grouped-line preconditioner needs %.2f GB: %s",
+                (bb + xb + fb + fb64 + sizeof(double) * (size_t)p.nchain) / 1e9, cudaGetErrorString(e));
   }
   ZGroupDev &g = c->zgd;
   for (int k = 0; k < kZgSide && e == cudaSuccess; ++k) {
