@@ -60,13 +60,12 @@ def fp32_apply_flops_per_dof(N):
 # from `ncu --set full -k regex:zgroup_packed_kernel` of `bench.py --mode
 # apply --workload single_coating`; absent where no capture of the current
 # kernel exists
-ZLINE_TRAFFIC = {("single_coating", "zgroup_packed_kernel<7>"): 342619136.0 + 10593280.0}
+ZLINE_TRAFFIC = {("single_coating", "zgroup_packed_kernel<7>"): 342965760.0 + 9518336.0}
 
 
-# DRAM bytes (read + write) of one FP32 apply (both launches), from ncu on the
-# single-coating mesh (variant 1 captured; the variants move the same bytes)
-APPLY_TRAFFIC = {("single_coating", f"apply_elem_kernel<7,float,{v}> + trace_add_kernel<7,float>"): 22863872.0
-                 for v in (0, 1)}
+# DRAM bytes (read + write) of one FP32 apply (both launches), from captures of
+# the same command; absent where no capture of the variant exists
+APPLY_TRAFFIC = {("single_coating", "apply_elem_kernel<7,float,0> + trace_add_kernel<7,float>"): 8209664.0 + 14674176.0}
 
 
 def measured_peaks():

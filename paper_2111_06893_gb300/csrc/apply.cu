@@ -27,10 +27,9 @@
 // D[N-1-a][N-1-b] = -D[a][b]: on the even and odd parts of a line they need
 // about half the multiplications (36 instead of 49 operations at N = 7).
 //
-// Bound: neither HBM nor the FMA pipe.  FP32 (2.0 M unknowns, p = 6): 7.9 M
-// warp instructions, of which 2.1 M shared or global accesses, against 43.6 M
-// of the form that rebuilt the neighbours' tractions; 17 + 6 us for the two
-// launches (51 us before).  59 M unknowns, p = 8: 335 + 108 us (1420 us).
+// Bound: neither HBM nor the FMA pipe.  FP32 (2.0 M unknowns, p = 6): 7.3 + 2.4 M
+// warp instructions against 43.6 M of the form that rebuilt the neighbours'
+// tractions; 17 + 7 us for the two launches (51 us before).  59 M unknowns, p = 8: 335 + 108 us (1420 us).
 // FP64 is bound by its pipe (two FMAs per clock and SM): 8.0 M unknowns,
 // p = 5: 1.10 ms (3.11 ms), about 65 FP64 operations per unknown (204).
 // The second launch starts while the first drains (its reads of the mesh
@@ -724,7 +723,7 @@ __device__ void fold_alpha(const PcgFold &f) {
 // FP32: variant 0 asks for three CTAs per SM (80 registers, some spilled at N
 // = 9), variant 1 for two (up to 128).  Both round alike (bit-identical
 // results); the autotuner times them on the mesh at hand (p = 6, 2.0 M
-// unknowns: 24.3 / 25.2 us; p = 8, 59 M: 547 / 451 us).
+// unknowns: 25.3 / 26.4 us; p = 8, 59 M: 578 / 454 us).
 template <typename T, int V>
 __host__ __device__ constexpr int apply_min_blocks() { return sizeof(T) == 8 ? 1 : (V == 0 ? 3 : 2); }
 

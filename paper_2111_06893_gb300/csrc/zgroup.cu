@@ -473,8 +473,8 @@ zgroup_packed_kernel(const DevMesh m1, const int *__restrict__ ginst, const DevM
 //   zg_chain_kernel  the two chains g and f of every group
 //   zg_final_kernel  x_s = a_s - Q_s g_{s-1} - W_s f_{s+1}, r.z and r.r, again
 //                    every slab on its own
-// All three are bound by the FP64 pipe (78, 80 and 88 % busy; 187 + 105 + 97 us
-// at 2.0 M unknowns, p = 6).  Loading the last launch's factors by bulk copies
+// All three are bound by the FP64 pipe (79, 65 and 88 % busy; 189 + 107 + 100 us
+// at 2.0 M unknowns, p = 6), the chains also by their dependent steps.  Loading the last launch's factors by bulk copies
 // through a ring, as the first does, was slower (441 against 383 us in all:
 // fewer CTAs per SM).
 // `chain` holds 12 g numbers per slab: c_s, then g_s; d_s, then f_s.
