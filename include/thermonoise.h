@@ -157,7 +157,8 @@ tn_status tn_apply_operator(tn_ctx *ctx, int precision, const void *u_dev, void 
  * of each, CUDA events on the
  * stream of the call, not while it is being captured; the call's y, or the
  * solver's FP32 workspace, is overwritten meanwhile) and keeps variant 1
- * only when it is faster by more than 2 %.
+ * only when it is faster by more than 2 %: a batch for all the degrees it times
+ * or none, by their sums, as degrees share a launch with one variant only.
  * tn_apply_tuning: variant[p - 2] for p = 2..8 is 0 or 1 once settled, -1
  * before; us (may be NULL) receives 14 doubles, the time per apply in
  * microseconds of variants 0 and 1 for each degree (0 where not timed).

@@ -723,19 +723,29 @@ static OpSys make_sys(const tn_ctx *c) {
 // Autotuner of the FP32 operator kernel: for every LGL count of the context
 // (the mesh, or each degree group of a batch) not yet settled, times both
 // occupancy variants on the vectors u -> y (y is overwritten) and keeps
-// variant 1 only when it is faster by more than 2 %.  Not called while st is
-// being captured into a graph.
+// variant 1 only when it is faster by more than 2 %, for a batch over all its
+// degrees timed: they share a launch only with one variant (24 mirrors: 57 us
+// with either throughout; each degree's own choice, 0 | 1 1 1 | 0 in three
+// launches, 72).  Not called while st is being captured into a graph.
 static tn_status ensure_tuned(tn_ctx *c, const float *u, float *y, cudaStream_t st) {
   const OpSys s = make_sys(c);
+  bool timed[10] = {false};
+  float sum[2] = {0.0f, 0.0f};
   for (int g = 0; g < (s.m ? 1 : s.ngroups); ++g) {
     const ApplyArgs a = s.args(g, g + 1, TN_F32, u, y);
     const int N = s.m ? s.m->N : s.gN[g];
     if (c->apply_set[N]) continue;
     float us[2] = {0.0f, 0.0f};
     CU_TRY(tn_tune_apply(a, st, us), "tuning");
-    c->apply_us[N][0] = us[0];
-    c->apply_us[N][1] = us[1];
-    c->apply_var[N] = us[1] < 0.98f * us[0] ? 1 : 0;
+    for (int v = 0; v < 2; ++v) {
+      c->apply_us[N][v] = us[v];
+      sum[v] += us[v];
+    }
+    timed[N] = true;
+  }
+  for (int N = 0; N < 10; ++N) {
+    if (!timed[N]) continue;
+    c->apply_var[N] = sum[1] < 0.98f * sum[0] ? 1 : 0;
     c->apply_set[N] = true;
   }
   return TN_OK;

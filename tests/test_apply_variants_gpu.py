@@ -75,3 +75,23 @@ def test_variants_of_a_large_batch_bit_identical():
     for i in range(len(descs)):
         a, b = (v[bc.dof_off[i]:bc.dof_off[i + 1]].double() for v in (ys[0], y64))
         assert float((a - b).abs().max() / b.abs().max()) < 2e-5, i
+
+
+def test_tuner_settles_a_batch_on_one_variant():
+    """By the sums over the degrees it times; a degree the caller has fixed
+    keeps its variant and is not timed."""
+    from paper_2111_06893_gb300 import thermonoise
+    descs = [W.sweep_instance(i) for i in range(40)]
+    for fixed in (None, 6):
+        bc = thermonoise.Context().build_batch(descs)
+        if fixed:
+            bc.set_apply_variant(fixed, 1)
+        bc.apply_operator(field(bc.ndof, torch.float32, seed=2))
+        t = bc.apply_tuning()
+        assert set(t) == {d["degree"] for d in descs} and len(t) == 5
+        timed = [v for p, v in t.items() if p != fixed]
+        us0, us1 = (sum(v["us"][i] for v in timed) for i in (0, 1))
+        assert us0 > 0 and us1 > 0
+        assert {v["variant"] for v in timed} == {1 if us1 < 0.98 * us0 else 0}
+        if fixed:
+            assert t[fixed] == {"variant": 1, "us": [0.0, 0.0]}
