@@ -866,13 +866,13 @@ int add_elems(int most, int E, int sms) { return std::min(most, std::max(1, E / 
 //   p = 8 (1165 threads per SM): 252.5 / 21.2 against 253.3 / 22.1
 //   pencils: 98 CTAs (p = 2, 2744 elements) 54.2 / 14.0 against 53.7 / 9.1; 275
 //   CTAs, p = 4: 164.7 / 20.6 against 165.6 / 19.4; 389, p = 6: 24.9 against 26.2
-//   batches (FP32, means over placements): 2 to 6 mirrors, few elements: 10.1 to
-//   22.7 against 10.3 to 24.5; 8 to 14, 283 to 501 CTAs: 40 to 54 against 31 to
-//   44; 24, 799 and 833 CTAs: 64.5 and 65.0 against 67.2 and 67.4
+//   batches, whose CTAs work on several elements each: FP32, 2 mirrors 10.1
+//   against 10.4, 6 22.7 against 24.5, 10 32.7 against 34.3, 24 52.7 against 55.3;
+//   FP64, 2 52.1 against 53.6, 24 726.9 against 730.5
 bool add_early(const ApplyArgs &a, int sms) {
   const int E = a.m ? a.m->E : a.elems;
   if (a.r) return !apply_small(E, sms) || E <= sms / 8;
-  if (!a.m) return apply_small(E, sms) || a.ncta > 5 * sms;
+  if (!a.m) return true;
   const int N = a.m->N;
   if (apply_small(E, sms)) return E <= sms / 8 || 3 * N * N * E > 600 * sms;
   return E / tn_apply_eb(N, false) > 2 * sms;
