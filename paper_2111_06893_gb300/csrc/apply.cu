@@ -864,8 +864,9 @@ int add_elems(int most, int E, int sms) { return std::min(most, std::max(1, E / 
 //   one element per CTA: 216 elements, p = 4: 56 / 7.0 against 25 / 7.2; 343 to
 //   512, p = 2, 3: 42 to 59 against 16 to 27; 8, p = 2: 14.6 against 15.6; 729,
 //   p = 8 (1165 threads per SM): 252.5 / 21.2 against 253.3 / 22.1
-//   pencils: 98 CTAs (p = 2, 2744 elements) 54.2 / 14.0 against 53.7 / 9.1; 275
-//   CTAs, p = 4: 164.7 / 20.6 against 165.6 / 19.4; 389, p = 6: 24.9 against 26.2
+//   pencils, FP32: 83 CTAs (p = 2, 2304 elements) 10.3 against 8.9; 140, p = 4,
+//   14.2 against 11.5; 180, p = 3, 11.5 against 12.3; 280, p = 6, 19.3 against 20.2;
+//   389, p = 6, 24.9 against 26.2 (not 288, p = 4: 20.7 against 19.3)
 //   batches, whose CTAs work on several elements each: FP32, 2 mirrors 10.1
 //   against 10.4, 6 22.7 against 24.5, 10 32.7 against 34.3, 24 52.7 against 55.3;
 //   FP64, 2 52.1 against 53.6, 24 726.9 against 730.5
@@ -875,8 +876,9 @@ bool add_early(const ApplyArgs &a, int sms) {
   if (!a.m) return true;
   const int N = a.m->N;
   if (apply_small(E, sms)) return E <= sms / 8 || 3 * N * N * E > 600 * sms;
-  return E / tn_apply_eb(N, false) > 2 * sms;
+  return E / tn_apply_eb(N, false) > sms;
 }
+
 template <int N, typename T, int UPD>
 __device__ __forceinline__ void trace_add_cta(const DevMesh &m1, const DevMesh *__restrict__ meshes,
                                               const int2 *__restrict__ work, const long long *__restrict__ dof_off,
