@@ -870,8 +870,8 @@ int add_elems(int most, int E, int sms) { return std::min(most, std::max(1, E / 
 //   batches, whose CTAs work on several elements each: FP32, 2 mirrors 10.1
 //   against 10.4, 6 22.7 against 24.5, 10 32.7 against 34.3, 24 52.7 against 55.3;
 //   FP64, 2 52.1 against 53.6, 24 726.9 against 730.5
-bool add_early(const ApplyArgs &a, int sms) {
-  const int E = a.m ? a.m->E : a.elems;
+bool add_early(const ApplyArgs &a) {
+  const int E = a.m ? a.m->E : a.elems, sms = a.sms;
   if (a.r) return !apply_small(E, sms) || E <= sms / 8;
   if (!a.m) return true;
   const int N = a.m->N;
@@ -1022,13 +1022,13 @@ cudaError_t launch_elem(const ApplyArgs &a, cudaStream_t st) {
 
 template <int N, typename T, int V>
 cudaError_t launch_mesh(const ApplyArgs &a, cudaStream_t st) {
-  return apply_small(a.m->E) ? launch_elem<N, T, 0, AM_SMALL>(a, st) : launch_elem<N, T, V, AM_PENCIL>(a, st);
+  return apply_small(a.m->E, a.sms) ? launch_elem<N, T, 0, AM_SMALL>(a, st) : launch_elem<N, T, V, AM_PENCIL>(a, st);
 }
 
 template <int N, typename T>
 cudaError_t launch_second(const ApplyArgs &a, cudaStream_t st) {
-  const int E = a.m->E, sms = tn_sm_count(), eb = add_elems(add_eb<N>(), E, sms), grid = (E + eb - 1) / eb;
-  const bool early = add_early(a, sms);
+  const int E = a.m->E, eb = add_elems(add_eb<N>(), E, a.sms), grid = (E + eb - 1) / eb;
+  const bool early = add_early(a);
   return a.r ? launch_pdl(trace_add_kernel<N, T, 1>, grid, kAddThreads, 0, st, *a.m, E, eb, early, (T *)a.y,
                           (const T *)a.trace, (T *)a.r, a.alpha, a.done)
              : launch_pdl(trace_add_kernel<N, T, 0>, grid, kAddThreads, 0, st, *a.m, E, eb, early, (T *)a.y,
@@ -1038,7 +1038,7 @@ cudaError_t launch_second(const ApplyArgs &a, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_second_batch(const ApplyArgs &a, cudaStream_t st) {
   if (a.nadd <= 0) return cudaSuccess;
-  const bool early = add_early(a, tn_sm_count());
+  const bool early = add_early(a);
   return a.r ? launch_pdl(trace_add_batch_kernel<T, 1>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
                           a.tr_off, a.adds, early, (T *)a.y, (const T *)a.trace, (T *)a.r, a.alpha, a.done)
              : launch_pdl(trace_add_batch_kernel<T, 0>, a.nadd, kAddThreads, 0, st, a.meshes, a.work, a.dof_off,
@@ -1294,7 +1294,7 @@ cudaError_t tn_upload_lgl_apply(const LglTables *t) {
 // variant 1 exists for FP32 only
 cudaError_t tn_launch_apply(const ApplyArgs &a, cudaStream_t st) {
   if (!a.m) {
-    if (tn_apply_few(a.elems))
+    if (apply_small(a.elems, a.sms))
       return a.prec == TN_F64 ? launch_batch<double, 0, AM_SMALL_BATCH>(a, st) : launch_batch<float, 0, AM_SMALL_BATCH>(a, st);
     if (a.prec == TN_F64) return launch_batch<double, 0, AM_PENCIL>(a, st);
     return a.var == 1 ? launch_batch<float, 1, AM_PENCIL>(a, st) : launch_batch<float, 0, AM_PENCIL>(a, st);

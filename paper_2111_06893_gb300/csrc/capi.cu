@@ -263,6 +263,7 @@ struct TraceBlocks {
 
 struct tn_ctx {
   int device = 0;
+  int sms = 0;  // its SMs
   Batch *batch = nullptr;
   cudaStream_t stream = nullptr;   // the caller's stream
   cudaStream_t sstream = nullptr;  // internal stream used for graph capture
@@ -717,6 +718,7 @@ static OpSys make_sys(const tn_ctx *c) {
   }
   s.zerr = c->wctl;
   s.trace = c->trace;
+  s.sms = c->sms;
   return s;
 }
 
@@ -791,6 +793,7 @@ tn_status tn_create(tn_ctx **out, int device, void *cuda_stream) {
   tn_ctx *c = new (std::nothrow) tn_ctx();
   if (!c) return fail(TN_ENOMEM, "host allocation failed");
   c->device = device;
+  c->sms = tn_sm_count();
   c->stream = (cudaStream_t)cuda_stream;
   cudaError_t e = cudaStreamCreateWithFlags(&c->sstream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming);

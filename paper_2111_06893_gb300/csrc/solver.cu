@@ -652,6 +652,7 @@ ApplyArgs OpSys::args(int g0, int g1, int prec, const void *u, void *y) const {
   a.u = u;
   a.y = y;
   a.trace = trace;
+  a.sms = sms;
   if (m) {
     a.var = mvar;
     return a;

@@ -188,6 +188,7 @@ struct ApplyArgs {
   const int4 *ctas = nullptr, *adds = nullptr;  // batch: CTAs of the apply and of tn_launch_trace_add
   int ncta = 0, nadd = 0;
   int elems = 0;                    // batch: all its elements (the forms taken depend on them)
+  int sms = 0;                      // SMs of the device
   int prec = TN_F64, var = 0;       // var: occupancy variant of the FP32 kernel (0 or 1, same results)
   const void *u = nullptr;
   void *y = nullptr, *trace = nullptr;  // trace: tn_trace_entries per element, of the vectors' precision

@@ -28,6 +28,7 @@ struct OpSys {
   void *trace = nullptr;  // traction scratch of the operator (FP64-sized; FP32 applies use half of it)
   const long long *tr_off = nullptr;  // batch: first trace entry of every mirror
   int n_elems = 0;        // elements of the mesh or of the whole batch
+  int sms = 0;            // SMs of the device
   int n_rz_parts = 0;     // single lines: partial sums of r.z written by one solve (r.r: as many, after them)
   int rz_parts(int prec) const { return grouped ? tn_zgroup_partials(zg, prec) : n_rz_parts; }
   TnWait *zerr = nullptr; // wait limit of the line solves; flag set by one whose staging wait ran out
